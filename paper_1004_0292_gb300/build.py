@@ -40,7 +40,7 @@ def _up_to_date(extra_flags) -> bool:
     if not os.path.exists(stamp) or open(stamp).read() != " ".join(extra_flags):
         return False
     t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(SRC, "*.h")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+    deps = sources() + glob.glob(os.path.join(SRC, "*.h")) + glob.glob(os.path.join(SRC, "*.cuh")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
     return all(os.path.getmtime(d) <= t for d in deps)
 
 

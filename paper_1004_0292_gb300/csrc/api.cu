@@ -127,6 +127,7 @@ extern "C" int ssqcd_upload_gauge(ssqcd_lattice lat, const double* links, int on
     user = lat->stage.as<double2>();
   }
   SS_TRY(pack_gauge64(user, lat->u64.as<double2>(), V, lat->stream));
+  SS_TRY(build_fix_links(lat));
   if (lat->precision == SSQCD_MIXED) {
     SS_TRY(lat->u16.alloc(sizeof(uint2) * 12 * (size_t)V));
     SS_TRY(pack_gauge16(lat->u64.as<double2>(), lat->u16.p, V, lat->stream));
@@ -151,18 +152,35 @@ int ssqcd::ensure_df_links(ssqcd_lattice lat) {
   return SSQCD_OK;
 }
 
+namespace {
+
+// out = A in in the caller's layout, host or device
+int apply_user(ssqcd_lattice lat, const double* in, double* out, int nrhs, int on_device) {
+  const double2* src = reinterpret_cast<const double2*>(in);
+  double2* dst = reinterpret_cast<double2*>(out);
+  AllocStream scope(lat->stream);
+  DevBuf a, b;
+  const size_t bytes = sizeof(double2) * 12 * (size_t)lat->g.V * nrhs;
+  if (!on_device) {
+    SS_TRY(a.alloc(bytes));
+    SS_TRY(b.alloc(bytes));
+    SS_CUDA(cudaMemcpyAsync(a.p, in, bytes, cudaMemcpyHostToDevice, lat->stream));
+    src = a.as<double2>();
+    dst = b.as<double2>();
+  }
+  SS_TRY(wilson64_lat(lat, src, true, dst, nrhs, lat->stream));
+  if (!on_device) SS_CUDA(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, lat->stream));
+  SS_CUDA(cudaStreamSynchronize(lat->stream));
+  return SSQCD_OK;
+}
+
+}  // namespace
+
 extern "C" int ssqcd_apply_H(ssqcd_lattice lat, const double* in, double* out, int nrhs, int on_device) {
   SS_TRY(check_lattice(lat, true));
   if (nrhs < 0 || (nrhs > 0 && (in == nullptr || out == nullptr))) return fail(SSQCD_ERR_ARG, "bad apply_H arguments");
   if (nrhs == 0) return SSQCD_OK;
-  DevBuf a, b;
-  SS_TRY(to_device_layout(lat, in, nrhs, on_device, a));
-  SS_TRY(b.alloc(a.bytes));
-  SS_TRY(wilson64(lat->g, lat->u64.as<double2>(), a.as<double2>(), b.as<double2>(), nrhs, 0.0, 1.0, nullptr,
-                  nullptr, lat->stream));
-  SS_TRY(from_device_layout(lat, b.as<double2>(), nrhs, on_device, out));
-  SS_CUDA(cudaStreamSynchronize(lat->stream));
-  return SSQCD_OK;
+  return apply_user(lat, in, out, nrhs, on_device);
 }
 
 extern "C" int ssqcd_apply_H_mixed(ssqcd_lattice lat, const double* in, double* out, int nrhs, int on_device) {
@@ -349,8 +367,7 @@ int finish_ritz(ssqcd_lattice lat, const DevBuf& X, const std::vector<double>& e
   std::vector<double> rs(cnt);
   DevBuf AX, th, rn;
   SS_TRY(AX.alloc(sizeof(double2) * n * cnt));
-  SS_TRY(wilson64(lat->g, lat->u64.as<double2>(), X.as<double2>(), AX.as<double2>(), cnt, 0.0, 1.0, nullptr,
-                  nullptr, st));
+  SS_TRY(wilson64_lat(lat, X.as<double2>(), false, AX.as<double2>(), cnt, st));
   SS_TRY(th.alloc(sizeof(double) * cnt));
   SS_TRY(rn.alloc(sizeof(double) * cnt));
   SS_CUDA(cudaMemcpyAsync(th.p, ev.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice, st));
@@ -404,8 +421,7 @@ int rayleigh_ritz_projected(ssqcd_lattice lat, const double2* S, int m, double r
     SS_TRY(wilson_df(lat->g, lat->udf.as<float4>(), T.as<float4>(), AT.as<float4>(), m, 0.0, 1.0, st));
     SS_TRY(gram_df(T.as<float4>(), m, AT.as<float4>(), m, n, Gd.as<double2>(), gs, st, true));
   } else {
-    SS_TRY(wilson64(lat->g, lat->u64.as<double2>(), T.as<double2>(), AT.as<double2>(), m, 0.0, 1.0, nullptr,
-                    nullptr, st));
+    SS_TRY(wilson64_lat(lat, T.as<double2>(), false, AT.as<double2>(), m, st));
     SS_TRY(gram(T.as<double2>(), m, AT.as<double2>(), m, n, Gd.as<double2>(), gs, st, true));
   }
   // (a copy to pageable host memory returns when it is complete: R is
@@ -492,8 +508,7 @@ int rayleigh_ritz_window(ssqcd_lattice lat, const double2* S, int m, double rank
   tmp.release();
   rank = r;
   SS_TRY(AQ.alloc(sizeof(double2) * n * r));
-  SS_TRY(wilson64(lat->g, lat->u64.as<double2>(), Q.as<double2>(), AQ.as<double2>(), r, 0.0, 1.0, nullptr, nullptr,
-                  st));
+  SS_TRY(wilson64_lat(lat, Q.as<double2>(), false, AQ.as<double2>(), r, st));
   SS_TRY(Gd.alloc(sizeof(double2) * r * r));
   SS_TRY(gram(Q.as<double2>(), r, AQ.as<double2>(), r, n, Gd.as<double2>(), scratch, st));
   std::vector<double2> At((size_t)r * r), W((size_t)r * r);
@@ -598,8 +613,7 @@ int rayleigh_ritz_window(ssqcd_lattice lat, const double2* S, int m, double rank
   SS_TRY(X.alloc(sizeof(double2) * n * cnt));
   SS_TRY(combine(Q.as<double2>(), r, n, Wd.as<double2>(), cnt, X.as<double2>(), st));
   SS_TRY(AX.alloc(sizeof(double2) * n * cnt));
-  SS_TRY(wilson64(lat->g, lat->u64.as<double2>(), X.as<double2>(), AX.as<double2>(), cnt, 0.0, 1.0, nullptr,
-                  nullptr, st));
+  SS_TRY(wilson64_lat(lat, X.as<double2>(), false, AX.as<double2>(), cnt, st));
   SS_TRY(th.alloc(sizeof(double) * cnt));
   SS_TRY(rn.alloc(sizeof(double) * cnt));
   SS_CUDA(cudaMemcpyAsync(th.p, ev.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice, st));
@@ -1631,6 +1645,12 @@ int server_enqueue(ssqcd_server srv, ssqcd_lattice lat, std::unique_ptr<ServerRe
   r->basis_cap = request_basis_cap(lat, Pb, srv->budget);
   r->est_bytes = estimate_request_bytes(lat, Pb, r->basis_cap);
   if (r->B < L) r->est_bytes += sizeof(double2) * 12 * (size_t)lat->g.V * r->P.MM * L * r->P.K;
+  // the digits of the seed direction (integer stencil), where the budget has
+  // room for them: a request that fits without them still runs
+  const size_t digits = lat->fix_ok && !is_mixed(lat->precision)
+                            ? (fix_field_bytes(lat->g.V) + fix_exp_bytes(lat->g.V)) * (size_t)r->B
+                            : 0;
+  if (r->est_bytes + digits <= srv->budget) r->est_bytes += digits;
   if (r->est_bytes > srv->budget)
     return fail(SSQCD_ERR_OOM, "request needs more device memory than the server budget");
   const size_t nd = 2ull * 12 * lat->g.V * L;  // doubles
@@ -1869,8 +1889,7 @@ extern "C" int ssqcd_time_stencil(ssqcd_lattice lat, int nrhs, int reps, double*
                                   b.as<float2>(), nrhs, 0.f, 1.f, st);
     }
     if (df) return wilson_df(lat->g, lat->udf.as<float4>(), a.as<float4>(), b.as<float4>(), nrhs, 0.0, 1.0, st);
-    return wilson64(lat->g, lat->u64.as<double2>(), a.as<double2>(), b.as<double2>(), nrhs, 0.0, 1.0, nullptr,
-                    nullptr, st);
+    return wilson64_lat(lat, a.as<double2>(), false, b.as<double2>(), nrhs, st);
   };
   for (int i = 0; i < 2; ++i) SS_TRY(once());
   cudaEvent_t e0, e1;

@@ -108,6 +108,9 @@ struct ssqcd_lattice_s {
   ssqcd::DevBuf u16;     // FP16 12-parameter links, SSQCD_MIXED only
   ssqcd::DevBuf u32;     // FP32 12-parameter links, SSQCD_MIXED_F32LINKS only
   ssqcd::DevBuf udf;     // float-float links [4][9][V] float4, built on first SSQCD_DF use
+  ssqcd::DevBuf ufix;    // links as 60-bit integers (wilson_fix.cuh), when fix_ok
+  ssqcd::DevBuf fnbr;    // its neighbour table
+  bool fix_ok = false;   // the links have unit rows and columns: the integer stencil serves the lattice
   int gauge_version = 0; // bumped by every upload
   int udf_version = -1;  // gauge_version udf was built from
   ssqcd::DevBuf stage;   // staging for host <-> device copies
@@ -132,6 +135,19 @@ int pack_gauge64(const double2* user, double2* dev, int V, cudaStream_t s);
 int wilson_blocks(const Geometry& g);
 int wilson64(const Geometry& g, const double2* u, const double2* in, double2* out, int nrhs,
              double c0, double c1, double* dot_partial, const int* skip_if_zero, cudaStream_t s);
+// out = A in through the form that suits the lattice: the integer stencil
+// (wilson_fix.cu) where its links allow it, else wilson64.  user: in and out
+// are in the caller's layout [nrhs][V][12], else [nrhs][12][V].
+int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s);
+// Integer stencil (wilson_fix.cu): fields as digits with one exponent a site,
+// bytes of each for one field; the links take three fields' bytes
+size_t fix_field_bytes(int V);
+size_t fix_exp_bytes(int V);
+int pack_fix(const double2* in, bool user, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
+int fix_split(int V, int nrhs);  // warps that share the hops of 16 sites: 1, 4 or 8
+int fix_block(int V, int nrhs);  // right-hand sides converted at a time
+// digits of the uploaded links (sets ufix, fix_ok)
+int build_fix_links(ssqcd_lattice lat);
 // link_bits 16: FP16 12-parameter links [4][3][V] uint2; 32: FP32 [4][3][V] float4
 int wilson32(const Geometry& g, const void* links, int link_bits, const float2* in, float2* out, int nrhs,
              float c0, float c1, float* dot_partial, const int* skip_if_zero, cudaStream_t s);

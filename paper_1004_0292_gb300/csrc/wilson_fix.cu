@@ -1,0 +1,354 @@
+// Stand-alone application of A = gamma5 (I - kappa D) to FP64 fields with the
+// integer stencil (wilson_fix.cuh), its link and spinor conversions, and the
+// choice between it and the FP64-pipe kernel (wilson.cu).
+#include <algorithm>
+
+#include "wilson_fix.cuh"
+
+namespace ssqcd {
+namespace {
+
+using namespace wfix;
+
+// FP64 links [4][9][V] -> digits; *bad is set when a link's rows or columns
+// are not of unit length to 2^-10 (the bounds of the integer sums, and their
+// accuracy, rest on it; every SU(3) field passes) or not finite: such a field
+// keeps the FP64 kernel.
+__global__ void pack_links_fix_kernel(const double2* __restrict__ u, int4* __restrict__ uf, int V, int* bad) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= 4LL * V) return;
+  const int mu = (int)(i / V), s = (int)(i % V);
+  double row[3] = {0.0, 0.0, 0.0}, col[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const double2 z = u[(size_t)(mu * 9 + e) * V + s];
+    const double n2 = z.x * z.x + z.y * z.y;
+    row[e / 3] += n2;
+    col[e % 3] += n2;
+    const long long xr = __double2ll_rn(z.x * 0x1p59) + (1ll << 29), xi = __double2ll_rn(z.y * 0x1p59) + (1ll << 29);
+    uf[link_at(fix_tiles(V), mu, s) + e * kTile] =
+        make_int4((int)(xr >> 30), (int)((unsigned)xr & 0x3fffffffu) - (1 << 29), (int)(xi >> 30),
+                  (int)((unsigned)xi & 0x3fffffffu) - (1 << 29));
+  }
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    ok = ok && fabs(row[k] - 1.0) <= 0x1p-10 && fabs(col[k] - 1.0) <= 0x1p-10;  // false for NaN
+  if (!ok) *bad = 1;
+}
+
+__global__ void neighbour_table_kernel(Geometry g, int* __restrict__ nbr) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int k = (int)(t / g.V), s = (int)(t % g.V);
+  if (k >= 8) return;
+  const wcore::Coords c = wcore::site_coords(s, g);
+  bool tw;
+  const int nb = k & 1 ? neighbour_rt<true>(s, c, g, k >> 1, tw) : neighbour_rt<false>(s, c, g, k >> 1, tw);
+  nbr[(size_t)(s >> 4) * (8 * kTile) + k * kTile + (s & 15)] = nb | (tw && g.bc_t < 0 ? kNegBit : 0);
+}
+
+// Fields to digits: four lanes a site (spin q), eight sites a warp.  USER: in
+// is [f][V][12] (the caller's layout), else [f][12][V].  Bound by memory: 16 B
+// read and 16 B written a component.
+template <bool USER>
+__global__ void __launch_bounds__(256)
+pack_fix_kernel(const double2* __restrict__ in, int4* __restrict__ dig, int* __restrict__ ex, int V) {
+  const int lane = threadIdx.x & 31, q = lane >> 3;
+  const int s = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 8 + (lane & 7);
+  const size_t f = blockIdx.y;
+  double2 v[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    v[a] = s >= V ? make_double2(0.0, 0.0)
+                  : USER ? __ldg(in + (f * V + s) * 12 + 3 * q + a) : __ldg(in + (f * 12 + 3 * q + a) * V + s);
+  const int e = quad_site_exp(v);
+  if (s >= V) return;
+  const int tiles = fix_tiles(V);
+  if (q == 0) ex[f * tiles * kTile + s] = e;
+  const int exmax = e + 1022;
+  const bool none = e == kZeroExp || e == kSpecialExp;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    dig[field_at(tiles, f, s) + (3 * q + a) * kTile] = none ? make_int4(0, 0, 0, 0) : to_digits(v[a], exmax);
+}
+
+// (D psi)(s), component comp, in FP64 from the links and the field as they
+// are: the sites next to a value the digits cannot hold (above 2^800, not
+// finite).  The sums are those of the FP64 kernel up to their order.
+template <bool USER>
+__device__ __noinline__ double2 hop_sum_fp64(const Geometry& g, const double2* __restrict__ u,
+                                             const double2* __restrict__ in, size_t f, int s, int comp) {
+  const int V = g.V;
+  const wcore::Coords c = wcore::site_coords(s, g);
+  const int spin = comp / 3, a = comp % 3;
+  double2 sum = make_double2(0.0, 0.0);
+  for (int hop = 0; hop < 8; ++hop) {
+    const int mu = hop >> 1;
+    const bool back = (hop & 1) != 0;
+    bool tw;
+    const int nb = back ? neighbour_rt<true>(s, c, g, mu, tw) : neighbour_rt<false>(s, c, g, mu, tw);
+    const bool neg = tw && g.bc_t < 0;
+    // the row of the half spinor this output takes, and the unit in front
+    const int r = spin < 2 ? spin : (mu < 2 ? 3 - spin : spin - 2);
+    const int lr = mu < 2 ? 1 - r : r;
+    const bool swap = (mu & 1) == 0;
+    const int sb = (mu == 1 && r == 0) || (mu == 2 && r == 1) ? -1 : 1;
+    const int sp = back ? sb : -sb;
+    double2 t = make_double2(0.0, 0.0);
+    for (int b = 0; b < 3; ++b) {
+      const int cu = r * 3 + b, cl = 6 + lr * 3 + b;
+      const double2 x = USER ? in[(f * V + nb) * 12 + cu] : in[(f * 12 + cu) * V + nb];
+      const double2 l = USER ? in[(f * V + nb) * 12 + cl] : in[(f * 12 + cl) * V + nb];
+      double2 h = swap ? make_double2(x.x - sp * l.y, x.y + sp * l.x) : make_double2(x.x + sp * l.x, x.y + sp * l.y);
+      if (neg) h = make_double2(-h.x, -h.y);
+      const double2 w = u[(size_t)(mu * 9 + (back ? 3 * b + a : 3 * a + b)) * V + (back ? nb : s)];
+      if (back)
+        wcore::cmac_conj(t, w, h);
+      else
+        wcore::cmac(t, w, h);
+    }
+    if (spin >= 2) {
+      const int eta = mu == 0 || (mu != 3 && r == 0) ? -1 : 1;
+      const double sg = back ? eta : -eta;
+      t = swap ? make_double2(-sg * t.y, sg * t.x) : make_double2(sg * t.x, sg * t.y);
+    }
+    sum.x += t.x;
+    sum.y += t.y;
+  }
+  return sum;
+}
+
+// out = A in for all right-hand sides.  A warp covers 16 sites of
+// one right-hand side (half-warp r: spin row r) and W warps share its hops;
+// RB right-hand sides of the same sites sit in one block, so that a link is
+// fetched from L2 once for them.  Consecutive blocks take the further
+// right-hand sides of the same sites (nrb of them).
+template <int W, bool USER>
+__global__ void __launch_bounds__(fix_threads(W), fix_min_blocks(W))
+wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const double2* __restrict__ in,
+                  double2* __restrict__ out, int nrhs, int RB, int nrb) {
+  constexpr int kWarps = fix_threads(W) / 32;
+  constexpr int kUnits = kWarps / W;  // (site group, rhs) units a block
+  // W > 1: the warps' hop sums; W = 1: two operand stages a warp
+  __shared__ longlong2 part[W > 1 ? kWarps * 6 * 32 : kWarps * kWarpStages];
+  __shared__ double2 stage[USER && W > 1 ? kUnits * kFixSites * 13 : 1];
+  const int V = g.V;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int unit = w / W, sub = w % W;
+  const int i = lane & (kFixSites - 1), r = lane >> 4;
+  const int blk = blockIdx.x / nrb;
+  const int f = (blockIdx.x % nrb) * RB + unit % RB;
+  const int s0 = (blk * (kUnits / RB) + unit / RB) * kFixSites;
+  const bool work = f < nrhs && s0 < V;
+  const int fc = min(f, nrhs - 1);
+  const int s = min(s0 + i, V - 1);
+  const double2* inf = in + (size_t)fc * 12 * V;
+  double2* outf = out + (size_t)fc * 12 * V;
+  // the sites' own components (USER): W > 1 an array of their own, W = 1 the
+  // stage of hop 6 once that is done
+  double2* st = W > 1 ? stage + (USER ? unit * kFixSites * 13 : 0) : reinterpret_cast<double2*>(part + w * kWarpStages);
+  if (W == 1 && !work) return;
+  const int own = work ? min(kFixSites, V - s0) * 12 : 0;  // components of the group's sites
+  auto stage_at = [](int t) { return t + ((unsigned)t * 21846u >> 18); };  // 13 (t / 12) + t % 12 for t < 192
+  if (USER && W > 1 && work) {  // the sites' own components, coalesced
+    const double2* src = inf + (size_t)s0 * 12;
+    for (int t = lane + 32 * sub, at = stage_at(t); t < kFixSites * 12; t += 32 * W, at = stage_at(t))
+      if (t < own) st[at] = src[t];
+  }
+  v.ex += (size_t)fc * v.tiles * kTile;
+  v.dig += field_at(v.tiles, fc, 0);
+  Hops h;
+  load_hops(v, s, h);
+  Acc3 up, lo;
+  if constexpr (W == 1) {
+    hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * kWarpStages), up, lo, [&](int4* to) {
+      if (USER) {
+        const int4* src = reinterpret_cast<const int4*>(inf + (size_t)s0 * 12);
+        for (int t = lane; t < own; t += 32) copy16(to + stage_at(t), src + t);
+      }
+      copy_commit();
+    });
+    copy_wait<0>();
+  } else {
+    hop_sums<W>(v, s, r, sub, h, up, lo);
+  }
+  const double hf = hop_factor(h.E, -g.kappa);
+  if (W > 1) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      part[(w * 6 + a) * 32 + lane] = make_longlong2(up.re[a], up.im[a]);
+      part[(w * 6 + 3 + a) * 32 + lane] = make_longlong2(lo.re[a], lo.im[a]);
+    }
+    __syncthreads();
+  } else {
+    __syncwarp();
+  }
+  // component k of this lane: 0..2 spin r, 3..5 spin 2 + r
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    longlong2 t;
+    if (W > 1) {
+      if (k % W != sub) continue;
+      t = part[(unit * W * 6 + k) * 32 + lane];
+#pragma unroll
+      for (int q = 1; q < W; ++q) {
+        const longlong2 p = part[((unit * W + q) * 6 + k) * 32 + lane];
+        t.x += p.x;
+        t.y += p.y;
+      }
+    } else {
+      t = k < 3 ? make_longlong2(up.re[k % 3], up.im[k % 3]) : make_longlong2(lo.re[k % 3], lo.im[k % 3]);
+    }
+    const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
+    if (!work || s0 + i >= V) continue;
+    const double2 p = USER ? st[i * 13 + comp] : inf[(size_t)comp * V + s];
+    double2 o;
+    o.x = hop_finish(hf, t.x, p.x);
+    o.y = hop_finish(hf, t.y, p.y);
+    if (k >= 3) o = make_double2(-o.x, -o.y);
+    if (USER)
+      st[i * 13 + comp] = o;
+    else
+      outf[(size_t)comp * V + s] = o;
+  }
+  if (work && s0 + i < V && h.E > kMaxExp) {  // next to a value the digits do not hold: FP64
+    for (int k = sub; k < 6; k += W) {
+      const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
+      const double2 p = USER ? in[((size_t)fc * V + s) * 12 + comp] : inf[(size_t)comp * V + s];
+      const double2 d = hop_sum_fp64<USER>(g, u64, in, fc, s, comp);
+      const double sg = k < 3 ? 1.0 : -1.0;
+      double2 o;
+      o.x = fma(sg, fma(-g.kappa, d.x, p.x), 0.0 * p.x);
+      o.y = fma(sg, fma(-g.kappa, d.y, p.y), 0.0 * p.y);
+      if (USER)
+        st[i * 13 + comp] = o;
+      else
+        outf[(size_t)comp * V + s] = o;
+    }
+  }
+  if (USER) {
+    if (W > 1)
+      __syncthreads();
+    else
+      __syncwarp();
+    double2* dst = outf + (size_t)s0 * 12;
+    for (int t = lane + 32 * sub; t < own; t += 32 * W) dst[t] = st[stage_at(t)];
+  }
+}
+
+template <int W>
+void launch_apply(bool user, const Geometry& g, const FixView& v, const double2* u64, const double2* in, double2* out,
+                  int nrhs, cudaStream_t s) {
+  constexpr int kUnits = fix_units(W);
+  const int groups = (g.V + kFixSites - 1) / kFixSites;
+  int RB = 1;
+  while (2 * RB <= kUnits && 2 * RB <= nrhs) RB *= 2;
+  const int nrb = (nrhs + RB - 1) / RB, gb = (groups + kUnits / RB - 1) / (kUnits / RB);
+  const unsigned blocks = (unsigned)gb * nrb;
+  if (user)
+    wilson_fix_kernel<W, true><<<blocks, fix_threads(W), 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
+  else
+    wilson_fix_kernel<W, false><<<blocks, fix_threads(W), 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
+}
+
+}  // namespace
+
+size_t fix_field_bytes(int V) { return sizeof(int4) * 12 * kTile * (size_t)fix_tiles(V); }
+size_t fix_exp_bytes(int V) { return sizeof(int) * kTile * (size_t)fix_tiles(V); }
+
+int pack_fix(const double2* in, bool user, int nrhs, int V, int4* dig, int* ex, cudaStream_t s) {
+  const dim3 grid((V + 63) / 64, nrhs);
+  if (user)
+    pack_fix_kernel<true><<<grid, 256, 0, s>>>(in, dig, ex, V);
+  else
+    pack_fix_kernel<false><<<grid, 256, 0, s>>>(in, dig, ex, V);
+  count_launches(1);
+  SS_CHECK_LAUNCH();
+  return SSQCD_OK;
+}
+
+// Warps that share the eight hops of 16 sites: 1 once the groups fill the
+// GPU's schedulers (8^4 x 4: 7.5 us against 9.4 with 4 and 11 with 8; 16^3 x 32:
+// 48 us against 57 and 70), 4 at half that, 8 below (8^4 x 1: 4.8 us against
+// 5.0 with 4 and 7.4 with 1).
+int fix_split(int V, int nrhs) {
+  const long long groups = (long long)fix_tiles(V) * nrhs;
+  return groups >= 608 ? 1 : groups >= 304 ? 4 : 8;
+}
+
+int wilson_fix(ssqcd_lattice lat, const int4* dig, const int* ex, const double2* in, bool user, double2* out, int nrhs,
+               cudaStream_t s) {
+  const Geometry& g = lat->g;
+  const double2* u64 = lat->u64.as<double2>();
+  const FixView v{lat->ufix.as<int4>(), lat->fnbr.as<int>(), dig, ex, fix_tiles(g.V)};
+  switch (fix_split(g.V, nrhs)) {
+    case 1: launch_apply<1>(user, g, v, u64, in, out, nrhs, s); break;
+    case 4: launch_apply<4>(user, g, v, u64, in, out, nrhs, s); break;
+    default: launch_apply<8>(user, g, v, u64, in, out, nrhs, s); break;
+  }
+  count_launches(1);
+  SS_CHECK_LAUNCH();
+  return SSQCD_OK;
+}
+
+// Scratch of the integer form for a block of right-hand sides: at most 1 GiB
+// at a time (a further block waits for the last one on the stream).
+int fix_block(int V, int nrhs) {
+  const size_t per = fix_field_bytes(V) + fix_exp_bytes(V);
+  const size_t fit = ((size_t)1 << 30) / per;
+  return (int)std::max<size_t>(1, std::min<size_t>({fit, (size_t)nrhs, (size_t)65535}));
+}
+
+int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s) {
+  const Geometry& g = lat->g;
+  if (nrhs <= 0) return SSQCD_OK;
+  AllocStream scope(s);
+  if (lat->fix_ok) {
+    const int nb = fix_block(g.V, nrhs);
+    DevBuf dig, ex;
+    // no room for the digits: the FP64 kernel needs none
+    if (dig.alloc(fix_field_bytes(g.V) * nb) == SSQCD_OK && ex.alloc(fix_exp_bytes(g.V) * nb) == SSQCD_OK) {
+      for (int f = 0; f < nrhs; f += nb) {
+        const int k = std::min(nb, nrhs - f);
+        const size_t off = (size_t)f * 12 * g.V;
+        SS_TRY(pack_fix(in + off, user, k, g.V, dig.as<int4>(), ex.as<int>(), s));
+        SS_TRY(wilson_fix(lat, dig.as<int4>(), ex.as<int>(), in + off, user, out + off, k, s));
+      }
+      return SSQCD_OK;
+    }
+  }
+  if (!user) return wilson64(g, lat->u64.as<double2>(), in, out, nrhs, 0.0, 1.0, nullptr, nullptr, s);
+  DevBuf a, b;
+  const size_t bytes = sizeof(double2) * 12 * (size_t)g.V * nrhs;
+  SS_TRY(a.alloc(bytes));
+  SS_TRY(b.alloc(bytes));
+  SS_TRY(pack_spinors(in, a.as<double2>(), nrhs, g.V, s));
+  SS_TRY(wilson64(g, lat->u64.as<double2>(), a.as<double2>(), b.as<double2>(), nrhs, 0.0, 1.0, nullptr, nullptr, s));
+  return unpack_spinors(b.as<double2>(), out, nrhs, g.V, s);
+}
+
+int build_fix_links(ssqcd_lattice lat) {
+  const int V = lat->g.V;
+  lat->fix_ok = false;
+  DevBuf bad;
+  if (bad.alloc(sizeof(int)) != SSQCD_OK || lat->fnbr.alloc(8 * fix_exp_bytes(V)) != SSQCD_OK ||
+      lat->ufix.alloc(3 * fix_field_bytes(V)) != SSQCD_OK)
+    return SSQCD_OK;  // no room: the FP64 kernel serves the lattice
+  int h = 0;
+  SS_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), lat->stream));
+  pack_links_fix_kernel<<<grid_for(4LL * V, 256), 256, 0, lat->stream>>>(lat->u64.as<double2>(), lat->ufix.as<int4>(),
+                                                                         V, bad.as<int>());
+  neighbour_table_kernel<<<grid_for(8LL * V, 256), 256, 0, lat->stream>>>(lat->g, lat->fnbr.as<int>());
+  count_launches(2);
+  SS_CHECK_LAUNCH();
+  SS_CUDA(cudaMemcpyAsync(&h, bad.p, sizeof(int), cudaMemcpyDeviceToHost, lat->stream));
+  SS_CUDA(cudaStreamSynchronize(lat->stream));
+  lat->fix_ok = h == 0;
+  if (!lat->fix_ok) {
+    lat->ufix.release();
+    lat->fnbr.release();
+  }
+  return SSQCD_OK;
+}
+
+}  // namespace ssqcd
