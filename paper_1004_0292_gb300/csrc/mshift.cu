@@ -62,6 +62,7 @@
 #include "floatfloat.cuh"
 #include "wilson_core.cuh"
 #include "wilson_df.cuh"
+#include "wilson_fix.cuh"
 
 namespace ssqcd {
 namespace {
@@ -334,6 +335,88 @@ struct Stencil64h {
         o.y = fma(sg, fma(mk, acc.y, pv.y), sigma * pv.y);
       }
       q[comp * g.V + s] = o;
+      d = fma(pv.x, o.x, fma(pv.y, o.y, d));
+    }
+    return d;
+  }
+};
+
+// FP64 by integers (wilson_fix.cuh): p's digits and exponents come from the
+// last kernel P; a warp covers 16 sites (half-warp r: spin row r) and W warps
+// share its eight hops, their exact integer sums meeting in shared memory.
+// The diagonal term and (p, q) take p in FP64.  Next to a site that the digits
+// cannot hold (above 2^800, not finite) q is NaN, which ends the recurrence as
+// a breakdown (such a p has no finite (p, p)).
+template <int W>
+struct StencilFix {
+  static constexpr bool kThreadPerSite = false;
+  static constexpr int kThreads = wfix::fix_threads(W);
+  static constexpr int kUnits = wfix::fix_units(W);
+  static constexpr int kSites = kUnits * wfix::kFixSites;
+  // W > 1: the warps' hop sums; W = 1: two operand stages a warp
+  static constexpr int kShElems = kThreads / 32 * (W > 1 ? 6 * 32 : wfix::kWarpStages);
+  static constexpr int kMinBlocks = wfix::fix_min_blocks(W);
+  wfix::FixView view;  // of source 0
+  __device__ __forceinline__ double run(const Geometry& g, const double2* __restrict__ p, double2* __restrict__ q,
+                                        double sigma, int, int, void* shm) const {
+    longlong2* part = static_cast<longlong2*>(shm);
+    const int V = g.V;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int unit = w / W, sub = w % W;
+    const int i = lane & (wfix::kFixSites - 1), r = lane >> 4;
+    const int s0 = (blockIdx.x * kUnits + unit) * wfix::kFixSites;
+    const int s = min(s0 + i, V - 1);
+    wfix::FixView v = view;
+    v.dig += wfix::field_at(v.tiles, blockIdx.y, 0);
+    v.ex += (size_t)blockIdx.y * v.tiles * wfix::kTile;
+    wfix::Hops h;
+    wfix::load_hops(v, s, h);
+    wfix::Acc3 up, lo;
+    if constexpr (W == 1)
+      wfix::hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * wfix::kWarpStages), up, lo,
+                           [](int4*) { wfix::copy_commit(); });
+    else
+      wfix::hop_sums<W>(v, s, r, sub, h, up, lo);
+    const double hf = h.E > wfix::kMaxExp ? __longlong_as_double(0x7ff8000000000000ll) : wfix::hop_factor(h.E, -g.kappa);
+    if (W > 1) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        part[(w * 6 + a) * 32 + lane] = make_longlong2(up.re[a], up.im[a]);
+        part[(w * 6 + 3 + a) * 32 + lane] = make_longlong2(lo.re[a], lo.im[a]);
+      }
+      __syncthreads();
+    }
+    double d = 0.0;
+    // component k of this lane: 0..2 spin r, 3..5 spin 2 + r
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      longlong2 t;
+      if (W > 1) {
+        if (k % W != sub) continue;
+        t = part[(unit * W * 6 + k) * 32 + lane];
+#pragma unroll
+        for (int m = 1; m < W; ++m) {
+          const longlong2 x = part[((unit * W + m) * 6 + k) * 32 + lane];
+          t.x += x.x;
+          t.y += x.y;
+        }
+      } else {
+        t = k < 3 ? make_longlong2(up.re[k % 3], up.im[k % 3]) : make_longlong2(lo.re[k % 3], lo.im[k % 3]);
+      }
+      if (s0 + i >= V) continue;
+      const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
+      const double2 pv = p[(size_t)comp * V + s];
+      double2 o;
+      o.x = wfix::hop_finish(hf, t.x, pv.x);
+      o.y = wfix::hop_finish(hf, t.y, pv.y);
+      if (sigma == 0.0) {  // the paper's seed shift: no sigma p term; the gamma5 sign as a negation
+        if (k < 3) o = make_double2(-o.x, -o.y);
+      } else {
+        const double sg = k < 3 ? -1.0 : 1.0;
+        o.x = fma(sg, o.x, sigma * pv.x);
+        o.y = fma(sg, o.y, sigma * pv.y);
+      }
+      q[(size_t)comp * V + s] = o;
       d = fma(pv.x, o.x, fma(pv.y, o.y, d));
     }
     return d;
@@ -767,6 +850,49 @@ cg_seed_p_kernel(Control c, const VR* __restrict__ r, VR* __restrict__ p, long l
       pe.y = fma(beta, pe.y, sc * x.y);
       pl[e] = pe;
     }
+  }
+  pdl_trigger();
+}
+
+// P for the integer stencil: p in FP64 and its digits and site exponents
+// (wilson_fix.cuh), four lanes a site (spin q), eight sites a warp.  A scale of
+// one -- nearly every iteration -- skips the product r s: FP64 issues two
+// operations a clock and SM, and the update needs no more than beta p + r.
+__global__ void __launch_bounds__(kUpdBlock)
+cg_seed_p_fix_kernel(Control c, const double2* __restrict__ r, double2* __restrict__ p, int4* __restrict__ dig,
+                     int* __restrict__ ex, int V) {
+  pdl_wait();
+  const int l = blockIdx.y;
+  const int ran = *c.ran, live_l = c.live[l];
+  const double scale_l = c.seed[l].scale, beta_l = c.seed[l].beta;
+  if (c.tab != nullptr) r = reinterpret_cast<const double2*>(c.rptr[0]);  // r_{k+1}: kernel B advanced the slots
+  if (ran == 0 || live_l == 0) return;
+  const int lane = threadIdx.x & 31, q = lane >> 3;
+  const int s = (blockIdx.x * (kUpdBlock / 32) + (threadIdx.x >> 5)) * 8 + (lane & 7);
+  const size_t o = ((size_t)l * 12 + 3 * q) * V + s;
+  const double beta = scale_l * beta_l;
+  double2 v[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (s < V) {
+      double2 x = r[o + (size_t)a * V];
+      const double2 y = p[o + (size_t)a * V];
+      if (scale_l != 1.0) x = make_double2(scale_l * x.x, scale_l * x.y);
+      v[a] = make_double2(fma(beta, y.x, x.x), fma(beta, y.y, x.y));
+      p[o + (size_t)a * V] = v[a];
+    } else {
+      v[a] = make_double2(0.0, 0.0);
+    }
+  }
+  const int e = wfix::quad_site_exp(v);
+  if (s < V) {
+    const bool none = e == wfix::kZeroExp || e == wfix::kSpecialExp;
+    const int tiles = wfix::fix_tiles(V);
+    if (q == 0) ex[(size_t)l * tiles * wfix::kTile + s] = e;
+    int4* d = dig + wfix::field_at(tiles, l, s) + 3 * q * wfix::kTile;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      d[a * wfix::kTile] = none ? make_int4(0, 0, 0, 0) : wfix::to_digits(v[a], e + 1022);
   }
   pdl_trigger();
 }
@@ -1910,6 +2036,9 @@ int update_blocks(long long n, int L, int ept) {
 
 namespace {
 
+// sites a block of StencilFix<W> covers
+int fix_sites(int w) { return wfix::fix_units(w) * wfix::kFixSites; }
+
 // The solve loop for one precision: VR is the type of the seed vectors (r, p,
 // q and the stencil), V2 that of the shift vectors (y, p-hat): double2 /
 // double2 (SSQCD_FP64), double2 / float2 (SSQCD_FP64_SHIFT32), double2 /
@@ -1930,6 +2059,7 @@ class CgRun final : public CgRunBase {
   static constexpr bool kShift32 = sizeof(V2) == sizeof(float2);    // shift vectors in FP32
   static constexpr bool kShiftDF = std::is_same<V2, float4>::value;  // shift vectors in float-float
   static constexpr bool kSeedDF = std::is_same<VR, float4>::value;   // seed vectors and stencil in float-float
+  static constexpr bool kSeed64 = std::is_same<VR, double2>::value;  // seed vectors and stencil in FP64
   static constexpr int kChunk = 16;  // even: every chunk starts at parity 0
   static constexpr int kSlots = 8;   // timing events per iteration: A, B, C, P start/stop
   static constexpr int kTimedEvery = 4;
@@ -1986,7 +2116,14 @@ class CgRun final : public CgRunBase {
     n_ = 12LL * g.V;
     const long long n = n_;
     const int NL = N * L;
+    if constexpr (kSeed64) {
+      // the integer stencil, when the links allow it and its digits fit
+      fix_ = lat->fix_ok && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
+             pex_.alloc(fix_exp_bytes(g.V) * L) == SSQCD_OK;
+      fix_w_ = fix_split(g.V, L);
+    }
     nbw_ = kFP32 ? (g.V + kSiteThreads - 1) / kSiteThreads
+           : fix_ ? (g.V + fix_sites(fix_w_) - 1) / fix_sites(fix_w_)
            : (kSeedDF || !balanced_stencil()) ? wilson_blocks(g)
                                               : (g.V + kSitesPerBlockH - 1) / kSitesPerBlockH;
     nbs_ = seed_blocks(n, L);
@@ -2100,6 +2237,9 @@ class CgRun final : public CgRunBase {
     init_control_kernel<<<1, 256, 0, st_>>>(c, vn2, L, N);
     SS_CHECK_LAUNCH();
     count_launches(2);
+    if constexpr (kSeed64) {
+      if (fix_) SS_TRY(pack_fix(p_.as<double2>(), false, L, g.V, pdig_.as<int4>(), pex_.as<int>(), st_));
+    }
 
     SS_CUDA(cudaEventCreate(&e0_));
     SS_CUDA(cudaEventCreate(&e1_));
@@ -2464,6 +2604,16 @@ class CgRun final : public CgRunBase {
     if (mark_on_) cudaEventRecordWithFlags(tev_[it * kSlots + slot], s, cudaEventRecordExternal);
   }
 
+  template <int W>
+  void launch_fix(dim3 grid, int par) {
+    if constexpr (kSeed64)
+      launch_chain(cg_stencil_kernel<StencilFix<W>, VR>, grid, StencilFix<W>::kThreads, st_, prio_a_,
+                   basis_ && use_pdl(), c_, L_, par, lat_->g,
+                   StencilFix<W>{wfix::FixView{lat_->ufix.as<int4>(), lat_->fnbr.as<int>(), pdig_.as<int4>(),
+                                               pex_.as<int>(), wfix::fix_tiles(lat_->g.V)}},
+                   sigma_, p_.as<VR>(), q_.as<VR>());
+  }
+
   void iteration(int it) {
     const Geometry& g = lat_->g;
     const long long n = n_;
@@ -2496,6 +2646,12 @@ class CgRun final : public CgRunBase {
         launch_chain(cg_stencil_kernel<StencilDF<4>, VR>, grid_a, kStencilThreadsDF, st, prio_a_,
                      basis_ && use_pdl(), c, L, par, g, StencilDF<4>{lat_->udf.as<float4>()}, sigma_, p_.as<VR>(),
                      q_.as<VR>());
+    } else if (fix_) {
+      switch (fix_w_) {
+        case 1: launch_fix<1>(grid_a, par); break;
+        case 4: launch_fix<4>(grid_a, par); break;
+        default: launch_fix<8>(grid_a, par); break;
+      }
     } else if (balanced_stencil()) {
       if (stencil_minb() == 8)
         launch_chain(cg_stencil_kernel<Stencil64h<8>, VR>, grid_a, kStencilThreads, st, prio_a_,
@@ -2516,7 +2672,17 @@ class CgRun final : public CgRunBase {
     mark(it, 3, st);
     cudaEventRecord(ev_[it], st);
     mark(it, 6, st);
-    launch_chain(cg_seed_p_kernel<VR>, grid_p, kUpdBlock, st, prio_hi_, basis_ && use_pdl(), c, r_out, p_.as<VR>(), n);
+    bool p_done = false;
+    if constexpr (kSeed64) {
+      if (fix_) {
+        launch_chain(cg_seed_p_fix_kernel, dim3((g.V + kUpdBlock / 4 - 1) / (kUpdBlock / 4), L), kUpdBlock, st, prio_hi_,
+                     basis_ && use_pdl(), c, r_out, p_.as<VR>(), pdig_.as<int4>(), pex_.as<int>(), g.V);
+        p_done = true;
+      }
+    }
+    if (!p_done)
+      launch_chain(cg_seed_p_kernel<VR>, grid_p, kUpdBlock, st, prio_hi_, basis_ && use_pdl(), c, r_out, p_.as<VR>(),
+                   n);
     mark(it, 7, st);
     if (basis_) {  // no shift-vector update: the shift scalars on the side stream
       cudaStreamWaitEvent(side_, ev_[it], 0);
@@ -2580,6 +2746,9 @@ class CgRun final : public CgRunBase {
   std::vector<std::unique_ptr<DevBuf>> blocks_;
   DevBuf tab_, gam_, count_;
   char** h_tab_ = nullptr;
+  bool fix_ = false;  // the integer stencil
+  int fix_w_ = 0;
+  DevBuf pdig_, pex_;  // p's digits and exponents
   DevBuf r_, p_, q_, ph_, y32_, x_, kx_, y_out_, ctl_;
   V2* yv_ = nullptr;
   Control c_{};
