@@ -136,7 +136,7 @@ extern "C" int ssqcd_upload_gauge(ssqcd_lattice lat, const double* links, int on
     SS_TRY(pack_gauge32(lat->u64.as<double2>(), lat->u32.p, V, lat->stream));
   }
   lat->gauge_version++;
-  if (lat->precision == SSQCD_DF) SS_TRY(ensure_df_links(lat));
+  if (lat->precision == SSQCD_DF && !lat->fix_ok) SS_TRY(ensure_df_links(lat));
   SS_CUDA(cudaStreamSynchronize(lat->stream));
   lat->has_gauge = true;
   return SSQCD_OK;
@@ -189,6 +189,8 @@ extern "C" int ssqcd_apply_H_mixed(ssqcd_lattice lat, const double* in, double* 
     return fail(SSQCD_ERR_ARG, "apply_H_mixed needs a mixed-precision or SSQCD_DF lattice");
   if (nrhs < 0 || (nrhs > 0 && (in == nullptr || out == nullptr))) return fail(SSQCD_ERR_ARG, "bad apply_H arguments");
   if (nrhs == 0) return SSQCD_OK;
+  // the integer stencil holds 60 bits a component: float-float's 48 and more
+  if (lat->precision == SSQCD_DF && lat->fix_ok) return apply_user(lat, in, out, nrhs, on_device);
   const long long n = 12LL * lat->g.V * nrhs;
   DevBuf a, a32, b32;
   SS_TRY(to_device_layout(lat, in, nrhs, on_device, a));
@@ -417,8 +419,7 @@ int rayleigh_ritz_projected(ssqcd_lattice lat, const double2* S, int m, double r
   SS_TRY(AT.alloc(sizeof(double2) * n * m));
   SS_TRY(Gd.alloc(sizeof(double2) * m * m));
   if (df) {
-    SS_TRY(ensure_df_links(lat));
-    SS_TRY(wilson_df(lat->g, lat->udf.as<float4>(), T.as<float4>(), AT.as<float4>(), m, 0.0, 1.0, st));
+    SS_TRY(wilson_df_lat(lat, T.as<float4>(), AT.as<float4>(), m, st));
     SS_TRY(gram_df(T.as<float4>(), m, AT.as<float4>(), m, n, Gd.as<double2>(), gs, st, true));
   } else {
     SS_TRY(wilson64_lat(lat, T.as<double2>(), false, AT.as<double2>(), m, st));
@@ -1876,7 +1877,6 @@ extern "C" int ssqcd_time_stencil(ssqcd_lattice lat, int nrhs, int reps, double*
   cudaStream_t st = lat->stream;
   const long long n = 12LL * lat->g.V * nrhs;
   const bool mixed = is_mixed(lat->precision), df = lat->precision == SSQCD_DF;
-  if (df) SS_TRY(ensure_df_links(lat));
   const size_t elem = mixed ? sizeof(float2) : sizeof(double2);
   DevBuf a, b;
   SS_TRY(a.alloc(elem * n));
@@ -1888,7 +1888,7 @@ extern "C" int ssqcd_time_stencil(ssqcd_lattice lat, int nrhs, int reps, double*
       return wilson32_kernel_only(lat->g, f16 ? lat->u16.p : lat->u32.p, f16 ? 16 : 32, a.as<float2>(),
                                   b.as<float2>(), nrhs, 0.f, 1.f, st);
     }
-    if (df) return wilson_df(lat->g, lat->udf.as<float4>(), a.as<float4>(), b.as<float4>(), nrhs, 0.0, 1.0, st);
+    if (df) return wilson_df_lat(lat, a.as<float4>(), b.as<float4>(), nrhs, st);
     return wilson64_lat(lat, a.as<double2>(), false, b.as<double2>(), nrhs, st);
   };
   for (int i = 0; i < 2; ++i) SS_TRY(once());

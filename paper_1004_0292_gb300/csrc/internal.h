@@ -109,7 +109,7 @@ struct ssqcd_lattice_s {
   ssqcd::DevBuf u32;     // FP32 12-parameter links, SSQCD_MIXED_F32LINKS only
   ssqcd::DevBuf udf;     // float-float links [4][9][V] float4, built on first SSQCD_DF use
   ssqcd::DevBuf ufix;    // links as 60-bit integers (wilson_fix.cuh), when fix_ok
-  ssqcd::DevBuf fnbr;    // its neighbour table
+  int* fnbr = nullptr;   // its neighbour table (inside ufix)
   bool fix_ok = false;   // the links have unit rows and columns: the integer stencil serves the lattice
   int gauge_version = 0; // bumped by every upload
   int udf_version = -1;  // gauge_version udf was built from
@@ -139,11 +139,13 @@ int wilson64(const Geometry& g, const double2* u, const double2* in, double2* ou
 // (wilson_fix.cu) where its links allow it, else wilson64.  user: in and out
 // are in the caller's layout [nrhs][V][12], else [nrhs][12][V].
 int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s);
+int wilson_df_lat(ssqcd_lattice lat, const float4* in, float4* out, int nrhs, cudaStream_t s);  // float-float fields
 // Integer stencil (wilson_fix.cu): fields as digits with one exponent a site,
 // bytes of each for one field; the links take three fields' bytes
 size_t fix_field_bytes(int V);
 size_t fix_exp_bytes(int V);
-int pack_fix(const double2* in, bool user, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
+int pack_fix(const double2* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
+int pack_fix(const float4* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
 int fix_split(int V, int nrhs);  // warps that share the hops of 16 sites: 1, 4 or 8
 int fix_block(int V, int nrhs);  // right-hand sides converted at a time
 // digits of the uploaded links (sets ufix, fix_ok)

@@ -77,7 +77,7 @@ struct SeedState {
   double beta;        // beta_k (valid after kernel B of iteration k)
   double scale;       // power of two applied to p by kernel C of this iteration and to r
                       // by kernel B of the next (C reads r scaled in registers)
-  double pad[3];      // pad[0] = 1 / rr, pad[1] = S = product of all scales so far
+  double pad[3];      // pad[1] = S = product of all scales so far
 };
 
 // Device-side control block of one solve (L sources, N shifts).  Every field
@@ -87,6 +87,7 @@ struct SeedState {
 struct Control {
   SeedState* seed;     // [L]
   double* alpha;       // [L]     alpha_k
+  double* inv_rr;      // [L]     1 / (r_k, r_k), kernel A
   double* vnorm2;      // [L]
   int* live;           // [L]     shifts still iterating
   int* live_total;     // [1]
@@ -233,8 +234,8 @@ __global__ void init_vectors_kernel(const double2* __restrict__ v, VR* __restric
 // A source with ||v|| = 0 has the exact solution y = 0 and starts frozen.
 __global__ void init_control_kernel(Control c, const double* __restrict__ vn2, int L, int N) {
   for (int t = threadIdx.x; t < L; t += blockDim.x) {
-    // rr_0, alpha_{-1} = 1, beta_{-1} = 0, scale 1, 1 / rr_0
-    c.seed[t] = SeedState{vn2[t], 1.0, 0.0, 0.0, 1.0, {vn2[t] > 0.0 ? 1.0 / vn2[t] : 0.0, 1.0, 0.0}};
+    // rr_0, alpha_{-1} = 1, beta_{-1} = 0, scale 1, S = 1
+    c.seed[t] = SeedState{vn2[t], 1.0, 0.0, 0.0, 1.0, {0.0, 1.0, 0.0}};
     c.alpha[t] = 0.0;
     c.vnorm2[t] = vn2[t];
     c.live[t] = vn2[t] > 0.0 ? N : 0;
@@ -341,14 +342,15 @@ struct Stencil64h {
   }
 };
 
-// FP64 by integers (wilson_fix.cuh): p's digits and exponents come from the
+// FP64 and float-float vectors by integers (wilson_fix.cuh): p's digits and exponents come from the
 // last kernel P; a warp covers 16 sites (half-warp r: spin row r) and W warps
 // share its eight hops, their exact integer sums meeting in shared memory.
-// The diagonal term and (p, q) take p in FP64.  Next to a site that the digits
+// The diagonal term and (p, q) take p in its own form.  Next to a site that the digits
 // cannot hold (above 2^800, not finite) q is NaN, which ends the recurrence as
 // a breakdown (such a p has no finite (p, p)).
-template <int W>
+template <int W, typename V2>
 struct StencilFix {
+  static constexpr bool kFF = std::is_same<V2, float4>::value;  // float-float vectors
   static constexpr bool kThreadPerSite = false;
   static constexpr int kThreads = wfix::fix_threads(W);
   static constexpr int kUnits = wfix::fix_units(W);
@@ -357,7 +359,7 @@ struct StencilFix {
   static constexpr int kShElems = kThreads / 32 * (W > 1 ? 6 * 32 : wfix::kWarpStages);
   static constexpr int kMinBlocks = wfix::fix_min_blocks(W);
   wfix::FixView view;  // of source 0
-  __device__ __forceinline__ double run(const Geometry& g, const double2* __restrict__ p, double2* __restrict__ q,
+  __device__ __forceinline__ double run(const Geometry& g, const V2* __restrict__ p, V2* __restrict__ q,
                                         double sigma, int, int, void* shm) const {
     longlong2* part = static_cast<longlong2*>(shm);
     const int V = g.V;
@@ -372,12 +374,22 @@ struct StencilFix {
     wfix::Hops h;
     wfix::load_hops(v, s, h);
     wfix::Acc3 up, lo;
-    if constexpr (W == 1)
+    if constexpr (W == 1) {
       wfix::hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * wfix::kWarpStages), up, lo,
-                           [](int4*) { wfix::copy_commit(); });
-    else
+                           [&](int4* to) {  // the diagonal term's p, a row of lanes a component
+#pragma unroll
+                             for (int k = 0; k < 6; ++k)
+                               wfix::copy16(to + k * 32 + lane, reinterpret_cast<const int4*>(p) + s +
+                                                                    (size_t)((k < 3 ? 0 : 6) + r * 3 + k % 3) * V);
+                             wfix::copy_commit();
+                           });
+      wfix::copy_wait<0>();  // each lane reads back its own copies
+    } else {
       wfix::hop_sums<W>(v, s, r, sub, h, up, lo);
-    const double hf = h.E > wfix::kMaxExp ? __longlong_as_double(0x7ff8000000000000ll) : wfix::hop_factor(h.E, -g.kappa);
+    }
+    const bool special = h.E > wfix::kMaxExp;
+    const double hf = special ? __longlong_as_double(0x7ff8000000000000ll) : wfix::hop_factor(h.E, -g.kappa);
+    float2 dff = make_float2(0.f, 0.f);
     if (W > 1) {
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -387,39 +399,57 @@ struct StencilFix {
       __syncthreads();
     }
     double d = 0.0;
-    // component k of this lane: 0..2 spin r, 3..5 spin 2 + r
+    // component k of this lane: 0..2 spin r, 3..5 spin 2 + r.  Z: sigma = 0, the
+    // paper's seed shift, leaves out the sigma p term (as a form of its own: an
+    // FP64 product under a predicate takes its pipe slot all the same)
+    auto finish = [&](auto zero) {
+      constexpr bool Z = decltype(zero)::value;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      longlong2 t;
-      if (W > 1) {
-        if (k % W != sub) continue;
-        t = part[(unit * W * 6 + k) * 32 + lane];
+      for (int k = 0; k < 6; ++k) {
+        longlong2 t;
+        if (W > 1) {
+          if (k % W != sub) continue;
+          t = part[(unit * W * 6 + k) * 32 + lane];
 #pragma unroll
-        for (int m = 1; m < W; ++m) {
-          const longlong2 x = part[((unit * W + m) * 6 + k) * 32 + lane];
-          t.x += x.x;
-          t.y += x.y;
+          for (int m = 1; m < W; ++m) {
+            const longlong2 x = part[((unit * W + m) * 6 + k) * 32 + lane];
+            t.x += x.x;
+            t.y += x.y;
+          }
+        } else {
+          t = k < 3 ? make_longlong2(up.re[k % 3], up.im[k % 3]) : make_longlong2(lo.re[k % 3], lo.im[k % 3]);
         }
-      } else {
-        t = k < 3 ? make_longlong2(up.re[k % 3], up.im[k % 3]) : make_longlong2(lo.re[k % 3], lo.im[k % 3]);
+        if (s0 + i >= V) continue;
+        const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
+        const V2 pv = W > 1 ? p[(size_t)comp * V + s]
+                            : reinterpret_cast<const V2*>(part + w * wfix::kWarpStages)[k * 32 + lane];
+        if constexpr (kFF) {
+          const float nan = __int_as_float(0x7fc00000);
+          const float4 hop = special ? make_float4(nan, nan, nan, nan) : wfix::hop_cff(t, h.E);
+          float4 o;
+          dff = ff::add(dff, finish_df(g, pv, ff::split(sigma), make_float2(-1.f, 0.f), comp, hop, o));
+          q[(size_t)comp * V + s] = o;
+        } else {
+          double2 o;
+          o.x = wfix::hop_finish(hf, t.x, pv.x);
+          o.y = wfix::hop_finish(hf, t.y, pv.y);
+          if constexpr (Z) {
+            if (k < 3) o = make_double2(-o.x, -o.y);
+          } else {
+            const double sg = k < 3 ? -1.0 : 1.0;
+            o.x = fma(sg, o.x, sigma * pv.x);
+            o.y = fma(sg, o.y, sigma * pv.y);
+          }
+          q[(size_t)comp * V + s] = o;
+          d = fma(pv.x, o.x, fma(pv.y, o.y, d));
+        }
       }
-      if (s0 + i >= V) continue;
-      const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
-      const double2 pv = p[(size_t)comp * V + s];
-      double2 o;
-      o.x = wfix::hop_finish(hf, t.x, pv.x);
-      o.y = wfix::hop_finish(hf, t.y, pv.y);
-      if (sigma == 0.0) {  // the paper's seed shift: no sigma p term; the gamma5 sign as a negation
-        if (k < 3) o = make_double2(-o.x, -o.y);
-      } else {
-        const double sg = k < 3 ? -1.0 : 1.0;
-        o.x = fma(sg, o.x, sigma * pv.x);
-        o.y = fma(sg, o.y, sigma * pv.y);
-      }
-      q[(size_t)comp * V + s] = o;
-      d = fma(pv.x, o.x, fma(pv.y, o.y, d));
-    }
-    return d;
+    };
+    if (kFF || sigma == 0.0)
+      finish(std::true_type{});
+    else
+      finish(std::false_type{});
+    return kFF ? (double)dff.x + (double)dff.y : d;
   }
 };
 
@@ -488,6 +518,40 @@ struct StencilDF {
   }
 };
 
+// Sums of the block partials [L][nb] into sums[L] by one block of W warps (the
+// tail that the whole GPU waits for): L sources share the warps -- with fewer
+// sources than warps each takes W / L of them, a contiguous part of its
+// partials a warp -- eight loads in flight a lane, a fixed order throughout.
+// spart: [W] doubles of shared memory.  Ends with a block barrier.
+template <int W>
+__device__ __forceinline__ void tail_sums(const double* __restrict__ partial, int nb, int L, double* sums,
+                                          double* spart) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int parts = L < W ? W / L : 1;
+  const int chunk = (nb + parts - 1) / parts;
+  for (int t = w; t < L * parts; t += W) {
+    const int ls = t / parts, b1 = min(nb, (t % parts + 1) * chunk);
+    double a = 0.0;
+    for (int b0 = (t % parts) * chunk + lane; b0 < b1; b0 += 32 * 8) {
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = b0 + 32 * i < b1 ? __ldcg(partial + (size_t)ls * nb + b0 + 32 * i) : 0.0;
+      a += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+    a = warp_sum(a);
+    if (lane == 0) (parts > 1 ? spart[t] : sums[ls]) = a;
+  }
+  __syncthreads();
+  if (parts > 1) {
+    if ((int)threadIdx.x < L) {
+      double a = spart[threadIdx.x * parts];
+      for (int i = 1; i < parts; ++i) a += spart[threadIdx.x * parts + i];
+      sums[threadIdx.x] = a;
+    }
+    __syncthreads();
+  }
+}
+
 template <typename Op, typename V2>
 __global__ void __launch_bounds__(Op::kThreads, Op::kMinBlocks)
 cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, const V2* __restrict__ p_all,
@@ -499,12 +563,17 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   }
   constexpr int kWarps = Op::kThreads / 32;
   __shared__ double2 sh[Op::kShElems];  // the op's reduction scratch
-  __shared__ double sred[kWarps];
+  __shared__ double sred[kWarps], spart[kWarps];
   __shared__ double sums[kMaxSources];
   __shared__ bool s_last;
   const int l = blockIdx.y;
   const int V = g.V;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // 1 / (r_k, r_k) for kernel B's beta: a division off both kernels' tails
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const double rr = c.seed[l].rr;
+    c.inv_rr[l] = rr > 0.0 ? 1.0 / rr : 0.0;
+  }
   double d_pq = 0.0;
   if (c.live[l] != 0) {
     const int s = Op::kThreadPerSite ? blockIdx.x * Op::kThreads + (int)threadIdx.x
@@ -529,24 +598,7 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  // warp w sums the partials of sources w, w + kWarps, ... in a fixed order,
-  // eight loads in flight a lane (this tail runs on one SM while the rest
-  // of the GPU waits for alpha)
-  for (int ls = w; ls < L; ls += kWarps) {
-    double a = 0.0;
-    for (int b0 = lane; b0 < nbw; b0 += 32 * 8) {
-      double t[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int b = b0 + 32 * i;
-        t[i] = b < nbw ? __ldcg(c.partial + (size_t)ls * nbw + b) : 0.0;
-      }
-      a += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
-    }
-    a = warp_sum(a);
-    if (lane == 0) sums[ls] = a;
-  }
-  __syncthreads();
+  tail_sums<kWarps>(c.partial, nbw, L, sums, spart);
   for (int ls = threadIdx.x; ls < L; ls += blockDim.x) {
     if (c.live[ls] == 0) continue;
     const double pq = sums[ls];
@@ -660,28 +712,51 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
       }
       acc0 = (double)hs + (double)hl;
     } else {
-      auto one = [&](long long e, double& acc) {
-        V2 x0 = rl[e];
-        const V2 y0 = ql[e];
-        x0.x = fma(-af, y0.x, sc * x0.x);
-        x0.y = fma(-af, y0.y, sc * x0.y);
-        ro[e] = x0;
-        const double xr = x0.x, xi = x0.y;
-        acc = fma(xr, xr, fma(xi, xi, acc));
-        if (xl != nullptr) {
-          const V2 pv = pl[e];
-          double2 xv = xl[e];
-          xv.x = fma(ax, (double)pv.x, xv.x);
-          xv.y = fma(ax, (double)pv.y, xv.y);
-          xl[e] = xv;
+      // Four elements a turn, their loads issued together.  The scale, one in
+      // nearly every iteration, and the mixed path's solution have loops of
+      // their own: FP64 issues two operations a clock and SM, whether or not a
+      // predicate lets them write, and four an element (two for r, two for
+      // its norm) already take as long as the element's 48 bytes.
+      auto sweep = [&](auto scaled) {
+        constexpr int kU = 4;
+        double au[kU] = {0.0, 0.0, 0.0, 0.0};
+        for (long long e = blockIdx.x * (long long)kSeedBlock + threadIdx.x; e < n; e += kU * stride) {
+          V2 x[kU], y[kU];
+#pragma unroll
+          for (int i = 0; i < kU; ++i)
+            if (e + i * stride < n) {
+              x[i] = rl[e + i * stride];
+              y[i] = ql[e + i * stride];
+            }
+#pragma unroll
+          for (int i = 0; i < kU; ++i) {
+            const long long ei = e + i * stride;
+            if (ei >= n) break;
+            V2 x0 = x[i];
+            if constexpr (decltype(scaled)::value) x0 = V2{sc * x0.x, sc * x0.y};
+            x0.x = fma(-af, y[i].x, x0.x);
+            x0.y = fma(-af, y[i].y, x0.y);
+            ro[ei] = x0;
+            const double xr = x0.x, xi = x0.y;
+            au[i] = fma(xr, xr, fma(xi, xi, au[i]));
+            if constexpr (sizeof(V2) == sizeof(float2)) {
+              if (xl != nullptr) {
+                const V2 pv = pl[ei];
+                double2 xv = xl[ei];
+                xv.x = fma(ax, (double)pv.x, xv.x);
+                xv.y = fma(ax, (double)pv.y, xv.y);
+                xl[ei] = xv;
+              }
+            }
+          }
         }
+        acc0 = au[0] + au[1];
+        acc1 = au[2] + au[3];
       };
-      long long e = blockIdx.x * (long long)kSeedBlock + threadIdx.x;
-      for (; e + stride < n; e += 2 * stride) {
-        one(e, acc0);
-        one(e + stride, acc1);
-      }
-      if (e < n) one(e, acc0);
+      if (sc == (T)1)
+        sweep(std::false_type{});
+      else
+        sweep(std::true_type{});
     }
   }
   double acc = warp_sum(acc0 + acc1);
@@ -700,23 +775,11 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
   if (!s_last) return;
   __threadfence();
   const int kb = c.tab != nullptr ? *c.seed_iters - 1 : 0;  // this iteration (Krylov-basis form)
-  for (int ls = w; ls < L; ls += kSeedBlock / 32) {
-    // the source's control words together with its partials
-    const double pad0 = c.seed[ls].pad[0], vn2 = c.vnorm2[ls];  // pad[0] holds 1 / rr_k
-    const int lv = c.live[ls];
-    double a0 = 0.0, a1 = 0.0;
-    int b = lane;
-    for (; b + 32 < nb; b += 64) {
-      a0 += __ldcg(c.partial_rr + (size_t)ls * nb + b);
-      a1 += __ldcg(c.partial_rr + (size_t)ls * nb + b + 32);
-    }
-    if (b < nb) a0 += __ldcg(c.partial_rr + (size_t)ls * nb + b);
-    const double a = warp_sum(a0 + a1);
-    if (lane == 0) {
-      sums[ls] = a;
-      s_beta[ls] = a * pad0;
-      s_scale[ls] = (lv != 0 && a < rescale_below * vn2 && a > 0.0) ? rescale_by : 1.0;
-    }
+  tail_sums<kSeedBlock / 32>(c.partial_rr, nb, L, sums, sred);
+  for (int ls = threadIdx.x; ls < L; ls += blockDim.x) {
+    const double a = sums[ls], vn2 = c.vnorm2[ls];
+    s_beta[ls] = a * c.inv_rr[ls];
+    s_scale[ls] = (c.live[ls] != 0 && a < rescale_below * vn2 && a > 0.0) ? rescale_by : 1.0;
   }
   if (c.tab != nullptr && threadIdx.x == 0) {  // slots of the next iteration
     const long long Ln = (long long)L * n;
@@ -736,7 +799,7 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
       rec[3] = sd.pad[1];
       if (c.live[ls] != 0) {
         const double rr = sums[ls] * sc * sc;
-        c.seed[ls] = SeedState{rr, c.alpha[ls], s_beta[ls], s_beta[ls], sc, {1.0 / rr, sd.pad[1] * sc, 0.0}};
+        c.seed[ls] = SeedState{rr, c.alpha[ls], s_beta[ls], s_beta[ls], sc, {0.0, sd.pad[1] * sc, 0.0}};
       }
     }
     if (threadIdx.x == 0) {
@@ -801,7 +864,7 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
       if (c.live[ls] != 0) {
         const double sc = s_scale[ls];
         const double rr = sums[ls] * sc * sc;
-        c.seed[ls] = SeedState{rr, c.alpha[ls], s_beta[ls], s_beta[ls], sc, {1.0 / rr, c.seed[ls].pad[1] * sc, 0.0}};
+        c.seed[ls] = SeedState{rr, c.alpha[ls], s_beta[ls], s_beta[ls], sc, {0.0, c.seed[ls].pad[1] * sc, 0.0}};
       }
       c.live[ls] = live;
     }
@@ -854,35 +917,51 @@ cg_seed_p_kernel(Control c, const VR* __restrict__ r, VR* __restrict__ p, long l
   pdl_trigger();
 }
 
-// P for the integer stencil: p in FP64 and its digits and site exponents
-// (wilson_fix.cuh), four lanes a site (spin q), eight sites a warp.  A scale of
-// one -- nearly every iteration -- skips the product r s: FP64 issues two
-// operations a clock and SM, and the update needs no more than beta p + r.
+// P for the integer stencil: p in its own form (FP64 or float-float) and its
+// digits and site exponents (wilson_fix.cuh), four lanes a site (spin q), eight
+// sites a warp.  A scale of one -- nearly every iteration -- skips the product
+// r s: FP64 issues two operations a clock and SM, and the update needs no more
+// than beta p + r.
+template <bool SCALED>
+__device__ __forceinline__ double2 seed_dir(double2 x, double2 y, double scale, double beta) {
+  if (SCALED) x = make_double2(scale * x.x, scale * x.y);
+  return make_double2(fma(beta, y.x, x.x), fma(beta, y.y, x.y));
+}
+template <bool SCALED>
+__device__ __forceinline__ float4 seed_dir(float4 x, float4 y, double scale, double beta) {
+  return ff::caxpy(SCALED ? ff::cscale2(x, (float)scale) : x, ff::split(beta), y);
+}
+template <typename V2>
 __global__ void __launch_bounds__(kUpdBlock)
-cg_seed_p_fix_kernel(Control c, const double2* __restrict__ r, double2* __restrict__ p, int4* __restrict__ dig,
+cg_seed_p_fix_kernel(Control c, const V2* __restrict__ r, V2* __restrict__ p, int4* __restrict__ dig,
                      int* __restrict__ ex, int V) {
   pdl_wait();
   const int l = blockIdx.y;
   const int ran = *c.ran, live_l = c.live[l];
   const double scale_l = c.seed[l].scale, beta_l = c.seed[l].beta;
-  if (c.tab != nullptr) r = reinterpret_cast<const double2*>(c.rptr[0]);  // r_{k+1}: kernel B advanced the slots
+  if (c.tab != nullptr) r = reinterpret_cast<const V2*>(c.rptr[0]);  // r_{k+1}: kernel B advanced the slots
   if (ran == 0 || live_l == 0) return;
   const int lane = threadIdx.x & 31, q = lane >> 3;
   const int s = (blockIdx.x * (kUpdBlock / 32) + (threadIdx.x >> 5)) * 8 + (lane & 7);
   const size_t o = ((size_t)l * 12 + 3 * q) * V + s;
-  const double beta = scale_l * beta_l;
-  double2 v[3];
+  V2 v[3] = {};
+  if (s < V) {
+    V2 x[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    if (s < V) {
-      double2 x = r[o + (size_t)a * V];
-      const double2 y = p[o + (size_t)a * V];
-      if (scale_l != 1.0) x = make_double2(scale_l * x.x, scale_l * x.y);
-      v[a] = make_double2(fma(beta, y.x, x.x), fma(beta, y.y, x.y));
-      p[o + (size_t)a * V] = v[a];
-    } else {
-      v[a] = make_double2(0.0, 0.0);
+    for (int a = 0; a < 3; ++a) {
+      x[a] = r[o + (size_t)a * V];
+      v[a] = p[o + (size_t)a * V];
     }
+    const double beta = scale_l * beta_l;
+    if (scale_l == 1.0) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[a] = seed_dir<false>(x[a], v[a], 1.0, beta);
+    } else {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[a] = seed_dir<true>(x[a], v[a], scale_l, beta);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) p[o + (size_t)a * V] = v[a];
   }
   const int e = wfix::quad_site_exp(v);
   if (s < V) {
@@ -891,8 +970,7 @@ cg_seed_p_fix_kernel(Control c, const double2* __restrict__ r, double2* __restri
     if (q == 0) ex[(size_t)l * tiles * wfix::kTile + s] = e;
     int4* d = dig + wfix::field_at(tiles, l, s) + 3 * q * wfix::kTile;
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-      d[a * wfix::kTile] = none ? make_int4(0, 0, 0, 0) : wfix::to_digits(v[a], e + 1022);
+    for (int a = 0; a < 3; ++a) d[a * wfix::kTile] = none ? make_int4(0, 0, 0, 0) : wfix::to_site_digits(v[a], e);
   }
   pdl_trigger();
 }
@@ -1467,7 +1545,7 @@ __global__ void df_to_f64_kernel(float4* __restrict__ y, long long count) {
 // the difference between it and the reduced-precision operator the
 // recursion uses (~3e-4 relative with FP16 links, ~1e-7 with FP32 links), and
 // replacing r would break the Krylov recurrence the shifted systems are
-// built on; the last block stores (r, r) and its reciprocal.  The stored r is
+// built on; the last block stores (r, r).  The stored r is
 // divided by the scale chosen in the last iteration, which kernel B applies.
 template <typename V2>
 __global__ void __launch_bounds__(kSeedBlock)
@@ -1517,7 +1595,6 @@ cg_reliable_kernel(Control c, int L, const double2* __restrict__ v, const double
     if (lane == 0 && ap && a > 0.0) {
       SeedState sn = sl;
       sn.rr = a;
-      sn.pad[0] = 1.0 / a;
       c.seed[ls] = sn;
       atomicAdd(c.seed_iters + 1, 1);  // reliable-update counter
     }
@@ -2096,7 +2173,9 @@ class CgRun final : public CgRunBase {
     max_iter_ = max_iter;
     st_ = st;
     // lattice-owned data first, outside the run's stream-ordered allocations
-    if constexpr (kSeedDF) SS_TRY(ensure_df_links(lat));
+    if constexpr (kSeedDF) {
+      if (!lat->fix_ok) SS_TRY(ensure_df_links(lat));
+    }
     AllocStream scope(st_);
     tma_ = kShiftDF && use_tma_update();
     {
@@ -2116,11 +2195,17 @@ class CgRun final : public CgRunBase {
     n_ = 12LL * g.V;
     const long long n = n_;
     const int NL = N * L;
-    if constexpr (kSeed64) {
-      // the integer stencil, when the links allow it and its digits fit
-      fix_ = lat->fix_ok && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
+    if constexpr (kSeed64 || kSeedDF) {
+      // the integer stencil, when the links allow it and its digits fit; for
+      // float-float vectors where it runs one warp a site group (below that,
+      // 8^4 x 2, the float-float stencil is as fast and needs no digits)
+      fix_ = lat->fix_ok && (kSeed64 || fix_split(g.V, L) == 1) && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
              pex_.alloc(fix_exp_bytes(g.V) * L) == SSQCD_OK;
       fix_w_ = fix_split(g.V, L);
+      if constexpr (kSeedDF) {
+        AllocStream plain(st_, false);  // lattice-owned
+        if (!fix_) SS_TRY(ensure_df_links(lat));
+      }
     }
     nbw_ = kFP32 ? (g.V + kSiteThreads - 1) / kSiteThreads
            : fix_ ? (g.V + fix_sites(fix_w_) - 1) / fix_sites(fix_w_)
@@ -2162,7 +2247,7 @@ class CgRun final : public CgRunBase {
       off += (bytes + 255) / 256 * 256;
       return o;
     };
-    const size_t o_seed = take(sizeof(SeedState) * L), o_alpha = take(sizeof(double) * L),
+    const size_t o_seed = take(sizeof(SeedState) * L), o_alpha = take(sizeof(double) * L), o_irr = take(sizeof(double) * L),
                  o_vn = take(sizeof(double) * L), o_live = take(sizeof(int) * L), o_tot = take(sizeof(int)),
                  o_ran = take(sizeof(int)), o_rran = take(sizeof(int) * 2), o_err = take(sizeof(int)),
                  o_si = take(sizeof(int) * 2), o_done = take(sizeof(unsigned) * 4),
@@ -2181,6 +2266,7 @@ class CgRun final : public CgRunBase {
     Control& c = c_;
     c.seed = reinterpret_cast<SeedState*>(base + o_seed);
     c.alpha = reinterpret_cast<double*>(base + o_alpha);
+    c.inv_rr = reinterpret_cast<double*>(base + o_irr);
     c.vnorm2 = reinterpret_cast<double*>(base + o_vn);
     c.live = reinterpret_cast<int*>(base + o_live);
     c.live_total = reinterpret_cast<int*>(base + o_tot);
@@ -2237,8 +2323,8 @@ class CgRun final : public CgRunBase {
     init_control_kernel<<<1, 256, 0, st_>>>(c, vn2, L, N);
     SS_CHECK_LAUNCH();
     count_launches(2);
-    if constexpr (kSeed64) {
-      if (fix_) SS_TRY(pack_fix(p_.as<double2>(), false, L, g.V, pdig_.as<int4>(), pex_.as<int>(), st_));
+    if constexpr (kSeed64 || kSeedDF) {
+      if (fix_) SS_TRY(pack_fix(p_.as<VR>(), L, g.V, pdig_.as<int4>(), pex_.as<int>(), st_));
     }
 
     SS_CUDA(cudaEventCreate(&e0_));
@@ -2606,12 +2692,22 @@ class CgRun final : public CgRunBase {
 
   template <int W>
   void launch_fix(dim3 grid, int par) {
-    if constexpr (kSeed64)
-      launch_chain(cg_stencil_kernel<StencilFix<W>, VR>, grid, StencilFix<W>::kThreads, st_, prio_a_,
-                   basis_ && use_pdl(), c_, L_, par, lat_->g,
-                   StencilFix<W>{wfix::FixView{lat_->ufix.as<int4>(), lat_->fnbr.as<int>(), pdig_.as<int4>(),
-                                               pex_.as<int>(), wfix::fix_tiles(lat_->g.V)}},
+    if constexpr (kSeed64 || kSeedDF) {
+      using Op = StencilFix<W, VR>;
+      launch_chain(cg_stencil_kernel<Op, VR>, grid, Op::kThreads, st_, prio_a_, basis_ && use_pdl(), c_, L_, par,
+                   lat_->g,
+                   Op{wfix::FixView{lat_->ufix.as<int4>(), lat_->fnbr, pdig_.as<int4>(), pex_.as<int>(),
+                                    wfix::fix_tiles(lat_->g.V)}},
                    sigma_, p_.as<VR>(), q_.as<VR>());
+    }
+  }
+
+  void launch_fix(dim3 grid, int par) {
+    switch (fix_w_) {
+      case 1: launch_fix<1>(grid, par); break;
+      case 4: launch_fix<4>(grid, par); break;
+      default: launch_fix<8>(grid, par); break;
+    }
   }
 
   void iteration(int it) {
@@ -2638,7 +2734,9 @@ class CgRun final : public CgRunBase {
         launch_chain(cg_stencil_kernel<Stencil32<LinksF32>, VR>, grid_a, kSiteThreads, st, prio_a_, basis_ && use_pdl(), c, L, par, g,
                     Stencil32<LinksF32>{LinksF32{lat_->u32.as<float4>(), g.V}}, sigma_, p_.as<VR>(), q_.as<VR>());
     } else if constexpr (kSeedDF) {
-      if (stencil_minb() == 3)
+      if (fix_)
+        launch_fix(grid_a, par);
+      else if (stencil_minb() == 3)
         launch_chain(cg_stencil_kernel<StencilDF<3>, VR>, grid_a, kStencilThreadsDF, st, prio_a_,
                      basis_ && use_pdl(), c, L, par, g, StencilDF<3>{lat_->udf.as<float4>()}, sigma_, p_.as<VR>(),
                      q_.as<VR>());
@@ -2647,11 +2745,7 @@ class CgRun final : public CgRunBase {
                      basis_ && use_pdl(), c, L, par, g, StencilDF<4>{lat_->udf.as<float4>()}, sigma_, p_.as<VR>(),
                      q_.as<VR>());
     } else if (fix_) {
-      switch (fix_w_) {
-        case 1: launch_fix<1>(grid_a, par); break;
-        case 4: launch_fix<4>(grid_a, par); break;
-        default: launch_fix<8>(grid_a, par); break;
-      }
+      launch_fix(grid_a, par);
     } else if (balanced_stencil()) {
       if (stencil_minb() == 8)
         launch_chain(cg_stencil_kernel<Stencil64h<8>, VR>, grid_a, kStencilThreads, st, prio_a_,
@@ -2673,9 +2767,9 @@ class CgRun final : public CgRunBase {
     cudaEventRecord(ev_[it], st);
     mark(it, 6, st);
     bool p_done = false;
-    if constexpr (kSeed64) {
+    if constexpr (kSeed64 || kSeedDF) {
       if (fix_) {
-        launch_chain(cg_seed_p_fix_kernel, dim3((g.V + kUpdBlock / 4 - 1) / (kUpdBlock / 4), L), kUpdBlock, st, prio_hi_,
+        launch_chain(cg_seed_p_fix_kernel<VR>, dim3((g.V + kUpdBlock / 4 - 1) / (kUpdBlock / 4), L), kUpdBlock, st, prio_hi_,
                      basis_ && use_pdl(), c, r_out, p_.as<VR>(), pdig_.as<int4>(), pex_.as<int>(), g.V);
         p_done = true;
       }

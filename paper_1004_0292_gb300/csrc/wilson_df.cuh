@@ -134,21 +134,27 @@ __device__ __forceinline__ void block_hops_df8(const LinksDF& lk, const float4* 
   __syncthreads();
 }
 
-// q_i = c0 p_i + c1 g5_i (p_i - kappa (D p)_i) for one spinor component i of
-// site s from its hop sum; returns the float-float share p_i^* q_i of (p, q)
-// (real part).
-__device__ __forceinline__ float2 finish_df1(const Geometry& g, const float4* __restrict__ p,
-                                             float4* __restrict__ q, float2 c0, float2 c1, int s, int i, float4 acc) {
+// q_i = c0 p_i + c1 g5_i (p_i - kappa (D p)_i) for one spinor component i from
+// p_i and its hop sum into o; returns the float-float share p_i^* q_i of
+// (p, q) (real part).
+__device__ __forceinline__ float2 finish_df(const Geometry& g, float4 pv, float2 c0, float2 c1, int i, float4 acc,
+                                            float4& o) {
   const float2 mk = ff::split(-g.kappa);
   const float2 sg = i < 6 ? c1 : ff::neg(c1);
-  const float4 pv = p[i * g.V + s];
   const float4 t = ff::caxpy(pv, mk, acc);  // p - kappa D p
   const float2 cs[2] = {c0, sg};
   const float2 br[2] = {ff::re(pv), ff::re(t)}, bi[2] = {ff::im(pv), ff::im(t)};
-  const float4 o = ff::make(ff::dot<2>(cs, br), ff::dot<2>(cs, bi));
-  q[i * g.V + s] = o;
+  o = ff::make(ff::dot<2>(cs, br), ff::dot<2>(cs, bi));
   const float2 a2[2] = {ff::re(pv), ff::im(pv)}, b2[2] = {ff::re(o), ff::im(o)};
   return ff::dot<2>(a2, b2);
+}
+// the same at site s of a field
+__device__ __forceinline__ float2 finish_df1(const Geometry& g, const float4* __restrict__ p,
+                                             float4* __restrict__ q, float2 c0, float2 c1, int s, int i, float4 acc) {
+  float4 o;
+  const float2 d = finish_df(g, p[i * g.V + s], c0, c1, i, acc, o);
+  q[i * g.V + s] = o;
+  return d;
 }
 
 }  // namespace wcore

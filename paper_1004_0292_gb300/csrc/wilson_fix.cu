@@ -2,7 +2,9 @@
 // integer stencil (wilson_fix.cuh), its link and spinor conversions, and the
 // choice between it and the FP64-pipe kernel (wilson.cu).
 #include <algorithm>
+#include <type_traits>
 
+#include "wilson_df.cuh"
 #include "wilson_fix.cuh"
 
 namespace ssqcd {
@@ -50,26 +52,24 @@ __global__ void neighbour_table_kernel(Geometry g, int* __restrict__ nbr) {
 // Fields to digits: four lanes a site (spin q), eight sites a warp.  USER: in
 // is [f][V][12] (the caller's layout), else [f][12][V].  Bound by memory: 16 B
 // read and 16 B written a component.
-template <bool USER>
+template <typename V2, bool USER>
 __global__ void __launch_bounds__(256)
-pack_fix_kernel(const double2* __restrict__ in, int4* __restrict__ dig, int* __restrict__ ex, int V) {
+pack_fix_kernel(const V2* __restrict__ in, int4* __restrict__ dig, int* __restrict__ ex, int V) {
   const int lane = threadIdx.x & 31, q = lane >> 3;
   const int s = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 8 + (lane & 7);
   const size_t f = blockIdx.y;
-  double2 v[3];
+  V2 v[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a)
-    v[a] = s >= V ? make_double2(0.0, 0.0)
-                  : USER ? __ldg(in + (f * V + s) * 12 + 3 * q + a) : __ldg(in + (f * 12 + 3 * q + a) * V + s);
+    v[a] = s >= V ? V2{} : USER ? __ldg(in + (f * V + s) * 12 + 3 * q + a) : __ldg(in + (f * 12 + 3 * q + a) * V + s);
   const int e = quad_site_exp(v);
   if (s >= V) return;
   const int tiles = fix_tiles(V);
   if (q == 0) ex[f * tiles * kTile + s] = e;
-  const int exmax = e + 1022;
   const bool none = e == kZeroExp || e == kSpecialExp;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
-    dig[field_at(tiles, f, s) + (3 * q + a) * kTile] = none ? make_int4(0, 0, 0, 0) : to_digits(v[a], exmax);
+    dig[field_at(tiles, f, s) + (3 * q + a) * kTile] = none ? make_int4(0, 0, 0, 0) : to_site_digits(v[a], e);
 }
 
 // (D psi)(s), component comp, in FP64 from the links and the field as they
@@ -118,20 +118,23 @@ __device__ __noinline__ double2 hop_sum_fp64(const Geometry& g, const double2* _
   return sum;
 }
 
-// out = A in for all right-hand sides.  A warp covers 16 sites of
+// out = A in for all right-hand sides (FP64, or float-float where V2 is
+// float4: every part but the integers in float-float).  A warp covers 16 sites of
 // one right-hand side (half-warp r: spin row r) and W warps share its hops;
 // RB right-hand sides of the same sites sit in one block, so that a link is
 // fetched from L2 once for them.  Consecutive blocks take the further
 // right-hand sides of the same sites (nrb of them).
-template <int W, bool USER>
+template <int W, typename V2, bool USER>
 __global__ void __launch_bounds__(fix_threads(W), fix_min_blocks(W))
-wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const double2* __restrict__ in,
-                  double2* __restrict__ out, int nrhs, int RB, int nrb) {
+wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const V2* __restrict__ in,
+                  V2* __restrict__ out, int nrhs, int RB, int nrb) {
+  constexpr bool kFF = std::is_same<V2, float4>::value;  // float-float fields
+  static_assert(!(kFF && USER), "the caller's fields are FP64");
   constexpr int kWarps = fix_threads(W) / 32;
   constexpr int kUnits = kWarps / W;  // (site group, rhs) units a block
   // W > 1: the warps' hop sums; W = 1: two operand stages a warp
   __shared__ longlong2 part[W > 1 ? kWarps * 6 * 32 : kWarps * kWarpStages];
-  __shared__ double2 stage[USER && W > 1 ? kUnits * kFixSites * 13 : 1];
+  __shared__ V2 stage[USER && W > 1 ? kUnits * kFixSites * 13 : 1];
   const int V = g.V;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int unit = w / W, sub = w % W;
@@ -142,16 +145,16 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
   const bool work = f < nrhs && s0 < V;
   const int fc = min(f, nrhs - 1);
   const int s = min(s0 + i, V - 1);
-  const double2* inf = in + (size_t)fc * 12 * V;
-  double2* outf = out + (size_t)fc * 12 * V;
+  const V2* inf = in + (size_t)fc * 12 * V;
+  V2* outf = out + (size_t)fc * 12 * V;
   // the sites' own components (USER): W > 1 an array of their own, W = 1 the
   // stage of hop 6 once that is done
-  double2* st = W > 1 ? stage + (USER ? unit * kFixSites * 13 : 0) : reinterpret_cast<double2*>(part + w * kWarpStages);
+  V2* st = W > 1 ? stage + (USER ? unit * kFixSites * 13 : 0) : reinterpret_cast<V2*>(part + w * kWarpStages);
   if (W == 1 && !work) return;
   const int own = work ? min(kFixSites, V - s0) * 12 : 0;  // components of the group's sites
   auto stage_at = [](int t) { return t + ((unsigned)t * 21846u >> 18); };  // 13 (t / 12) + t % 12 for t < 192
   if (USER && W > 1 && work) {  // the sites' own components, coalesced
-    const double2* src = inf + (size_t)s0 * 12;
+    const V2* src = inf + (size_t)s0 * 12;
     for (int t = lane + 32 * sub, at = stage_at(t); t < kFixSites * 12; t += 32 * W, at = stage_at(t))
       if (t < own) st[at] = src[t];
   }
@@ -201,17 +204,23 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
     }
     const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
     if (!work || s0 + i >= V) continue;
-    const double2 p = USER ? st[i * 13 + comp] : inf[(size_t)comp * V + s];
-    double2 o;
-    o.x = hop_finish(hf, t.x, p.x);
-    o.y = hop_finish(hf, t.y, p.y);
-    if (k >= 3) o = make_double2(-o.x, -o.y);
-    if (USER)
-      st[i * 13 + comp] = o;
-    else
-      outf[(size_t)comp * V + s] = o;
+    if constexpr (kFF) {
+      float4 d = hop_cff(t, h.E > kMaxExp ? kZeroExp : h.E);
+      if (h.E > kMaxExp) d = make_float4(nanf(""), nanf(""), nanf(""), nanf(""));
+      wcore::finish_df1(g, inf, outf, make_float2(0.f, 0.f), make_float2(1.f, 0.f), s, comp, d);
+    } else {
+      const double2 p = USER ? st[i * 13 + comp] : inf[(size_t)comp * V + s];
+      double2 o;
+      o.x = hop_finish(hf, t.x, p.x);
+      o.y = hop_finish(hf, t.y, p.y);
+      if (k >= 3) o = make_double2(-o.x, -o.y);
+      if (USER)
+        st[i * 13 + comp] = o;
+      else
+        outf[(size_t)comp * V + s] = o;
+    }
   }
-  if (work && s0 + i < V && h.E > kMaxExp) {  // next to a value the digits do not hold: FP64
+  if constexpr (!kFF) if (work && s0 + i < V && h.E > kMaxExp) {  // next to a value the digits do not hold: FP64
     for (int k = sub; k < 6; k += W) {
       const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
       const double2 p = USER ? in[((size_t)fc * V + s) * 12 + comp] : inf[(size_t)comp * V + s];
@@ -231,24 +240,64 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
       __syncthreads();
     else
       __syncwarp();
-    double2* dst = outf + (size_t)s0 * 12;
+    V2* dst = outf + (size_t)s0 * 12;
     for (int t = lane + 32 * sub; t < own; t += 32 * W) dst[t] = st[stage_at(t)];
   }
 }
 
-template <int W>
-void launch_apply(bool user, const Geometry& g, const FixView& v, const double2* u64, const double2* in, double2* out,
-                  int nrhs, cudaStream_t s) {
+template <int W, typename V2, bool USER>
+void launch_apply(const Geometry& g, const FixView& v, const double2* u64, const V2* in, V2* out, int nrhs,
+                  cudaStream_t s) {
   constexpr int kUnits = fix_units(W);
-  const int groups = (g.V + kFixSites - 1) / kFixSites;
+  const int groups = fix_tiles(g.V);
   int RB = 1;
   while (2 * RB <= kUnits && 2 * RB <= nrhs) RB *= 2;
   const int nrb = (nrhs + RB - 1) / RB, gb = (groups + kUnits / RB - 1) / (kUnits / RB);
   const unsigned blocks = (unsigned)gb * nrb;
-  if (user)
-    wilson_fix_kernel<W, true><<<blocks, fix_threads(W), 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
-  else
-    wilson_fix_kernel<W, false><<<blocks, fix_threads(W), 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
+  wilson_fix_kernel<W, V2, USER><<<blocks, fix_threads(W), 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
+}
+
+template <typename V2, bool USER>
+int pack_fields(const V2* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s) {
+  pack_fix_kernel<V2, USER><<<dim3((V + 63) / 64, nrhs), 256, 0, s>>>(in, dig, ex, V);
+  count_launches(1);
+  SS_CHECK_LAUNCH();
+  return SSQCD_OK;
+}
+
+// digits of the block of fields, then the stencil
+template <typename V2, bool USER>
+int apply_block(ssqcd_lattice lat, const V2* in, V2* out, int nrhs, int4* dig, int* ex, cudaStream_t s) {
+  const Geometry& g = lat->g;
+  const double2* u64 = lat->u64.as<double2>();
+  SS_TRY((pack_fields<V2, USER>(in, nrhs, g.V, dig, ex, s)));
+  const FixView v{lat->ufix.as<int4>(), lat->fnbr, dig, ex, fix_tiles(g.V)};
+  switch (fix_split(g.V, nrhs)) {
+    case 1: launch_apply<1, V2, USER>(g, v, u64, in, out, nrhs, s); break;
+    case 4: launch_apply<4, V2, USER>(g, v, u64, in, out, nrhs, s); break;
+    default: launch_apply<8, V2, USER>(g, v, u64, in, out, nrhs, s); break;
+  }
+  count_launches(1);
+  SS_CHECK_LAUNCH();
+  return SSQCD_OK;
+}
+
+// The integer form for all right-hand sides, a block at a time; false in *done
+// when there is no room for the digits.
+template <typename V2, bool USER>
+int apply_fix(ssqcd_lattice lat, const V2* in, V2* out, int nrhs, cudaStream_t s, bool* done) {
+  const int V = lat->g.V, nb = fix_block(V, nrhs);
+  const size_t db = fix_field_bytes(V) * nb;
+  DevBuf ws;
+  *done = false;
+  if (ws.alloc(db + fix_exp_bytes(V) * nb) != SSQCD_OK) return SSQCD_OK;
+  for (int f = 0; f < nrhs; f += nb) {
+    const size_t off = (size_t)f * 12 * V;
+    SS_TRY((apply_block<V2, USER>(lat, in + off, out + off, std::min(nb, nrhs - f), ws.as<int4>(),
+                                  reinterpret_cast<int*>(ws.as<char>() + db), s)));
+  }
+  *done = true;
+  return SSQCD_OK;
 }
 
 }  // namespace
@@ -256,15 +305,19 @@ void launch_apply(bool user, const Geometry& g, const FixView& v, const double2*
 size_t fix_field_bytes(int V) { return sizeof(int4) * 12 * kTile * (size_t)fix_tiles(V); }
 size_t fix_exp_bytes(int V) { return sizeof(int) * kTile * (size_t)fix_tiles(V); }
 
-int pack_fix(const double2* in, bool user, int nrhs, int V, int4* dig, int* ex, cudaStream_t s) {
-  const dim3 grid((V + 63) / 64, nrhs);
-  if (user)
-    pack_fix_kernel<true><<<grid, 256, 0, s>>>(in, dig, ex, V);
-  else
-    pack_fix_kernel<false><<<grid, 256, 0, s>>>(in, dig, ex, V);
-  count_launches(1);
-  SS_CHECK_LAUNCH();
-  return SSQCD_OK;
+// Scratch of the integer form for a block of right-hand sides: at most 1 GiB
+// at a time (a further block waits for the last one on the stream).
+int fix_block(int V, int nrhs) {
+  const size_t per = fix_field_bytes(V) + fix_exp_bytes(V);
+  const size_t fit = ((size_t)1 << 30) / per;
+  return (int)std::max<size_t>(1, std::min<size_t>({fit, (size_t)nrhs, (size_t)65535}));
+}
+
+int pack_fix(const double2* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s) {
+  return pack_fields<double2, false>(in, nrhs, V, dig, ex, s);
+}
+int pack_fix(const float4* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s) {
+  return pack_fields<float4, false>(in, nrhs, V, dig, ex, s);
 }
 
 // Warps that share the eight hops of 16 sites: 1 once the groups fill the
@@ -276,46 +329,17 @@ int fix_split(int V, int nrhs) {
   return groups >= 608 ? 1 : groups >= 304 ? 4 : 8;
 }
 
-int wilson_fix(ssqcd_lattice lat, const int4* dig, const int* ex, const double2* in, bool user, double2* out, int nrhs,
-               cudaStream_t s) {
-  const Geometry& g = lat->g;
-  const double2* u64 = lat->u64.as<double2>();
-  const FixView v{lat->ufix.as<int4>(), lat->fnbr.as<int>(), dig, ex, fix_tiles(g.V)};
-  switch (fix_split(g.V, nrhs)) {
-    case 1: launch_apply<1>(user, g, v, u64, in, out, nrhs, s); break;
-    case 4: launch_apply<4>(user, g, v, u64, in, out, nrhs, s); break;
-    default: launch_apply<8>(user, g, v, u64, in, out, nrhs, s); break;
-  }
-  count_launches(1);
-  SS_CHECK_LAUNCH();
-  return SSQCD_OK;
-}
-
-// Scratch of the integer form for a block of right-hand sides: at most 1 GiB
-// at a time (a further block waits for the last one on the stream).
-int fix_block(int V, int nrhs) {
-  const size_t per = fix_field_bytes(V) + fix_exp_bytes(V);
-  const size_t fit = ((size_t)1 << 30) / per;
-  return (int)std::max<size_t>(1, std::min<size_t>({fit, (size_t)nrhs, (size_t)65535}));
-}
-
 int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s) {
   const Geometry& g = lat->g;
   if (nrhs <= 0) return SSQCD_OK;
   AllocStream scope(s);
   if (lat->fix_ok) {
-    const int nb = fix_block(g.V, nrhs);
-    DevBuf dig, ex;
-    // no room for the digits: the FP64 kernel needs none
-    if (dig.alloc(fix_field_bytes(g.V) * nb) == SSQCD_OK && ex.alloc(fix_exp_bytes(g.V) * nb) == SSQCD_OK) {
-      for (int f = 0; f < nrhs; f += nb) {
-        const int k = std::min(nb, nrhs - f);
-        const size_t off = (size_t)f * 12 * g.V;
-        SS_TRY(pack_fix(in + off, user, k, g.V, dig.as<int4>(), ex.as<int>(), s));
-        SS_TRY(wilson_fix(lat, dig.as<int4>(), ex.as<int>(), in + off, user, out + off, k, s));
-      }
-      return SSQCD_OK;
-    }
+    bool done = false;
+    if (user)
+      SS_TRY((apply_fix<double2, true>(lat, in, out, nrhs, s, &done)));
+    else
+      SS_TRY((apply_fix<double2, false>(lat, in, out, nrhs, s, &done)));
+    if (done) return SSQCD_OK;
   }
   if (!user) return wilson64(g, lat->u64.as<double2>(), in, out, nrhs, 0.0, 1.0, nullptr, nullptr, s);
   DevBuf a, b;
@@ -327,27 +351,44 @@ int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, 
   return unpack_spinors(b.as<double2>(), out, nrhs, g.V, s);
 }
 
+int wilson_df_lat(ssqcd_lattice lat, const float4* in, float4* out, int nrhs, cudaStream_t s) {
+  if (nrhs <= 0) return SSQCD_OK;
+  if (lat->fix_ok) {
+    AllocStream scope(s);
+    bool done = false;
+    SS_TRY((apply_fix<float4, false>(lat, in, out, nrhs, s, &done)));
+    if (done) return SSQCD_OK;
+  }
+  {
+    AllocStream plain(s, false);  // lattice-owned
+    SS_TRY(ensure_df_links(lat));
+  }
+  return wilson_df(lat->g, lat->udf.as<float4>(), in, out, nrhs, 0.0, 1.0, s);
+}
+
 int build_fix_links(ssqcd_lattice lat) {
   const int V = lat->g.V;
   lat->fix_ok = false;
-  DevBuf bad;
-  if (bad.alloc(sizeof(int)) != SSQCD_OK || lat->fnbr.alloc(8 * fix_exp_bytes(V)) != SSQCD_OK ||
-      lat->ufix.alloc(3 * fix_field_bytes(V)) != SSQCD_OK)
-    return SSQCD_OK;  // no room: the FP64 kernel serves the lattice
+  lat->fnbr = nullptr;
+  // links, neighbour table and the check's flag in one allocation
+  const size_t lb = 3 * fix_field_bytes(V), nb = 8 * fix_exp_bytes(V);
+  if (lat->ufix.alloc(lb + nb + sizeof(int)) != SSQCD_OK) return SSQCD_OK;  // no room: the FP64 kernel serves
+  int* nbr = reinterpret_cast<int*>(lat->ufix.as<char>() + lb);
+  int* bad = reinterpret_cast<int*>(lat->ufix.as<char>() + lb + nb);
   int h = 0;
-  SS_CUDA(cudaMemsetAsync(bad.p, 0, sizeof(int), lat->stream));
+  SS_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), lat->stream));
   pack_links_fix_kernel<<<grid_for(4LL * V, 256), 256, 0, lat->stream>>>(lat->u64.as<double2>(), lat->ufix.as<int4>(),
-                                                                         V, bad.as<int>());
-  neighbour_table_kernel<<<grid_for(8LL * V, 256), 256, 0, lat->stream>>>(lat->g, lat->fnbr.as<int>());
+                                                                         V, bad);
+  neighbour_table_kernel<<<grid_for(8LL * V, 256), 256, 0, lat->stream>>>(lat->g, nbr);
   count_launches(2);
   SS_CHECK_LAUNCH();
-  SS_CUDA(cudaMemcpyAsync(&h, bad.p, sizeof(int), cudaMemcpyDeviceToHost, lat->stream));
+  SS_CUDA(cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, lat->stream));
   SS_CUDA(cudaStreamSynchronize(lat->stream));
   lat->fix_ok = h == 0;
-  if (!lat->fix_ok) {
+  if (lat->fix_ok)
+    lat->fnbr = nbr;
+  else
     lat->ufix.release();
-    lat->fnbr.release();
-  }
   return SSQCD_OK;
 }
 

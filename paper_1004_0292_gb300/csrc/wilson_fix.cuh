@@ -1,4 +1,4 @@
-// Integer form of the Wilson stencil for FP64 data (A = gamma5 (I - kappa D),
+// Integer form of the Wilson stencil for FP64 and float-float data (A = gamma5 (I - kappa D),
 // the operator of wilson_core.cuh).
 //
 // GB300 issues 2 FP64 operations a clock and SM and 32 wide integer
@@ -29,6 +29,7 @@
 // order, so every split of the hops over warps gives the same bits.
 #pragma once
 
+#include "floatfloat.cuh"
 #include "internal.h"
 #include "wilson_core.cuh"
 
@@ -72,22 +73,54 @@ __device__ __forceinline__ int4 to_digits(double2 v, int exmax) {
   return make_int4(a.x, a.y, b.x, b.y);
 }
 
+__device__ __forceinline__ int4 to_site_digits(double2 v, int e) { return to_digits(v, e + 1022); }
+
+// Float-float reals (hi + lo): the site exponent from the hi parts, and the
+// digits as the sum of both parts' integers (exact above 2^-60 of the site's
+// largest).
+__device__ __forceinline__ long long float_to_fix(float v, int exmax) {
+  const int b = __float_as_int(v), ex = (b >> 23) & 0xff;
+  const unsigned long long m = (unsigned long long)((b & 0x7fffff) | (ex ? 0x800000 : 0)) << 35;
+  const int d = min(exmax - max(ex, 1), 63);
+  const long long x = (long long)((m + ((1ull << d) >> 1)) >> d);
+  const long long sg = b >> 31;
+  return (x ^ sg) - sg;
+}
+__device__ __forceinline__ int2 to_digits(float hi, float lo, int exmax) {
+  const long long x = float_to_fix(hi, exmax) + float_to_fix(lo, exmax) + (1ll << 29);
+  return make_int2((int)(x >> 30), (int)((unsigned)x & 0x3fffffffu) - (1 << 29));
+}
+__device__ __forceinline__ int4 to_site_digits(float4 v, int e) {
+  const int2 a = to_digits(v.x, v.z, e + 126), b = to_digits(v.y, v.w, e + 126);
+  return make_int4(a.x, a.y, b.x, b.y);
+}
+
 // Four lanes a site (lane = 8 q + j: spin q of site j of eight), three
 // components each: the site's exponent, the same in its four lanes.
-__device__ __forceinline__ int quad_site_exp(const double2 (&v)[3]) {
+__device__ __forceinline__ void site_key(const double2& v, int& key, int& low) {
+  key = max(key, max(abs_key(v.x), abs_key(v.y)));
+  low |= __double2loint(v.x) | __double2loint(v.y);
+}
+__device__ __forceinline__ void site_key(const float4& v, int& key, int&) {
+  key = max(key, max(__float_as_int(v.x) & 0x7fffffff, __float_as_int(v.y) & 0x7fffffff));
+}
+__device__ __forceinline__ int key_exp(double2, int key, int nz) { return site_exp(key, nz != 0); }
+__device__ __forceinline__ int key_exp(float4, int key, int) {
+  const int ex = key >> 23;
+  return key == 0 ? kZeroExp : ex == 255 ? kSpecialExp : max(ex, 1) - 126;
+}
+template <typename V2>
+__device__ __forceinline__ int quad_site_exp(const V2 (&v)[3]) {
   int key = 0, low = 0;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    key = max(key, max(abs_key(v[a].x), abs_key(v[a].y)));
-    low |= __double2loint(v[a].x) | __double2loint(v[a].y);
-  }
+  for (int a = 0; a < 3; ++a) site_key(v[a], key, low);
   int nz = (key | low) != 0;
 #pragma unroll
   for (int o = 8; o <= 16; o <<= 1) {
     key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
     nz |= __shfl_xor_sync(0xffffffffu, nz, o);
   }
-  return site_exp(key, nz != 0);
+  return key_exp(v[0], key, nz);
 }
 
 // ---- layout -----------------------------------------------------------------------------
@@ -411,6 +444,23 @@ __device__ __forceinline__ double hop_finish(double f, long long t, double psi) 
   const double d = (double)t;
   const int hw = __double2hiint(d);
   return fma(f, __hiloint2double(t == 0 ? hw : hw - (200 << 20), __double2loint(d)), psi);
+}
+
+// The same for float-float fields: a hop sum T 2^(E - 57) as float-float, from
+// its three 21-bit parts (exact in FP32), scaled in two steps.
+__device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) << 23); }
+__device__ __forceinline__ float2 hop_ff(long long t, float s1, float s2) {
+  const float a = (float)(int)(t >> 42) * 0x1p42f, b = (float)((int)(t >> 21) & 0x1fffff) * 0x1p21f;
+  const float c = (float)((int)t & 0x1fffff);
+  float s, e, h, l;
+  ff::fast_two_sum(a, b, s, e);
+  ff::fast_two_sum(s, __fadd_rn(e, c), h, l);
+  return make_float2(h * s1 * s2, l * s1 * s2);
+}
+__device__ __forceinline__ float4 hop_cff(longlong2 t, int E) {
+  const int k = E == kZeroExp ? 0 : E - 57, k1 = k / 2;
+  const float s1 = pow2f(k1), s2 = pow2f(k - k1);
+  return ff::make(hop_ff(t.x, s1, s2), hop_ff(t.y, s1, s2));
 }
 
 }  // namespace wfix
