@@ -266,12 +266,22 @@ extern "C" int ssqcd_moments(ssqcd_lattice lat, int N, int M, int L, const doubl
       zi = ni;
     }
   }
+  // the same sum for every component: the caller's order of them does for both
+  AllocStream scope(lat->stream);
   DevBuf yd, sd, scratch;
-  SS_TRY(to_device_layout(lat, y, L * N, on_device, yd));
   const long long n = 12LL * lat->g.V;
-  SS_TRY(sd.alloc(sizeof(double2) * n * M * L));
-  SS_TRY(moments_device(yd.as<double2>(), N, M, L, n, coef.data(), sd.as<double2>(), scratch, lat->stream));
-  SS_TRY(from_device_layout(lat, sd.as<double2>(), L * M, on_device, s_hat));
+  const double2* src = reinterpret_cast<const double2*>(y);
+  double2* dst = reinterpret_cast<double2*>(s_hat);
+  if (!on_device) {
+    SS_TRY(yd.alloc(sizeof(double2) * n * N * L));
+    SS_TRY(sd.alloc(sizeof(double2) * n * M * L));
+    SS_CUDA(cudaMemcpyAsync(yd.p, y, sizeof(double2) * n * N * L, cudaMemcpyHostToDevice, lat->stream));
+    src = yd.as<double2>();
+    dst = sd.as<double2>();
+  }
+  SS_TRY(moments_device(src, N, M, L, n, coef.data(), dst, scratch, lat->stream));
+  if (!on_device)
+    SS_CUDA(cudaMemcpyAsync(s_hat, dst, sizeof(double2) * n * M * L, cudaMemcpyDeviceToHost, lat->stream));
   SS_CUDA(cudaStreamSynchronize(lat->stream));
   return SSQCD_OK;
 }
@@ -282,8 +292,7 @@ int moments_device(const double2* y, int N, int M, int L, long long n, const dou
                    DevBuf& scratch, cudaStream_t s) {
   SS_TRY(scratch.alloc(sizeof(double2) * (size_t)N * M));
   SS_CUDA(cudaMemcpyAsync(scratch.p, coef_host, sizeof(double2) * (size_t)N * M, cudaMemcpyHostToDevice, s));
-  for (int l = 0; l < L; ++l)
-    SS_TRY(combine(y + (long long)l * N * n, N, n, scratch.as<double2>(), M, s_hat + (long long)l * M * n, s));
+  SS_TRY(combine(y, N, n, scratch.as<double2>(), M, s_hat, s, L));
   // the coefficient upload must finish before `scratch` can be reused by the caller
   SS_CUDA(cudaStreamSynchronize(s));
   return SSQCD_OK;

@@ -620,8 +620,14 @@ int cgs2(const double2* S, int m, long long n, double2* Q, double2* R, DevBuf& s
   return SSQCD_OK;
 }
 
-int combine(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s) {
-  if (ms <= 0 || mc <= 0 || n <= 0) return SSQCD_OK;
+namespace {
+
+// Terms (complex multiply-adds) from which the tensor-core combination pays: its
+// four launches and the read of its error word take ~40 us, what the FP64 pipe
+// (four operations a term, 152 x 2 a clock) does for six million terms.
+constexpr double kTcCombineTerms = 8e6;
+
+int combine_fp64(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s) {
   const int cy = (mc + kCC - 1) / kCC;
   long long bx = (n + 255) / 256;
   const long long cap = (4LL * 152 + cy - 1) / cy;
@@ -640,6 +646,26 @@ int combine(const double2* S, int ms, long long n, const double2* C, int mc, dou
   count_launches(1);
   SS_CHECK_LAUNCH();
   return SSQCD_OK;
+}
+
+}  // namespace
+
+int combine(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s, int nl) {
+  if (ms <= 0 || mc <= 0 || n <= 0 || nl <= 0) return SSQCD_OK;
+  if (combine_tc_enabled() && combine_tc_applicable(n, 1, ms) && (double)nl * ms * mc * (double)n >= kTcCombineTerms) {
+    DevBuf work;
+    if (work.alloc(combine_tc_work_bytes(nl, ms)) == SSQCD_OK) {
+      bool suits = false;
+      SS_TRY(combine_tc_vectors(S, ms, n, C, mc, Q, nl, work.p, s, &suits));
+      if (suits) return SSQCD_OK;
+    }
+  }
+  if (nl > 1) {
+    for (int l = 0; l < nl; ++l)
+      SS_TRY(combine_fp64(S + (long long)l * ms * n, ms, n, C, mc, Q + (long long)l * mc * n, s));
+    return SSQCD_OK;
+  }
+  return combine_fp64(S, ms, n, C, mc, Q, s);
 }
 
 int col_residual_norms(const double2* AX, const double2* X, const double* theta, int m, long long n,

@@ -1,20 +1,25 @@
-// Moment combination on the tensor cores (tcgen05), FP64 stored residuals
-// with real coefficients (the line-pair contours):
+// Combinations of FP64 vectors on the tensor cores (tcgen05), with real or
+// complex coefficients:
 //
-//   out[l][o][e] = sum_{s < count[l]} C[l][o][s] r_s[l][e]     (Eq. 2 through
-//   the Krylov-basis identity: every shifted solution is a combination of
-//   the seed residuals)
+//   out[l][o][e] = sum_{s < count[l]} C[l][o][s] r_s[l][e]
+//
+// -- the moments of Eq. 2 and the shifted solutions from the stored seed
+// residuals (the Krylov-basis identity: every shifted solution is a
+// combination of the seed residuals), the moments from solutions in hand, the
+// basis combinations of Rayleigh-Ritz.  A complex coefficient is two real ones
+// (its real and imaginary part combine the same vectors); the epilogue adds
+// the two sums, which sit in neighbouring lanes.
 //
 // GB300's tensor cores have no fast FP64 rate, so the FP64 products are
-// split exactly into bf16 pieces (the error-free splitting of Ozaki et al.,
+// split exactly into fp16 pieces (the error-free splitting of Ozaki et al.,
 // "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication and its applications", 2012):
 //
 // * Each residual r_s (real and imaginary parts as separate rows) is scaled
 //   by tau_s = 2^e_s >= max |r_s| and rounded to a 56-bit fixed-point
 //   integer X = round(|r| 2^(56 - e_s)), whose seven base-256 digits
-//   d_0 .. d_6 (d_0 <= 256) are the bf16 slices A_p = sign d_p (integers,
-//   exact in bf16).
+//   d_0 .. d_6 are the fp16 slices A_p = sign d_p (integers of 8 bits, exact
+//   in fp16, which a byte permutation and one paired multiply-add make).
 // * Each coefficient column o, B[s][o] = C[l][o][s] tau_s, is scaled by
 //   sigma_o = 2^g_o >= max_s |B[s][o]| and split the same way into B_q.
 // * A_p B_q sums 16-bit integer products; 256 of them stay below 2^24, so
@@ -33,10 +38,17 @@
 // within a residual, the fixed-point grid leaves the small ones fewer bits
 // (2.4e-15 against 6.5e-16).
 //
-// One persistent CTA per SM (18 warps):
-// * warp 9, lane 0: bulk copies (cp.async.bulk) of a tile's 16 slots x 128
-//   rows of FP64 into a ring of kF64Stages stages;
-// * warps 10-17: cut the stage into the seven A slices (core-matrix layout,
+// Measured (2502 slots of 786,432 complex elements, 31.5 GB, 16 real outputs,
+// scale pass included): 18.5 ms, 1.7 TB/s.  Before: 34.6 ms -- the scale pass
+// compared in FP64 (15 ms; 5 by integers), one lane issued the copies, each
+// behind a dependent load of the block table (3200 cycles a K-step), and the
+// epilogue converted to 64-bit integers on the FP64 pipe.  The slicing warps'
+// ALU work (~25 instructions an element) and the scale pass bound it now.
+//
+// One persistent CTA per SM (26 warps):
+// * warp 9: bulk copies (cp.async.bulk, a lane a slot) of a tile's 16 slots x
+//   128 rows of FP64 into a ring of kF64Stages stages;
+// * warps 10-25: cut the stage into the seven A slices (core-matrix layout,
 //   K-major, no swizzle) and copy the K-step's B slices (prepared once per
 //   launch in the same layout) into a ring of kSliceStages stages;
 // * warp 8, lane 0: issues seven tcgen05.mma (M = 128, N = 16 (7 - p),
@@ -48,10 +60,13 @@
 // Every wait is bounded (1 s of device time); past it the kernel sets *err,
 // lets its issued copies and MMAs finish, frees its tensor memory and
 // returns.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdlib>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -69,8 +84,8 @@ constexpr int kEpiWarps = 8;
 constexpr int kMmaWarp = 8;
 constexpr int kLoadWarp = 9;
 constexpr int kSliceWarp0 = 10;
-constexpr int kSliceWarps = 8;
-constexpr int kTcThreads = (kSliceWarp0 + kSliceWarps) * 32;  // 576
+constexpr int kSliceWarps = 16;
+constexpr int kTcThreads = (kSliceWarp0 + kSliceWarps) * 32;  // 832
 constexpr int kTmemCols = 512;
 constexpr int kABytes = kRows * kKStep * 2;       // one bf16 slice: 4096 B
 constexpr int kBRows = kSlices * kOut;            // 112
@@ -113,9 +128,9 @@ __device__ __forceinline__ void bar_arrive_tx(unsigned long long* b, unsigned by
 __device__ __forceinline__ bool bar_test(unsigned long long* b, unsigned parity) {
   unsigned ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
-      : "r"(su32(b)), "r"(parity)
+      : "r"(su32(b)), "r"(parity), "r"(2000u)  // the thread may sleep up to 2 us between tests
       : "memory");
   return ok != 0;
 }
@@ -141,6 +156,7 @@ __device__ __forceinline__ bool bar_wait(unsigned long long* b, unsigned parity,
 // the same for all 32 lanes of a warp together: every lane observes the
 // phase (so every lane may read what it guards) and all leave together
 __device__ __forceinline__ bool bar_wait_warp(unsigned long long* b, unsigned parity, volatile int* abort) {
+  if (__all_sync(0xffffffffu, bar_test(b, parity))) return true;
   const unsigned long long t0 = gtimer();
   for (long long i = 0; i < kTcSpin; ++i) {
     if (__all_sync(0xffffffffu, bar_test(b, parity))) return true;
@@ -167,10 +183,10 @@ __device__ __forceinline__ unsigned long long smem_desc(const void* p, unsigned 
          (1ull << 46);
 }
 // Instruction descriptor of kind::f16: fp32 accumulator (bits [4, 6) = 1),
-// A and B bf16 ([7, 10) = 1, [10, 13) = 1), both K-major (bits 15, 16 = 0),
+// A and B fp16 ([7, 10) = 0, [10, 13) = 0), both K-major (bits 15, 16 = 0),
 // N >> 3 at [17, 23), M >> 4 at [24, 29).
-__host__ __device__ constexpr unsigned idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
+__host__ __device__ constexpr unsigned idesc_f16(int M, int N) {
+  return (1u << 4) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
 __device__ __forceinline__ void tc_mma(unsigned d_tmem, unsigned long long a, unsigned long long b, unsigned idesc,
                                        unsigned acc) {
@@ -187,22 +203,14 @@ __device__ __forceinline__ void tc_commit(unsigned long long* bar) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// a[i] += 2^sh x (the 8 consecutive fp32 columns of this thread's lane),
-// each column an integer of magnitude <= 2^24 (exact conversion); load,
-// wait, conversion and addition in one statement
-__device__ __forceinline__ void tc_ld8_add(unsigned taddr, unsigned sh, long long (&a)[8]) {
+// the 8 consecutive fp32 columns of this thread's lane; load and wait in one
+// statement
+__device__ __forceinline__ void tc_ld8(unsigned taddr, float (&t)[8]) {
   asm volatile(
-      "{\n .reg .f32 t<8>;\n .reg .s64 c<8>;\n"
-      " tcgen05.ld.sync.aligned.32x32b.x8.b32 {t0, t1, t2, t3, t4, t5, t6, t7}, [%8];\n"
-      " tcgen05.wait::ld.sync.aligned;\n"
-      " cvt.rni.s64.f32 c0, t0;\n cvt.rni.s64.f32 c1, t1;\n cvt.rni.s64.f32 c2, t2;\n cvt.rni.s64.f32 c3, t3;\n"
-      " cvt.rni.s64.f32 c4, t4;\n cvt.rni.s64.f32 c5, t5;\n cvt.rni.s64.f32 c6, t6;\n cvt.rni.s64.f32 c7, t7;\n"
-      " shl.b64 c0, c0, %9;\n shl.b64 c1, c1, %9;\n shl.b64 c2, c2, %9;\n shl.b64 c3, c3, %9;\n"
-      " shl.b64 c4, c4, %9;\n shl.b64 c5, c5, %9;\n shl.b64 c6, c6, %9;\n shl.b64 c7, c7, %9;\n"
-      " add.s64 %0, %0, c0;\n add.s64 %1, %1, c1;\n add.s64 %2, %2, c2;\n add.s64 %3, %3, c3;\n"
-      " add.s64 %4, %4, c4;\n add.s64 %5, %5, c5;\n add.s64 %6, %6, c6;\n add.s64 %7, %7, c7;\n}\n"
-      : "+l"(a[0]), "+l"(a[1]), "+l"(a[2]), "+l"(a[3]), "+l"(a[4]), "+l"(a[5]), "+l"(a[6]), "+l"(a[7])
-      : "r"(taddr), "r"(sh)
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=f"(t[0]), "=f"(t[1]), "=f"(t[2]), "=f"(t[3]), "=f"(t[4]), "=f"(t[5]), "=f"(t[6]), "=f"(t[7])
+      : "r"(taddr)
       : "memory");
 }
 
@@ -213,70 +221,121 @@ __host__ __device__ constexpr int core_off(int row, int k) {
 }
 constexpr unsigned kLbo = 128, kSbo = 256;
 
-// bf16 bits of the signed integer digit d (0 <= d <= 256): d converted
-// exactly to fp32 by the 2^23 offset, the sign set, the upper half kept
-// (d has at most 9 significant bits and a power of two when it has 9)
-__device__ __forceinline__ unsigned digit_f32(unsigned d, unsigned sgn) {
-  const float f = __int_as_float(0x4B000000 | (int)d) - 8388608.0f;
-  return (unsigned)__float_as_int(f) | sgn;
+// 56-bit fixed point X = round(|x| 2^(56 - e)), ties up, for |x| < 2^e (then
+// X < 2^56): the mantissa m at bit 4, shifted right by e + 1022 - E >= 0 (one
+// bit less than its place), plus one, halved.  Without branches: the lanes of
+// a warp hold elements of different exponents.  Zero and subnormals (E = 0)
+// give 0: e >= -950 (tc_scales_kernel), so that they are shifted out.
+__device__ __forceinline__ uint2 fixed56(double x, int e) {
+  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+  const int E = (int)((hw >> 20) & 0x7FF);
+  const unsigned k = min((unsigned)(e + 1022 - E), 63u);
+  const unsigned long long m = (unsigned long long)__funnelshift_l(lw, (hw & 0xFFFFFu) | 0x100000u, 4) << 32 | (lw << 4);
+  const unsigned long long X = ((m >> k) + 1) >> 1;
+  return make_uint2((unsigned)X, (unsigned)(X >> 32));
 }
-__device__ __forceinline__ unsigned pack_bf16(unsigned lo_f32, unsigned hi_f32) {
-  return __byte_perm(lo_f32, hi_f32, 0x7632);
+// Signed digits (complex combinations): X with its sign plus the bias that
+// makes every base-256 digit d a byte d + 128 and the top one (|d| <= 256) a
+// field d + 512 of bits 48 ...  The digits' products then average to zero, so
+// that the dropped levels do: with magnitudes and signs they add up
+// coherently, the larger part of the error of a short sum.
+__device__ __forceinline__ uint2 signed_digits(uint2 X, double x) {
+  const long long sg = __double2hiint(x) >> 31;
+  const long long v = (((long long)X.y << 32 | X.x) ^ sg) - sg + 0x0200808080808080ll;
+  return make_uint2((unsigned)v, (unsigned)((unsigned long long)v >> 32));
 }
-// 56-bit fixed point |x| 2^(56 - e), rounded to nearest (ties up); the sign
-// bit in sgn (bit 31).  |x| <= 2^e is required (then X <= 2^56).  Without
-// branches: the lanes of a warp hold elements of different exponents.
-__device__ __forceinline__ unsigned long long fixed56(double x, int e, unsigned& sgn) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  sgn = (unsigned)(bits >> 32) & 0x80000000u;
-  const int E = (int)((bits >> 52) & 0x7FF);
-  const unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  const int sh = E - 1019 - e;                  // X = m 2^sh
-  const int ls = min(max(sh, 0), 4), rs = min(max(-sh, 0), 62);
-  const unsigned long long half = rs > 0 ? (1ull << (rs - 1)) : 0ull;
-  const unsigned long long X = ((m << ls) + half) >> rs;
-  // zero (and subnormals, far below any scale here) and shifts past the last digit
-  return (E == 0 || sh <= -60) ? 0ull : X;
+template <int P>
+__device__ __forceinline__ unsigned signed_pair(uint2 a, uint2 b) {
+  constexpr int byte = 6 - P, k = byte & 3;
+  unsigned v;
+  __half2 off;
+  if constexpr (P == 0) {
+    v = __byte_perm(a.y, b.y, 0x7632) | 0x64006400u;
+    off = __half2half2(__ushort_as_half(0xE600));  // -1536
+  } else {
+    const unsigned wa = byte >= 4 ? a.y : a.x, wb = byte >= 4 ? b.y : b.x;
+    v = (__byte_perm(wa, wb, k | k << 4 | (4 + k) << 8 | (4 + k) << 12) & 0x00FF00FFu) | 0x64006400u;
+    off = __half2half2(__ushort_as_half(0xE480));  // -1152
+  }
+  const __half2 d = __hadd2(*reinterpret_cast<const __half2*>(&v), off);
+  return *reinterpret_cast<const unsigned*>(&d);
+}
+// Slice P of two elements, their digits (byte 6 - P of X) with their signs as
+// two fp16 integers: the bytes under the exponent of 1024, times the signs,
+// less 1024 (exact).  s1: (+-1, +-1), s2: (-+1024, -+1024).
+template <int P>
+__device__ __forceinline__ unsigned digit_pair(uint2 a, uint2 b, __half2 s1, __half2 s2) {
+  constexpr int byte = 6 - P, k = byte & 3;
+  const unsigned wa = byte >= 4 ? a.y : a.x, wb = byte >= 4 ? b.y : b.x;
+  const unsigned v = (__byte_perm(wa, wb, k | k << 4 | (4 + k) << 8 | (4 + k) << 12) & 0x00FF00FFu) | 0x64006400u;
+  const __half2 d = __hfma2(*reinterpret_cast<const __half2*>(&v), s1, s2);
+  return *reinterpret_cast<const unsigned*>(&d);
 }
 
 // ---- scales and coefficient slices --------------------------------------------------------
-__device__ __forceinline__ const double* slot_ptr(char* const* tab, int basis_log, long long n, int L, int l, int s) {
+// Where the vectors are: slot s of source l in the basis blocks tab[s >> log],
+// [slot][L][n] each, or (tab null) at base, [l][slots][n].
+struct SlotMap {
+  char* const* tab;
+  int basis_log, L;
+  const double2* base;
+  long long slots;
+};
+__device__ __forceinline__ const double* slot_ptr(const SlotMap& m, long long n, int l, int s) {
+  if (m.tab == nullptr) return reinterpret_cast<const double*>(m.base + (l * m.slots + s) * n);
+  char* const* tab = m.tab;
+  const int basis_log = m.basis_log, L = m.L;
   const int mask = (1 << basis_log) - 1;
   return reinterpret_cast<const double*>(tab[s >> basis_log]) + 2 * (((long long)(s & mask) * L + l) * n);
 }
 
-// mx[l'][s] = max |component| of r_s of source l0 + l' (as the bits of a
-// non-negative double, so that integer atomicMax orders them); grid
-// (x: element blocks, y: slot, z: source)
-__global__ void tc_maxabs_kernel(char* const* __restrict__ tab, int basis_log, long long n, int L, int l0,
-                                 const int* __restrict__ count, int S, unsigned long long* __restrict__ mx) {
+// Real output o of a pass: the part o & 1 of the complex coefficient o / 2
+// (cplx), or the real part of coefficient o.
+struct CoefView {
+  const double2* c;
+  long long sl, so, ss;  // strides of source, output, slot
+  bool cplx;
+  __device__ __forceinline__ double get(int l, int o, int s) const {
+    const double2 v = c[l * sl + (cplx ? o >> 1 : o) * so + s * ss];
+    return cplx && (o & 1) ? v.y : v.x;
+  }
+};
+__device__ __forceinline__ int slots_of(const int* count, int l, int S) { return count != nullptr ? count[l] : S; }
+
+// mx[l'][s] = the largest high word (exponent and leading mantissa bits, sign
+// off) of a component of r_s of source l0 + l'; infinities and NaN are at
+// least kBadKey; ex[l'][s] (may be null) the sum of the components' exponent
+// fields.  By integers: FP64 comparisons run on a pipe of two a clock
+// and SM (2.1 TB/s with them).  grid (x: element blocks, y: slot, z: source)
+constexpr unsigned kBadKey = 0x7FF00000u;
+__global__ void __launch_bounds__(256)
+tc_maxabs_kernel(SlotMap map, long long n, int l0, const int* __restrict__ count, int S, unsigned* __restrict__ mx,
+                 unsigned long long* __restrict__ ex) {
   const int s = blockIdx.y, lz = blockIdx.z, l = l0 + lz;
-  if (s >= count[l]) return;
-  const double2* r = reinterpret_cast<const double2*>(slot_ptr(tab, basis_log, n, L, l, s));
-  double m = 0.0;
-  bool bad = false;  // a NaN or infinity (fmax would drop a NaN)
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const double2 v = r[e];
-    bad |= !isfinite(v.x) || !isfinite(v.y);
-    m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
-  }
+  if (s >= slots_of(count, l, S)) return;
+  const uint4* r = reinterpret_cast<const uint4*>(slot_ptr(map, n, l, s));
+  unsigned m = 0, se = 0;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += 4 * stride) {
+    uint4 v[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  bad = __any_sync(0xffffffffu, bad);
-  __shared__ double wm[32];
-  __shared__ int wb[32];
-  if ((threadIdx.x & 31) == 0) {
-    wm[threadIdx.x >> 5] = m;
-    wb[threadIdx.x >> 5] = bad ? 1 : 0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      m = fmax(m, wm[w]);
-      bad |= wb[w] != 0;
+    for (int i = 0; i < 4; ++i) v[i] = e + i * stride < n ? __ldg(r + e + i * stride) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const unsigned a = v[i].y & 0x7FFFFFFFu, b = v[i].w & 0x7FFFFFFFu;
+      m = max(m, max(a, b));
+      se += (a >> 20) + (b >> 20);
     }
-    // a non-finite element marks the slot with +infinity (above every finite bit pattern)
-    atomicMax(mx + (size_t)lz * S + s, bad ? 0x7FF0000000000000ull : (unsigned long long)__double_as_longlong(m));
+    if (se >= 1u << 26) {  // 32 lanes of this still fit 32 bits
+      if (ex != nullptr) atomicAdd(ex + (size_t)lz * S + s, (unsigned long long)se);
+      se = 0;
+    }
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(mx + (size_t)lz * S + s, m);
+  if (ex != nullptr) {
+    se = __reduce_add_sync(0xffffffffu, se);
+    if ((threadIdx.x & 31) == 0) atomicAdd(ex + (size_t)lz * S + s, (unsigned long long)se);
   }
 }
 
@@ -287,27 +346,42 @@ __device__ __forceinline__ int exp_above(double x) {
   return e;
 }
 
+// A vector suits the fixed point of its largest component when its components
+// are on average at most kMaxSpread binades below it: then max / rms <= 2^5, the
+// grid's error, 2^-57 of the largest, is below 2^-52 of the rms, and FP64's own
+// rounding of the sum is no smaller (a Gaussian vector: 3 to 4 binades).  A
+// point-like vector is far above it.
+constexpr int kMaxSpread = 5;
+constexpr int kErrWait = 1, kErrSpread = 2;  // bits of the error word
+
 // e[l'][s] (slot scales) and sig[l'][o] = 2^g_o >= max_s |C[l][o][s] 2^e_s|;
 // one block of 256 threads per (source, output).  A non-finite residual
 // element or coefficient makes sig NaN, so that the outputs of that source
 // come out NaN as the FP64 sum's would (the slices themselves stay finite).
-__global__ void tc_scales_kernel(const unsigned long long* __restrict__ mx, const double2* __restrict__ C, int O,
-                                 int S, int l0, const int* __restrict__ count, int* __restrict__ eslot,
-                                 double* __restrict__ sig) {
+__global__ void tc_scales_kernel(const unsigned* __restrict__ mx, CoefView C, int O, int S, int l0,
+                                 const int* __restrict__ count, int* __restrict__ eslot, double* __restrict__ sig,
+                                 const unsigned long long* __restrict__ ex, long long n, int* __restrict__ err) {
   const int lz = blockIdx.x / kOut, o = blockIdx.x % kOut, l = l0 + lz;
-  const int cnt = count[l];
+  const int cnt = slots_of(count, l, S);
   double m = 0.0;
   bool bad = false;
   for (int s = threadIdx.x; s < cnt; s += blockDim.x) {
-    const double ms = __longlong_as_double((long long)mx[(size_t)lz * S + s]);
-    const bool fin = isfinite(ms);
-    const int e = fin ? exp_above(ms) : 0;
+    const unsigned key = mx[(size_t)lz * S + s];
+    const bool fin = key < kBadKey;
+    const int e = fin && key != 0 ? max((int)(key >> 20) - 1022, -950) : 0;  // 2^(e - 1) <= max < 2^e
     bad |= !fin;
+    if (ex != nullptr && o == 0 && key != 0 &&
+        (unsigned long long)(key >> 20) * (unsigned long long)(2 * n) >
+            ex[(size_t)lz * S + s] + (unsigned long long)kMaxSpread * (unsigned long long)(2 * n))
+      atomicOr(err, kErrSpread);
     if (o == 0) eslot[(size_t)lz * S + s] = e;
     if (o < O) {
-      const double c = C[((size_t)l * O + o) * S + s].x;
-      bad |= !isfinite(c);
-      if (isfinite(c)) m = fmax(m, fabs(ldexp(c, e)));
+      // the two parts of a complex coefficient share their scale
+      for (int k = 0; k < (C.cplx ? 2 : 1); ++k) {
+        const double c = C.get(l, o ^ k, s);
+        bad |= !isfinite(c);
+        if (isfinite(c)) m = fmax(m, fabs(ldexp(c, e)));
+      }
     }
   }
 #pragma unroll
@@ -325,6 +399,7 @@ __global__ void tc_scales_kernel(const unsigned long long* __restrict__ mx, cons
       m = fmax(m, wm[w]);
       bad |= wb[w] != 0;
     }
+    if (ex != nullptr && (bad || !isfinite(m) || abs(exp_above(m)) > 950)) atomicOr(err, kErrSpread);
     // every output of the source: a bad slot of this source poisons them all
     sig[(size_t)lz * kOut + o] = (bad || !isfinite(m)) ? __longlong_as_double(0x7FF8000000000000ll)
                                                        : ldexp(1.0, exp_above(m));
@@ -335,44 +410,78 @@ __global__ void tc_scales_kernel(const unsigned long long* __restrict__ mx, cons
 // q * 16 + o of the N x 16 operand holds digit q of C[l][o][s] 2^(e_s - g_o)
 // for the slots s = 16 kk + k; thread t writes the 8 slots k = 8 (t & 1) ..
 // of row t / 2 (16 bytes of one core matrix).
-__global__ void tc_bslices_kernel(const double2* __restrict__ C, int O, int S, int l0, const int* __restrict__ count,
+__global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* __restrict__ count,
                                   const int* __restrict__ eslot, const double* __restrict__ sig, int ksteps_cap,
                                   unsigned char* __restrict__ bimg) {
   const int kk = blockIdx.x, lz = blockIdx.y, l = l0 + lz;
   const int t = threadIdx.x, row = t >> 1, h = t & 1;
   const int q = row / kOut, o = row % kOut;
-  const int cnt = count[l];
-  unsigned w[4];
-  unsigned f[8];
+  const int cnt = slots_of(count, l, S);
+  __align__(16) __half f[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int s = kk * kKStep + 8 * h + i;
-    unsigned d = 0, sgn = 0;
+    int d = 0;
     if (o < O && s < cnt) {
       const int g = exp_above(sig[(size_t)lz * kOut + o]) - 1;  // sig = 2^g
-      const double b = ldexp(C[((size_t)l * O + o) * S + s].x, eslot[(size_t)lz * S + s] - g);
-      sgn = b < 0.0 ? 0x80000000u : 0u;
-      const unsigned long long X = (unsigned long long)llrint(ldexp(fabs(b), 56));
-      d = q == 0 ? (unsigned)(X >> 48) : (unsigned)((X >> (48 - 8 * q)) & 0xFFu);
+      const double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * S + s] - g);
+      if (C.cplx) {  // signed digits
+        long long X = llrint(ldexp(b, 56));
+        for (int k = 6; k >= q; --k) {
+          d = k == 0 ? (int)X : (int)((X + 128) & 0xFF) - 128;
+          X = (X - d) >> 8;
+        }
+      } else {
+        const unsigned long long X = (unsigned long long)llrint(ldexp(fabs(b), 56));
+        d = (int)((X >> (48 - 8 * q)) & 0xFFu);
+        if (b < 0.0) d = -d;
+      }
     }
-    f[i] = digit_f32(d, sgn);
+    f[i] = __int2half_rn(d);
   }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) w[k] = pack_bf16(f[2 * k], f[2 * k + 1]);
   unsigned char* dst = bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes + core_off(row, 8 * h);
-  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(f);
+}
+
+// A sum xh 2^32 + xl (|xh| < 2^50) times 2^e as a double, rounded to nearest
+// from its leading 64 bits, by integers: the FP64 pipe, two a clock and SM, would
+// take a third of the time of a short sum.
+__device__ __forceinline__ double sum_to_double(long long xh, long long xl, int e) {
+  long long t = xh + (xl >> 32);
+  unsigned r = (unsigned)xl;
+  const unsigned sg = (unsigned)(t >> 63) & 0x80000000u;
+  if (t < 0) {
+    t = ~t + (r == 0 ? 1 : 0);
+    r = 0u - r;
+  }
+  const int lz = __clzll(t);
+  const int k = 95 - lz + e + 1023;  // biased exponent of the leading bit
+  if (t == 0 || k <= 0 || k >= 2046) {
+    const double v = ldexp(fma((double)t, 0x1p32, (double)r), e);
+    return sg ? -v : v;
+  }
+  unsigned long long m = (unsigned long long)t << lz;
+  m |= lz <= 32 ? (unsigned long long)(r >> (32 - lz)) : (unsigned long long)r << (lz - 32);
+  m = (m >> 11) + ((m >> 10) & 1);
+  const unsigned long long bits = ((unsigned long long)(k - 1) << 52) + m;
+  return __hiloint2double((int)((unsigned)(bits >> 32) | sg), (int)(unsigned)bits);
 }
 
 // ---- the combination ------------------------------------------------------------------------
+// CPLX: complex coefficients (O real outputs, two for each complex one) and
+// signed digits.  SHORT: at most 64 slots, so that a chunk's sums, below 2^22,
+// turn into integers by an FP32 addition instead of a conversion (16 a clock
+// and SM).
+template <bool CPLX, bool SHORT>
 __global__ void __launch_bounds__(kTcThreads, 1)
-combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int L, int l0, int nl,
-                  const int* __restrict__ count, int S, const int* __restrict__ eslot,
-                  const unsigned char* __restrict__ bimg, int ksteps_cap, const double* __restrict__ sig, int O,
-                  double2* __restrict__ out, int* __restrict__ err) {
+combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restrict__ count, int S,
+                  const int* __restrict__ eslot, const unsigned char* __restrict__ bimg, int ksteps_cap,
+                  const double* __restrict__ sig, int O, long long out_l, double2* __restrict__ out,
+                  int* __restrict__ err) {
   extern __shared__ unsigned char tc_smem_raw[];
   TcShared* sh = reinterpret_cast<TcShared*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long tiles_per_src = (2 * n) / kRows;
+  const long long tiles_per_src = (2 * n + kRows - 1) / kRows;  // the last one may be short
   const long long tiles = tiles_per_src * nl;
   volatile int* abort = &sh->abort;
 
@@ -404,29 +513,33 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
 
   auto give_up = [&]() {
     *abort = 1;
-    atomicExch(err, 3);
+    atomicOr(err, kErrWait);
   };
 
   if (warp == kLoadWarp) {
-    // ---- bulk copies of the FP64 residual rows ----
-    if (lane == 0) {
+    // ---- bulk copies of the FP64 residual rows: lane j issues slot j's ----
+    // (one lane for all sixteen was the kernel's pace: each copy's address
+    // takes a dependent load of the block table, ~3200 cycles a K-step)
+    {
       long long fc = 0;
       bool ok = true;
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         const int lz = (int)(t / tiles_per_src), l = l0 + lz;
         const long long row0 = (t % tiles_per_src) * kRows;
-        const int cnt = count[l], ks = (cnt + kKStep - 1) / kKStep;
+        const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
         for (int kk = 0; kk < ks; ++kk, ++fc) {
           const int st = (int)(fc % kF64Stages);
-          if (fc >= kF64Stages && !bar_wait(sh->empty_f + st, (unsigned)((fc / kF64Stages - 1) & 1), abort)) {
+          const int nv = min(kKStep, cnt - kk * kKStep);
+          const double* src = lane < nv ? slot_ptr(map, n, l, kk * kKStep + lane) + row0 : nullptr;
+          // rows of a short tile past the end keep what the stage held: their sums are not stored
+          const unsigned bytes = (unsigned)min((long long)kRows, 2 * n - row0) * 8u;
+          if (fc >= kF64Stages && !bar_wait_warp(sh->empty_f + st, (unsigned)((fc / kF64Stages - 1) & 1), abort)) {
             ok = false;
             break;
           }
-          const int nv = min(kKStep, cnt - kk * kKStep);
-          bar_arrive_tx(sh->full_f + st, (unsigned)nv * kRows * 8u);
-          for (int j = 0; j < nv; ++j)
-            bulk_copy(sh->f64[st].v[j], slot_ptr(tab, basis_log, n, L, l, kk * kKStep + j) + row0, kRows * 8u,
-                      sh->full_f + st);
+          if (lane == 0) bar_arrive_tx(sh->full_f + st, (unsigned)nv * bytes);
+          __syncwarp();
+          if (lane < nv) bulk_copy(sh->f64[st].v[lane], src, bytes, sh->full_f + st);
         }
       }
       if (!ok) {
@@ -441,29 +554,44 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
       }
     }
   } else if (warp >= kSliceWarp0) {
-    // ---- slices: thread u <-> row u % 128, slots 8 (u / 128) .. + 7 of a K-step ----
+    // ---- slices: thread u <-> row u % 128, slots kPer (u / 128) .. of a K-step ----
+    constexpr int kPer = kKStep * kRows / (kSliceWarps * 32);  // 4 or 8 slots a thread
     const int u = threadIdx.x - kSliceWarp0 * 32;
     const int row = u & (kRows - 1), h = u >> 7;
     long long fc = 0, sc = 0;
     bool ok = true;
     for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int lz = (int)(t / tiles_per_src), l = l0 + lz;
-      const int cnt = count[l], ks = (cnt + kKStep - 1) / kKStep;
+      const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
       for (int kk = 0; kk < ks; ++kk, ++fc, ++sc) {
         const int fs = (int)(fc % kF64Stages), ss = (int)(sc % kSliceStages);
+        const int nv = min(kKStep, cnt - kk * kKStep);
+        int es[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+          es[i] = kPer * h + i < nv ? __ldg(eslot + (size_t)lz * S + kk * kKStep + kPer * h + i) : 0;
         if (!bar_wait_warp(sh->full_f + fs, (unsigned)((fc / kF64Stages) & 1), abort)) {
           ok = false;
           break;
         }
-        const int nv = min(kKStep, cnt - kk * kKStep);
-        unsigned long long X[8];
-        unsigned sg[8];
+        uint2 X[kPer];
+        __half2 s1[kPer / 2], s2[kPer / 2];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int j = 8 * h + i;
-          X[i] = 0ull;
-          sg[i] = 0u;
-          if (j < nv) X[i] = fixed56(sh->f64[fs].v[j][row], __ldg(eslot + (size_t)lz * S + kk * kKStep + j), sg[i]);
+        for (int i = 0; i < kPer; i += 2) {
+          const int j = kPer * h + i;
+          const double a = j < nv ? sh->f64[fs].v[j][row] : 0.0, b = j + 1 < nv ? sh->f64[fs].v[j + 1][row] : 0.0;
+          X[i] = fixed56(a, es[i]);
+          X[i + 1] = fixed56(b, es[i + 1]);
+          if constexpr (CPLX) {
+            X[i] = signed_digits(X[i], a);
+            X[i + 1] = signed_digits(X[i + 1], b);
+          } else {
+            const unsigned sg =
+                ((unsigned)__double2hiint(a) >> 16 & 0x8000u) | ((unsigned)__double2hiint(b) & 0x80000000u);
+            const unsigned o1 = 0x3C003C00u ^ sg, o2 = 0xE400E400u ^ sg;
+            s1[i / 2] = *reinterpret_cast<const __half2*>(&o1);
+            s2[i / 2] = *reinterpret_cast<const __half2*>(&o2);
+          }
         }
         __syncwarp();
         if (lane == 0) bar_arrive(sh->empty_f + fs);
@@ -472,17 +600,29 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
           ok = false;
           break;
         }
+        auto put = [&](auto pc) {
+          constexpr int p = decltype(pc)::value;
+          unsigned w[kPer / 2];
 #pragma unroll
-        for (int p = 0; p < kSlices; ++p) {
-          unsigned f[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const unsigned d = p == 0 ? (unsigned)(X[i] >> 48) : (unsigned)((X[i] >> (48 - 8 * p)) & 0xFFu);
-            f[i] = digit_f32(d, sg[i]);
+          for (int i = 0; i < kPer / 2; ++i) {
+            if constexpr (CPLX)
+              w[i] = signed_pair<p>(X[2 * i], X[2 * i + 1]);
+            else
+              w[i] = digit_pair<p>(X[2 * i], X[2 * i + 1], s1[i], s2[i]);
           }
-          *reinterpret_cast<uint4*>(sh->sl[ss].a[p] + core_off(row, 8 * h)) =
-              make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
-        }
+          unsigned char* dst = sh->sl[ss].a[p] + core_off(row, kPer * h);
+          if constexpr (kPer == 8)
+            *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+          else
+            *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+        };
+        put(std::integral_constant<int, 0>{});
+        put(std::integral_constant<int, 1>{});
+        put(std::integral_constant<int, 2>{});
+        put(std::integral_constant<int, 3>{});
+        put(std::integral_constant<int, 4>{});
+        put(std::integral_constant<int, 5>{});
+        put(std::integral_constant<int, 6>{});
         if (u < kBBytes / 16)
           reinterpret_cast<uint4*>(sh->sl[ss].b)[u] =
               __ldg(reinterpret_cast<const uint4*>(bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes) + u);
@@ -499,7 +639,7 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
       bool ok = true;
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         const int l = l0 + (int)(t / tiles_per_src);
-        const int cnt = count[l], ks = (cnt + kKStep - 1) / kKStep;
+        const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
         for (int kk = 0; kk < ks; ++kk, ++sc) {
           const int ss = (int)(sc % kSliceStages);
           if (kk % kChunkSteps == 0) {
@@ -519,7 +659,7 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
 #pragma unroll
           for (int p = 0; p < kSlices; ++p)
             tc_mma(tmem + (unsigned)col_base(p), smem_desc(sh->sl[ss].a[p], kLbo, kSbo), bd,
-                   idesc_bf16(kRows, kOut * (kSlices - p)), acc);
+                   idesc_f16(kRows, kOut * (kSlices - p)), acc);
           tc_commit(sh->empty_s + ss);
           if (kk % kChunkSteps == kChunkSteps - 1 || kk == ks - 1) {
             tc_commit(&sh->tmem_full);
@@ -543,7 +683,7 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
     for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int lz = (int)(t / tiles_per_src), l = l0 + lz;
       const long long row0 = (t % tiles_per_src) * kRows;
-      const int cnt = count[l], ks = (cnt + kKStep - 1) / kKStep;
+      const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
       const int nch = (ks + kChunkSteps - 1) / kChunkSteps;
       // level sums combined exactly as they arrive: xh = I_0 2^16 + I_1 2^8 +
       // I_2 (< 2^48), xl = I_3 2^24 + I_4 2^16 + I_5 2^8 + I_6 (< 2^56)
@@ -556,16 +696,29 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
           break;
         }
         tc_fence_after();
+        // level by level: the pairs of a level add up in 32 bits
 #pragma unroll
-        for (int p = 0; p < kSlices; ++p)
+        for (int lv = 0; lv < kSlices; ++lv) {
+          unsigned a[8];
 #pragma unroll
-          for (int q = 0; q < kSlices - p; ++q) {
-            const unsigned ta = lane_addr + (unsigned)(col_base(p) + kOut * q + 8 * half);
-            if (p + q <= 2)
-              tc_ld8_add(ta, 8u * (2 - p - q), xh);
-            else
-              tc_ld8_add(ta, 8u * (6 - p - q), xl);
+          for (int p = 0; p <= lv; ++p) {
+            float f[8];
+            tc_ld8(lane_addr + (unsigned)(col_base(p) + kOut * (lv - p) + 8 * half), f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const unsigned v = SHORT ? __float_as_uint(f[i] + 12582912.0f) : (unsigned)__float2int_rn(f[i]);
+              a[i] = p == 0 ? v : a[i] + v;
+            }
           }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (SHORT) a[i] -= (lv + 1) * 0x4B400000u;
+            if (lv <= 2)
+              xh[i] += (long long)(int)a[i] * (1 << 8 * (2 - lv));
+            else
+              xl[i] += (long long)(int)a[i] * (1 << 8 * (6 - lv));
+          }
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) bar_arrive(&sh->tmem_empty);
@@ -575,14 +728,35 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
       long long r = row0 + 32 * quarter + lane;  // real row: element r / 2, part r % 2
       int lo = l, lzo = lz;
       asm volatile("" : "+l"(r), "+r"(lo), "+r"(lzo));
+      if constexpr (!CPLX) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int o = 8 * half + i;
-        if (o < O) {
-          // sum_l I_l 2^(-8 l) = 2^-16 xh + 2^-48 xl
-          double v = fma((double)xl[i], 0x1p-48, (double)xh[i] * 0x1p-16);
-          v *= sig[(size_t)lzo * kOut + o] * 0x1p-16;
-          reinterpret_cast<double*>(out + ((size_t)lo * O + o) * n)[r] = v;
+        for (int i = 0; i < 8; ++i) {
+          const int o = 8 * half + i;
+          if (o < O && r < 2 * n) {
+            // sum_l I_l 2^(-8 l) = 2^-16 xh + 2^-48 xl
+            double v = fma((double)xl[i], 0x1p-48, (double)xh[i] * 0x1p-16);
+            v *= sig[(size_t)lzo * kOut + o] * 0x1p-16;
+            reinterpret_cast<double*>(out + lo * out_l + (long long)o * n)[r] = v;
+          }
+        }
+      } else {
+        // (c x).re = Re c x.re - Im c x.im, (c x).im = Re c x.im + Im c x.re: the
+        // element's two parts sit in lanes 2 j and 2 j + 1, the sums with Re c
+        // and Im c have one scale and add as integers
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+          const int o = 8 * half + i;
+          if (o < O) {
+            const long long m = lane & 1 ? 0 : -1;
+            const long long bh = __shfl_xor_sync(0xffffffffu, xh[i + 1], 1);
+            const long long bl = __shfl_xor_sync(0xffffffffu, xl[i + 1], 1);
+            const double sc = sig[(size_t)lzo * kOut + o];
+            // sig 2^-64 (2^32 xh + xl); a scale that is no number poisons the sum
+            double v = sum_to_double(xh[i] + (bh ^ m) - m, xl[i] + (bl ^ m) - m,
+                                     (int)((unsigned)__double2hiint(sc) >> 20) - 1023 - 64);
+            if (sc != sc) v = sc;
+            if (r < 2 * n) reinterpret_cast<double*>(out + lo * out_l + (long long)(o / 2) * n)[r] = v;
+          }
         }
       }
     }
@@ -597,7 +771,8 @@ combine_tc_kernel(char* const* __restrict__ tab, int basis_log, long long n, int
 }
 
 struct TcWork {
-  unsigned long long* mx;
+  unsigned long long* ex;
+  unsigned* mx;
   int* eslot;
   double* sig;
   unsigned char* bimg;
@@ -607,8 +782,10 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 TcWork carve(void* w, int nl, int S, int ksteps_cap) {
   char* p = static_cast<char*>(w);
   TcWork t;
-  t.mx = reinterpret_cast<unsigned long long*>(p);
+  t.ex = reinterpret_cast<unsigned long long*>(p);
   p += align256(sizeof(unsigned long long) * (size_t)nl * S);
+  t.mx = reinterpret_cast<unsigned*>(p);
+  p += align256(sizeof(unsigned) * (size_t)nl * S);
   t.eslot = reinterpret_cast<int*>(p);
   p += align256(sizeof(int) * (size_t)nl * S);
   t.sig = reinterpret_cast<double*>(p);
@@ -631,46 +808,85 @@ bool combine_tc_enabled() {
 }
 
 bool combine_tc_applicable(long long n, int O, int S) {
-  return O >= 1 && O <= kOut && n > 0 && (2 * n) % kRows == 0 && S >= 1 && S <= kMaxCount;
+  return O >= 1 && O <= kOut && n > 0 && S >= 1 && S <= kMaxCount;
 }
 
 size_t combine_tc_work_bytes(int nl, int S) {
   const int ks = (S + kKStep - 1) / kKStep;
-  return align256(sizeof(unsigned long long) * (size_t)nl * S) + align256(sizeof(int) * (size_t)nl * S) +
+  return align256(sizeof(unsigned long long) * (size_t)nl * S) + align256(sizeof(unsigned) * (size_t)nl * S) + align256(sizeof(int) * (size_t)nl * S) +
          align256(sizeof(double) * (size_t)nl * kOut) + 256 + (size_t)nl * ks * kBBytes;
 }
+
+namespace {
+
+// The scale pass, then a launch for every kOut real (kOut / 2 complex) outputs.
+// suits (may be null): set to false, the outputs then not to be used, when a
+// vector has too wide a spread (kMaxSpread), an infinity or a NaN.
+int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const int* count, double2* out,
+                long long out_l, int l0, int nl, void* work, cudaStream_t st, bool* suits) {
+  const int ks = (S + kKStep - 1) / kKStep;
+  TcWork w = carve(work, nl, S, ks);
+  unsigned long long* ex = suits != nullptr ? w.ex : nullptr;
+  SS_CUDA(cudaMemsetAsync(w.mx, 0, sizeof(unsigned) * (size_t)nl * S, st));
+  if (ex != nullptr) SS_CUDA(cudaMemsetAsync(ex, 0, sizeof(unsigned long long) * (size_t)nl * S, st));
+  SS_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), st));
+  // blocks of at least 4 elements a thread
+  const unsigned gx = (unsigned)std::max(1LL, std::min(64LL, (n + 1023) / 1024));
+  tc_maxabs_kernel<<<dim3(gx, S, nl), 256, 0, st>>>(map, n, l0, count, S, w.mx, ex);
+  SS_CHECK_LAUNCH();
+  const size_t smem = sizeof(TcShared) + 1024;
+  auto* kern = C.cplx ? (S <= 64 ? combine_tc_kernel<true, true> : combine_tc_kernel<true, false>)
+                      : (S <= 64 ? combine_tc_kernel<false, true> : combine_tc_kernel<false, false>);
+  SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // the same every time
+  int dev = 0, sms = 0;
+  SS_CUDA(cudaGetDevice(&dev));
+  SS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const long long tiles = ((2 * n + kRows - 1) / kRows) * nl;
+  const int grid = (int)(tiles < sms ? tiles : sms);
+  const int per = C.cplx ? kOut / 2 : kOut;
+  for (int o0 = 0; o0 < O; o0 += per) {
+    CoefView Cp = C;
+    Cp.c += o0 * C.so;
+    const int Op = (C.cplx ? 2 : 1) * std::min(per, O - o0);
+    tc_scales_kernel<<<nl * kOut, 256, 0, st>>>(w.mx, Cp, Op, S, l0, count, w.eslot, w.sig, ex, n, w.err);
+    SS_CHECK_LAUNCH();
+    tc_bslices_kernel<<<dim3(ks, nl), 2 * kBRows, 0, st>>>(Cp, Op, S, l0, count, w.eslot, w.sig, ks, w.bimg);
+    SS_CHECK_LAUNCH();
+    kern<<<grid, kTcThreads, smem, st>>>(map, n, l0, nl, count, S, w.eslot, w.bimg, ks, w.sig, Op, out_l,
+                                         out + (long long)o0 * n, w.err);
+    SS_CHECK_LAUNCH();
+    count_launches(3);
+  }
+  count_launches(1);
+  int h_err = 0;
+  SS_CUDA(cudaMemcpyAsync(&h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SS_CUDA(cudaStreamSynchronize(st));
+  if (h_err & kErrWait) return fail(SSQCD_ERR_NOCONV, "combination (tensor cores): a device-side wait hit its limit");
+  if (suits != nullptr) *suits = h_err == 0;
+  return SSQCD_OK;
+}
+
+}  // namespace
 
 int combine_tc(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
                const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st) {
   if (!combine_tc_applicable(n, O, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
-  const int ks = (S + kKStep - 1) / kKStep;
-  TcWork w = carve(work, nl, S, ks);
-  SS_CUDA(cudaMemsetAsync(w.mx, 0, sizeof(unsigned long long) * (size_t)nl * S, st));
-  SS_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), st));
-  tc_maxabs_kernel<<<dim3(64, S, nl), 256, 0, st>>>(tab, basis_log, n, L, l0, count, S, w.mx);
-  SS_CHECK_LAUNCH();
-  tc_scales_kernel<<<nl * kOut, 256, 0, st>>>(w.mx, C, O, S, l0, count, w.eslot, w.sig);
-  SS_CHECK_LAUNCH();
-  tc_bslices_kernel<<<dim3(ks, nl), 2 * kBRows, 0, st>>>(C, O, S, l0, count, w.eslot, w.sig, ks, w.bimg);
-  SS_CHECK_LAUNCH();
-  static const size_t smem = sizeof(TcShared) + 1024;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(combine_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  SS_CUDA(attr);
-  int dev = 0, sms = 0;
-  SS_CUDA(cudaGetDevice(&dev));
-  SS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const long long tiles = (2 * n / kRows) * nl;
-  const int grid = (int)(tiles < sms ? tiles : sms);
-  combine_tc_kernel<<<grid, kTcThreads, smem, st>>>(tab, basis_log, n, L, l0, nl, count, S, w.eslot, w.bimg, ks,
-                                                  w.sig, O, out, w.err);
-  SS_CHECK_LAUNCH();
-  count_launches(4);
-  int h_err = 0;
-  SS_CUDA(cudaMemcpyAsync(&h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  SS_CUDA(cudaStreamSynchronize(st));
-  if (h_err != 0) return fail(SSQCD_ERR_NOCONV, "moment combination (tensor cores): a device-side wait hit its limit");
-  return SSQCD_OK;
+  return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, false}, O, S, count,
+                     out, (long long)O * n, l0, nl, work, st, nullptr);
+}
+
+int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
+                       const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits) {
+  if (O < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
+  return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, true}, O, S, count,
+                     out, (long long)O * n, l0, nl, work, st, suits);
+}
+
+int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,
+                       cudaStream_t st, bool* suits) {
+  if (O < 1 || nl < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
+  return combine_all(SlotMap{nullptr, 0, 1, x, S}, n, CoefView{C, 0, 1, O, true}, O, S, nullptr, out, (long long)O * n,
+                     0, nl, work, st, suits);
 }
 
 }  // namespace ssqcd

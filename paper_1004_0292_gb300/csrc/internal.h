@@ -176,8 +176,10 @@ int sum_partials(const double* partial, int nvec, int nblocks, double* out, cuda
 // formed, the others are left zero (the upper triangle is always complete)
 int gram(const double2* X, int mx, const double2* Y, int my, long long n, double2* G, DevBuf& scratch,
          cudaStream_t s, bool herm = false);
-// Q[c] = sum_a S[a] C[a][c] (C ms x mc row-major, device)
-int combine(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s);
+// Q[l][c] = sum_a S[l][a] C[a][c] (C ms x mc row-major, device) for nl blocks
+// of vectors: on the tensor cores where the work and the vectors suit them
+// (then synchronises s), else on the FP64 pipe
+int combine(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s, int nl = 1);
 // CGS2 QR of the m vectors S (device): Q [m][n] with orthonormal (or zero)
 // vectors and R (m x m row-major, device, upper triangular), S = Q R.
 // group_ready (optional): events after which column groups of `group`
@@ -257,7 +259,7 @@ int basis_moments(const KrylovBasis& b, const double2* coef_host, int M, double2
 // throughout, for comparison)
 bool real_moments_enabled();
 
-// The moment combination on the tensor cores (combine_tc.cu): FP64 residuals
+// Combinations on the tensor cores (combine_tc.cu): FP64 residuals
 // (tab: the basis block table, 2^basis_log slots a block, [slot][L][n]),
 // real coefficients C[l][o][s] (.x), O <= 16 outputs, out[l][o][n] for the
 // sources l0 .. l0 + nl - 1; work: combine_tc_work_bytes(nl, S) bytes.
@@ -267,6 +269,14 @@ bool combine_tc_applicable(long long n, int O, int S);
 size_t combine_tc_work_bytes(int nl, int S);
 int combine_tc(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
                const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st);
+// The same with complex coefficients and any number of outputs (8 a launch).
+// *suits = false (the outputs then not to be used) when a vector does not suit
+// a fixed point relative to its largest component: point-like, not finite.
+int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
+                       const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits);
+// out[l][o] = sum_s C[s][o] x[l][s] for l < nl, vectors of n complex elements
+int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,
+                       cudaStream_t st, bool* suits);
 
 // Solves for L sources already packed on device (v: [L][12][V]); y out
 // [L][N][12][V] (device, FP64).  iters/xi: host arrays [L*N] (may be null).
