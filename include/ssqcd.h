@@ -129,8 +129,12 @@ typedef struct {
                              (32 N L n bytes: up to 32 N iterations) or 4 GiB
                              if more, at most half the free device memory.  A solve that
                              reaches it forms y_j and p-hat_j from the stored
-                             residuals and continues with the per-iteration
-                             updates (the same eigenpairs, other rounding)     */
+                             residuals and continues from them: SSQCD_FP64 with
+                             the residuals of the next iterations in the same
+                             memory, again up to the cap (from nine blocks of
+                             sixteen iterations), otherwise with the
+                             per-iteration updates (the same eigenpairs, other
+                             rounding)                                         */
   int    source_block;    /* 0 (default): all L sources in one shifted-CG run.
                              B with 0 < B < L: the sources run in blocks of B,
                              one shifted-CG run per block, each block's moments
@@ -192,8 +196,9 @@ typedef struct {
                                form: opts.basis)                                  */
   long long timed_shift_updates; /* (source, shift) updates in the timed iterations */
   int    basis;           /* 1: moments from the stored seed residuals; 2: began
-                             so and switched to shift-vector updates at the
-                             memory cap; 0: shift-vector updates throughout    */
+                             so and formed the shift vectors at the memory cap
+                             (opts.basis_max_bytes); 0: shift-vector updates
+                             throughout                                        */
   double basis_bytes;     /* device memory the stored residuals took at most  */
   int    n_converged;     /* accepted pairs with residual <= opts.converged_tol
                              (Rayleigh-Ritz only; the Hankel extraction has no

@@ -471,8 +471,8 @@ __device__ __forceinline__ double sum_to_double(long long xh, long long xl, int 
 // CPLX: complex coefficients (O real outputs, two for each complex one) and
 // signed digits.  SHORT: at most 64 slots, so that a chunk's sums, below 2^22,
 // turn into integers by an FP32 addition instead of a conversion (16 a clock
-// and SM).
-template <bool CPLX, bool SHORT>
+// and SM).  ACC: the sums are added to out.
+template <bool CPLX, bool SHORT, bool ACC>
 __global__ void __launch_bounds__(kTcThreads, 1)
 combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restrict__ count, int S,
                   const int* __restrict__ eslot, const unsigned char* __restrict__ bimg, int ksteps_cap,
@@ -755,7 +755,10 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
             double v = sum_to_double(xh[i] + (bh ^ m) - m, xl[i] + (bl ^ m) - m,
                                      (int)((unsigned)__double2hiint(sc) >> 20) - 1023 - 64);
             if (sc != sc) v = sc;
-            if (r < 2 * n) reinterpret_cast<double*>(out + lo * out_l + (long long)(o / 2) * n)[r] = v;
+            if (r < 2 * n) {
+              double* at = reinterpret_cast<double*>(out + lo * out_l + (long long)(o / 2) * n) + r;
+              *at = ACC ? *at + v : v;
+            }
           }
         }
       }
@@ -821,9 +824,11 @@ namespace {
 
 // The scale pass, then a launch for every kOut real (kOut / 2 complex) outputs.
 // suits (may be null): set to false, the outputs then not to be used, when a
-// vector has too wide a spread (kMaxSpread), an infinity or a NaN.
+// vector has too wide a spread (kMaxSpread), an infinity or a NaN; with add
+// (complex coefficients: the sums are added to out) that is found out before
+// out is touched.
 int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const int* count, double2* out,
-                long long out_l, int l0, int nl, void* work, cudaStream_t st, bool* suits) {
+                long long out_l, int l0, int nl, void* work, cudaStream_t st, bool* suits, bool add = false) {
   const int ks = (S + kKStep - 1) / kKStep;
   TcWork w = carve(work, nl, S, ks);
   unsigned long long* ex = suits != nullptr ? w.ex : nullptr;
@@ -835,8 +840,10 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
   tc_maxabs_kernel<<<dim3(gx, S, nl), 256, 0, st>>>(map, n, l0, count, S, w.mx, ex);
   SS_CHECK_LAUNCH();
   const size_t smem = sizeof(TcShared) + 1024;
-  auto* kern = C.cplx ? (S <= 64 ? combine_tc_kernel<true, true> : combine_tc_kernel<true, false>)
-                      : (S <= 64 ? combine_tc_kernel<false, true> : combine_tc_kernel<false, false>);
+  auto* kern = add       ? combine_tc_kernel<true, false, true>
+               : C.cplx  ? (S <= 64 ? combine_tc_kernel<true, true, false> : combine_tc_kernel<true, false, false>)
+               : S <= 64 ? combine_tc_kernel<false, true, false>
+                         : combine_tc_kernel<false, false, false>;
   SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // the same every time
   int dev = 0, sms = 0;
   SS_CUDA(cudaGetDevice(&dev));
@@ -844,6 +851,21 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
   const long long tiles = ((2 * n + kRows - 1) / kRows) * nl;
   const int grid = (int)(tiles < sms ? tiles : sms);
   const int per = C.cplx ? kOut / 2 : kOut;
+  int h_err = 0;
+  if (add) {  // every output's scales first
+    for (int o0 = 0; o0 < O; o0 += per) {
+      CoefView Cp = C;
+      Cp.c += o0 * C.so;
+      tc_scales_kernel<<<nl * kOut, 256, 0, st>>>(w.mx, Cp, 2 * std::min(per, O - o0), S, l0, count, w.eslot, w.sig, ex, n,
+                                                  w.err);
+      SS_CHECK_LAUNCH();
+      count_launches(1);
+    }
+    SS_CUDA(cudaMemcpyAsync(&h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SS_CUDA(cudaStreamSynchronize(st));
+    if (suits != nullptr) *suits = h_err == 0;
+    if (h_err != 0) return SSQCD_OK;
+  }
   for (int o0 = 0; o0 < O; o0 += per) {
     CoefView Cp = C;
     Cp.c += o0 * C.so;
@@ -858,7 +880,6 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     count_launches(3);
   }
   count_launches(1);
-  int h_err = 0;
   SS_CUDA(cudaMemcpyAsync(&h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
   SS_CUDA(cudaStreamSynchronize(st));
   if (h_err & kErrWait) return fail(SSQCD_ERR_NOCONV, "combination (tensor cores): a device-side wait hit its limit");
@@ -876,10 +897,11 @@ int combine_tc(char* const* tab, int basis_log, long long n, int L, const double
 }
 
 int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
-                       const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits) {
+                       const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits,
+                       bool add) {
   if (O < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
   return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, true}, O, S, count,
-                     out, (long long)O * n, l0, nl, work, st, suits);
+                     out, (long long)O * n, l0, nl, work, st, suits, add);
 }
 
 int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,

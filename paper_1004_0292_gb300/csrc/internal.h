@@ -17,6 +17,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <memory>
+#include <mutex>
 #include <utility>
 #include <string>
 #include <vector>
@@ -114,6 +115,9 @@ struct ssqcd_lattice_s {
   int gauge_version = 0; // bumped by every upload
   int udf_version = -1;  // gauge_version udf was built from
   ssqcd::DevBuf stage;   // staging for host <-> device copies
+  // work spaces of finished apply calls, kept for the next ones (take_workspace)
+  std::mutex ws_mutex;
+  std::vector<std::unique_ptr<ssqcd::DevBuf>> ws;
 };
 
 namespace ssqcd {
@@ -138,7 +142,9 @@ int wilson64(const Geometry& g, const double2* u, const double2* in, double2* ou
 // out = A in through the form that suits the lattice: the integer stencil
 // (wilson_fix.cu) where its links allow it, else wilson64.  user: in and out
 // are in the caller's layout [nrhs][V][12], else [nrhs][12][V].
-int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s);
+// work (may be null): apply_workspace_bytes, else they are allocated on s.
+int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s,
+                 void* work = nullptr);
 int wilson_df_lat(ssqcd_lattice lat, const float4* in, float4* out, int nrhs, cudaStream_t s);  // float-float fields
 // Integer stencil (wilson_fix.cu): fields as digits with one exponent a site,
 // bytes of each for one field; the links take three fields' bytes
@@ -148,6 +154,13 @@ int pack_fix(const double2* in, int nrhs, int V, int4* dig, int* ex, cudaStream_
 int pack_fix(const float4* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
 int fix_split(int V, int nrhs);  // warps that share the hops of 16 sites: 1, 4 or 8
 int fix_block(int V, int nrhs);  // right-hand sides converted at a time
+// A work space of the lattice with at least `bytes`: one that an earlier call
+// gave back, or a new one.  give_workspace takes it back once its stream has
+// been waited for; at most four of at most 256 MiB are kept, until the lattice
+// goes.  (An allocation and its release cost 50 to 150 us, a small apply 15.)
+int take_workspace(ssqcd_lattice lat, size_t bytes, std::unique_ptr<DevBuf>* out);
+void give_workspace(ssqcd_lattice lat, std::unique_ptr<DevBuf> ws);
+size_t apply_workspace_bytes(ssqcd_lattice lat, int nrhs);  // digits of a block
 // digits of the uploaded links (sets ufix, fix_ok)
 int build_fix_links(ssqcd_lattice lat);
 // link_bits 16: FP16 12-parameter links [4][3][V] uint2; 32: FP32 [4][3][V] float4
@@ -272,8 +285,10 @@ int combine_tc(char* const* tab, int basis_log, long long n, int L, const double
 // The same with complex coefficients and any number of outputs (8 a launch).
 // *suits = false (the outputs then not to be used) when a vector does not suit
 // a fixed point relative to its largest component: point-like, not finite.
+// add: the sums are added to out, which is as it was when they do not suit.
 int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
-                       const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits);
+                       const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits,
+                       bool add = false);
 // out[l][o] = sum_s C[s][o] x[l][s] for l < nl, vectors of n complex elements
 int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,
                        cudaStream_t st, bool* suits);
@@ -294,10 +309,12 @@ class CgRunBase {
   virtual bool take_basis(KrylovBasis* out) = 0;
 };
 // basis_cap: bytes the stored residuals may take (Krylov-basis form, FP64 and
-// DF precisions); 0 selects the per-iteration shift-vector updates
+// DF precisions); 0 selects the per-iteration shift-vector updates.  want_y:
+// the solutions are wanted, not the stored residuals; their memory and that of
+// p-hat is taken at once, so that the residuals only use what is left
 int make_cg_run(ssqcd_lattice lat, int N, const double2* z_host, int L, const double2* v, double sigma, double tol,
                 int max_iter, int precision, int reliable_every, double basis_cap, cudaStream_t st,
-                std::unique_ptr<CgRunBase>* out);
+                std::unique_ptr<CgRunBase>* out, bool want_y = false);
 // the basis_cap of a solve from its options and size (n, N points, L
 // sources): 0 when the form does not apply
 double basis_cap_for(int precision, int basis, double basis_max_bytes, long long n, int N, int L);

@@ -1604,38 +1604,46 @@ cg_reliable_kernel(Control c, int L, const double2* __restrict__ v, const double
 }
 
 // ---- Krylov-basis form: coefficients and the combination of stored residuals ----------
+// A run whose residuals reach their memory cap goes on in segments: from
+// iteration k0 the state is y_j, p-hat_j (k0) and the residuals stored since,
+//   y_j = y_j(k0) + g_j(k0) p-hat_j(k0) + sum_{s > k0} g_j(s) scs(s) r_s
+// with the same backward recurrence, and p-hat_j likewise.  The first segment
+// has k0 = 0, y = 0 and p-hat = r_0.
+//
 // g_j(s) scs(s) for every (source, shift) pair, one thread each: the backward
 // recurrence g_j(s) = a_j(s) + b_j(s) g_j(s+1) from s = K_j = iters_j - 1
-// (zero above); gam [L N][S].
-__global__ void basis_gamma_kernel(Control c, int L, int N, int S, double2* __restrict__ gam) {
+// (zero above) down to k0; gam [L N][S], slot s at s - k0.  Slot k0 of a later
+// segment is left out (zero): its coefficient, p-hat's, goes to gp.
+__global__ void basis_gamma_kernel(Control c, int L, int N, int S, double2* __restrict__ gam, int k0,
+                                   double2* __restrict__ gp) {
   const int qi = blockIdx.x * blockDim.x + threadIdx.x;
   const int NL = N * L;
   if (qi >= NL) return;
   const int l = qi / N;
   const int K = c.iters[qi] - 1;
-  double2* gq = gam + (size_t)qi * S;
-  for (int s = S - 1; s > K; --s) gq[s] = make_double2(0.0, 0.0);
+  double2* gq = gam + (size_t)qi * S - k0;
+  for (int s = S - 1 + k0; s > max(K, k0 - 1); --s) gq[s] = make_double2(0.0, 0.0);
   // the recurrence is a chain of dependent FMAs (64 cycles each); the loads
   // of the coefficients it needs are independent of it, so they are issued
   // kG steps ahead
   constexpr int kG = 8;
   double gx = 0.0, gy = 0.0;
-  for (int s1 = K; s1 >= 0; s1 -= kG) {
+  for (int s1 = K; s1 >= k0; s1 -= kG) {
     double2 a[kG], b[kG];
     double sc[kG];
 #pragma unroll
     for (int i = 0; i < kG; ++i) {
       const int s = s1 - i;
-      if (s >= 0) {
+      if (s >= k0) {
         a[i] = basis_coef(c, s, NL, 0)[qi];
         b[i] = basis_coef(c, s, NL, 1)[qi];
-        sc[i] = s == 0 ? 1.0 : basis_scale(c, s - 1, NL, L)[l];
+        sc[i] = s == k0 ? 1.0 : basis_scale(c, s - 1, NL, L)[l];
       }
     }
 #pragma unroll
     for (int i = 0; i < kG; ++i) {
       const int s = s1 - i;
-      if (s >= 0) {
+      if (s >= k0) {
         const double nx = fma(b[i].x, gx, fma(-b[i].y, gy, a[i].x));
         const double ny = fma(b[i].x, gy, fma(b[i].y, gx, a[i].y));
         gx = nx;
@@ -1644,33 +1652,66 @@ __global__ void basis_gamma_kernel(Control c, int L, int N, int S, double2* __re
       }
     }
   }
+  if (gp != nullptr) {
+    gp[qi] = make_double2(gx, gy);
+    if (S > 0) gq[k0] = make_double2(0.0, 0.0);
+  }
 }
 
 // Coefficients of p-hat_j after k iterations for the shifts still live:
-// p-hat_j(k) = sum_{s <= k} (prod_{m=s}^{k-1} b_j(m)) scs(s) r_s; zero for
-// frozen shifts (their p-hat is never used again); P [L N][S].
-__global__ void basis_phat_kernel(Control c, int L, int N, int k, int S, double2* __restrict__ P) {
+// p-hat_j(k) = (prod_{m=k0}^{k-1} b_j(m)) p-hat_j(k0)
+//              + sum_{k0 < s <= k} (prod_{m=s}^{k-1} b_j(m)) scs(s) r_s;
+// zero for frozen shifts (their p-hat is never used again); P [L N][S], pp the
+// first product (null in the first segment: slot 0 holds p-hat_j(0)).
+__global__ void basis_phat_kernel(Control c, int L, int N, int k, int S, double2* __restrict__ P, int k0,
+                                  double2* __restrict__ pp) {
   const int qi = blockIdx.x * blockDim.x + threadIdx.x;
   const int NL = N * L;
   if (qi >= NL) return;
   const int l = qi / N;
   const bool live = c.act[qi] != 0;
-  double2* pq = P + (size_t)qi * S;
+  double2* pq = P + (size_t)qi * S - k0;
   double px = 1.0, py = 0.0;
-  for (int s = S - 1; s >= 0; --s) {
+  for (int s = S - 1 + k0; s >= k0; --s) {
     if (!live || s > k) {
       pq[s] = make_double2(0.0, 0.0);
       continue;
     }
-    const double sc = s == 0 ? 1.0 : basis_scale(c, s - 1, NL, L)[l];
+    const double sc = s == k0 ? 1.0 : basis_scale(c, s - 1, NL, L)[l];
     pq[s] = make_double2(px * sc, py * sc);
-    if (s > 0) {
+    if (s > k0) {
       const double2 b = basis_coef(c, s - 1, NL, 1)[qi];
       const double nx = b.x * px - b.y * py, ny = b.x * py + b.y * px;
       px = nx;
       py = ny;
     }
   }
+  if (pp != nullptr) {
+    pp[qi] = live ? make_double2(px, py) : make_double2(0.0, 0.0);
+    pq[k0] = make_double2(0.0, 0.0);
+  }
+}
+
+// A segment's share of the old state, every (source, shift) pair (blockIdx.y):
+// y += gp p-hat, then p-hat = pp p-hat (pp may be null: not wanted any more).
+__global__ void __launch_bounds__(kUpdBlock)
+segment_state_kernel(const double2* __restrict__ gp, const double2* __restrict__ pp, double2* __restrict__ y,
+                     double2* __restrict__ ph, long long n) {
+  const size_t q = blockIdx.y;
+  const double2 g = gp[q], b = pp != nullptr ? pp[q] : make_double2(0.0, 0.0);
+  for (long long e = blockIdx.x * (long long)kUpdBlock + threadIdx.x; e < n; e += (long long)gridDim.x * kUpdBlock) {
+    const double2 x = ph[q * n + e];
+    double2 v = y[q * n + e];
+    v.x = fma(g.x, x.x, fma(-g.y, x.y, v.x));
+    v.y = fma(g.x, x.y, fma(g.y, x.x, v.y));
+    y[q * n + e] = v;
+    if (pp != nullptr) ph[q * n + e] = make_double2(b.x * x.x - b.y * x.y, b.x * x.y + b.y * x.x);
+  }
+}
+__global__ void __launch_bounds__(kUpdBlock)
+add_vectors_kernel(double2* __restrict__ y, const double2* __restrict__ x, long long count) {
+  for (long long e = blockIdx.x * (long long)kUpdBlock + threadIdx.x; e < count; e += (long long)gridDim.x * kUpdBlock)
+    y[e] = make_double2(y[e].x + x[e].x, y[e].y + x[e].y);
 }
 
 // Moment coefficients of one window: G[l][m][s] = sum_j W[j][m] gam[l][j][s]
@@ -2159,8 +2200,9 @@ class CgRun final : public CgRunBase {
   }
 
   int init(ssqcd_lattice lat, int N, const double2* z_host, int L, const double2* v, double sigma, double tol,
-           int max_iter, int reliable_every, double basis_cap, cudaStream_t st) {
+           int max_iter, int reliable_every, double basis_cap, cudaStream_t st, bool want_y) {
     lat_ = lat;
+    want_y_ = want_y;
     // the Krylov-basis form: 16-byte seed vectors (FP64 or float-float) and
     // shift vectors of the same type, no reliable updates
     basis_ = basis_cap > 0.0 && kBasisCapable && reliable_every <= 0;
@@ -2223,6 +2265,7 @@ class CgRun final : public CgRunBase {
 
     SS_TRY(p_.alloc(sizeof(VR) * n * L));
     SS_TRY(q_.alloc(sizeof(VR) * n * L));
+    if (basis_ && want_y_) SS_TRY(alloc_update_vectors());
     if (basis_) {
       // block table (pinned host mirror, written once per entry) and the
       // first two blocks: slot 0 and the first chunk's residuals
@@ -2232,7 +2275,7 @@ class CgRun final : public CgRunBase {
       SS_TRY(tab_.alloc(sizeof(char*) * tab_cap_));
       SS_CUDA(cudaMallocHost(&h_tab_, sizeof(char*) * (tab_cap_ + 2)));  // + the first two slot pointers
       SS_TRY(ensure_blocks(kChunk + 1));
-      if (!basis_) return fail(SSQCD_ERR_OOM, "stored residuals: the memory cap is below two blocks");
+      if (!basis_ || blocks_.size() < 2) return fail(SSQCD_ERR_OOM, "stored residuals: the memory cap is below two blocks");
     } else {
       SS_TRY(alloc_update_vectors());
     }
@@ -2581,20 +2624,37 @@ class CgRun final : public CgRunBase {
   }
 
   // Blocks for every slot up to kend (and the coefficient records of the
-  // iterations before it); at the memory cap, switch to the update form.
+  // iterations before it); at the memory cap, the next segment.
   int ensure_blocks(int kend) {
-    const size_t need = (size_t)(kend >> kBasisLog) + 1;
-    while (blocks_.size() < need) {
-      if (blocks_.size() >= tab_cap_) return fail(SSQCD_ERR_ARG, "stored residuals: block table full");
-      if ((double)(basis_bytes_ + blk_bytes_) > basis_cap_ && blocks_.size() >= 2) return switch_to_updates();
-      auto b = std::make_unique<DevBuf>();
-      SS_TRY(b->alloc(blk_bytes_));
-      const size_t i = blocks_.size();
+    while (basis_ && blocks_.size() < (size_t)(kend >> kBasisLog) + 1 - blk0_) {
+      if (blk0_ + blocks_.size() >= tab_cap_) return fail(SSQCD_ERR_ARG, "stored residuals: block table full");
+      std::unique_ptr<DevBuf> b;
+      if (!spare_.empty()) {
+        b = std::move(spare_.back());
+        spare_.pop_back();
+      } else if ((double)(basis_bytes_ + blk_bytes_) <= basis_cap_ || blocks_.size() < 2) {
+        b = std::make_unique<DevBuf>();
+        const int st = b->alloc(blk_bytes_);
+        if (st != SSQCD_OK) {
+          // where the solutions' memory is at hand, no more room is the cap
+          if (!want_y_ || blocks_.size() < 3) return st;
+          b.reset();
+          basis_cap_ = (double)basis_bytes_;
+        } else {
+          basis_bytes_ += blk_bytes_;
+          basis_peak_ = std::max(basis_peak_, basis_bytes_);
+        }
+      }
+      if (b == nullptr) {
+        bool over = false;
+        SS_TRY(next_segment(&over));
+        if (over) return SSQCD_OK;
+        continue;
+      }
+      const size_t i = blk0_ + blocks_.size();
       h_tab_[i] = b->as<char>();
       SS_CUDA(cudaMemcpyAsync(tab_.as<char*>() + i, h_tab_ + i, sizeof(char*), cudaMemcpyHostToDevice, st_));
       blocks_.push_back(std::move(b));
-      basis_bytes_ += blk_bytes_;
-      basis_peak_ = std::max(basis_peak_, basis_bytes_);
     }
     return SSQCD_OK;
   }
@@ -2612,7 +2672,7 @@ class CgRun final : public CgRunBase {
     for (int qi = 0; qi < NL; ++qi) {
       int c = it_all[qi];
       if (with_live && act_all[qi]) c = k + 1;
-      cnt[qi / N_] = std::max(cnt[qi / N_], c);
+      cnt[qi / N_] = std::max(cnt[qi / N_], c - k0_);
     }
     int S = 1;
     for (int v : cnt) S = std::max(S, v);
@@ -2624,7 +2684,8 @@ class CgRun final : public CgRunBase {
   }
 
   // End of a run in the Krylov-basis form: the coefficient of every slot in
-  // every solution (the moments are formed from them later).
+  // every solution (the moments are formed from them later), or the solutions
+  // where they are wanted or begun.
   int finish_basis() {
     int k = 0;
     SS_CUDA(cudaMemcpy(&k, c_.seed_iters, sizeof(int), cudaMemcpyDeviceToHost));
@@ -2632,51 +2693,109 @@ class CgRun final : public CgRunBase {
     SS_TRY(slot_counts(k, false, it_all, act_all, &basis_S_));
     const int NL = N_ * L_;
     SS_TRY(gam_.alloc(sizeof(double2) * (size_t)NL * basis_S_));
-    basis_gamma_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, basis_S_, gam_.as<double2>());
+    const bool old = k0_ > 0;
+    DevBuf gp;
+    if (old) SS_TRY(gp.alloc(sizeof(double2) * NL));
+    basis_gamma_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, basis_S_, gam_.as<double2>(), k0_,
+                                                          gp.as<double2>());
     SS_CHECK_LAUNCH();
     count_launches(1);
+    if (!old && !want_y_) return SSQCD_OK;
+    if constexpr (kBasisCapable) {
+      if (old) SS_TRY(add_old_state(gp.as<double2>(), nullptr));
+      SS_TRY(combine_solutions(gam_, basis_S_, yv_, old));
+    }
+    blocks_.clear();
+    spare_.clear();
+    gam_.release();
+    basis_ = false;
     return SSQCD_OK;
   }
 
-  // out[l][j] = sum_s g[l][j][s] r_s: FP64 vectors on the tensor cores where they
-  // suit them (12^4, 4 sources, 32 points, 992 slots: 157 ms on the FP64 pipe)
-  int combine_solutions(const DevBuf& g, int S, V2* out) {
+  int add_old_state(const double2* gp, const double2* pp) {
+    if constexpr (std::is_same<V2, double2>::value) {
+      segment_state_kernel<<<dim3((unsigned)std::min((n_ + kUpdBlock - 1) / kUpdBlock, 64LL), N_ * L_), kUpdBlock, 0,
+                             st_>>>(gp, pp, yv_, ph_.as<V2>(), n_);
+      SS_CHECK_LAUNCH();
+      count_launches(1);
+    }
+    return SSQCD_OK;
+  }
+
+  // out[l][j] = (out[l][j] +) sum_s g[l][j][s] r_s over the segment's slots: on the
+  // tensor cores where the residuals suit them (12^4, 4 sources, 32 points, 992
+  // slots: 28 ms against 157 on the FP64 pipe)
+  int combine_solutions(const DevBuf& g, int S, V2* out, bool add) {
+    char* const* tab = tab_.as<char*>() + blk0_;
     if constexpr (std::is_same<V2, double2>::value && std::is_same<VR, double2>::value) {
       DevBuf work;
       if (combine_tc_enabled() && combine_tc_applicable(n_, 1, S) &&
           work.alloc(combine_tc_work_bytes(L_, S)) == SSQCD_OK) {
         bool suits = false;
-        SS_TRY(combine_tc_complex(tab_.as<char*>(), kBasisLog, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), out, 0,
-                                  L_, work.p, st_, &suits));
+        SS_TRY(combine_tc_complex(tab, kBasisLog, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), out, 0, L_, work.p,
+                                  st_, &suits, add));
         if (suits) return SSQCD_OK;
       }
+      if (add) {
+        DevBuf t;
+        const long long cnt = n_ * N_ * L_;
+        SS_TRY(t.alloc(sizeof(double2) * cnt));
+        SS_TRY((launch_combine<VR, V2>(tab, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), t.as<double2>(), st_)));
+        add_vectors_kernel<<<1216, kUpdBlock, 0, st_>>>(out, t.as<double2>(), cnt);
+        SS_CHECK_LAUNCH();
+        count_launches(1);
+        return SSQCD_OK;
+      }
     }
-    return launch_combine<VR, V2>(tab_.as<char*>(), n_, L_, g.as<double2>(), N_, S, count_.as<int>(), out, st_);
+    return launch_combine<VR, V2>(tab, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), out, st_);
   }
 
-  // At the memory cap: form y_j and p-hat_j from the stored residuals, put
-  // r_k into the parity buffer the next iteration reads, free the blocks and
-  // continue with the per-iteration updates (new chunk graphs).
-  int switch_to_updates() {
+  // At the memory cap: form y_j and p-hat_j from the segment's residuals.  FP64
+  // runs then begin the next segment with the blocks they have, r_k where it
+  // is; float-float ones free the blocks and continue with the per-iteration
+  // updates (new chunk graphs).  *over: no shift is live any more.
+  int next_segment(bool* over) {
     SS_CUDA(cudaStreamSynchronize(st_));
-    int k = 0;
+    int k = 0, live = 0, err = 0;
     SS_CUDA(cudaMemcpy(&k, c_.seed_iters, sizeof(int), cudaMemcpyDeviceToHost));
+    SS_CUDA(cudaMemcpy(&live, c_.live_total, sizeof(int), cudaMemcpyDeviceToHost));
+    SS_CUDA(cudaMemcpy(&err, c_.err, sizeof(int), cudaMemcpyDeviceToHost));
+    *over = live == 0 || err != 0;  // what is launched now does nothing
+    if (*over) return SSQCD_OK;
     std::vector<int> it_all, act_all;
     int S = 0;
     SS_TRY(slot_counts(k, true, it_all, act_all, &S));
-    SS_TRY(alloc_update_vectors());
+    const bool old = k0_ > 0;
+    if (!old && !want_y_) SS_TRY(alloc_update_vectors());
     const int NL = N_ * L_;
-    DevBuf gy, gp;
+    DevBuf gy, gp, go;
     SS_TRY(gy.alloc(sizeof(double2) * (size_t)NL * S));
     SS_TRY(gp.alloc(sizeof(double2) * (size_t)NL * S));
-    basis_gamma_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, S, gy.as<double2>());
+    if (old) SS_TRY(go.alloc(2 * sizeof(double2) * NL));
+    basis_gamma_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, S, gy.as<double2>(), k0_, go.as<double2>());
     SS_CHECK_LAUNCH();
-    basis_phat_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, k, S, gp.as<double2>());
+    basis_phat_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, k, S, gp.as<double2>(), k0_,
+                                                         old ? go.as<double2>() + NL : nullptr);
     SS_CHECK_LAUNCH();
     count_launches(2);
     if constexpr (kBasisCapable) {
-      SS_TRY(combine_solutions(gy, S, yv_));
-      SS_TRY(combine_solutions(gp, S, ph_.as<V2>()));
+      if (old) SS_TRY(add_old_state(go.as<double2>(), go.as<double2>() + NL));
+      SS_TRY(combine_solutions(gy, S, yv_, old));
+      SS_TRY(combine_solutions(gp, S, ph_.as<V2>(), old));
+    }
+    basis_state_ = 2;
+    // every launched chunk has run in full (shifts are live), so k is a chunk's
+    // end and r_k the first slot of its block.  Segments of 128 iterations and
+    // more: a segment's combinations read its residuals 4 N L / 16 times.
+    const size_t keep = (size_t)(k >> kBasisLog) - blk0_;
+    if (std::is_same<V2, double2>::value && k % kBasisBlock == 0 && keep >= 8) {
+      std::vector<std::unique_ptr<DevBuf>> rest;
+      for (size_t i = 0; i < blocks_.size(); ++i) (i < keep ? spare_ : rest).push_back(std::move(blocks_[i]));
+      blocks_.swap(rest);
+      blk0_ += keep;
+      k0_ = k;
+      SS_CUDA(cudaStreamSynchronize(st_));
+      return SSQCD_OK;
     }
     const char* rk = h_tab_[k >> kBasisLog] + (size_t)(k & (kBasisBlock - 1)) * L_ * n_ * sizeof(VR);
     SS_CUDA(cudaMemcpyAsync(r_.p, rk, sizeof(VR) * L_ * n_, cudaMemcpyDeviceToDevice, st_));
@@ -2684,9 +2803,9 @@ class CgRun final : public CgRunBase {
     gy.release();
     gp.release();
     blocks_.clear();
+    spare_.clear();
     basis_bytes_ = 0;
     basis_ = false;
-    basis_state_ = 2;
     c_.tab = nullptr;
     c_.split = 0;  // kernel B takes the shift scalars again
     if (gexec_ != nullptr) cudaGraphExecDestroy(gexec_);
@@ -2852,7 +2971,10 @@ class CgRun final : public CgRunBase {
   int basis_state_ = 0, basis_S_ = 0;
   double basis_cap_ = 0.0;
   size_t blk_vec_ = 0, blk_bytes_ = 0, tab_cap_ = 0, basis_bytes_ = 0, basis_peak_ = 0;
-  std::vector<std::unique_ptr<DevBuf>> blocks_;
+  std::vector<std::unique_ptr<DevBuf>> blocks_, spare_;  // of the segment; to be used again
+  size_t blk0_ = 0;      // block of the segment's first slot
+  int k0_ = 0;           // its first iteration
+  bool want_y_ = false;  // the solutions, not the stored residuals, are wanted
   DevBuf tab_, gam_, count_;
   char** h_tab_ = nullptr;
   bool fix_ = false;  // the integer stencil
@@ -2879,7 +3001,7 @@ class CgRun final : public CgRunBase {
 
 int make_cg_run(ssqcd_lattice lat, int N, const double2* z_host, int L, const double2* v, double sigma, double tol,
                 int max_iter, int precision, int reliable_every, double basis_cap, cudaStream_t st,
-                std::unique_ptr<CgRunBase>* out) {
+                std::unique_ptr<CgRunBase>* out, bool want_y) {
   if (!valid_precision(precision)) return fail(SSQCD_ERR_ARG, "unknown precision");
   if (is_mixed(precision) && precision != lat->precision)
     return fail(SSQCD_ERR_ARG, "a mixed-precision solve needs a lattice created with that precision");
@@ -2889,7 +3011,7 @@ int make_cg_run(ssqcd_lattice lat, int N, const double2* z_host, int L, const do
   auto make = [&](auto* run) -> int {
     std::unique_ptr<CgRunBase> holder(run);
     if (!run) return fail(SSQCD_ERR_OOM, "host allocation failed");
-    SS_TRY(run->init(lat, N, z_host, L, v, sigma, tol, max_iter, reliable_every, basis_cap, st));
+    SS_TRY(run->init(lat, N, z_host, L, v, sigma, tol, max_iter, reliable_every, basis_cap, st, want_y));
     *out = std::move(holder);
     return SSQCD_OK;
   };
@@ -2919,12 +3041,35 @@ int drive(CgRunBase* run) {
 
 }  // namespace
 
+namespace {
+
+// Memory for the stored residuals of a run that wants the solutions, 0 for the
+// update form: a twentieth of the time an iteration's update takes goes into
+// the combination per iteration (8^4 x 4, 32 shifts: 102 us against 5), but it
+// has launches and coefficients of its own, ~200 us, that a run of few or short
+// vectors does not earn back.
+double solutions_cap(long long n, int N, int L, int precision) {
+  if (!(precision == SSQCD_FP64 || precision == SSQCD_FP64_DFSHIFT) || !combine_tc_enabled() || N < 4 || (double)n * N * L < 4e5) return 0.0;
+  const double cap = basis_cap_for(SSQCD_FP64, 1, 0.0, n, N, L);
+  return cap >= 12.0 * 16.0 * 16.0 * (double)n * L ? cap : 0.0;  // at least twelve blocks
+}
+
+}  // namespace
+
 int shifted_cg_device(ssqcd_lattice lat, int N, const double2* z_host, int L, const double2* v, double sigma,
                       double tol, int max_iter, int precision, int reliable_every, DevBuf& y, int* iters_host,
                       double2* xi_host, ShiftedCGOut* out) {
   std::unique_ptr<CgRunBase> run;
-  SS_TRY(make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, precision, reliable_every, 0.0, lat->stream,
-                     &run));
+  // The solutions out of stored residuals, a combination at the end (and at
+  // every cap) instead of an update of y and p-hat in every iteration.  The
+  // seed is FP64 with float-float shift vectors as well, and the solutions then
+  // FP64 throughout.
+  const double cap = solutions_cap(12LL * lat->g.V, N, L, precision);
+  int made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, cap > 0.0 ? SSQCD_FP64 : precision, reliable_every,
+                         cap, lat->stream, &run, cap > 0.0);
+  if (made == SSQCD_ERR_OOM && cap > 0.0)  // the update form needs less
+    made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, precision, reliable_every, 0.0, lat->stream, &run);
+  SS_TRY(made);
   const int status = drive(run.get());
   if (status != SSQCD_OK && status != SSQCD_ERR_BREAKDOWN && status != SSQCD_ERR_NOCONV) return status;
   const int s2 = run->finish(y, iters_host, xi_host, out);

@@ -285,16 +285,17 @@ int apply_block(ssqcd_lattice lat, const V2* in, V2* out, int nrhs, int4* dig, i
 // The integer form for all right-hand sides, a block at a time; false in *done
 // when there is no room for the digits.
 template <typename V2, bool USER>
-int apply_fix(ssqcd_lattice lat, const V2* in, V2* out, int nrhs, cudaStream_t s, bool* done) {
+int apply_fix(ssqcd_lattice lat, const V2* in, V2* out, int nrhs, cudaStream_t s, bool* done, void* work) {
   const int V = lat->g.V, nb = fix_block(V, nrhs);
   const size_t db = fix_field_bytes(V) * nb;
   DevBuf ws;
   *done = false;
-  if (ws.alloc(db + fix_exp_bytes(V) * nb) != SSQCD_OK) return SSQCD_OK;
+  if (work == nullptr && ws.alloc(db + fix_exp_bytes(V) * nb) != SSQCD_OK) return SSQCD_OK;
+  char* dig = work != nullptr ? static_cast<char*>(work) : ws.as<char>();
   for (int f = 0; f < nrhs; f += nb) {
     const size_t off = (size_t)f * 12 * V;
-    SS_TRY((apply_block<V2, USER>(lat, in + off, out + off, std::min(nb, nrhs - f), ws.as<int4>(),
-                                  reinterpret_cast<int*>(ws.as<char>() + db), s)));
+    SS_TRY((apply_block<V2, USER>(lat, in + off, out + off, std::min(nb, nrhs - f),
+                                  reinterpret_cast<int4*>(dig), reinterpret_cast<int*>(dig + db), s)));
   }
   *done = true;
   return SSQCD_OK;
@@ -329,16 +330,16 @@ int fix_split(int V, int nrhs) {
   return groups >= 608 ? 1 : groups >= 304 ? 4 : 8;
 }
 
-int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s) {
+int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s, void* work) {
   const Geometry& g = lat->g;
   if (nrhs <= 0) return SSQCD_OK;
   AllocStream scope(s);
   if (lat->fix_ok) {
     bool done = false;
     if (user)
-      SS_TRY((apply_fix<double2, true>(lat, in, out, nrhs, s, &done)));
+      SS_TRY((apply_fix<double2, true>(lat, in, out, nrhs, s, &done, work)));
     else
-      SS_TRY((apply_fix<double2, false>(lat, in, out, nrhs, s, &done)));
+      SS_TRY((apply_fix<double2, false>(lat, in, out, nrhs, s, &done, work)));
     if (done) return SSQCD_OK;
   }
   if (!user) return wilson64(g, lat->u64.as<double2>(), in, out, nrhs, 0.0, 1.0, nullptr, nullptr, s);
@@ -356,7 +357,7 @@ int wilson_df_lat(ssqcd_lattice lat, const float4* in, float4* out, int nrhs, cu
   if (lat->fix_ok) {
     AllocStream scope(s);
     bool done = false;
-    SS_TRY((apply_fix<float4, false>(lat, in, out, nrhs, s, &done)));
+    SS_TRY((apply_fix<float4, false>(lat, in, out, nrhs, s, &done, nullptr)));
     if (done) return SSQCD_OK;
   }
   {
@@ -364,6 +365,43 @@ int wilson_df_lat(ssqcd_lattice lat, const float4* in, float4* out, int nrhs, cu
     SS_TRY(ensure_df_links(lat));
   }
   return wilson_df(lat->g, lat->udf.as<float4>(), in, out, nrhs, 0.0, 1.0, s);
+}
+
+size_t apply_workspace_bytes(ssqcd_lattice lat, int nrhs) {
+  if (!lat->fix_ok) return 0;
+  const int nb = fix_block(lat->g.V, nrhs);
+  return (fix_field_bytes(lat->g.V) + fix_exp_bytes(lat->g.V)) * nb;
+}
+
+int take_workspace(ssqcd_lattice lat, size_t bytes, std::unique_ptr<DevBuf>* out) {
+  {
+    std::lock_guard<std::mutex> lock(lat->ws_mutex);
+    for (size_t i = 0; i < lat->ws.size(); ++i)
+      if (lat->ws[i]->bytes >= bytes) {
+        *out = std::move(lat->ws[i]);
+        lat->ws.erase(lat->ws.begin() + i);
+        return SSQCD_OK;
+      }
+  }
+  auto b = std::make_unique<DevBuf>();
+  // plain allocation: it may be used on any stream and by any thread next
+  AllocStream plain(nullptr, false);
+  SS_TRY(b->alloc(bytes));
+  *out = std::move(b);
+  return SSQCD_OK;
+}
+
+void give_workspace(ssqcd_lattice lat, std::unique_ptr<DevBuf> ws) {
+  if (ws == nullptr || ws->bytes > ((size_t)256 << 20)) return;
+  std::unique_ptr<DevBuf> out;  // released outside the lock
+  std::lock_guard<std::mutex> lock(lat->ws_mutex);
+  lat->ws.push_back(std::move(ws));
+  if (lat->ws.size() > 4) {  // the smallest goes
+    auto it = std::min_element(lat->ws.begin(), lat->ws.end(),
+                               [](const auto& a, const auto& b) { return a->bytes < b->bytes; });
+    out = std::move(*it);
+    lat->ws.erase(it);
+  }
 }
 
 int build_fix_links(ssqcd_lattice lat) {

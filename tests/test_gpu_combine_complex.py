@@ -9,6 +9,7 @@ import pytest
 from tests._lib import gpu_module
 
 import synthetic
+from oracle import wilson
 
 pytestmark = pytest.mark.gpu
 
@@ -87,10 +88,12 @@ def test_vectors_that_keep_the_fp64_sum(ss, kind):
     assert np.all(np.abs(got - ref) <= (N + M + 16) * 2.0 ** -53 * size)
 
 
+# a cap of a few blocks of stored residuals: y and p-hat come from the
+# combination and the run goes on with updates; a cap of nine or more: it goes
+# on in segments, several of them here (~370 and more iterations)
+@pytest.mark.parametrize("blocks", [6.5, 9.5, 11.5])
 @pytest.mark.parametrize("dims,L", [((5, 4, 3, 8), 2), ((8, 8, 8, 8), 1)])
-def test_solutions_formed_at_the_memory_cap(ss, dims, L):
-    # a cap of a few blocks of stored residuals: y and p-hat come from the
-    # combination, the run goes on with updates and ends where the others do
+def test_solutions_formed_at_the_memory_cap(ss, dims, L, blocks):
     U = synthetic.gauge_field(dims, "smooth", seed=5, eps=0.3)
     v = synthetic.gaussian_sources(dims, L, seed=6)
     lat = ss.create_lattice(dims, 0.12, -1)
@@ -98,8 +101,41 @@ def test_solutions_formed_at_the_memory_cap(ss, dims, L):
     n = 12 * synthetic.volume(dims)
     block = 16 * 16 * n * L + 2 * 16 * 16 * 16 * L + 4096
     base, st0 = ss.ss_moments(lat, (0.10, 0.13), 16, 4, v, basis=0)
-    got, st1 = ss.ss_moments(lat, (0.10, 0.13), 16, 4, v, basis=1, basis_max_bytes=6.5 * block)
+    got, st1 = ss.ss_moments(lat, (0.10, 0.13), 16, 4, v, basis=1, basis_max_bytes=blocks * block)
     assert st0["basis"] == 0 and st1["basis"] == 2
     for l in range(L):
         for k in range(4):
             assert np.linalg.norm(got[l, k] - base[l, k]) <= 1e-8 * np.linalg.norm(base[l, k])
+
+
+@pytest.mark.parametrize("dims,L,N", [((8, 8, 8, 8), 1, 8), ((8, 8, 8, 8), 1, 9), ((8, 8, 8, 9), 2, 12)])
+def test_shifted_solutions_from_stored_residuals(ss, dims, L, N):
+    # both sides of the size from which shifted_cg forms the solutions from the
+    # residuals; a source of zeros, frozen from the start, beside the others
+    U = synthetic.gauge_field(dims, "smooth", seed=5, eps=0.3)
+    v = synthetic.gaussian_sources(dims, L, seed=6)
+    if L > 1:
+        v[0] = 0
+    z = 0.11 + 0.02 * np.linspace(-1, 1, N) + 0.01j * (-1.0) ** np.arange(N)
+    lat = ss.create_lattice(dims, 0.12, -1)
+    ss.upload_gauge(lat, U)
+    code, y, iters, xi, seed_iters = ss.shifted_cg(lat, z, v, tol=1e-10)
+    assert code == ss.OK and seed_iters == iters.max()
+    for l in range(L):
+        for j in range(N):
+            if not v[l].any():
+                assert not y[l, j].any() and iters[l, j] == 0
+                continue
+            r = v[l] - (z[j] * y[l, j] - wilson.apply_H(U, y[l, j], 0.12, dims, -1))
+            # the stopping rule and the drift of the indefinite seed's recurrence, whose
+            # residual passes peaks of a hundred ||v||: 100 it 2^-52 ||A|| ||y||
+            drift = 100 * seed_iters * 2.0 ** -52 * 2.1 * np.linalg.norm(y[l, j])
+            assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(v[l]) + drift
+    # stopped early: the last iterate, as the update form leaves it
+    code, y1, it1, _, _ = ss.shifted_cg(lat, z, v, tol=1e-10, max_iter=40)
+    assert code == ss.ERR_NOCONV and it1.max() == 40
+    live = v[-1]
+    code, y2, it2, _, _ = ss.shifted_cg(lat, z[:3], live[None], tol=1e-10, max_iter=40)  # three points: updates
+    assert code == ss.ERR_NOCONV
+    for j in range(3):
+        assert np.linalg.norm(y1[-1, j] - y2[0, j]) <= 1e-10 * np.linalg.norm(y2[0, j])
