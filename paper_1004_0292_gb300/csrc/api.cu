@@ -158,19 +158,32 @@ namespace {
 int apply_user(ssqcd_lattice lat, const double* in, double* out, int nrhs, int on_device) {
   const double2* src = reinterpret_cast<const double2*>(in);
   double2* dst = reinterpret_cast<double2*>(out);
-  AllocStream scope(lat->stream);
-  DevBuf a, b;
   const size_t bytes = sizeof(double2) * 12 * (size_t)lat->g.V * nrhs;
-  if (!on_device) {
-    SS_TRY(a.alloc(bytes));
-    SS_TRY(b.alloc(bytes));
-    SS_CUDA(cudaMemcpyAsync(a.p, in, bytes, cudaMemcpyHostToDevice, lat->stream));
-    src = a.as<double2>();
-    dst = b.as<double2>();
+  size_t digits = apply_workspace_bytes(lat, nrhs);
+  std::unique_ptr<DevBuf> ws;
+  size_t need = digits + (on_device ? 0 : 2 * bytes);
+  if (need > 0 && take_workspace(lat, need, &ws) != SSQCD_OK) {
+    // no room for all of it: without the digits the FP64 kernel serves
+    need -= digits;
+    digits = 0;
+    if (need > 0) SS_TRY(take_workspace(lat, need, &ws));
   }
-  SS_TRY(wilson64_lat(lat, src, true, dst, nrhs, lat->stream));
-  if (!on_device) SS_CUDA(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, lat->stream));
-  SS_CUDA(cudaStreamSynchronize(lat->stream));
+  char* host = ws != nullptr ? ws->as<char>() + digits : nullptr;
+  auto run = [&]() -> int {
+    if (!on_device) {
+      src = reinterpret_cast<const double2*>(host);
+      dst = reinterpret_cast<double2*>(host + bytes);
+      SS_CUDA(cudaMemcpyAsync(host, in, bytes, cudaMemcpyHostToDevice, lat->stream));
+    }
+    SS_TRY(wilson64_lat(lat, src, true, dst, nrhs, lat->stream, digits > 0 ? ws->p : nullptr));
+    if (!on_device) SS_CUDA(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, lat->stream));
+    return SSQCD_OK;
+  };
+  const int st = run();
+  const cudaError_t e = cudaStreamSynchronize(lat->stream);
+  if (e == cudaSuccess) give_workspace(lat, std::move(ws));
+  SS_TRY(st);
+  SS_CUDA(e);
   return SSQCD_OK;
 }
 
@@ -267,7 +280,6 @@ extern "C" int ssqcd_moments(ssqcd_lattice lat, int N, int M, int L, const doubl
     }
   }
   // the same sum for every component: the caller's order of them does for both
-  AllocStream scope(lat->stream);
   DevBuf yd, sd, scratch;
   const long long n = 12LL * lat->g.V;
   const double2* src = reinterpret_cast<const double2*>(y);
