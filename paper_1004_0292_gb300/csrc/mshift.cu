@@ -267,7 +267,11 @@ __global__ void init_control_kernel(Control c, const double* __restrict__ vn2, i
 // ---- A. stencil q = K p + (p, q) partials; last block: alpha_k ---------------------
 // Stencil of one block for one source: q = sigma p - gamma5 (p - kappa D p) at
 // spin w's three components of site s; returns this thread's share of (p, q).
+// stencils that load nothing ahead of the control words
+struct NoPre {};
 struct Stencil64 {
+  using Pre = NoPre;
+  __device__ __forceinline__ void pre(const Geometry&, Pre&) const {}
   static constexpr bool kThreadPerSite = false;
   static constexpr int kThreads = kStencilThreads;
   static constexpr int kSites = kSitesPerBlock;
@@ -275,7 +279,7 @@ struct Stencil64 {
   static constexpr int kMinBlocks = 4;  // <= 128 registers (four 128-thread blocks per SM)
   const double2* __restrict__ u;
   __device__ __forceinline__ double run(const Geometry& g, const double2* __restrict__ p, double2* __restrict__ q,
-                                        double sigma, int s, int w, void* shm) const {
+                                        double sigma, int s, int w, void* shm, NoPre&) const {
     double2 acc[3];
     block_hops64(Links64{u, g.V}, p, s, g, static_cast<double2*>(shm), acc);
     double d = 0.0;
@@ -303,6 +307,8 @@ struct Stencil64 {
 // 8^4 x 4 rhs) by default, 8 (64 registers, a few spilled) for comparison
 template <int MinB>
 struct Stencil64h {
+  using Pre = NoPre;
+  __device__ __forceinline__ void pre(const Geometry&, Pre&) const {}
   static constexpr bool kThreadPerSite = false;
   static constexpr int kThreads = kStencilThreads;
   static constexpr int kSites = kSitesPerBlockH;
@@ -310,7 +316,7 @@ struct Stencil64h {
   static constexpr int kMinBlocks = MinB;
   const double2* __restrict__ u;
   __device__ __forceinline__ double run(const Geometry& g, const double2* __restrict__ p, double2* __restrict__ q,
-                                        double sigma, int, int, void* shm) const {
+                                        double sigma, int, int, void* shm, NoPre&) const {
     double2* sh = static_cast<double2*>(shm);
     const int s0 = blockIdx.x * kSitesPerBlockH;
     block_hops64h(Links64{u, g.V}, p, s0, g, sh);
@@ -359,20 +365,32 @@ struct StencilFix {
   static constexpr int kShElems = kThreads / 32 * (W > 1 ? 6 * 32 : wfix::kWarpStages);
   static constexpr int kMinBlocks = wfix::fix_min_blocks(W);
   wfix::FixView view;  // of source 0
+  __device__ __forceinline__ int site(int V) const {
+    const int w = threadIdx.x >> 5;
+    return min((int)(blockIdx.x * kUnits + w / W) * wfix::kFixSites + (int)(threadIdx.x & (wfix::kFixSites - 1)), V - 1);
+  }
+  // the neighbours, loaded beside the control words of the kernel's start
+  using Pre = wfix::Hops;
+  __device__ __forceinline__ void pre(const Geometry& g, Pre& h) const { wfix::load_neighbours(view, site(g.V), h); }
   __device__ __forceinline__ double run(const Geometry& g, const V2* __restrict__ p, V2* __restrict__ q,
-                                        double sigma, int, int, void* shm) const {
+                                        double sigma, int, int, void* shm, Pre& h) const {
     longlong2* part = static_cast<longlong2*>(shm);
     const int V = g.V;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int unit = w / W, sub = w % W;
     const int i = lane & (wfix::kFixSites - 1), r = lane >> 4;
     const int s0 = (blockIdx.x * kUnits + unit) * wfix::kFixSites;
-    const int s = min(s0 + i, V - 1);
+    const int s = site(V);
     wfix::FixView v = view;
     v.dig += wfix::field_at(v.tiles, blockIdx.y, 0);
     v.ex += (size_t)blockIdx.y * v.tiles * wfix::kTile;
-    wfix::Hops h;
-    wfix::load_hops(v, s, h);
+    // p at the components this lane finishes (W > 1; W = 1 copies it beside hop 7)
+    V2 own[W > 1 ? (5 + W) / W : 1];
+    if (W > 1) {
+#pragma unroll
+      for (int k = sub, j = 0; j < (5 + W) / W; k += W, ++j)
+        if (k < 6) own[j] = p[(size_t)((k < 3 ? 0 : 6) + r * 3 + k % 3) * V + s];
+    }
     wfix::Acc3 up, lo;
     if constexpr (W == 1) {
       wfix::hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * wfix::kWarpStages), up, lo,
@@ -421,8 +439,7 @@ struct StencilFix {
         }
         if (s0 + i >= V) continue;
         const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
-        const V2 pv = W > 1 ? p[(size_t)comp * V + s]
-                            : reinterpret_cast<const V2*>(part + w * wfix::kWarpStages)[k * 32 + lane];
+        const V2 pv = W > 1 ? own[k / W] : reinterpret_cast<const V2*>(part + w * wfix::kWarpStages)[k * 32 + lane];
         if constexpr (kFF) {
           const float nan = __int_as_float(0x7fc00000);
           const float4 hop = special ? make_float4(nan, nan, nan, nan) : wfix::hop_cff(t, h.E);
@@ -456,6 +473,8 @@ struct StencilFix {
 // FP32 spinors (mixed precisions): one thread per site (memory-bound form)
 template <typename LK>
 struct Stencil32 {
+  using Pre = NoPre;
+  __device__ __forceinline__ void pre(const Geometry&, Pre&) const {}
   static constexpr int kThreads = kSiteThreads;
   static constexpr int kMinBlocks = 1;
   static constexpr bool kThreadPerSite = true;
@@ -463,7 +482,7 @@ struct Stencil32 {
   static constexpr int kShElems = 1;
   LK lk;
   __device__ __forceinline__ double run(const Geometry& g, const float2* __restrict__ p, float2* __restrict__ q,
-                                        double sigma, int s, int, void*) const {
+                                        double sigma, int s, int, void*, NoPre&) const {
     double d = 0.0;
     if (s < g.V) {
       float2 acc[12];
@@ -493,6 +512,8 @@ struct Stencil32 {
 // 57.2 us at 3 blocks an SM, <= 85 registers, 1.12 waves); 3 for comparison
 template <int MinB>
 struct StencilDF {
+  using Pre = NoPre;
+  __device__ __forceinline__ void pre(const Geometry&, Pre&) const {}
   static constexpr bool kThreadPerSite = false;
   static constexpr int kThreads = kStencilThreadsDF;
   static constexpr int kSites = kSitesPerBlock;
@@ -500,7 +521,7 @@ struct StencilDF {
   static constexpr int kMinBlocks = MinB;
   const float4* __restrict__ u;
   __device__ __forceinline__ double run(const Geometry& g, const float4* __restrict__ p, float4* __restrict__ q,
-                                        double sigma, int s, int w, void* shm) const {
+                                        double sigma, int s, int w, void* shm, NoPre&) const {
     float4* sh = static_cast<float4*>(shm);
     const int lane = threadIdx.x & 31;
     block_hops_df8(LinksDF{u, g.V}, p, s, g, sh);
@@ -517,6 +538,15 @@ struct StencilDF {
     return d;
   }
 };
+
+// The block's ticket: releases its thread's partial sums and, for the last one,
+// acquires the others' (the block barrier after it passes both on to the
+// block), in one operation instead of one between two full fences.
+__device__ __forceinline__ unsigned ticket(unsigned* done) {
+  unsigned old;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(done) : "memory");
+  return old;
+}
 
 // Sums of the block partials [L][nb] into sums[L] by one block of W warps (the
 // tail that the whole GPU waits for): L sources share the warps -- with fewer
@@ -556,8 +586,11 @@ template <typename Op, typename V2>
 __global__ void __launch_bounds__(Op::kThreads, Op::kMinBlocks)
 cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, const V2* __restrict__ p_all,
                   V2* __restrict__ q_all) {
+  typename Op::Pre ahead;
+  op.pre(g, ahead);  // what no kernel of the loop writes
   pdl_wait();
-  if (*c.err != 0 || *c.live_total == 0) {
+  const int err = *c.err, live_total = *c.live_total, live_l = c.live[blockIdx.y];
+  if (err != 0 || live_total == 0) {
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *c.ran = c.rec_ran[par] = 0;
     return;
   }
@@ -575,11 +608,15 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
     c.inv_rr[l] = rr > 0.0 ? 1.0 / rr : 0.0;
   }
   double d_pq = 0.0;
-  if (c.live[l] != 0) {
+  if (live_l != 0) {
     const int s = Op::kThreadPerSite ? blockIdx.x * Op::kThreads + (int)threadIdx.x
                                      : blockIdx.x * Op::kSites + lane;
-    d_pq = op.run(g, p_all + (size_t)l * 12 * V, q_all + (size_t)l * 12 * V, sigma, s, w, sh);
+    d_pq = op.run(g, p_all + (size_t)l * 12 * V, q_all + (size_t)l * 12 * V, sigma, s, w, sh, ahead);
   }
+  // what the last block's tail needs of a source, loaded ahead of it
+  const int lt = min((int)threadIdx.x, L - 1);
+  const double rr_t = c.seed[lt].rr;
+  const int live_t = c.live[lt];
   d_pq = warp_sum(d_pq);
   if (lane == 0) sred[w] = d_pq;
   __syncthreads();
@@ -591,24 +628,23 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
     static_assert(kWarps == 4 || kWarps == 8, "four or eight warps");
     c.partial[(size_t)l * nbw + blockIdx.x] = t;
     pdl_trigger();
-    __threadfence();
-    const unsigned ticket = atomicAdd(&c.done[0], 1u);
-    s_last = ticket == gridDim.x * gridDim.y - 1;
+    s_last = ticket(&c.done[0]) == gridDim.x * gridDim.y - 1;
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   tail_sums<kWarps>(c.partial, nbw, L, sums, spart);
-  for (int ls = threadIdx.x; ls < L; ls += blockDim.x) {
-    if (c.live[ls] == 0) continue;
+  static_assert(kMaxSources <= Op::kThreads, "a thread a source");
+  if ((int)threadIdx.x < L && live_t != 0) {
+    const int ls = threadIdx.x;
     const double pq = sums[ls];
-    const double rr = c.seed[ls].rr;
+    const double rr = rr_t;
     if (!(fabs(pq) >= 1e-30 * rr)) {  // breakdown (also catches NaN)
       atomicExch(c.err, 1);
-      continue;
+    } else {
+      const double alpha = rr / pq;
+      c.alpha[ls] = alpha;
+      if (c.split) c.alpha_rec[par * L + ls] = alpha;
     }
-    c.alpha[ls] = rr / pq;
-    if (c.split) c.alpha_rec[par * L + ls] = rr / pq;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -638,9 +674,13 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
                const V2* __restrict__ q, const V2* __restrict__ p, long long n, double rescale_below,
                double rescale_by) {
   pdl_wait();
-  // the control words this block needs, loaded together (one round trip)
+  // The control words this block needs, loaded together (one round trip), and
+  // further down those of the last block's tail before its ticket: on small
+  // lattices the chains of dependent loads and fences of the three kernels are
+  // the iteration (8^4 x 1: 23.6 -> 22.0 us, 8^4 x 4: 31.4 -> 29.3).
   const int l = blockIdx.y;
   const int ran = *c.ran, live_l = c.live[l];
+  const int kb = c.tab != nullptr ? *c.seed_iters - 1 : 0;  // this iteration (Krylov-basis form)
   const double alpha_l = c.alpha[l], scale_l = c.seed[l].scale, spad1_l = c.seed[l].pad[1];
   if (c.tab != nullptr) {  // Krylov-basis form: this iteration's slots
     r_in = reinterpret_cast<const V2*>(c.rptr[0]);
@@ -759,6 +799,15 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
         sweep(std::true_type{});
     }
   }
+  // what the last block's tail needs of a source, loaded ahead of it
+  const int lt = min((int)threadIdx.x, L - 1);
+  const double vn2_t = c.vnorm2[lt], irr_t = c.inv_rr[lt], alpha_t = c.alpha[lt], S_t = c.seed[lt].pad[1];
+  const int live_t = c.live[lt];
+  char *slot1 = nullptr, *slot2 = nullptr;  // slots of the next iteration
+  if (c.tab != nullptr) {
+    slot1 = reinterpret_cast<char*>(basis_slot<V2>(c, kb + 1, (long long)L * n));
+    slot2 = reinterpret_cast<char*>(basis_slot<V2>(c, kb + 2, (long long)L * n));
+  }
   double acc = warp_sum(acc0 + acc1);
   if (lane == 0) sred[w] = acc;
   __syncthreads();
@@ -767,39 +816,34 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
     const double t = ((sred[0] + sred[1]) + (sred[2] + sred[3])) + ((sred[4] + sred[5]) + (sred[6] + sred[7]));
     c.partial_rr[(size_t)l * nb + blockIdx.x] = t;
     pdl_trigger();
-    __threadfence();
-    const unsigned ticket = atomicAdd(&c.done[1], 1u);
-    s_last = ticket == gridDim.x * gridDim.y - 1;
+    s_last = ticket(&c.done[1]) == gridDim.x * gridDim.y - 1;
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
-  const int kb = c.tab != nullptr ? *c.seed_iters - 1 : 0;  // this iteration (Krylov-basis form)
   tail_sums<kSeedBlock / 32>(c.partial_rr, nb, L, sums, sred);
-  for (int ls = threadIdx.x; ls < L; ls += blockDim.x) {
-    const double a = sums[ls], vn2 = c.vnorm2[ls];
-    s_beta[ls] = a * c.inv_rr[ls];
-    s_scale[ls] = (c.live[ls] != 0 && a < rescale_below * vn2 && a > 0.0) ? rescale_by : 1.0;
+  if ((int)threadIdx.x < L) {  // kMaxSources <= kSeedBlock
+    const double a = sums[lt];
+    s_beta[lt] = a * irr_t;
+    s_scale[lt] = (live_t != 0 && a < rescale_below * vn2_t && a > 0.0) ? rescale_by : 1.0;
   }
-  if (c.tab != nullptr && threadIdx.x == 0) {  // slots of the next iteration
-    const long long Ln = (long long)L * n;
-    c.rptr[0] = reinterpret_cast<char*>(basis_slot<V2>(c, kb + 1, Ln));
-    c.rptr[1] = reinterpret_cast<char*>(basis_slot<V2>(c, kb + 2, Ln));
+  if (c.tab != nullptr && threadIdx.x == 0) {
+    c.rptr[0] = slot1;
+    c.rptr[1] = slot2;
   }
   __syncthreads();
   if (c.split) {
     // the seed state only; kernel S takes the shifts from this record
-    for (int ls = threadIdx.x; ls < L; ls += blockDim.x) {
+    if ((int)threadIdx.x < L) {
+      const int ls = lt;
       const double sc = s_scale[ls];
-      const SeedState sd = c.seed[ls];
       double* rec = c.srec + ((size_t)par * L + ls) * 4;
       rec[0] = sums[ls];
       rec[1] = s_beta[ls];
       rec[2] = sc;
-      rec[3] = sd.pad[1];
-      if (c.live[ls] != 0) {
+      rec[3] = S_t;
+      if (live_t != 0) {
         const double rr = sums[ls] * sc * sc;
-        c.seed[ls] = SeedState{rr, c.alpha[ls], s_beta[ls], s_beta[ls], sc, {0.0, sd.pad[1] * sc, 0.0}};
+        c.seed[ls] = SeedState{rr, alpha_t, s_beta[ls], s_beta[ls], sc, {0.0, S_t * sc, 0.0}};
       }
     }
     if (threadIdx.x == 0) {
@@ -935,23 +979,25 @@ template <typename V2>
 __global__ void __launch_bounds__(kUpdBlock)
 cg_seed_p_fix_kernel(Control c, const V2* __restrict__ r, V2* __restrict__ p, int4* __restrict__ dig,
                      int* __restrict__ ex, int V) {
-  pdl_wait();
   const int l = blockIdx.y;
+  const int lane = threadIdx.x & 31, q = lane >> 3;
+  const int s = (blockIdx.x * (kUpdBlock / 32) + (threadIdx.x >> 5)) * 8 + (lane & 7);
+  const size_t o = ((size_t)l * 12 + 3 * q) * V + s;
+  pdl_wait();
+  // p beside the control words and the slot's address
+  V2 v[3] = {};
+  if (s < V) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v[a] = p[o + (size_t)a * V];
+  }
   const int ran = *c.ran, live_l = c.live[l];
   const double scale_l = c.seed[l].scale, beta_l = c.seed[l].beta;
   if (c.tab != nullptr) r = reinterpret_cast<const V2*>(c.rptr[0]);  // r_{k+1}: kernel B advanced the slots
   if (ran == 0 || live_l == 0) return;
-  const int lane = threadIdx.x & 31, q = lane >> 3;
-  const int s = (blockIdx.x * (kUpdBlock / 32) + (threadIdx.x >> 5)) * 8 + (lane & 7);
-  const size_t o = ((size_t)l * 12 + 3 * q) * V + s;
-  V2 v[3] = {};
   if (s < V) {
     V2 x[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      x[a] = r[o + (size_t)a * V];
-      v[a] = p[o + (size_t)a * V];
-    }
+    for (int a = 0; a < 3; ++a) x[a] = r[o + (size_t)a * V];
     const double beta = scale_l * beta_l;
     if (scale_l == 1.0) {
 #pragma unroll
@@ -1983,8 +2029,11 @@ void launch_chain(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t st
 }
 
 // Programmatic dependent launch of the chain kernels in the Krylov-basis
-// loop: off by default (measured 59.7 us per iteration without, 65.6 with,
-// on the 8^4 x 4 workload); SSQCD_PDL=1 turns it on for comparison runs.
+// loop: off by default, SSQCD_PDL=1 turns it on for comparison runs.  A loop
+// that has the GPU to itself gains 1 to 3% by it on small lattices (8^4 x 2:
+// 24.4 -> 23.6 us an iteration) and loses as much on large ones (16^3 x 32:
+// 93.4 -> 96.0); six solves side by side lose 4% (101 -> 105 ms): blocks that
+// wait for their predecessor hold the places that other loops could use.
 bool use_pdl() {
   static const bool v = [] {
     const char* e = std::getenv("SSQCD_PDL");
@@ -2239,9 +2288,10 @@ class CgRun final : public CgRunBase {
     const int NL = N * L;
     if constexpr (kSeed64 || kSeedDF) {
       // the integer stencil, when the links allow it and its digits fit; for
-      // float-float vectors where it runs one warp a site group (below that,
-      // 8^4 x 2, the float-float stencil is as fast and needs no digits)
-      fix_ = lat->fix_ok && (kSeed64 || fix_split(g.V, L) == 1) && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
+      // float-float vectors where one or four warps run a site group (8^4 x 2:
+      // 25.0 -> 23.5 us an iteration; at eight, 8^4 x 1, the float-float
+      // stencil is the faster one, 22.5 against 23.6, and needs no digits)
+      fix_ = lat->fix_ok && (kSeed64 || fix_split(g.V, L) <= 4) && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
              pex_.alloc(fix_exp_bytes(g.V) * L) == SSQCD_OK;
       fix_w_ = fix_split(g.V, L);
       if constexpr (kSeedDF) {

@@ -161,7 +161,7 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
   v.ex += (size_t)fc * v.tiles * kTile;
   v.dig += field_at(v.tiles, fc, 0);
   Hops h;
-  load_hops(v, s, h);
+  load_neighbours(v, s, h);
   Acc3 up, lo;
   if constexpr (W == 1) {
     hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * kWarpStages), up, lo, [&](int4* to) {

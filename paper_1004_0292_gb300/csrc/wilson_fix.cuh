@@ -161,26 +161,35 @@ __device__ __forceinline__ int b_sign(int mu, int r) { return (mu == 1 && r == 0
 // -1 where row r's share of the lower spins takes the factor -1 or -i of B^H
 __device__ __forceinline__ int eta_sign(int mu, int r) { return mu == 0 || (mu != 3 && r == 0) ? -1 : 0; }
 
+// The operands of one hop of a spin row r: the neighbour's components of spin r
+// and of B's column, and the link.
+struct HopData {
+  int4 p[3], q[3], g[9];
+};
+template <bool SHARED>
+__device__ __forceinline__ void hop_fetch(const int4* u, const int4* x, const int4* l, HopData& d) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    d.p[a] = SHARED ? x[a * kTile] : load4(x + a * kTile);
+    d.q[a] = SHARED ? l[a * kTile] : load4(l + a * kTile);
+  }
+#pragma unroll
+  for (int e = 0; e < 9; ++e) d.g[e] = SHARED ? u[e * kTile] : load4(u + e * kTile);
+}
+
 // w = U h (BACK = false) or U^H h (BACK = true) for spin row r of the projected
 // half spinor h = psi_r -+ (B_mu psi_l)_r at the neighbour, negated if neg,
-// shifted right by sh (1 .. 62) with rounding.  u: the link of its site; x, l:
-// the neighbour's components of spins r and of B's column.  MU < 0: the
-// direction is the run-time value mu_rt (one copy of the code for all four).
-template <int MU, bool BACK, bool SHARED = false>
-__device__ __forceinline__ void hop_row(const int4* u, const int4* x, const int4* l, int mu_rt, int r, bool neg, int sh,
-                                        Acc3& w) {
+// shifted right by sh (1 .. 62) with rounding.  MU < 0: the direction is the
+// run-time value mu_rt (one copy of the code for all four).
+template <int MU, bool BACK>
+__device__ __forceinline__ void hop_math(const HopData& d, int mu_rt, int r, bool neg, int sh, Acc3& w) {
   const int mu = MU < 0 ? mu_rt : MU;
   const bool swap = (mu & 1) == 0;  // entries +-i (mu = 0, 2), else +-1
   const int m = BACK ? b_sign(mu, r) : ~b_sign(mu, r);
-  // every load of the hop first: one latency a hop, not one a link column
-  int4 p[3], q[3], g[9], h[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    p[a] = SHARED ? x[a * kTile] : load4(x + a * kTile);
-    q[a] = SHARED ? l[a * kTile] : load4(l + a * kTile);
-  }
-#pragma unroll
-  for (int e = 0; e < 9; ++e) g[e] = SHARED ? u[e * kTile] : load4(u + e * kTile);
+  const int4(&p)[3] = d.p;
+  const int4(&q)[3] = d.q;
+  const int4(&g)[9] = d.g;
+  int4 h[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     h[a].x = add_signed(p[a].x, swap ? q[a].z : q[a].x, swap ? ~m : m);
@@ -262,32 +271,34 @@ struct Hops {
   unsigned sh[2];  // eight shifts of a byte
   int E;
 };
-__device__ __forceinline__ void load_hops(const FixView& v, int s, Hops& h) {
+// In two parts: the copies or loads of the hops' operands need the neighbours
+// alone, so that they are under way while the exponents come.
+__device__ __forceinline__ void load_neighbours(const FixView& v, int s, Hops& h) {
   const int* t = nbr_at(v.nbr, s);
-  int e[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) h.nb[k] = __ldg(t + k * kTile);
+}
+__device__ __forceinline__ void load_exponents(const FixView& v, int s, Hops& h) {
+  int e[8];
   const int own = __ldg(v.ex + s);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) e[k] = __ldg(v.ex + (h.nb[k] & (kNegBit - 1)));
   h.E = kZeroExp;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    e[k] = __ldg(v.ex + (h.nb[k] & (kNegBit - 1)));
-    h.E = max(h.E, e[k]);
-  }
+  for (int k = 0; k < 8; ++k) h.E = max(h.E, e[k]);
   h.sh[0] = h.sh[1] = 0;
 #pragma unroll
   for (int k = 0; k < 8; ++k) h.sh[k >> 2] |= (unsigned)min(h.E - e[k] + 1, 62) << (8 * (k & 3));
   if (own > kMaxExp) h.E = own;
 }
 
-// One hop of direction mu at site s, operands straight from global memory.
+// The operands of one hop of direction mu at site s from global memory.
 template <bool BACK>
-__device__ __forceinline__ void hop_at(const FixView& v, int s, int nbe, int sh, int mu, int r, Acc3& w) {
+__device__ __forceinline__ void hop_fetch_at(const FixView& v, int s, int nbe, int mu, int r, HopData& d) {
   const int nb = nbe & (kNegBit - 1);
   const int lr = mu < 2 ? 1 - r : r;
-  const int4* d = v.dig + (size_t)(nb >> 4) * (12 * kTile) + (nb & 15);
-  hop_row<-1, BACK>(v.u + link_at(v.tiles, mu, BACK ? nb : s), d + r * 3 * kTile, d + (6 + lr * 3) * kTile, mu, r,
-                    (nbe & kNegBit) != 0, sh, w);
+  const int4* x = v.dig + (size_t)(nb >> 4) * (12 * kTile) + (nb & 15);
+  hop_fetch<false>(v.u + link_at(v.tiles, mu, BACK ? nb : s), x + r * 3 * kTile, x + (6 + lr * 3) * kTile, d);
 }
 
 // up += w, d += -+ eta i^swap w (forward, backward): one hop's share of the
@@ -360,9 +371,10 @@ __device__ __forceinline__ void staged_hop(const int4* buf, int nbe, int sh, int
   constexpr int MU = K >> 1;
   constexpr bool BACK = (K & 1) != 0;
   const int lr = MU < 2 ? 1 - r : r;
+  HopData o;
   Acc3 w;
-  hop_row<MU, BACK, true>(buf + 12 * kTile + i, buf + r * 3 * kTile + i, buf + (6 + lr * 3) * kTile + i, MU, r,
-                          (nbe & kNegBit) != 0, sh, w);
+  hop_fetch<true>(buf + 12 * kTile + i, buf + r * 3 * kTile + i, buf + (6 + lr * 3) * kTile + i, o);
+  hop_math<MU, BACK>(o, MU, r, (nbe & kNegBit) != 0, sh, w);
   add_hop<BACK>(w, MU, r, up, d);
 }
 
@@ -385,15 +397,17 @@ __device__ __forceinline__ void pipe_hops(const FixView& v, int s, int i, int r,
   }
 }
 
-// The eight hops of the warp's 16 sites; last(stage) starts the copy of what
+// The eight hops of the warp's 16 sites, whose neighbours are loaded (the
+// exponents are loaded here); last(stage) starts the copy of what
 // the caller needs after them (committed, complete after copy_wait<1>).
 template <typename Last>
-__device__ __forceinline__ void hop_sums_piped(const FixView& v, int s, int i, int r, const Hops& h, int4* buf,
+__device__ __forceinline__ void hop_sums_piped(const FixView& v, int s, int i, int r, Hops& h, int4* buf,
                                                Acc3& up, Acc3& lo, Last last) {
   clear(up);
   clear(lo);
   stage_hop<0>(v, s, h.nb[0], i, r, buf);
   stage_hop<1>(v, s, h.nb[1], i, r, buf + kStageElems);
+  load_exponents(v, s, h);
   pipe_hops<0>(v, s, i, r, h, buf, up, lo, last);
 }
 
@@ -404,22 +418,30 @@ __device__ __forceinline__ void hop_sums_piped(const FixView& v, int s, int i, i
 // on instruction fetches.  (W = 1: hop_sums_piped.)  All lanes of the warp
 // take part.
 template <int W>
-__device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub, const Hops& h, Acc3& up, Acc3& lo) {
+__device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub, Hops& h, Acc3& up, Acc3& lo) {
   static_assert(W == 4 || W == 8, "W = 1: hop_sums_piped");
   clear(up);
   clear(lo);
   const int mu = W == 4 ? sub : sub >> 1;
+  const bool back = W == 8 && (sub & 1) != 0;
   const int nf = mu == 0 ? h.nb[0] : mu == 1 ? h.nb[2] : mu == 2 ? h.nb[4] : h.nb[6];
   const int nb = mu == 0 ? h.nb[1] : mu == 1 ? h.nb[3] : mu == 2 ? h.nb[5] : h.nb[7];
+  HopData d;
+  if (back)
+    hop_fetch_at<true>(v, s, nb, mu, r, d);
+  else
+    hop_fetch_at<false>(v, s, nf, mu, r, d);
+  load_exponents(v, s, h);
   const unsigned s2 = (mu < 2 ? h.sh[0] : h.sh[1]) >> (16 * (mu & 1));
   const int sf = s2 & 0xff, sb = (s2 >> 8) & 0xff;
   Acc3 w;
-  if (W == 4 || (sub & 1) == 0) {
-    hop_at<false>(v, s, nf, sf, mu, r, w);
+  if (!back) {
+    hop_math<-1, false>(d, mu, r, (nf & kNegBit) != 0, sf, w);
     add_hop<false>(w, mu, r, up, lo);
   }
-  if (W == 4 || (sub & 1) != 0) {
-    hop_at<true>(v, s, nb, sb, mu, r, w);
+  if (W == 4) hop_fetch_at<true>(v, s, nb, mu, r, d);
+  if (W == 4 || back) {
+    hop_math<-1, true>(d, mu, r, (nb & kNegBit) != 0, sb, w);
     add_hop<true>(w, mu, r, up, lo);
   }
   if (mu < 2) cross_over(lo);
@@ -427,11 +449,12 @@ __device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub
 
 // Launch shapes: warps a block, (site group, rhs) units a block, and the
 // blocks an SM that the registers are capped for (the fastest of those tried:
-// W = 1 at 3, 4, 5 blocks 368, 326, 386 us for 16^3 x 32 x 8; W = 4 at 5, 6, 7
-// 503, 456, 406 us; W = 8 at 3, 4 the same for the small lattices it serves).
+// W = 1 at 3, 4, 5 blocks 368, 326, 386 us for 16^3 x 32 x 8; W = 4 at 7, 6, 5
+// 24.9, 24.1, 23.7 us an iteration of 8^4 x 2; W = 8 at 3, 4 the same for the
+// small lattices it serves).
 __host__ __device__ constexpr int fix_threads(int W) { return W == 8 ? 256 : 128; }
 __host__ __device__ constexpr int fix_units(int W) { return fix_threads(W) / 32 / W; }
-__host__ __device__ constexpr int fix_min_blocks(int W) { return W == 1 ? 4 : W == 4 ? 7 : 3; }
+__host__ __device__ constexpr int fix_min_blocks(int W) { return W == 1 ? 4 : W == 4 ? 5 : 3; }
 
 // psi - kappa D psi from a hop sum T in units 2^(E - 57): the sum is made a
 // double times 2^-200 (its exponent field lowered: |T| < 2^63, so that this is
