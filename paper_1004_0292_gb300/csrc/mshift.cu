@@ -448,8 +448,8 @@ struct StencilFix {
           q[(size_t)comp * V + s] = o;
         } else {
           double2 o;
-          o.x = wfix::hop_finish(hf, t.x, pv.x);
-          o.y = wfix::hop_finish(hf, t.y, pv.y);
+          o.x = wfix::hop_finish<true>(hf, t.x, pv.x);
+          o.y = wfix::hop_finish<true>(hf, t.y, pv.y);
           if constexpr (Z) {
             if (k < 3) o = make_double2(-o.x, -o.y);
           } else {

@@ -211,8 +211,8 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
     } else {
       const double2 p = USER ? st[i * 13 + comp] : inf[(size_t)comp * V + s];
       double2 o;
-      o.x = hop_finish(hf, t.x, p.x);
-      o.y = hop_finish(hf, t.y, p.y);
+      o.x = k < 3 ? hop_finish<false>(hf, t.x, p.x) : hop_finish<true>(hf, t.x, p.x);
+      o.y = k < 3 ? hop_finish<false>(hf, t.y, p.y) : hop_finish<true>(hf, t.y, p.y);
       if (k >= 3) o = make_double2(-o.x, -o.y);
       if (USER)
         st[i * 13 + comp] = o;

@@ -457,13 +457,35 @@ __host__ __device__ constexpr int fix_units(int W) { return fix_threads(W) / 32 
 __host__ __device__ constexpr int fix_min_blocks(int W) { return W == 1 ? 4 : W == 4 ? 5 : 3; }
 
 // psi - kappa D psi from a hop sum T in units 2^(E - 57): the sum is made a
-// double times 2^-200 (its exponent field lowered: |T| < 2^63, so that this is
-// exact) and the factor -kappa 2^(E + 143) is a normal number for every E.
+// double times 2^-200 (exact up to its rounding: |T| < 2^63) and the factor
+// -kappa 2^(E + 143) is a normal number for every E.
 __device__ __forceinline__ double hop_factor(int E, double mkappa) {
   const int k = E == kZeroExp || E > kMaxExp ? 0 : E + 143;
   return mkappa * __hiloint2double((k + 1023) << 20, 0);
 }
+// t 2^-200 rounded to nearest (halves away from zero), put together from
+// integers: the conversion instruction takes two of the FP64 pipe's slots, 128
+// cycles of a warp, which was half of that pipe's work in the CG loop's stencil.
+__device__ __forceinline__ double scaled_double(long long t) {
+  const long long sign = t >> 63;
+  const unsigned long long a = (unsigned long long)((t ^ sign) - sign);
+  unsigned hi = (unsigned)(a >> 32), lo = (unsigned)a;
+  const bool low = hi == 0;
+  hi = low ? lo : hi;
+  lo = low ? 0u : lo;
+  const int n = __clz((int)hi);  // 32: t = 0
+  const unsigned uh = __funnelshift_l(lo, hi, n), ul = __funnelshift_l(0u, lo, n);
+  // the leading one lies at bit 52 and adds one to the exponent field, as does a carry out of the rounding
+  const unsigned long long m =
+      ((unsigned long long)((uh >> 11) + ((unsigned)((low ? 853 : 885) - n) << 20)) << 32 | __funnelshift_r(ul, uh, 11)) +
+      (ul >> 10 & 1);
+  const unsigned top = (uh == 0 ? 0u : (unsigned)(m >> 32)) | ((unsigned)sign & 0x80000000u);
+  return __hiloint2double((int)top, (int)(unsigned)m);
+}
+// INT: by integers, else by the conversion instruction and its exponent field lowered
+template <bool INT>
 __device__ __forceinline__ double hop_finish(double f, long long t, double psi) {
+  if (INT) return fma(f, scaled_double(t), psi);
   const double d = (double)t;
   const int hw = __double2hiint(d);
   return fma(f, __hiloint2double(t == 0 ? hw : hw - (200 << 20), __double2loint(d)), psi);
