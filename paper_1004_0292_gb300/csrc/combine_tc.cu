@@ -76,37 +76,56 @@ namespace {
 constexpr int kRows = 128;         // real rows (64 complex elements) per tile
 constexpr int kKStep = 16;         // slots per MMA (K of kind::f16)
 constexpr int kSlices = 7;         // base-256 digits of the 56-bit fixed point
-constexpr int kOut = 16;           // outputs per launch
-constexpr int kChunkSteps = 16;    // K-steps per accumulator flush (256 slots)
+constexpr int kOut = 16;           // real outputs per launch
+constexpr int kWideOut = 32;       // of the wide form
 constexpr int kF64Stages = 4;
-constexpr int kSliceStages = 4;
-constexpr int kEpiWarps = 8;
-constexpr int kMmaWarp = 8;
-constexpr int kLoadWarp = 9;
-constexpr int kSliceWarp0 = 10;
-constexpr int kSliceWarps = 16;
-constexpr int kTcThreads = (kSliceWarp0 + kSliceWarps) * 32;  // 832
+constexpr int kEpiWarps = 8;       // warps 0 ..
+constexpr int kSliceWarps = 16;    // warps 8 ..
+constexpr int kMmaWarp = kEpiWarps + kSliceWarps;
+constexpr int kLoadWarp = kMmaWarp + 1;
 constexpr int kTmemCols = 512;
-constexpr int kABytes = kRows * kKStep * 2;       // one bf16 slice: 4096 B
-constexpr int kBRows = kSlices * kOut;            // 112
-constexpr int kBBytes = kBRows * kKStep * 2;      // 3584 B
+constexpr int kABytes = kRows * kKStep * 2;       // one fp16 slice: 4096 B
+// The two forms of the kernel.  Narrow: 16 real outputs, every pair (p, q) a
+// block of 16 accumulator columns of its own.  Wide (more than 8 complex
+// outputs): 32 real outputs, the pairs of a level in one block of 32.
+template <bool WIDE>
+struct Form {
+  static constexpr int kO = WIDE ? kWideOut : kOut;
+  static constexpr int kBRows = kSlices * kO;         // 112, 224
+  static constexpr int kBBytes = kBRows * kKStep * 2;  // 3584, 7168 B
+  // wide: rows of zeros ahead of B's, so that every slice's product spans all levels
+  static constexpr int kPadBytes = WIDE ? (kSlices - 1) * kO * kKStep * 2 : 0;
+  static constexpr int kSliceStages = WIDE ? 3 : 4;
+  // K-steps per accumulator flush.  Narrow: 256 products of 16 bits.  Wide: a
+  // level's products of signed digits, at most 2 * 2^15 + 5 * 2^14 a slot, of 96 slots.
+  static constexpr int kChunkSteps = WIDE ? 6 : 16;
+  static constexpr int kBuffers = WIDE ? 2 : 1;  // of accumulators
+  static constexpr int kBufferCols = 256;
+  static constexpr int kThreads = WIDE ? 896 : 832;  // whole warpgroups where registers move between them
+  static constexpr int kEpiOuts = kO / 2;             // real outputs an epilogue thread
+  // wide: registers a thread at launch, of the epilogue and of the others
+  static constexpr int kRegs = 72, kEpiRegs = 112, kOtherRegs = 56;
+  static_assert(kEpiWarps * 32 * kEpiRegs + (896 - kEpiWarps * 32) * kOtherRegs <= 896 * kRegs, "register split");
+};
 constexpr int kMaxCount = 65535;                  // slots (grid.y of the scale kernel)
 constexpr unsigned long long kTcWaitNs = 1000000000ull;
 constexpr long long kTcSpin = 1LL << 26;
 
+template <bool WIDE>
 struct __align__(1024) SliceStage {
   unsigned char a[kSlices][kABytes];
-  unsigned char b[kBBytes];
+  unsigned char b[Form<WIDE>::kPadBytes + Form<WIDE>::kBBytes];
 };
 struct __align__(1024) F64Stage {
   double v[kKStep][kRows];
 };
+template <bool WIDE>
 struct TcShared {
   F64Stage f64[kF64Stages];
-  SliceStage sl[kSliceStages];
+  SliceStage<WIDE> sl[Form<WIDE>::kSliceStages];
   unsigned long long full_f[kF64Stages], empty_f[kF64Stages];
-  unsigned long long full_s[kSliceStages], empty_s[kSliceStages];
-  unsigned long long tmem_full, tmem_empty, mma_done;
+  unsigned long long full_s[Form<WIDE>::kSliceStages], empty_s[Form<WIDE>::kSliceStages];
+  unsigned long long tmem_full[2], tmem_empty[2], mma_done;
   unsigned tmem_base;
   int abort;
 };
@@ -210,6 +229,17 @@ __device__ __forceinline__ void tc_ld8(unsigned taddr, float (&t)[8]) {
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
       "tcgen05.wait::ld.sync.aligned;\n"
       : "=f"(t[0]), "=f"(t[1]), "=f"(t[2]), "=f"(t[3]), "=f"(t[4]), "=f"(t[5]), "=f"(t[6]), "=f"(t[7])
+      : "r"(taddr)
+      : "memory");
+}
+
+__device__ __forceinline__ void tc_ld16(unsigned taddr, float (&t)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=f"(t[0]), "=f"(t[1]), "=f"(t[2]), "=f"(t[3]), "=f"(t[4]), "=f"(t[5]), "=f"(t[6]), "=f"(t[7]), "=f"(t[8]),
+        "=f"(t[9]), "=f"(t[10]), "=f"(t[11]), "=f"(t[12]), "=f"(t[13]), "=f"(t[14]), "=f"(t[15])
       : "r"(taddr)
       : "memory");
 }
@@ -358,10 +388,11 @@ constexpr int kErrWait = 1, kErrSpread = 2;  // bits of the error word
 // one block of 256 threads per (source, output).  A non-finite residual
 // element or coefficient makes sig NaN, so that the outputs of that source
 // come out NaN as the FP64 sum's would (the slices themselves stay finite).
+template <int OUT>
 __global__ void tc_scales_kernel(const unsigned* __restrict__ mx, CoefView C, int O, int S, int l0,
                                  const int* __restrict__ count, int* __restrict__ eslot, double* __restrict__ sig,
                                  const unsigned long long* __restrict__ ex, long long n, int* __restrict__ err) {
-  const int lz = blockIdx.x / kOut, o = blockIdx.x % kOut, l = l0 + lz;
+  const int lz = blockIdx.x / OUT, o = blockIdx.x % OUT, l = l0 + lz;
   const int cnt = slots_of(count, l, S);
   double m = 0.0;
   bool bad = false;
@@ -401,21 +432,22 @@ __global__ void tc_scales_kernel(const unsigned* __restrict__ mx, CoefView C, in
     }
     if (ex != nullptr && (bad || !isfinite(m) || abs(exp_above(m)) > 950)) atomicOr(err, kErrSpread);
     // every output of the source: a bad slot of this source poisons them all
-    sig[(size_t)lz * kOut + o] = (bad || !isfinite(m)) ? __longlong_as_double(0x7FF8000000000000ll)
+    sig[(size_t)lz * OUT + o] = (bad || !isfinite(m)) ? __longlong_as_double(0x7FF8000000000000ll)
                                                        : ldexp(1.0, exp_above(m));
   }
 }
 
-// B image of K-step kk for source l0 + l' (grid (kk, l'), 224 threads): row
-// q * 16 + o of the N x 16 operand holds digit q of C[l][o][s] 2^(e_s - g_o)
+// B image of K-step kk for source l0 + l' (grid (kk, l'), 14 OUT threads): row
+// q * OUT + o of the N x 16 operand holds digit q of C[l][o][s] 2^(e_s - g_o)
 // for the slots s = 16 kk + k; thread t writes the 8 slots k = 8 (t & 1) ..
 // of row t / 2 (16 bytes of one core matrix).
+template <int OUT>
 __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* __restrict__ count,
                                   const int* __restrict__ eslot, const double* __restrict__ sig, int ksteps_cap,
                                   unsigned char* __restrict__ bimg) {
   const int kk = blockIdx.x, lz = blockIdx.y, l = l0 + lz;
   const int t = threadIdx.x, row = t >> 1, h = t & 1;
-  const int q = row / kOut, o = row % kOut;
+  const int q = row / OUT, o = row % OUT;
   const int cnt = slots_of(count, l, S);
   __align__(16) __half f[8];
 #pragma unroll
@@ -423,7 +455,7 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
     const int s = kk * kKStep + 8 * h + i;
     int d = 0;
     if (o < O && s < cnt) {
-      const int g = exp_above(sig[(size_t)lz * kOut + o]) - 1;  // sig = 2^g
+      const int g = exp_above(sig[(size_t)lz * OUT + o]) - 1;  // sig = 2^g
       const double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * S + s] - g);
       if (C.cplx) {  // signed digits
         long long X = llrint(ldexp(b, 56));
@@ -439,7 +471,7 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
     }
     f[i] = __int2half_rn(d);
   }
-  unsigned char* dst = bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes + core_off(row, 8 * h);
+  unsigned char* dst = bimg + ((size_t)lz * ksteps_cap + kk) * (kSlices * OUT * kKStep * 2) + core_off(row, 8 * h);
   *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(f);
 }
 
@@ -472,14 +504,18 @@ __device__ __forceinline__ double sum_to_double(long long xh, long long xl, int 
 // signed digits.  SHORT: at most 64 slots, so that a chunk's sums, below 2^22,
 // turn into integers by an FP32 addition instead of a conversion (16 a clock
 // and SM).  ACC: the sums are added to out.
-template <bool CPLX, bool SHORT, bool ACC>
-__global__ void __launch_bounds__(kTcThreads, 1)
+template <bool CPLX, bool SHORT, bool ACC, bool WIDE>
+__global__ void __launch_bounds__(Form<WIDE>::kThreads, 1)
 combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restrict__ count, int S,
                   const int* __restrict__ eslot, const unsigned char* __restrict__ bimg, int ksteps_cap,
                   const double* __restrict__ sig, int O, long long out_l, double2* __restrict__ out,
                   int* __restrict__ err) {
   extern __shared__ unsigned char tc_smem_raw[];
-  TcShared* sh = reinterpret_cast<TcShared*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
+  using F = Form<WIDE>;
+  static_assert(CPLX || !WIDE, "the wide form's bound is that of signed digits");
+  constexpr int kSliceStages = F::kSliceStages, kChunkSteps = F::kChunkSteps, kBBytes = F::kBBytes;
+  constexpr int kE = F::kEpiOuts;
+  TcShared<WIDE>* sh = reinterpret_cast<TcShared<WIDE>*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long tiles_per_src = (2 * n + kRows - 1) / kRows;  // the last one may be short
   const long long tiles = tiles_per_src * nl;
@@ -494,8 +530,10 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
       bar_init(sh->full_s + i, kSliceWarps);
       bar_init(sh->empty_s + i, 1);
     }
-    bar_init(&sh->tmem_full, 1);
-    bar_init(&sh->tmem_empty, kEpiWarps);
+    for (int i = 0; i < F::kBuffers; ++i) {
+      bar_init(sh->tmem_full + i, 1);
+      bar_init(sh->tmem_empty + i, kEpiWarps);
+    }
     bar_init(&sh->mma_done, 1);
     sh->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -507,6 +545,12 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     tc_fence_before();
   }
+  if (WIDE) {  // the zero rows ahead of B's
+    constexpr int kPad = F::kPadBytes / 16;
+    for (int i = threadIdx.x; i < kSliceStages * kPad; i += F::kThreads)
+      reinterpret_cast<uint4*>(sh->sl[i / max(kPad, 1)].b)[i % max(kPad, 1)] = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
   __syncthreads();
   tc_fence_after();
   const unsigned tmem = sh->tmem_base;
@@ -516,47 +560,119 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
     atomicOr(err, kErrWait);
   };
 
-  if (warp == kLoadWarp) {
-    // ---- bulk copies of the FP64 residual rows: lane j issues slot j's ----
-    // (one lane for all sixteen was the kernel's pace: each copy's address
-    // takes a dependent load of the block table, ~3200 cycles a K-step)
-    {
-      long long fc = 0;
-      bool ok = true;
-      for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        const int lz = (int)(t / tiles_per_src), l = l0 + lz;
-        const long long row0 = (t % tiles_per_src) * kRows;
-        const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
-        for (int kk = 0; kk < ks; ++kk, ++fc) {
-          const int st = (int)(fc % kF64Stages);
-          const int nv = min(kKStep, cnt - kk * kKStep);
-          const double* src = lane < nv ? slot_ptr(map, n, l, kk * kKStep + lane) + row0 : nullptr;
-          // rows of a short tile past the end keep what the stage held: their sums are not stored
-          const unsigned bytes = (unsigned)min((long long)kRows, 2 * n - row0) * 8u;
-          if (fc >= kF64Stages && !bar_wait_warp(sh->empty_f + st, (unsigned)((fc / kF64Stages - 1) & 1), abort)) {
-            ok = false;
-            break;
-          }
-          if (lane == 0) bar_arrive_tx(sh->full_f + st, (unsigned)nv * bytes);
-          __syncwarp();
-          if (lane < nv) bulk_copy(sh->f64[st].v[lane], src, bytes, sh->full_f + st);
+  // Wide: the epilogue's sums take the registers that the others can spare
+  // (what they give up is at least what it takes: Form).
+  if (warp < kEpiWarps) {
+    if (WIDE) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(F::kEpiRegs));
+    // ---- epilogue: warp w reads lanes 32 (w % 4) .., outputs 8 (w / 4) .. ----
+    const int quarter = warp & 3, half = warp >> 2;
+    const unsigned lane_addr = tmem + ((unsigned)(32 * quarter) << 16);
+    long long cc = 0;
+    bool ok = true;
+    for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      const int lz = (int)(t / tiles_per_src), l = l0 + lz;
+      const long long row0 = (t % tiles_per_src) * kRows;
+      const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
+      const int nch = (ks + kChunkSteps - 1) / kChunkSteps;
+      // level sums combined exactly as they arrive: xh = I_0 2^16 + I_1 2^8 +
+      // I_2 (< 2^48), xl = I_3 2^24 + I_4 2^16 + I_5 2^8 + I_6 (< 2^56)
+      long long xh[kE], xl[kE];
+#pragma unroll
+      for (int i = 0; i < kE; ++i) xh[i] = xl[i] = 0;
+      for (int c = 0; c < nch; ++c, ++cc) {
+        if (!bar_wait_warp(sh->tmem_full + cc % F::kBuffers, (unsigned)((cc / F::kBuffers) & 1), abort)) {
+          ok = false;
+          break;
         }
+        tc_fence_after();
+        // level by level: the pairs of a level add up in 32 bits
+#pragma unroll
+        for (int lv = 0; lv < kSlices; ++lv) {
+          if constexpr (WIDE) {
+            const unsigned at =
+                lane_addr + (unsigned)(cc % F::kBuffers * F::kBufferCols + lv * F::kO + kE * half);
+            float f[16];
+            tc_ld16(at, f);
+#pragma unroll
+            for (int i = 0; i < kE; ++i) {
+              const int v = __float2int_rn(f[i]);
+              if (lv <= 2)
+                xh[i] += (long long)v * (1 << 8 * (2 - lv));
+              else
+                xl[i] += (long long)v * (1 << 8 * (6 - lv));
+            }
+            continue;
+          }
+          unsigned a[8];
+#pragma unroll
+          for (int p = 0; p <= lv; ++p) {
+            float f[8];
+            tc_ld8(lane_addr + (unsigned)(col_base(p) + kOut * (lv - p) + 8 * half), f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const unsigned v = SHORT ? __float_as_uint(f[i] + 12582912.0f) : (unsigned)__float2int_rn(f[i]);
+              a[i] = p == 0 ? v : a[i] + v;
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (SHORT) a[i] -= (lv + 1) * 0x4B400000u;
+            if (lv <= 2)
+              xh[i] += (long long)(int)a[i] * (1 << 8 * (2 - lv));
+            else
+              xl[i] += (long long)(int)a[i] * (1 << 8 * (6 - lv));
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) bar_arrive(sh->tmem_empty + cc % F::kBuffers);
       }
-      if (!ok) {
-        give_up();
-        // the copies already issued land before the CTA can exit
-        for (long long q = fc - 1; q >= 0 && q >= fc - kF64Stages; --q) {
-          const int st = (int)(q % kF64Stages);
-          const unsigned long long t0 = gtimer();
-          while (!bar_test(sh->full_f + st, (unsigned)((q / kF64Stages) & 1)) && gtimer() - t0 < kTcWaitNs) {
+      if (!ok) break;
+      // the output addresses are formed here, not kept live across the chunks
+      long long r = row0 + 32 * quarter + lane;  // real row: element r / 2, part r % 2
+      int lo = l, lzo = lz;
+      asm volatile("" : "+l"(r), "+r"(lo), "+r"(lzo));
+      if constexpr (!CPLX) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int o = 8 * half + i;
+          if (o < O && r < 2 * n) {
+            // sum_l I_l 2^(-8 l) = 2^-16 xh + 2^-48 xl
+            double v = fma((double)xl[i], 0x1p-48, (double)xh[i] * 0x1p-16);
+            v *= sig[(size_t)lzo * kOut + o] * 0x1p-16;
+            reinterpret_cast<double*>(out + lo * out_l + (long long)o * n)[r] = v;
+          }
+        }
+      } else {
+        // (c x).re = Re c x.re - Im c x.im, (c x).im = Re c x.im + Im c x.re: the
+        // element's two parts sit in lanes 2 j and 2 j + 1, the sums with Re c
+        // and Im c have one scale and add as integers
+#pragma unroll
+        for (int i = 0; i < kE; i += 2) {
+          const int o = kE * half + i;
+          if (o < O) {
+            const long long m = lane & 1 ? 0 : -1;
+            const long long bh = __shfl_xor_sync(0xffffffffu, xh[i + 1], 1);
+            const long long bl = __shfl_xor_sync(0xffffffffu, xl[i + 1], 1);
+            const double sc = sig[(size_t)lzo * F::kO + o];
+            // sig 2^-64 (2^32 xh + xl); a scale that is no number poisons the sum
+            double v = sum_to_double(xh[i] + (bh ^ m) - m, xl[i] + (bl ^ m) - m,
+                                     (int)((unsigned)__double2hiint(sc) >> 20) - 1023 - 64);
+            if (sc != sc) v = sc;
+            if (r < 2 * n) {
+              double* at = reinterpret_cast<double*>(out + lo * out_l + (long long)(o / 2) * n) + r;
+              *at = ACC ? *at + v : v;
+            }
           }
         }
       }
     }
-  } else if (warp >= kSliceWarp0) {
+    if (!ok) give_up();
+  } else if (warp < kMmaWarp) {
+    if (WIDE) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::kOtherRegs));
     // ---- slices: thread u <-> row u % 128, slots kPer (u / 128) .. of a K-step ----
     constexpr int kPer = kKStep * kRows / (kSliceWarps * 32);  // 4 or 8 slots a thread
-    const int u = threadIdx.x - kSliceWarp0 * 32;
+    const int u = threadIdx.x - kEpiWarps * 32;
     const int row = u & (kRows - 1), h = u >> 7;
     long long fc = 0, sc = 0;
     bool ok = true;
@@ -624,7 +740,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
         put(std::integral_constant<int, 5>{});
         put(std::integral_constant<int, 6>{});
         if (u < kBBytes / 16)
-          reinterpret_cast<uint4*>(sh->sl[ss].b)[u] =
+          reinterpret_cast<uint4*>(sh->sl[ss].b + F::kPadBytes)[u] =
               __ldg(reinterpret_cast<const uint4*>(bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes) + u);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
@@ -632,7 +748,46 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
       }
     }
     if (!ok) give_up();
-  } else if (warp == kMmaWarp) {
+  } else {
+    if (WIDE) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::kOtherRegs));
+    if (warp == kLoadWarp) {
+    // ---- bulk copies of the FP64 residual rows: lane j issues slot j's ----
+    // (one lane for all sixteen was the kernel's pace: each copy's address
+    // takes a dependent load of the block table, ~3200 cycles a K-step)
+    {
+      long long fc = 0;
+      bool ok = true;
+      for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        const int lz = (int)(t / tiles_per_src), l = l0 + lz;
+        const long long row0 = (t % tiles_per_src) * kRows;
+        const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
+        for (int kk = 0; kk < ks; ++kk, ++fc) {
+          const int st = (int)(fc % kF64Stages);
+          const int nv = min(kKStep, cnt - kk * kKStep);
+          const double* src = lane < nv ? slot_ptr(map, n, l, kk * kKStep + lane) + row0 : nullptr;
+          // rows of a short tile past the end keep what the stage held: their sums are not stored
+          const unsigned bytes = (unsigned)min((long long)kRows, 2 * n - row0) * 8u;
+          if (fc >= kF64Stages && !bar_wait_warp(sh->empty_f + st, (unsigned)((fc / kF64Stages - 1) & 1), abort)) {
+            ok = false;
+            break;
+          }
+          if (lane == 0) bar_arrive_tx(sh->full_f + st, (unsigned)nv * bytes);
+          __syncwarp();
+          if (lane < nv) bulk_copy(sh->f64[st].v[lane], src, bytes, sh->full_f + st);
+        }
+      }
+      if (!ok) {
+        give_up();
+        // the copies already issued land before the CTA can exit
+        for (long long q = fc - 1; q >= 0 && q >= fc - kF64Stages; --q) {
+          const int st = (int)(q % kF64Stages);
+          const unsigned long long t0 = gtimer();
+          while (!bar_test(sh->full_f + st, (unsigned)((q / kF64Stages) & 1)) && gtimer() - t0 < kTcWaitNs) {
+          }
+        }
+      }
+    }
+    } else if (warp == kMmaWarp) {
     // ---- MMA issue (one thread) ----
     if (lane == 0) {
       long long sc = 0, cc = 0;
@@ -643,7 +798,8 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
         for (int kk = 0; kk < ks; ++kk, ++sc) {
           const int ss = (int)(sc % kSliceStages);
           if (kk % kChunkSteps == 0) {
-            if (cc >= 1 && !bar_wait(&sh->tmem_empty, (unsigned)((cc - 1) & 1), abort)) {
+            if (cc >= F::kBuffers &&
+                !bar_wait(sh->tmem_empty + cc % F::kBuffers, (unsigned)((cc / F::kBuffers - 1) & 1), abort)) {
               ok = false;
               break;
             }
@@ -655,14 +811,21 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
           }
           tc_fence_after();
           const unsigned acc = (kk % kChunkSteps) != 0 ? 1u : 0u;
-          const unsigned long long bd = smem_desc(sh->sl[ss].b, kLbo, kSbo);
 #pragma unroll
-          for (int p = 0; p < kSlices; ++p)
-            tc_mma(tmem + (unsigned)col_base(p), smem_desc(sh->sl[ss].a[p], kLbo, kSbo), bd,
-                   idesc_f16(kRows, kOut * (kSlices - p)), acc);
+          for (int p = 0; p < kSlices; ++p) {
+            const unsigned long long ad = smem_desc(sh->sl[ss].a[p], kLbo, kSbo);
+            if constexpr (WIDE)
+              // all levels, the first p times zero rows: products of one shape and place run in order
+              tc_mma(tmem + (unsigned)(cc % F::kBuffers * F::kBufferCols), ad,
+                     smem_desc(sh->sl[ss].b + F::kPadBytes - p * (F::kO * kKStep * 2), kLbo, kSbo),
+                     idesc_f16(kRows, F::kBRows), p > 0 ? 1u : acc);
+            else
+              tc_mma(tmem + (unsigned)col_base(p), ad, smem_desc(sh->sl[ss].b, kLbo, kSbo),
+                     idesc_f16(kRows, kOut * (kSlices - p)), acc);
+          }
           tc_commit(sh->empty_s + ss);
           if (kk % kChunkSteps == kChunkSteps - 1 || kk == ks - 1) {
-            tc_commit(&sh->tmem_full);
+            tc_commit(sh->tmem_full + cc % F::kBuffers);
             ++cc;
           }
         }
@@ -674,96 +837,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
       while (!bar_test(&sh->mma_done, 0u) && gtimer() - t0 < kTcWaitNs) {
       }
     }
-  } else {
-    // ---- epilogue: warp w reads lanes 32 (w % 4) .., outputs 8 (w / 4) .. ----
-    const int quarter = warp & 3, half = warp >> 2;
-    const unsigned lane_addr = tmem + ((unsigned)(32 * quarter) << 16);
-    long long cc = 0;
-    bool ok = true;
-    for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-      const int lz = (int)(t / tiles_per_src), l = l0 + lz;
-      const long long row0 = (t % tiles_per_src) * kRows;
-      const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
-      const int nch = (ks + kChunkSteps - 1) / kChunkSteps;
-      // level sums combined exactly as they arrive: xh = I_0 2^16 + I_1 2^8 +
-      // I_2 (< 2^48), xl = I_3 2^24 + I_4 2^16 + I_5 2^8 + I_6 (< 2^56)
-      long long xh[8], xl[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) xh[i] = xl[i] = 0;
-      for (int c = 0; c < nch; ++c, ++cc) {
-        if (!bar_wait_warp(&sh->tmem_full, (unsigned)(cc & 1), abort)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        // level by level: the pairs of a level add up in 32 bits
-#pragma unroll
-        for (int lv = 0; lv < kSlices; ++lv) {
-          unsigned a[8];
-#pragma unroll
-          for (int p = 0; p <= lv; ++p) {
-            float f[8];
-            tc_ld8(lane_addr + (unsigned)(col_base(p) + kOut * (lv - p) + 8 * half), f);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const unsigned v = SHORT ? __float_as_uint(f[i] + 12582912.0f) : (unsigned)__float2int_rn(f[i]);
-              a[i] = p == 0 ? v : a[i] + v;
-            }
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            if (SHORT) a[i] -= (lv + 1) * 0x4B400000u;
-            if (lv <= 2)
-              xh[i] += (long long)(int)a[i] * (1 << 8 * (2 - lv));
-            else
-              xl[i] += (long long)(int)a[i] * (1 << 8 * (6 - lv));
-          }
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) bar_arrive(&sh->tmem_empty);
-      }
-      if (!ok) break;
-      // the output addresses are formed here, not kept live across the chunks
-      long long r = row0 + 32 * quarter + lane;  // real row: element r / 2, part r % 2
-      int lo = l, lzo = lz;
-      asm volatile("" : "+l"(r), "+r"(lo), "+r"(lzo));
-      if constexpr (!CPLX) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int o = 8 * half + i;
-          if (o < O && r < 2 * n) {
-            // sum_l I_l 2^(-8 l) = 2^-16 xh + 2^-48 xl
-            double v = fma((double)xl[i], 0x1p-48, (double)xh[i] * 0x1p-16);
-            v *= sig[(size_t)lzo * kOut + o] * 0x1p-16;
-            reinterpret_cast<double*>(out + lo * out_l + (long long)o * n)[r] = v;
-          }
-        }
-      } else {
-        // (c x).re = Re c x.re - Im c x.im, (c x).im = Re c x.im + Im c x.re: the
-        // element's two parts sit in lanes 2 j and 2 j + 1, the sums with Re c
-        // and Im c have one scale and add as integers
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-          const int o = 8 * half + i;
-          if (o < O) {
-            const long long m = lane & 1 ? 0 : -1;
-            const long long bh = __shfl_xor_sync(0xffffffffu, xh[i + 1], 1);
-            const long long bl = __shfl_xor_sync(0xffffffffu, xl[i + 1], 1);
-            const double sc = sig[(size_t)lzo * kOut + o];
-            // sig 2^-64 (2^32 xh + xl); a scale that is no number poisons the sum
-            double v = sum_to_double(xh[i] + (bh ^ m) - m, xl[i] + (bl ^ m) - m,
-                                     (int)((unsigned)__double2hiint(sc) >> 20) - 1023 - 64);
-            if (sc != sc) v = sc;
-            if (r < 2 * n) {
-              double* at = reinterpret_cast<double*>(out + lo * out_l + (long long)(o / 2) * n) + r;
-              *at = ACC ? *at + v : v;
-            }
-          }
-        }
-      }
     }
-    if (!ok) give_up();
   }
   __syncthreads();
   if (warp == kMmaWarp) {
@@ -792,7 +866,7 @@ TcWork carve(void* w, int nl, int S, int ksteps_cap) {
   t.eslot = reinterpret_cast<int*>(p);
   p += align256(sizeof(int) * (size_t)nl * S);
   t.sig = reinterpret_cast<double*>(p);
-  p += align256(sizeof(double) * (size_t)nl * kOut);
+  p += align256(sizeof(double) * (size_t)nl * kWideOut);
   t.err = reinterpret_cast<int*>(p);
   p += 256;
   t.bimg = reinterpret_cast<unsigned char*>(p);
@@ -817,7 +891,7 @@ bool combine_tc_applicable(long long n, int O, int S) {
 size_t combine_tc_work_bytes(int nl, int S) {
   const int ks = (S + kKStep - 1) / kKStep;
   return align256(sizeof(unsigned long long) * (size_t)nl * S) + align256(sizeof(unsigned) * (size_t)nl * S) + align256(sizeof(int) * (size_t)nl * S) +
-         align256(sizeof(double) * (size_t)nl * kOut) + 256 + (size_t)nl * ks * kBBytes;
+         align256(sizeof(double) * (size_t)nl * kWideOut) + 256 + (size_t)nl * ks * Form<true>::kBBytes;
 }
 
 namespace {
@@ -839,25 +913,27 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
   const unsigned gx = (unsigned)std::max(1LL, std::min(64LL, (n + 1023) / 1024));
   tc_maxabs_kernel<<<dim3(gx, S, nl), 256, 0, st>>>(map, n, l0, count, S, w.mx, ex);
   SS_CHECK_LAUNCH();
-  const size_t smem = sizeof(TcShared) + 1024;
-  auto* kern = add       ? combine_tc_kernel<true, false, true>
-               : C.cplx  ? (S <= 64 ? combine_tc_kernel<true, true, false> : combine_tc_kernel<true, false, false>)
-               : S <= 64 ? combine_tc_kernel<false, true, false>
-                         : combine_tc_kernel<false, false, false>;
-  SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // the same every time
   int dev = 0, sms = 0;
   SS_CUDA(cudaGetDevice(&dev));
   SS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const long long tiles = ((2 * n + kRows - 1) / kRows) * nl;
   const int grid = (int)(tiles < sms ? tiles : sms);
-  const int per = C.cplx ? kOut / 2 : kOut;
+  // a pass: its first output, its outputs, and whether it is a wide one
+  auto wide_at = [&](int o0) { return C.cplx && O - o0 > kOut / 2; };
+  auto outs_at = [&](int o0) { return std::min(O - o0, !C.cplx ? kOut : wide_at(o0) ? kWideOut / 2 : kOut / 2); };
+  auto scales = [&](int o0) {
+    CoefView Cp = C;
+    Cp.c += o0 * C.so;
+    const int Op = (C.cplx ? 2 : 1) * outs_at(o0);
+    if (wide_at(o0))
+      tc_scales_kernel<kWideOut><<<nl * kWideOut, 256, 0, st>>>(w.mx, Cp, Op, S, l0, count, w.eslot, w.sig, ex, n, w.err);
+    else
+      tc_scales_kernel<kOut><<<nl * kOut, 256, 0, st>>>(w.mx, Cp, Op, S, l0, count, w.eslot, w.sig, ex, n, w.err);
+  };
   int h_err = 0;
   if (add) {  // every output's scales first
-    for (int o0 = 0; o0 < O; o0 += per) {
-      CoefView Cp = C;
-      Cp.c += o0 * C.so;
-      tc_scales_kernel<<<nl * kOut, 256, 0, st>>>(w.mx, Cp, 2 * std::min(per, O - o0), S, l0, count, w.eslot, w.sig, ex, n,
-                                                  w.err);
+    for (int o0 = 0; o0 < O; o0 += outs_at(o0)) {
+      scales(o0);
       SS_CHECK_LAUNCH();
       count_launches(1);
     }
@@ -866,16 +942,35 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     if (suits != nullptr) *suits = h_err == 0;
     if (h_err != 0) return SSQCD_OK;
   }
-  for (int o0 = 0; o0 < O; o0 += per) {
+  for (int o0 = 0; o0 < O; o0 += outs_at(o0)) {
+    const bool wide = wide_at(o0);
     CoefView Cp = C;
     Cp.c += o0 * C.so;
-    const int Op = (C.cplx ? 2 : 1) * std::min(per, O - o0);
-    tc_scales_kernel<<<nl * kOut, 256, 0, st>>>(w.mx, Cp, Op, S, l0, count, w.eslot, w.sig, ex, n, w.err);
+    const int Op = (C.cplx ? 2 : 1) * outs_at(o0);
+    auto* kern = wide    ? (add ? combine_tc_kernel<true, false, true, true> : combine_tc_kernel<true, false, false, true>)
+                 : add    ? combine_tc_kernel<true, false, true, false>
+                 : C.cplx ? (S <= 64 ? combine_tc_kernel<true, true, false, false>
+                                     : combine_tc_kernel<true, false, false, false>)
+                 : S <= 64 ? combine_tc_kernel<false, true, false, false>
+                           : combine_tc_kernel<false, false, false, false>;
+    const size_t smem = (wide ? sizeof(TcShared<true>) : sizeof(TcShared<false>)) + 1024;
+    SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // the same every time
+    if (wide) {  // its warps share out the registers of the launch
+      cudaFuncAttributes at;
+      SS_CUDA(cudaFuncGetAttributes(&at, kern));
+      if (at.numRegs < Form<true>::kRegs) return fail(SSQCD_ERR_CUDA, "combination (tensor cores): too few registers");
+    }
+    scales(o0);
     SS_CHECK_LAUNCH();
-    tc_bslices_kernel<<<dim3(ks, nl), 2 * kBRows, 0, st>>>(Cp, Op, S, l0, count, w.eslot, w.sig, ks, w.bimg);
+    if (wide)
+      tc_bslices_kernel<kWideOut><<<dim3(ks, nl), 2 * Form<true>::kBRows, 0, st>>>(Cp, Op, S, l0, count, w.eslot, w.sig,
+                                                                                   ks, w.bimg);
+    else
+      tc_bslices_kernel<kOut><<<dim3(ks, nl), 2 * Form<false>::kBRows, 0, st>>>(Cp, Op, S, l0, count, w.eslot, w.sig, ks,
+                                                                                w.bimg);
     SS_CHECK_LAUNCH();
-    kern<<<grid, kTcThreads, smem, st>>>(map, n, l0, nl, count, S, w.eslot, w.bimg, ks, w.sig, Op, out_l,
-                                         out + (long long)o0 * n, w.err);
+    kern<<<grid, wide ? Form<true>::kThreads : Form<false>::kThreads, smem, st>>>(
+        map, n, l0, nl, count, S, w.eslot, w.bimg, ks, w.sig, Op, out_l, out + (long long)o0 * n, w.err);
     SS_CHECK_LAUNCH();
     count_launches(3);
   }

@@ -52,6 +52,19 @@ def test_moments_of_vectors(ss, dims, L, N, M, device):
     assert np.all(np.abs(got - ref) <= (N + M + 16) * 2.0 ** -53 * np.max(size, axis=(2, 3, 4), keepdims=True))
 
 
+# more than eight outputs: 16 a pass, chunks of 96 vectors in two accumulators
+@pytest.mark.parametrize("dims,L,N,M", [
+    ((5, 7, 3, 11), 1, 95, 9), ((5, 7, 3, 11), 1, 96, 16), ((5, 7, 3, 11), 2, 97, 25), ((3, 5, 7, 4), 2, 193, 24),
+    ((4, 4, 4, 5), 3, 289, 11), ((16, 8, 8, 9), 1, 2, 40), ((3, 3, 3, 5), 2, 600, 33),
+])
+def test_wide_passes(ss, dims, L, N, M):
+    w, zeta, y = _inputs(dims, L, N, seed=2)
+    lat = ss.create_lattice(dims, 0.12, -1)
+    got = ss.moments(lat, w, zeta, y, M)
+    ref, size = _reference(w, zeta, y, M)
+    assert np.all(np.abs(got - ref) <= (N + M + 16) * 2.0 ** -53 * np.max(size, axis=(2, 3, 4), keepdims=True))
+
+
 @pytest.mark.parametrize("kind", ["point", "wide", "inf", "nan", "zero vector", "inf weight"])
 def test_vectors_that_keep_the_fp64_sum(ss, kind):
     dims, L, N, M = (8, 8, 8, 8), 2, 32, 8
