@@ -524,10 +524,10 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
   if (threadIdx.x == 0) {
     for (int i = 0; i < kF64Stages; ++i) {
       bar_init(sh->full_f + i, 1);
-      bar_init(sh->empty_f + i, kSliceWarps);
+      bar_init(sh->empty_f + i, kSliceWarps / 2);
     }
     for (int i = 0; i < kSliceStages; ++i) {
-      bar_init(sh->full_s + i, kSliceWarps);
+      bar_init(sh->full_s + i, kSliceWarps / 2);
       bar_init(sh->empty_s + i, 1);
     }
     for (int i = 0; i < F::kBuffers; ++i) {
@@ -670,9 +670,13 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
     if (!ok) give_up();
   } else if (warp < kMmaWarp) {
     if (WIDE) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::kOtherRegs));
-    // ---- slices: thread u <-> row u % 128, slots kPer (u / 128) .. of a K-step ----
-    constexpr int kPer = kKStep * kRows / (kSliceWarps * 32);  // 4 or 8 slots a thread
-    const int u = threadIdx.x - kEpiWarps * 32;
+    // ---- slices: the two halves of the warps take K-steps in turn; thread u
+    // of a half <-> row u % 128, slots 8 (u / 128) .. (16-byte stores without
+    // conflicts; one half's waits pass while the other works) ----
+    constexpr int kPer = 8;
+    static_assert(kPer * kSliceWarps / 2 * 32 == kKStep * kRows, "a K-step for half of the warps");
+    const int turn = (warp - kEpiWarps) / (kSliceWarps / 2);
+    const int u = (threadIdx.x - kEpiWarps * 32) & (kSliceWarps * 16 - 1);
     const int row = u & (kRows - 1), h = u >> 7;
     long long fc = 0, sc = 0;
     bool ok = true;
@@ -680,6 +684,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
       const int lz = (int)(t / tiles_per_src), l = l0 + lz;
       const int cnt = slots_of(count, l, S), ks = (cnt + kKStep - 1) / kKStep;
       for (int kk = 0; kk < ks; ++kk, ++fc, ++sc) {
+        if ((int)(fc & 1) != turn) continue;
         const int fs = (int)(fc % kF64Stages), ss = (int)(sc % kSliceStages);
         const int nv = min(kKStep, cnt - kk * kKStep);
         int es[kPer];
@@ -727,10 +732,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
               w[i] = digit_pair<p>(X[2 * i], X[2 * i + 1], s1[i], s2[i]);
           }
           unsigned char* dst = sh->sl[ss].a[p] + core_off(row, kPer * h);
-          if constexpr (kPer == 8)
-            *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-          else
-            *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+          *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         };
         put(std::integral_constant<int, 0>{});
         put(std::integral_constant<int, 1>{});
@@ -739,9 +741,10 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
         put(std::integral_constant<int, 4>{});
         put(std::integral_constant<int, 5>{});
         put(std::integral_constant<int, 6>{});
-        if (u < kBBytes / 16)
-          reinterpret_cast<uint4*>(sh->sl[ss].b + F::kPadBytes)[u] =
-              __ldg(reinterpret_cast<const uint4*>(bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes) + u);
+#pragma unroll
+        for (int i = u; i < kBBytes / 16; i += kSliceWarps * 16)
+          reinterpret_cast<uint4*>(sh->sl[ss].b + F::kPadBytes)[i] =
+              __ldg(reinterpret_cast<const uint4*>(bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes) + i);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) bar_arrive(sh->full_s + ss);
