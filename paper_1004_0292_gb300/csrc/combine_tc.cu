@@ -46,12 +46,12 @@
 // ALU work (~25 instructions an element) and the scale pass bound it now.
 //
 // One persistent CTA per SM (26 warps):
-// * warp 9: bulk copies (cp.async.bulk, a lane a slot) of a tile's 16 slots x
+// * warp 25: bulk copies (cp.async.bulk, a lane a slot) of a tile's 16 slots x
 //   128 rows of FP64 into a ring of kF64Stages stages;
-// * warps 10-25: cut the stage into the seven A slices (core-matrix layout,
-//   K-major, no swizzle) and copy the K-step's B slices (prepared once per
-//   launch in the same layout) into a ring of kSliceStages stages;
-// * warp 8, lane 0: issues seven tcgen05.mma (M = 128, N = 16 (7 - p),
+// * warps 8-23: cut the stage into the seven A slices (core-matrix layout,
+//   K-major, no swizzle) in a ring of kSliceStages stages, into which the
+//   K-step's B slices (prepared once per launch in the same layout) are copied;
+// * warp 24, lane 0: issues seven tcgen05.mma (M = 128, N = 16 (7 - p),
 //   K = 16) a K-step into 448 tensor-memory columns, and commits the stage
 //   and, every 256 slots, the accumulators;
 // * warps 0-7: read the accumulators (tcgen05.ld; warp w: lanes 32 (w % 4),
@@ -124,7 +124,8 @@ struct TcShared {
   F64Stage f64[kF64Stages];
   SliceStage<WIDE> sl[Form<WIDE>::kSliceStages];
   unsigned long long full_f[kF64Stages], empty_f[kF64Stages];
-  unsigned long long full_s[Form<WIDE>::kSliceStages], empty_s[Form<WIDE>::kSliceStages];
+  unsigned long long full_s[Form<WIDE>::kSliceStages], full_b[Form<WIDE>::kSliceStages];
+  unsigned long long empty_s[Form<WIDE>::kSliceStages];
   unsigned long long tmem_full[2], tmem_empty[2], mma_done;
   unsigned tmem_base;
   int abort;
@@ -251,54 +252,63 @@ __host__ __device__ constexpr int core_off(int row, int k) {
 }
 constexpr unsigned kLbo = 128, kSbo = 256;
 
-// 56-bit fixed point X = round(|x| 2^(56 - e)), ties up, for |x| < 2^e (then
-// X < 2^56): the mantissa m at bit 4, shifted right by e + 1022 - E >= 0 (one
-// bit less than its place), plus one, halved.  Without branches: the lanes of
-// a warp hold elements of different exponents.  Zero and subnormals (E = 0)
+// 57-bit fixed point floor(|x| 2^(57 - e)) for |x| < 2^e: the mantissa at bit
+// 4, shifted right by e + 1022 - E >= 0.  Without branches: the lanes of a
+// warp hold elements of different exponents.  Zero and subnormals (E = 0)
 // give 0: e >= -950 (tc_scales_kernel), so that they are shifted out.
-__device__ __forceinline__ uint2 fixed56(double x, int e) {
+// Whatever x and e are, it is below 2^57.
+__device__ __forceinline__ unsigned long long fixed57(double x, int e) {
   const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
   const int E = (int)((hw >> 20) & 0x7FF);
   const unsigned k = min((unsigned)(e + 1022 - E), 63u);
-  const unsigned long long m = (unsigned long long)__funnelshift_l(lw, (hw & 0xFFFFFu) | 0x100000u, 4) << 32 | (lw << 4);
-  const unsigned long long X = ((m >> k) + 1) >> 1;
-  return make_uint2((unsigned)X, (unsigned)(X >> 32));
+  return ((unsigned long long)__funnelshift_l(lw, (hw & 0xFFFFFu) | 0x100000u, 4) << 32 | (lw << 4)) >> k;
 }
-// Signed digits (complex combinations): X with its sign plus the bias that
-// makes every base-256 digit d a byte d + 128 and the top one (|d| <= 256) a
-// field d + 512 of bits 48 ...  The digits' products then average to zero, so
-// that the dropped levels do: with magnitudes and signs they add up
-// coherently, the larger part of the error of a short sum.
-__device__ __forceinline__ uint2 signed_digits(uint2 X, double x) {
-  const long long sg = __double2hiint(x) >> 31;
-  const long long v = (((long long)X.y << 32 | X.x) ^ sg) - sg + 0x0200808080808080ll;
-  return make_uint2((unsigned)v, (unsigned)((unsigned long long)v >> 32));
+__device__ __forceinline__ uint2 halves(unsigned long long v) { return make_uint2((unsigned)v, (unsigned)(v >> 32)); }
+// X = round(|x| 2^(56 - e)), ties up
+__device__ __forceinline__ uint2 fixed56(double x, int e) { return halves((fixed57(x, e) + 1) >> 1); }
+// Signed digits (complex combinations): X with its sign, rounded to nearest,
+// plus the bias that makes every base-256 digit d a byte d + 128 and the top
+// one (|d| <= 256) a field d + 512 of bits 48 ...  The digits' products then
+// average to zero, so that the dropped levels do: with magnitudes and signs
+// they add up coherently, the larger part of the error of a short sum.
+__device__ __forceinline__ uint2 signed_digits(double x, int e) {
+  const unsigned long long t = fixed57(x, e);
+  const unsigned sg = (unsigned)(__double2hiint(x) >> 31);
+  // a negative x's floor is the complement; twice the bias plus the rounding's one
+  constexpr unsigned long long c = 0x0401010101010101ull;
+  return halves((((t >> 32 ^ sg) << 32 | ((unsigned)t ^ sg)) + c) >> 1);
+}
+// The digits of two elements side by side, so that a byte permutation with the
+// exponent byte of 1024 makes a pair of fp16 numbers 1024 + byte: p[0], p[1]
+// from the low words, p[2] the lower half of the high ones.
+struct BytePairs {
+  unsigned p[3], top;
+};
+__device__ __forceinline__ BytePairs byte_pairs(uint2 a, uint2 b) {
+  BytePairs r;
+  r.p[0] = __byte_perm(a.x, b.x, 0x5140);
+  r.p[1] = __byte_perm(a.x, b.x, 0x7362);
+  r.p[2] = __byte_perm(a.y, b.y, 0x5140);
+  r.top = __byte_perm(a.y, b.y, 0x7632);
+  return r;
+}
+// 1024 + byte 6 - P of both (P = 0: 1024 + the top 16 bits)
+template <int P>
+__device__ __forceinline__ __half2 with_exponent(const BytePairs& r) {
+  constexpr int byte = 6 - P;
+  const unsigned v = P == 0 ? r.top | 0x64006400u : __byte_perm(r.p[byte >> 1], 0x64646464u, byte & 1 ? 0x4342 : 0x4140);
+  return *reinterpret_cast<const __half2*>(&v);
 }
 template <int P>
-__device__ __forceinline__ unsigned signed_pair(uint2 a, uint2 b) {
-  constexpr int byte = 6 - P, k = byte & 3;
-  unsigned v;
-  __half2 off;
-  if constexpr (P == 0) {
-    v = __byte_perm(a.y, b.y, 0x7632) | 0x64006400u;
-    off = __half2half2(__ushort_as_half(0xE600));  // -1536
-  } else {
-    const unsigned wa = byte >= 4 ? a.y : a.x, wb = byte >= 4 ? b.y : b.x;
-    v = (__byte_perm(wa, wb, k | k << 4 | (4 + k) << 8 | (4 + k) << 12) & 0x00FF00FFu) | 0x64006400u;
-    off = __half2half2(__ushort_as_half(0xE480));  // -1152
-  }
-  const __half2 d = __hadd2(*reinterpret_cast<const __half2*>(&v), off);
+__device__ __forceinline__ unsigned signed_pair(const BytePairs& r) {
+  const __half2 d = __hadd2(with_exponent<P>(r), __half2half2(__ushort_as_half(P == 0 ? 0xE600 : 0xE480)));  // -1536, -1152
   return *reinterpret_cast<const unsigned*>(&d);
 }
-// Slice P of two elements, their digits (byte 6 - P of X) with their signs as
-// two fp16 integers: the bytes under the exponent of 1024, times the signs,
-// less 1024 (exact).  s1: (+-1, +-1), s2: (-+1024, -+1024).
+// The digits with their signs: the bytes under the exponent of 1024, times the
+// signs, less 1024 (exact).  s1: (+-1, +-1), s2: (-+1024, -+1024).
 template <int P>
-__device__ __forceinline__ unsigned digit_pair(uint2 a, uint2 b, __half2 s1, __half2 s2) {
-  constexpr int byte = 6 - P, k = byte & 3;
-  const unsigned wa = byte >= 4 ? a.y : a.x, wb = byte >= 4 ? b.y : b.x;
-  const unsigned v = (__byte_perm(wa, wb, k | k << 4 | (4 + k) << 8 | (4 + k) << 12) & 0x00FF00FFu) | 0x64006400u;
-  const __half2 d = __hfma2(*reinterpret_cast<const __half2*>(&v), s1, s2);
+__device__ __forceinline__ unsigned digit_pair(const BytePairs& r, __half2 s1, __half2 s2) {
+  const __half2 d = __hfma2(with_exponent<P>(r), s1, s2);
   return *reinterpret_cast<const unsigned*>(&d);
 }
 
@@ -330,6 +340,8 @@ struct CoefView {
     return cplx && (o & 1) ? v.y : v.x;
   }
 };
+// slots in whole K-steps: the stride of the slot scales
+__host__ __device__ __forceinline__ int padded(int S) { return (S + kKStep - 1) / kKStep * kKStep; }
 __device__ __forceinline__ int slots_of(const int* count, int l, int S) { return count != nullptr ? count[l] : S; }
 
 // mx[l'][s] = the largest high word (exponent and leading mantissa bits, sign
@@ -405,7 +417,7 @@ __global__ void tc_scales_kernel(const unsigned* __restrict__ mx, CoefView C, in
         (unsigned long long)(key >> 20) * (unsigned long long)(2 * n) >
             ex[(size_t)lz * S + s] + (unsigned long long)kMaxSpread * (unsigned long long)(2 * n))
       atomicOr(err, kErrSpread);
-    if (o == 0) eslot[(size_t)lz * S + s] = e;
+    if (o == 0) eslot[(size_t)lz * padded(S) + s] = e;
     if (o < O) {
       // the two parts of a complex coefficient share their scale
       for (int k = 0; k < (C.cplx ? 2 : 1); ++k) {
@@ -456,7 +468,7 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
     int d = 0;
     if (o < O && s < cnt) {
       const int g = exp_above(sig[(size_t)lz * OUT + o]) - 1;  // sig = 2^g
-      const double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * S + s] - g);
+      const double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * padded(S) + s] - g);
       if (C.cplx) {  // signed digits
         long long X = llrint(ldexp(b, 56));
         for (int k = 6; k >= q; --k) {
@@ -528,6 +540,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
     }
     for (int i = 0; i < kSliceStages; ++i) {
       bar_init(sh->full_s + i, kSliceWarps / 2);
+      bar_init(sh->full_b + i, 1);
       bar_init(sh->empty_s + i, 1);
     }
     for (int i = 0; i < F::kBuffers; ++i) {
@@ -678,7 +691,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
     const int turn = (warp - kEpiWarps) / (kSliceWarps / 2);
     const int u = (threadIdx.x - kEpiWarps * 32) & (kSliceWarps * 16 - 1);
     const int row = u & (kRows - 1), h = u >> 7;
-    long long fc = 0, sc = 0;
+    long long fc = 0, sc = 0, copied = -1;
     bool ok = true;
     for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int lz = (int)(t / tiles_per_src), l = l0 + lz;
@@ -686,27 +699,24 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
       for (int kk = 0; kk < ks; ++kk, ++fc, ++sc) {
         if ((int)(fc & 1) != turn) continue;
         const int fs = (int)(fc % kF64Stages), ss = (int)(sc % kSliceStages);
-        const int nv = min(kKStep, cnt - kk * kKStep);
-        int es[kPer];
-#pragma unroll
-        for (int i = 0; i < kPer; ++i)
-          es[i] = kPer * h + i < nv ? __ldg(eslot + (size_t)lz * S + kk * kKStep + kPer * h + i) : 0;
+        // past the last slot: any scale and any numbers, finite digits that meet zeros in B
+        const int4* ep = reinterpret_cast<const int4*>(eslot + (size_t)lz * padded(S) + kk * kKStep + kPer * h);
+        const int4 e0 = __ldg(ep), e1 = __ldg(ep + 1);
+        const int es[kPer] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
         if (!bar_wait_warp(sh->full_f + fs, (unsigned)((fc / kF64Stages) & 1), abort)) {
           ok = false;
           break;
         }
-        uint2 X[kPer];
+        BytePairs X[kPer / 2];
         __half2 s1[kPer / 2], s2[kPer / 2];
 #pragma unroll
         for (int i = 0; i < kPer; i += 2) {
           const int j = kPer * h + i;
-          const double a = j < nv ? sh->f64[fs].v[j][row] : 0.0, b = j + 1 < nv ? sh->f64[fs].v[j + 1][row] : 0.0;
-          X[i] = fixed56(a, es[i]);
-          X[i + 1] = fixed56(b, es[i + 1]);
+          const double a = sh->f64[fs].v[j][row], b = sh->f64[fs].v[j + 1][row];
           if constexpr (CPLX) {
-            X[i] = signed_digits(X[i], a);
-            X[i + 1] = signed_digits(X[i + 1], b);
+            X[i / 2] = byte_pairs(signed_digits(a, es[i]), signed_digits(b, es[i + 1]));
           } else {
+            X[i / 2] = byte_pairs(fixed56(a, es[i]), fixed56(b, es[i + 1]));
             const unsigned sg =
                 ((unsigned)__double2hiint(a) >> 16 & 0x8000u) | ((unsigned)__double2hiint(b) & 0x80000000u);
             const unsigned o1 = 0x3C003C00u ^ sg, o2 = 0xE400E400u ^ sg;
@@ -721,15 +731,21 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
           ok = false;
           break;
         }
+        if (u == 0) {
+          bar_arrive_tx(sh->full_b + ss, kBBytes);
+          bulk_copy(sh->sl[ss].b + F::kPadBytes, bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes, kBBytes,
+                    sh->full_b + ss);
+          copied = sc;
+        }
         auto put = [&](auto pc) {
           constexpr int p = decltype(pc)::value;
           unsigned w[kPer / 2];
 #pragma unroll
           for (int i = 0; i < kPer / 2; ++i) {
             if constexpr (CPLX)
-              w[i] = signed_pair<p>(X[2 * i], X[2 * i + 1]);
+              w[i] = signed_pair<p>(X[i]);
             else
-              w[i] = digit_pair<p>(X[2 * i], X[2 * i + 1], s1[i], s2[i]);
+              w[i] = digit_pair<p>(X[i], s1[i], s2[i]);
           }
           unsigned char* dst = sh->sl[ss].a[p] + core_off(row, kPer * h);
           *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -741,16 +757,22 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
         put(std::integral_constant<int, 4>{});
         put(std::integral_constant<int, 5>{});
         put(std::integral_constant<int, 6>{});
-#pragma unroll
-        for (int i = u; i < kBBytes / 16; i += kSliceWarps * 16)
-          reinterpret_cast<uint4*>(sh->sl[ss].b + F::kPadBytes)[i] =
-              __ldg(reinterpret_cast<const uint4*>(bimg + ((size_t)lz * ksteps_cap + kk) * kBBytes) + i);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) bar_arrive(sh->full_s + ss);
       }
     }
-    if (!ok) give_up();
+    if (!ok) {
+      give_up();
+      // the copies of coefficients already issued land before the CTA can exit
+      for (long long q = copied; q >= 0 && q > copied - kSliceStages; --q) {
+        if (((q ^ copied) & 1) != 0) continue;  // the other half's
+        const unsigned long long t0 = gtimer();
+        while (!bar_test(sh->full_b + q % kSliceStages, (unsigned)((q / kSliceStages) & 1)) &&
+               gtimer() - t0 < kTcWaitNs) {
+        }
+      }
+    }
   } else {
     if (WIDE) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(F::kOtherRegs));
     if (warp == kLoadWarp) {
@@ -808,7 +830,8 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
             }
             tc_fence_after();
           }
-          if (!bar_wait(sh->full_s + ss, (unsigned)((sc / kSliceStages) & 1), abort)) {
+          if (!bar_wait(sh->full_s + ss, (unsigned)((sc / kSliceStages) & 1), abort) ||
+              !bar_wait(sh->full_b + ss, (unsigned)((sc / kSliceStages) & 1), abort)) {
             ok = false;
             break;
           }
@@ -867,7 +890,7 @@ TcWork carve(void* w, int nl, int S, int ksteps_cap) {
   t.mx = reinterpret_cast<unsigned*>(p);
   p += align256(sizeof(unsigned) * (size_t)nl * S);
   t.eslot = reinterpret_cast<int*>(p);
-  p += align256(sizeof(int) * (size_t)nl * S);
+  p += align256(sizeof(int) * (size_t)nl * padded(S));
   t.sig = reinterpret_cast<double*>(p);
   p += align256(sizeof(double) * (size_t)nl * kWideOut);
   t.err = reinterpret_cast<int*>(p);
@@ -893,7 +916,8 @@ bool combine_tc_applicable(long long n, int O, int S) {
 
 size_t combine_tc_work_bytes(int nl, int S) {
   const int ks = (S + kKStep - 1) / kKStep;
-  return align256(sizeof(unsigned long long) * (size_t)nl * S) + align256(sizeof(unsigned) * (size_t)nl * S) + align256(sizeof(int) * (size_t)nl * S) +
+  return align256(sizeof(unsigned long long) * (size_t)nl * S) + align256(sizeof(unsigned) * (size_t)nl * S) +
+         align256(sizeof(int) * (size_t)nl * padded(S)) +
          align256(sizeof(double) * (size_t)nl * kWideOut) + 256 + (size_t)nl * ks * Form<true>::kBBytes;
 }
 
