@@ -266,7 +266,7 @@ __device__ __forceinline__ unsigned long long fixed57(double x, int e) {
 __device__ __forceinline__ uint2 halves(unsigned long long v) { return make_uint2((unsigned)v, (unsigned)(v >> 32)); }
 // X = round(|x| 2^(56 - e)), ties up
 __device__ __forceinline__ uint2 fixed56(double x, int e) { return halves((fixed57(x, e) + 1) >> 1); }
-// Signed digits (complex combinations): X with its sign, rounded to nearest,
+// Signed digits (complex and float-float combinations): X with its sign, rounded to nearest,
 // plus the bias that makes every base-256 digit d a byte d + 128 and the top
 // one (|d| <= 256) a field d + 512 of bits 48 ...  The digits' products then
 // average to zero, so that the dropped levels do: with magnitudes and signs
@@ -277,6 +277,19 @@ __device__ __forceinline__ uint2 signed_digits(double x, int e) {
   // a negative x's floor is the complement; twice the bias plus the rounding's one
   constexpr unsigned long long c = 0x0401010101010101ull;
   return halves((((t >> 32 ^ sg) << 32 | ((unsigned)t ^ sg)) + c) >> 1);
+}
+// The same of a float-float number h + l, |h| < 2^e: both mantissas on the
+// 57-bit grid, what is left of them below it cut off.
+__device__ __forceinline__ long long float57(float f, int e) {
+  const unsigned b = __float_as_uint(f);
+  const int E = (int)((b >> 23) & 0xFF);
+  const unsigned m = (b & 0x7FFFFFu) | (unsigned)min(E, 1) << 23;
+  const unsigned k = min((unsigned)(e + 126 - max(E, 1)), 63u);
+  const long long sg = (int)b >> 31;
+  return ((long long)(((unsigned long long)m << 33) >> k) ^ sg) - sg;
+}
+__device__ __forceinline__ uint2 signed_digits(float h, float l, int e) {
+  return halves((unsigned long long)(float57(h, e) + float57(l, e) + 0x0401010101010101ll) >> 1);
 }
 // The digits of two elements side by side, so that a byte permutation with the
 // exponent byte of 1024 makes a pair of fp16 numbers 1024 + byte: p[0], p[1]
@@ -335,6 +348,7 @@ struct CoefView {
   const double2* c;
   long long sl, so, ss;  // strides of source, output, slot
   bool cplx;
+  bool sgn;  // signed digits
   __device__ __forceinline__ double get(int l, int o, int s) const {
     const double2 v = c[l * sl + (cplx ? o >> 1 : o) * so + s * ss];
     return cplx && (o & 1) ? v.y : v.x;
@@ -349,7 +363,10 @@ __device__ __forceinline__ int slots_of(const int* count, int l, int S) { return
 // least kBadKey; ex[l'][s] (may be null) the sum of the components' exponent
 // fields.  By integers: FP64 comparisons run on a pipe of two a clock
 // and SM (2.1 TB/s with them).  grid (x: element blocks, y: slot, z: source)
+// FF: float-float vectors (re, im, their lower parts), the upper parts' keys and
+// exponents as doubles have them.
 constexpr unsigned kBadKey = 0x7FF00000u;
+template <bool FF>
 __global__ void __launch_bounds__(256)
 tc_maxabs_kernel(SlotMap map, long long n, int l0, const int* __restrict__ count, int S, unsigned* __restrict__ mx,
                  unsigned long long* __restrict__ ex) {
@@ -364,9 +381,12 @@ tc_maxabs_kernel(SlotMap map, long long n, int l0, const int* __restrict__ count
     for (int i = 0; i < 4; ++i) v[i] = e + i * stride < n ? __ldg(r + e + i * stride) : make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const unsigned a = v[i].y & 0x7FFFFFFFu, b = v[i].w & 0x7FFFFFFFu;
+      const unsigned a = (FF ? v[i].x : v[i].y) & 0x7FFFFFFFu, b = (FF ? v[i].y : v[i].w) & 0x7FFFFFFFu;
       m = max(m, max(a, b));
-      se += (a >> 20) + (b >> 20);
+      if (FF)
+        se += (a >> 23 != 0 ? (a >> 23) + 896 : 0) + (b >> 23 != 0 ? (b >> 23) + 896 : 0);
+      else
+        se += (a >> 20) + (b >> 20);
     }
     if (se >= 1u << 26) {  // 32 lanes of this still fit 32 bits
       if (ex != nullptr) atomicAdd(ex + (size_t)lz * S + s, (unsigned long long)se);
@@ -374,6 +394,7 @@ tc_maxabs_kernel(SlotMap map, long long n, int l0, const int* __restrict__ count
     }
   }
   m = __reduce_max_sync(0xffffffffu, m);
+  if (FF) m = (unsigned)__double2hiint((double)__uint_as_float(m));
   if ((threadIdx.x & 31) == 0) atomicMax(mx + (size_t)lz * S + s, m);
   if (ex != nullptr) {
     se = __reduce_add_sync(0xffffffffu, se);
@@ -469,7 +490,7 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
     if (o < O && s < cnt) {
       const int g = exp_above(sig[(size_t)lz * OUT + o]) - 1;  // sig = 2^g
       const double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * padded(S) + s] - g);
-      if (C.cplx) {  // signed digits
+      if (C.sgn) {
         long long X = llrint(ldexp(b, 56));
         for (int k = 6; k >= q; --k) {
           d = k == 0 ? (int)X : (int)((X + 128) & 0xFF) - 128;
@@ -513,10 +534,10 @@ __device__ __forceinline__ double sum_to_double(long long xh, long long xl, int 
 
 // ---- the combination ------------------------------------------------------------------------
 // CPLX: complex coefficients (O real outputs, two for each complex one) and
-// signed digits.  SHORT: at most 64 slots, so that a chunk's sums, below 2^22,
+// signed digits.  FF: float-float vectors, signed digits.  SHORT: at most 64 slots, so that a chunk's sums, below 2^22,
 // turn into integers by an FP32 addition instead of a conversion (16 a clock
 // and SM).  ACC: the sums are added to out.
-template <bool CPLX, bool SHORT, bool ACC, bool WIDE>
+template <bool CPLX, bool SHORT, bool ACC, bool WIDE, bool FF>
 __global__ void __launch_bounds__(Form<WIDE>::kThreads, 1)
 combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restrict__ count, int S,
                   const int* __restrict__ eslot, const unsigned char* __restrict__ bimg, int ksteps_cap,
@@ -713,7 +734,11 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
         for (int i = 0; i < kPer; i += 2) {
           const int j = kPer * h + i;
           const double a = sh->f64[fs].v[j][row], b = sh->f64[fs].v[j + 1][row];
-          if constexpr (CPLX) {
+          if constexpr (FF) {
+            const float* fa = reinterpret_cast<const float*>(sh->f64[fs].v[j]) + 4 * (row >> 1) + (row & 1);
+            const float* fb = fa + 2 * kRows;
+            X[i / 2] = byte_pairs(signed_digits(fa[0], fa[2], es[i]), signed_digits(fb[0], fb[2], es[i + 1]));
+          } else if constexpr (CPLX) {
             X[i / 2] = byte_pairs(signed_digits(a, es[i]), signed_digits(b, es[i + 1]));
           } else {
             X[i / 2] = byte_pairs(fixed56(a, es[i]), fixed56(b, es[i + 1]));
@@ -742,7 +767,7 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
           unsigned w[kPer / 2];
 #pragma unroll
           for (int i = 0; i < kPer / 2; ++i) {
-            if constexpr (CPLX)
+            if constexpr (CPLX || FF)
               w[i] = signed_pair<p>(X[i]);
             else
               w[i] = digit_pair<p>(X[i], s1[i], s2[i]);
@@ -929,7 +954,8 @@ namespace {
 // (complex coefficients: the sums are added to out) that is found out before
 // out is touched.
 int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const int* count, double2* out,
-                long long out_l, int l0, int nl, void* work, cudaStream_t st, bool* suits, bool add = false) {
+                long long out_l, int l0, int nl, void* work, cudaStream_t st, bool* suits, bool add = false,
+                bool ff = false) {
   const int ks = (S + kKStep - 1) / kKStep;
   TcWork w = carve(work, nl, S, ks);
   unsigned long long* ex = suits != nullptr ? w.ex : nullptr;
@@ -938,7 +964,8 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
   SS_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), st));
   // blocks of at least 4 elements a thread
   const unsigned gx = (unsigned)std::max(1LL, std::min(64LL, (n + 1023) / 1024));
-  tc_maxabs_kernel<<<dim3(gx, S, nl), 256, 0, st>>>(map, n, l0, count, S, w.mx, ex);
+  auto* maxabs = ff ? tc_maxabs_kernel<true> : tc_maxabs_kernel<false>;
+  maxabs<<<dim3(gx, S, nl), 256, 0, st>>>(map, n, l0, count, S, w.mx, ex);
   SS_CHECK_LAUNCH();
   int dev = 0, sms = 0;
   SS_CUDA(cudaGetDevice(&dev));
@@ -974,12 +1001,14 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     CoefView Cp = C;
     Cp.c += o0 * C.so;
     const int Op = (C.cplx ? 2 : 1) * outs_at(o0);
-    auto* kern = wide    ? (add ? combine_tc_kernel<true, false, true, true> : combine_tc_kernel<true, false, false, true>)
-                 : add    ? combine_tc_kernel<true, false, true, false>
-                 : C.cplx ? (S <= 64 ? combine_tc_kernel<true, true, false, false>
-                                     : combine_tc_kernel<true, false, false, false>)
-                 : S <= 64 ? combine_tc_kernel<false, true, false, false>
-                           : combine_tc_kernel<false, false, false, false>;
+    auto* kern = wide    ? (add ? combine_tc_kernel<true, false, true, true, false>
+                               : combine_tc_kernel<true, false, false, true, false>)
+                 : add    ? combine_tc_kernel<true, false, true, false, false>
+                 : C.cplx ? (S <= 64 ? combine_tc_kernel<true, true, false, false, false>
+                                     : combine_tc_kernel<true, false, false, false, false>)
+                 : ff     ? combine_tc_kernel<false, false, false, false, true>
+                 : S <= 64 ? combine_tc_kernel<false, true, false, false, false>
+                           : combine_tc_kernel<false, false, false, false, false>;
     const size_t smem = (wide ? sizeof(TcShared<true>) : sizeof(TcShared<false>)) + 1024;
     SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // the same every time
     if (wide) {  // its warps share out the registers of the launch
@@ -1012,24 +1041,24 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
 }  // namespace
 
 int combine_tc(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
-               const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st) {
+               const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool ff, bool* suits) {
   if (!combine_tc_applicable(n, O, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
-  return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, false}, O, S, count,
-                     out, (long long)O * n, l0, nl, work, st, nullptr);
+  return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, false, ff}, O, S, count,
+                     out, (long long)O * n, l0, nl, work, st, suits, false, ff);
 }
 
 int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
                        const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits,
                        bool add) {
   if (O < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
-  return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, true}, O, S, count,
+  return combine_all(SlotMap{tab, basis_log, L, nullptr, 0}, n, CoefView{C, (long long)O * S, S, 1, true, true}, O, S, count,
                      out, (long long)O * n, l0, nl, work, st, suits, add);
 }
 
 int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,
                        cudaStream_t st, bool* suits) {
   if (O < 1 || nl < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
-  return combine_all(SlotMap{nullptr, 0, 1, x, S}, n, CoefView{C, 0, 1, O, true}, O, S, nullptr, out, (long long)O * n,
+  return combine_all(SlotMap{nullptr, 0, 1, x, S}, n, CoefView{C, 0, 1, O, true, true}, O, S, nullptr, out, (long long)O * n,
                      0, nl, work, st, suits);
 }
 

@@ -272,17 +272,18 @@ int basis_moments(const KrylovBasis& b, const double2* coef_host, int M, double2
 // throughout, for comparison)
 bool real_moments_enabled();
 
-// Combinations on the tensor cores (combine_tc.cu): FP64 residuals
+// Combinations on the tensor cores (combine_tc.cu): FP64 (ff: float-float) residuals
 // (tab: the basis block table, 2^basis_log slots a block, [slot][L][n]),
 // real coefficients C[l][o][s] (.x), O <= 16 outputs, out[l][o][n] for the
 // sources l0 .. l0 + nl - 1; work: combine_tc_work_bytes(nl, S) bytes.
-// Synchronises st (reads the kernel's error word).
+// suits: as below, or null.  Synchronises st (reads the kernel's error word).
 bool combine_tc_enabled();
 bool combine_tc_applicable(long long n, int O, int S);
 size_t combine_tc_work_bytes(int nl, int S);
 int combine_tc(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
-               const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st);
-// The same with complex coefficients and any number of outputs (8 a launch).
+               const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool ff = false,
+               bool* suits = nullptr);
+// The same with complex coefficients and any number of outputs (8 or 16 a launch).
 // *suits = false (the outputs then not to be used) when a vector does not suit
 // a fixed point relative to its largest component: point-like, not finite.
 // add: the sums are added to out, which is as it was when they do not suit.

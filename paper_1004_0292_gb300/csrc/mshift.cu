@@ -3177,9 +3177,12 @@ int basis_moments(const KrylovBasis& b, const double2* coef_host, int M, double2
   const size_t w_bytes = (sizeof(double2) * (size_t)N * M + 255) / 256 * 256;
   const long long cnt = (long long)L * M * S;
   const bool rc = real_coef && real_moments_enabled();
-  // FP64 residuals with real coefficients: the tensor-core combination
-  // (unless SSQCD_MOMENTS_TC=0), one source a launch, each with its work space
-  const bool tc = !b.df && rc && combine_tc_enabled() && combine_tc_applicable(b.n, M, S);
+  // Real coefficients: the tensor-core combination (unless
+  // SSQCD_MOMENTS_TC=0).  Float-float residuals take it with more than eight
+  // moments, where the FP32 pipes read them twice (16^3 x 32 x 8 sources, 2500
+  // residuals: 16 moments 1028 -> 566 ms; 8 moments are as fast there, 20.0
+  // against 21.9 ms a source), and when its fixed point suits them.
+  const bool tc = rc && (!b.df || M > 8) && combine_tc_enabled() && combine_tc_applicable(b.n, M, S);
   const size_t g_bytes = (sizeof(double2) * (size_t)cnt + (b.df ? sizeof(float2) * (size_t)cnt : 0) + 255) / 256 * 256;
   const size_t tc_src = tc ? (combine_tc_work_bytes(1, S) + 255) / 256 * 256 : 0;
   // W, G and (float-float residuals) Re G as float-float pairs
@@ -3192,53 +3195,55 @@ int basis_moments(const KrylovBasis& b, const double2* coef_host, int M, double2
   basis_window_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(b.gam.as<double2>(), W, N, M, L, S, G);
   SS_CHECK_LAUNCH();
   count_launches(1);
-  if (b.df && rc) {
-    coef_real_to_ff_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(G, cnt, Gr);
-    SS_CHECK_LAUNCH();
-    count_launches(1);
-  }
-  auto one = [&](int l0, int nl, cudaStream_t s) -> int {
-    if (b.df) {
-      // outputs a thread accumulates: 8 (default) or 4 (SSQCD_COMB_DF_OUT=4:
-      // fewer registers, more resident warps, the residuals read twice as often)
-      static const int out_df = [] {
-        const char* e = std::getenv("SSQCD_COMB_DF_OUT");
-        return (e != nullptr && std::atoi(e) == 4) ? 4 : 8;
-      }();
-      const int per = out_df;
-      const dim3 grid((unsigned)((b.n + kCombThreads - 1) / kCombThreads), nl, (M + per - 1) / per);
-      char* const* tab = b.tab.as<char*>();
-      const int* count = b.count.as<int>();
-      // SSQCD_COMB_DF_TILE=32: real coefficients in tiles of 32 (comparison runs)
-      static const bool tile32 = [] {
-        const char* e = std::getenv("SSQCD_COMB_DF_TILE");
-        return e != nullptr && std::atoi(e) == 32;
-      }();
-      if (per == 4 && rc)
-        basis_combine_df_kernel<4, true, kCombTileRC>
-            <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
-      else if (per == 4)
-        basis_combine_df_kernel<4, false, kCombTile>
-            <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
-      else if (rc && tile32)
-        basis_combine_df_kernel<8, true, kCombTile>
-            <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
-      else if (rc)
-        basis_combine_df_kernel<8, true, kCombTileRC>
-            <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
-      else
-        basis_combine_df_kernel<8, false, kCombTile>
-            <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
+  auto on_fp32 = [&](int l0, int nl, cudaStream_t s) -> int {
+    if (rc) {
+      const long long at = (long long)l0 * M * S, of = (long long)nl * M * S;  // these sources'
+      coef_real_to_ff_kernel<<<(unsigned)((of + 255) / 256), 256, 0, s>>>(G + at, of, Gr + at);
       SS_CHECK_LAUNCH();
       count_launches(1);
-      return SSQCD_OK;
     }
+    // outputs a thread accumulates: 8 (default) or 4 (SSQCD_COMB_DF_OUT=4:
+    // fewer registers, more resident warps, the residuals read twice as often)
+    static const int out_df = [] {
+      const char* e = std::getenv("SSQCD_COMB_DF_OUT");
+      return (e != nullptr && std::atoi(e) == 4) ? 4 : 8;
+    }();
+    const int per = out_df;
+    const dim3 grid((unsigned)((b.n + kCombThreads - 1) / kCombThreads), nl, (M + per - 1) / per);
+    char* const* tab = b.tab.as<char*>();
+    const int* count = b.count.as<int>();
+    // SSQCD_COMB_DF_TILE=32: real coefficients in tiles of 32 (comparison runs)
+    static const bool tile32 = [] {
+      const char* e = std::getenv("SSQCD_COMB_DF_TILE");
+      return e != nullptr && std::atoi(e) == 32;
+    }();
+    if (per == 4 && rc)
+      basis_combine_df_kernel<4, true, kCombTileRC>
+          <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
+    else if (per == 4)
+      basis_combine_df_kernel<4, false, kCombTile>
+          <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
+    else if (rc && tile32)
+      basis_combine_df_kernel<8, true, kCombTile>
+          <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
+    else if (rc)
+      basis_combine_df_kernel<8, true, kCombTileRC>
+          <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
+    else
+      basis_combine_df_kernel<8, false, kCombTile>
+          <<<grid, kCombThreads, 0, s>>>(tab, b.n, L, G, Gr, M, S, count, s_hat, l0);
+    SS_CHECK_LAUNCH();
+    count_launches(1);
+    return SSQCD_OK;
+  };
+  auto one = [&](int l0, int nl, cudaStream_t s) -> int {
     if (tc) {
-      for (int l = l0; l < l0 + nl; ++l)
-        SS_TRY(combine_tc(b.tab.as<char*>(), kBasisLog, b.n, L, G, M, S, b.count.as<int>(), s_hat, l, 1,
-                          tcw + tc_src * (size_t)l, s));
-      return SSQCD_OK;
+      bool suits = true;
+      SS_TRY(combine_tc(b.tab.as<char*>(), kBasisLog, b.n, L, G, M, S, b.count.as<int>(), s_hat, l0, nl,
+                        tcw + tc_src * (size_t)l0, s, b.df, b.df ? &suits : nullptr));
+      return suits ? SSQCD_OK : on_fp32(l0, nl, s);
     }
+    if (b.df) return on_fp32(l0, nl, s);
     return launch_combine<double2, double2>(b.tab.as<char*>(), b.n, L, G, M, S, b.count.as<int>(), s_hat, s, l0,
                                             nl, rc);
   };

@@ -152,3 +152,29 @@ def test_shifted_solutions_from_stored_residuals(ss, dims, L, N):
     assert code == ss.ERR_NOCONV
     for j in range(3):
         assert np.linalg.norm(y1[-1, j] - y2[0, j]) <= 1e-10 * np.linalg.norm(y2[0, j])
+
+
+# float-float residuals: the update form's moments come from float-float shift
+# vectors of the same seed recurrence.  Point sources: their first residuals
+# keep the FP32 pipes' combination; a source of zeros; 16 and 17 moments are on
+# both sides of what the tensor cores take.
+@pytest.mark.parametrize("kind", ["gauss", "point", "zero"])
+@pytest.mark.parametrize("dims,L,M", [((5, 4, 3, 8), 3, 5), ((8, 8, 8, 8), 1, 8), ((3, 3, 5, 8), 2, 16), ((3, 3, 5, 8), 2, 17)])
+def test_moments_of_floatfloat_residuals(ss, dims, L, M, kind):
+    U = synthetic.gauge_field(dims, "smooth", seed=5, eps=0.3)
+    v = synthetic.gaussian_sources(dims, L, seed=6)
+    if kind == "point":
+        v[:] = 0
+        for l in range(L):
+            v[l, 3 * l + 1, l, 0] = 1.0
+    elif kind == "zero":
+        v[-1] = 0
+    lat = ss.create_lattice(dims, 0.12, -1, precision=ss.DF)
+    ss.upload_gauge(lat, U)
+    base, st0 = ss.ss_moments(lat, (0.10, 0.13), 20, M, v, basis=0)
+    got, st1 = ss.ss_moments(lat, (0.10, 0.13), 20, M, v, basis=1)
+    assert st0["basis"] == 0 and st1["basis"] == 1
+    for l in range(L):
+        for k in range(M):
+            # the stopping rule's residual, as for the FP64 solutions above
+            assert np.linalg.norm(got[l, k] - base[l, k]) <= 1e-8 * np.linalg.norm(base[l, k])
