@@ -616,7 +616,6 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   // what the last block's tail needs of a source, loaded ahead of it
   const int lt = min((int)threadIdx.x, L - 1);
   const double rr_t = c.seed[lt].rr;
-  const int live_t = c.live[lt];
   d_pq = warp_sum(d_pq);
   if (lane == 0) sred[w] = d_pq;
   __syncthreads();
@@ -632,6 +631,10 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   }
   __syncthreads();
   if (!s_last) return;
+  // Kernel S of the iteration before may clear a count meanwhile: a block that
+  // reads zero adds nothing to its source's sum, so that the count read after
+  // every block's has to say whether the sum is used.
+  const int live_t = __ldcg(c.live + lt);
   tail_sums<kWarps>(c.partial, nbw, L, sums, spart);
   static_assert(kMaxSources <= Op::kThreads, "a thread a source");
   if ((int)threadIdx.x < L && live_t != 0) {
@@ -802,7 +805,6 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
   // what the last block's tail needs of a source, loaded ahead of it
   const int lt = min((int)threadIdx.x, L - 1);
   const double vn2_t = c.vnorm2[lt], irr_t = c.inv_rr[lt], alpha_t = c.alpha[lt], S_t = c.seed[lt].pad[1];
-  const int live_t = c.live[lt];
   char *slot1 = nullptr, *slot2 = nullptr;  // slots of the next iteration
   if (c.tab != nullptr) {
     slot1 = reinterpret_cast<char*>(basis_slot<V2>(c, kb + 1, (long long)L * n));
@@ -820,6 +822,7 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
   }
   __syncthreads();
   if (!s_last) return;
+  const int live_t = __ldcg(c.live + lt);  // after every block's, as in A
   tail_sums<kSeedBlock / 32>(c.partial_rr, nb, L, sums, sred);
   if ((int)threadIdx.x < L) {  // kMaxSources <= kSeedBlock
     const double a = sums[lt];
