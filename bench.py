@@ -93,9 +93,14 @@ UPDATE_BYTES_PER_UNIT = 64
 # + 24 = 888 FP64 instructions; counted as 1368 flop/site/rhs (FMA = 2); bytes:
 # spinor in 192 B + out 192 B + links 576 B (shared by the rhs) per site.
 STENCIL_FLOP_PER_SITE = 1368
-# DRAM traffic of one launch of the FP64 stencil kernel (cg_stencil_kernel<Stencil64h>,
-# 1 rhs, 16^3 x 32) from a one-pass ncu capture; None until captured for the current kernel.
-STENCIL_FP64_TRAFFIC = 102877184.0 + 11855872.0  # ncu: dram read 102.88 MB + write 11.86 MB
+# The stencil of FP64 lattices in 60-bit fixed point (cg_stencil_kernel<StencilFix<1>>): a
+# hop takes 3 products of 32-bit digits for each of the 18 x 4 real products of its two
+# link-times-spin-row products; the wide multiply-add runs at 32 lanes a clock and SM.
+STENCIL_MADS_PER_SITE = 8 * 2 * 9 * 4 * 3
+WIDE_MAD_PEAK = 152 * 32 * 2.07e9 / 1e12
+# DRAM traffic of one launch of that kernel (1 rhs, 16^3 x 32) from an ncu capture;
+# None until captured for the current kernel.
+STENCIL_FP64_TRAFFIC = None
 # DRAM traffic of one launch of each update kernel with all 128 (source,
 # shift) pairs live on this workload (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum, one capture per kernel; the algorithmic bytes of such
@@ -226,7 +231,7 @@ def moments_flops(w, st, n):
 def moments_roofline(w, st, n, mom_tf, step_ms, peaks):
     """Roofline line of the moment combination.  With real coefficients and
     FP64 residuals it runs on the tensor cores (combine_tc_kernel, unless
-    SSQCD_MOMENTS_TC=0): exact bf16 slices, so its roof is reading the
+    SSQCD_MOMENTS_TC=0): exact fp16 slices, so its roof is reading the
     stored residuals once (16 B a complex element and slot, each window);
     the phase also holds the scale pass, which reads them once more a
     window.  Otherwise the FP64-pipe kernel, bound by the FP64 rate."""
@@ -236,7 +241,7 @@ def moments_roofline(w, st, n, mom_tf, step_ms, peaks):
         gbs = nbytes / (st["ms_moments"] / 1e3) / 1e9
         return {
             "kernel": "combine_tc_kernel (moments on the tensor cores: the FP64 residuals and real coefficients "
-                      "cut exactly into seven 8-bit bf16 slices, 28 slice-pair tcgen05.mma into tensor memory, "
+                      "cut exactly into seven 8-bit fp16 slices, 28 slice-pair tcgen05.mma into tensor memory, "
                       "exact integer sums; with its scale pass, one read of the residuals more)",
             "bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": gbs / peaks["hbm_gbs"], "traffic": None,
@@ -326,8 +331,9 @@ def run_ours(args):
     # shifted-CG runs one after another: groups of block_streams runs of Lb sources side by side
     n_groups = -(-w["L"] // (Lb * w.get("block_streams", 1)))
     sten_flops = it_tot * V * Lb * STENCIL_FLOP_PER_SITE
-    sten_bytes = it_tot * V * (Lb * 2 * 192 + 576)
+    sten_bytes = it_tot * V * (Lb * 3 * 192 + 576)  # p and its digits in, q out, the links' digits
     sten_tf = sten_flops / (ms_sten / 1e3) / 1e12 if ms_sten > 0 else None
+    sten_mads = it_tot * V * Lb * STENCIL_MADS_PER_SITE / (ms_sten / 1e3) / 1e12 if ms_sten > 0 else None
 
     # ---- end to end through the C ABI with host buffers ----
     e2e = None
@@ -388,15 +394,14 @@ def run_ours(args):
         }
         # the float-float arm's dominant kernel: its stencil (one rhs a launch)
         sten_us_m = 1e3 * sum(x["ms_k_stencil"] for x in s_m) / it_m
-        sten_gbs_m = V * (Lb * 2 * 192 + 576) / (sten_us_m * 1e-6) / 1e9 if sten_us_m > 0 else None
+        sten_gbs_m = V * (Lb * 3 * 192 + 576) / (sten_us_m * 1e-6) / 1e9 if sten_us_m > 0 else None
         mixed["stencil"] = {
-            "kernel": "cg_stencil_kernel<StencilDF<4>> (q = K p in float-float with the (p, q) partials; 32 "
-                      "sites and 8 warps, one hop each, a block)",
-            "bound": "FP32 issue and latency (float-float chains; the FP32 pipes run at 64x the FP64 rate)",
+            "kernel": "cg_stencil_kernel<StencilFix<1, float4>> (q = K p with the (p, q) partials: hops in 60-bit "
+                      "fixed point, the rest in float-float)",
+            "bound": "integer multiply-adds and their latency at 16 warps an SM",
             "avg_launch_us": sten_us_m, "rhs_per_launch": Lb, "hbm_achieved_gbs": sten_gbs_m,
             "hbm_frac": sten_gbs_m / peaks["hbm_gbs"] if sten_gbs_m else None,
-            "note": "algorithmic bytes 192 in + 192 out + 576 links (float-float, 16 B a complex element) a "
-                    "site; profiles/stencil_floatfloat_16x16x16x32.md",
+            "note": "algorithmic bytes 192 + 192 in (p and its digits) + 192 out + 576 links a site",
             "share_of_step": (sten_us_m * p_m[-1]["iterations"] * w["L"] / Lb) / 1e3 / (ms_m / args.steps),
         }
         del lat_m
@@ -443,17 +448,19 @@ def run_ours(args):
             "cg_us_per_iteration": 1e3 * last["ms_cg"] / max(1, last["iterations"]) / n_groups,
             "stored_residual_bytes_per_block": last["basis_bytes"],
             "roofline": {
-                "kernel": "cg_stencil_kernel<Stencil64h> (q = K p with the (p, q) partials, FP64, 16 sites a block; "
-                          "the step's dominant kernel: 2 x L x iterations launches)",
-                "bound": "alu", "achieved": sten_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": sten_tf / FP64_PEAK_TFLOPS if sten_tf else None, "traffic": STENCIL_FP64_TRAFFIC,
-                "traffic_note": "dram read + write of one launch (1 rhs, 16^3 x 32) from a one-pass ncu capture "
-                                "(profiles/launches_fp64_16x16x16x32_headline.md); algorithmic 192 + 192 + 576 B a "
-                                "site = 125.8 MB",
-                "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (no FP64 entry in "
+                "kernel": "cg_stencil_kernel<StencilFix<1>> (q = K p with the (p, q) partials: hops in 60-bit fixed "
+                          "point on the integer multiply-adds; the step's dominant kernel: 2 x L x iterations launches)",
+                "bound": "alu", "achieved": sten_mads, "peak": WIDE_MAD_PEAK,
+                "unit": "T 32 x 32 + 64-bit integer multiply-adds/s",
+                "frac": sten_mads / WIDE_MAD_PEAK if sten_mads else None, "traffic": STENCIL_FP64_TRAFFIC,
+                "traffic_note": "no capture of this kernel on this workload; algorithmic 192 + 192 B of digits and p in, "
+                                "192 out, 576 of links a site = 151 MB",
+                "peak_source": "derived: 152 SMs x 32 lanes/clk (measured by a probe) x 2.07 GHz (no integer entry in "
                                "MEASURED_PEAKS.json)",
-                "flop_count": "1368 a site and rhs (the Wilson hop's 1320 plus gamma5 and the diagonal; FMA = 2); "
-                              "~910 FP64 instructions, so 0.75 of the flop peak is the instruction-issue bound",
+                "op_count": "1728 a site and rhs: 8 hops x 18 complex products x 4 real ones x 3 digit products",
+                "fp64_equivalent_tflops": sten_tf,
+                "fp64_equivalent_note": "1368 flop a site and rhs (the Wilson hop's 1320 plus gamma5 and the diagonal; "
+                                        "FMA = 2), beside the FP64 pipe's 1.259 TFLOP/s",
                 "avg_launch_us": 1e3 * ms_sten / max(1, it_tot), "rhs_per_launch": Lb,
                 "hbm_achieved_gbs": sten_bytes / (ms_sten / 1e3) / 1e9 if ms_sten > 0 else None,
                 "launch_time_source": "a separate step with the library's kernel timing on (one run at a time): "
@@ -522,8 +529,10 @@ def run_config2(ss, stream, flush, args, world, peaks):
             it_tot = sum(s["launches_update"] for s in stats)
             ms_sten = sum(s["ms_k_stencil"] for s in stats)
             tf = it_tot * V * w["L"] * STENCIL_FLOP_PER_SITE / (ms_sten / 1e3) / 1e12
-            ent["stencil"] = {"kernel": "cg_stencil_kernel<Stencil64h>", "bound": "alu", "achieved_tflops": tf,
-                              "frac": tf / FP64_PEAK_TFLOPS, "traffic": None,
+            mads = tf / STENCIL_FLOP_PER_SITE * STENCIL_MADS_PER_SITE
+            ent["stencil"] = {"kernel": "cg_stencil_kernel<StencilFix<1>>", "bound": "alu", "achieved": mads,
+                              "unit": "T 32 x 32 + 64-bit integer multiply-adds/s", "frac": mads / WIDE_MAD_PEAK,
+                              "fp64_equivalent_tflops": tf, "traffic": None,
                               "avg_launch_us": 1e3 * ms_sten / max(1, it_tot)}
             ent["kernel_us_per_iteration"] = {
                 "stencil": 1e3 * ms_sten / max(1, it_tot),

@@ -416,7 +416,7 @@ struct StencilFix {
       }
       __syncthreads();
     }
-    double d = 0.0;
+    double d = 0.0, d2 = 0.0;
     // component k of this lane: 0..2 spin r, 3..5 spin 2 + r.  Z: sigma = 0, the
     // paper's seed shift, leaves out the sigma p term (as a form of its own: an
     // FP64 product under a predicate takes its pipe slot all the same)
@@ -458,7 +458,8 @@ struct StencilFix {
             o.y = fma(sg, o.y, sigma * pv.y);
           }
           q[(size_t)comp * V + s] = o;
-          d = fma(pv.x, o.x, fma(pv.y, o.y, d));
+          d = fma(pv.x, o.x, d);  // two sums: half the chain, and its rounding
+          d2 = fma(pv.y, o.y, d2);
         }
       }
     };
@@ -466,7 +467,7 @@ struct StencilFix {
       finish(std::true_type{});
     else
       finish(std::false_type{});
-    return kFF ? (double)dff.x + (double)dff.y : d;
+    return kFF ? (double)dff.x + (double)dff.y : d + d2;
   }
 };
 
@@ -793,8 +794,8 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
             }
           }
         }
-        acc0 = au[0] + au[1];
-        acc1 = au[2] + au[3];
+        acc0 = au[0] + au[2];
+        acc1 = au[1] + au[3];
       };
       if (sc == (T)1)
         sweep(std::false_type{});
@@ -1659,51 +1660,68 @@ cg_reliable_kernel(Control c, int L, const double2* __restrict__ v, const double
 // with the same backward recurrence, and p-hat_j likewise.  The first segment
 // has k0 = 0, y = 0 and p-hat = r_0.
 //
-// g_j(s) scs(s) for every (source, shift) pair, one thread each: the backward
-// recurrence g_j(s) = a_j(s) + b_j(s) g_j(s+1) from s = K_j = iters_j - 1
-// (zero above) down to k0; gam [L N][S], slot s at s - k0.  Slot k0 of a later
-// segment is left out (zero): its coefficient, p-hat's, goes to gp.
-__global__ void basis_gamma_kernel(Control c, int L, int N, int S, double2* __restrict__ gam, int k0,
-                                   double2* __restrict__ gp) {
-  const int qi = blockIdx.x * blockDim.x + threadIdx.x;
-  const int NL = N * L;
-  if (qi >= NL) return;
-  const int l = qi / N;
-  const int K = c.iters[qi] - 1;
-  double2* gq = gam + (size_t)qi * S - k0;
-  for (int s = S - 1 + k0; s > max(K, k0 - 1); --s) gq[s] = make_double2(0.0, 0.0);
-  // the recurrence is a chain of dependent FMAs (64 cycles each); the loads
-  // of the coefficients it needs are independent of it, so they are issued
-  // kG steps ahead
-  constexpr int kG = 8;
-  double gx = 0.0, gy = 0.0;
-  for (int s1 = K; s1 >= k0; s1 -= kG) {
-    double2 a[kG], b[kG];
-    double sc[kG];
-#pragma unroll
-    for (int i = 0; i < kG; ++i) {
-      const int s = s1 - i;
-      if (s >= k0) {
-        a[i] = basis_coef(c, s, NL, 0)[qi];
-        b[i] = basis_coef(c, s, NL, 1)[qi];
-        sc[i] = s == k0 ? 1.0 : basis_scale(c, s - 1, NL, L)[l];
+// g_j(s) scs(s) for every (source, shift) pair: the backward recurrence
+// g_j(s) = a_j(s) + b_j(s) g_j(s+1) from s = K_j = iters_j - 1 (zero above)
+// down to k0; gam [L N][S], slot s at s - k0.  Slot k0 of a later segment is
+// left out (zero): its coefficient, p-hat's, goes to gp.
+//
+// The recurrence is a chain of FP64 multiply-adds, and a warp's takes 64
+// cycles: a block's warp 0 runs kGammaQ pairs, the real parts in its lower and
+// the imaginary parts in its upper lanes (two instructions a step, not four),
+// through tiles of shared memory that the other warps fill ahead and empty,
+// times the scales, behind it (780 slots of 8^4: 330 -> 128 us; a thread a pair
+// with its loads eight steps ahead before, 208 with three warps for the tiles).
+constexpr int kGammaQ = 16, kGammaT = 32, kGammaBlock = 32 + kGammaQ * kGammaT;
+__global__ void __launch_bounds__(kGammaBlock)
+basis_gamma_kernel(Control c, int L, int N, int S, double2* __restrict__ gam, int k0, double2* __restrict__ gp) {
+  __shared__ double2 sa[2][kGammaT][kGammaQ], sb[2][kGammaT][kGammaQ];
+  __shared__ double2 sg[2][kGammaT][kGammaQ];
+  __shared__ int s_K[kGammaQ];
+  const int NL = N * L, q0 = blockIdx.x * kGammaQ, top = S - 1 + k0;
+  const int tiles = (S + kGammaT - 1) / kGammaT;  // tile t: s = top - t kGammaT - i
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, u = threadIdx.x - 32;
+  if (threadIdx.x < kGammaQ) s_K[threadIdx.x] = q0 + (int)threadIdx.x < NL ? c.iters[q0 + threadIdx.x] - 1 : k0 - 1;
+  __syncthreads();
+  double g = 0.0;  // this lane's part
+  for (int t = -1; t <= tiles; ++t) {
+    if (w == 0) {
+      if (t >= 0 && t < tiles) {
+        const int q = lane & (kGammaQ - 1);
+        const bool im = lane >= kGammaQ;
+#pragma unroll 8
+        for (int i = 0; i < kGammaT; ++i) {
+          const double2 a = sa[t & 1][i][q], b = sb[t & 1][i][q];
+          const double o = __shfl_xor_sync(0xffffffffu, g, kGammaQ);
+          g = fma(b.x, g, fma(im ? b.y : -b.y, o, im ? a.y : a.x));
+          reinterpret_cast<double*>(&sg[t & 1][i][q])[im] = g;
+        }
+      }
+    } else {
+      if (t + 1 < tiles) {
+        for (int x = u; x < kGammaT * kGammaQ; x += kGammaBlock - 32) {
+          const int i = x / kGammaQ, q = x % kGammaQ, s = top - (t + 1) * kGammaT - i;
+          const bool ok = s >= k0 && s <= s_K[q];
+          sa[(t + 1) & 1][i][q] = ok ? basis_coef(c, s, NL, 0)[q0 + q] : make_double2(0.0, 0.0);
+          sb[(t + 1) & 1][i][q] = ok ? basis_coef(c, s, NL, 1)[q0 + q] : make_double2(0.0, 0.0);
+        }
+      }
+      if (t >= 1) {
+        for (int x = u; x < kGammaT * kGammaQ; x += kGammaBlock - 32) {
+          const int q = x / kGammaT, i = x % kGammaT, s = top - (t - 1) * kGammaT - i, qi = q0 + q;
+          if (qi >= NL || s < k0) continue;
+          const double2 v = sg[(t - 1) & 1][i][q];
+          double2 o = make_double2(0.0, 0.0);
+          if (s == k0 && gp != nullptr) {
+            gp[qi] = v;
+          } else if (s <= s_K[q]) {
+            const double sc = s == k0 ? 1.0 : basis_scale(c, s - 1, NL, L)[qi / N];
+            o = make_double2(v.x * sc, v.y * sc);
+          }
+          gam[(size_t)qi * S + (s - k0)] = o;
+        }
       }
     }
-#pragma unroll
-    for (int i = 0; i < kG; ++i) {
-      const int s = s1 - i;
-      if (s >= k0) {
-        const double nx = fma(b[i].x, gx, fma(-b[i].y, gy, a[i].x));
-        const double ny = fma(b[i].x, gy, fma(b[i].y, gx, a[i].y));
-        gx = nx;
-        gy = ny;
-        gq[s] = make_double2(gx * sc[i], gy * sc[i]);
-      }
-    }
-  }
-  if (gp != nullptr) {
-    gp[qi] = make_double2(gx, gy);
-    if (S > 0) gq[k0] = make_double2(0.0, 0.0);
+    __syncthreads();
   }
 }
 
@@ -2749,7 +2767,7 @@ class CgRun final : public CgRunBase {
     const bool old = k0_ > 0;
     DevBuf gp;
     if (old) SS_TRY(gp.alloc(sizeof(double2) * NL));
-    basis_gamma_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, basis_S_, gam_.as<double2>(), k0_,
+    basis_gamma_kernel<<<(NL + kGammaQ - 1) / kGammaQ, kGammaBlock, 0, st_>>>(c_, L_, N_, basis_S_, gam_.as<double2>(), k0_,
                                                           gp.as<double2>());
     SS_CHECK_LAUNCH();
     count_launches(1);
@@ -2825,7 +2843,7 @@ class CgRun final : public CgRunBase {
     SS_TRY(gy.alloc(sizeof(double2) * (size_t)NL * S));
     SS_TRY(gp.alloc(sizeof(double2) * (size_t)NL * S));
     if (old) SS_TRY(go.alloc(2 * sizeof(double2) * NL));
-    basis_gamma_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, S, gy.as<double2>(), k0_, go.as<double2>());
+    basis_gamma_kernel<<<(NL + kGammaQ - 1) / kGammaQ, kGammaBlock, 0, st_>>>(c_, L_, N_, S, gy.as<double2>(), k0_, go.as<double2>());
     SS_CHECK_LAUNCH();
     basis_phat_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, k, S, gp.as<double2>(), k0_,
                                                          old ? go.as<double2>() + NL : nullptr);
