@@ -14,7 +14,7 @@ Rayleigh-Ritz, acceptance, eigenpair readback):
   time (opts.source_block = 1), two such runs side by side on their own
   streams (opts.block_streams = 2), so that the stored seed residuals of the
   two fit the device memory; FP64 throughout ("plain"), the moment
-  combination on the tensor cores through an exact bf16 splitting of the
+  combination on the tensor cores through an exact fp16 splitting of the
   FP64 operands (as accurate as the FP64 sum; SSQCD_MOMENTS_TC=0 runs it
   on the FP64 pipe).
 

@@ -214,7 +214,7 @@ typedef struct {
                              With real coefficients and FP64 residuals the
                              combination runs on the tensor cores: residuals
                              and coefficients are split exactly into seven
-                             8-bit bf16 slices on power-of-two grids and the
+                             8-bit fp16 slices on power-of-two grids and the
                              slice products summed exactly, so the moments
                              lie within 2^-56 of the operand scales of the
                              FP64 sum (SSQCD_MOMENTS_TC=0 in the environment:

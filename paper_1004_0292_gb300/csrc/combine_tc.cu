@@ -38,25 +38,33 @@
 // within a residual, the fixed-point grid leaves the small ones fewer bits
 // (2.4e-15 against 6.5e-16).
 //
-// Measured (2502 slots of 786,432 complex elements, 31.5 GB, 16 real outputs,
-// scale pass included): 18.5 ms, 1.7 TB/s.  Before: 34.6 ms -- the scale pass
-// compared in FP64 (15 ms; 5 by integers), one lane issued the copies, each
-// behind a dependent load of the block table (3200 cycles a K-step), and the
-// epilogue converted to 64-bit integers on the FP64 pipe.  The slicing warps'
-// ALU work (~25 instructions an element) and the scale pass bound it now.
+// Measured (2502 slots of 786,432 complex elements, 31.5 GB, 16 real outputs):
+// 15.1 ms, 2.1 TB/s, and 5.0 ms of scale pass.  Before: 34.6 ms -- the scale
+// pass compared in FP64 (15 ms; 5 by integers), one lane issued the copies, each
+// behind a dependent load of the block table (3200 cycles a K-step), the epilogue
+// converted to 64-bit integers on the FP64 pipe, and a digit took twice the
+// integer operations.  Those of the slicing warps (~20 an element, the integer
+// pipe 69% busy) and the scale pass bound it now.
 //
-// One persistent CTA per SM (26 warps):
+// One persistent CTA per SM (26 warps; wide form 28):
 // * warp 25: bulk copies (cp.async.bulk, a lane a slot) of a tile's 16 slots x
 //   128 rows of FP64 into a ring of kF64Stages stages;
 // * warps 8-23: cut the stage into the seven A slices (core-matrix layout,
-//   K-major, no swizzle) in a ring of kSliceStages stages, into which the
-//   K-step's B slices (prepared once per launch in the same layout) are copied;
-// * warp 24, lane 0: issues seven tcgen05.mma (M = 128, N = 16 (7 - p),
-//   K = 16) a K-step into 448 tensor-memory columns, and commits the stage
-//   and, every 256 slots, the accumulators;
+//   K-major, no swizzle) in a ring of kSliceStages stages, half of them a K-step
+//   in turn; the K-step's B slices (prepared once per launch in the same layout)
+//   are copied beside them;
+// * warp 24, lane 0: issues seven tcgen05.mma (M = 128, N = 16 (7 - p), K = 16) a
+//   K-step into 448 tensor-memory columns, and commits the stage and, every 256
+//   slots, the accumulators;
 // * warps 0-7: read the accumulators (tcgen05.ld; warp w: lanes 32 (w % 4),
 //   outputs 8 (w / 4) ..), add them exactly into X_hi and X_lo, and at the
 //   end of a tile form and store the outputs.
+// Wide form (more than eight complex outputs; Form): the cut is what a pass costs,
+// whatever its outputs, so that 16 complex ones at a time halve it (64 outputs of
+// 1000 slots x 4 sources of 12^4: 77 -> 42 ms, then 31 with the rest).  Its 28 pairs
+// do not fit tensor memory: the pairs of a level share an accumulator, by rows of
+// zeros ahead of B's, for 96 slots; two accumulators, so that the epilogue, with
+// registers of the other warps, and the products overlap.
 // Every wait is bounded (1 s of device time); past it the kernel sets *err,
 // lets its issued copies and MMAs finish, frees its tensor memory and
 // returns.

@@ -22,7 +22,8 @@
 // Two forms of the loop; every kernel finishes its reduction in its last
 // block (fixed summation order, no host round trip).
 //
-// Update form (opts.basis = 0; the path of ssqcd_shifted_cg): per iteration
+// Update form (opts.basis = 0; ssqcd_shifted_cg of small systems, few shifts
+// or FP32): per iteration
 //   A. stencil q = K p for every source with block partials of (p, q); the
 //      last block forms alpha_k = (r, r) / (p, q) (breakdown check);
 //   B. seed update r -= alpha q with partials of ||r||^2; meanwhile the
@@ -34,7 +35,8 @@
 //   P. seed direction p = r + beta p;
 //   C. fused update, on a side stream beside A, B, P of the next iteration:
 //      for every listed shift y_j += a_j p-hat_j, p-hat_j = r + b_j p-hat_j.
-// Krylov-basis form (default for FP64 and float-float solves): A, B, P as
+// Krylov-basis form (default for FP64 and float-float solves, and for the
+// larger ssqcd_shifted_cg of FP64 lattices): A, B, P as
 // above, B writing r_{k+1} into a stored slot, and S (the shift scalars:
 // xi_{k+1}, a_j, b_j into per-iteration records, the freeze test) on the
 // side stream; the shift vectors are never formed -- see "Krylov-basis form"

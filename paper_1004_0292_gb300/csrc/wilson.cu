@@ -3,7 +3,7 @@
 // sides, in FP64 (FP64 links) or FP32 (FP16 12-parameter links).  The device
 // building blocks and the work split are described in wilson_core.cuh.
 //
-// FP64: on GB300 FP64 runs at 1/64 of the FP32 rate (~1.2 TFLOP/s measured),
+// FP64 (links that the integer stencil of wilson_fix.cuh does not take): on GB300 FP64 runs at 1/64 of the FP32 rate (~1.2 TFLOP/s measured),
 // so this kernel is bound by the FP64 pipe, not by HBM: per site and rhs
 // 8 x (12 projection adds + 72 link FMA/MUL + 24 reconstruction adds) + 18
 // combine adds + 24 FMA ~ 906 FP64 instructions against 192 B (spinor in) +
