@@ -360,7 +360,8 @@ template <int W, typename V2>
 struct StencilFix {
   static constexpr bool kFF = std::is_same<V2, float4>::value;  // float-float vectors
   static constexpr bool kThreadPerSite = false;
-  static constexpr int kThreads = wfix::fix_threads(W);
+  static_assert(W == 1 || W == 4, "one or four warps a site group");
+  static constexpr int kThreads = wfix::kFixThreads;
   static constexpr int kUnits = wfix::fix_units(W);
   static constexpr int kSites = kUnits * wfix::kFixSites;
   // W > 1: the warps' hop sums; W = 1: two operand stages a warp
@@ -405,7 +406,7 @@ struct StencilFix {
                            });
       wfix::copy_wait<0>();  // each lane reads back its own copies
     } else {
-      wfix::hop_sums<W>(v, s, r, sub, h, up, lo);
+      wfix::hop_sums(v, s, r, sub, h, up, lo);
     }
     const bool special = h.E > wfix::kMaxExp;
     const double hf = special ? __longlong_as_double(0x7ff8000000000000ll) : wfix::hop_factor(h.E, -g.kappa);
@@ -460,8 +461,11 @@ struct StencilFix {
             o.y = fma(sg, o.y, sigma * pv.y);
           }
           q[(size_t)comp * V + s] = o;
-          d = fma(pv.x, o.x, d);  // two sums: half the chain, and its rounding
-          d2 = fma(pv.y, o.y, d2);
+          d = fma(pv.x, o.x, d);
+          if (W == 1)  // twelve terms a lane: two sums, half the chain and its rounding
+            d2 = fma(pv.y, o.y, d2);
+          else  // four terms at most
+            d = fma(pv.y, o.y, d);
         }
       }
     };
@@ -2310,11 +2314,10 @@ class CgRun final : public CgRunBase {
     const long long n = n_;
     const int NL = N * L;
     if constexpr (kSeed64 || kSeedDF) {
-      // the integer stencil, when the links allow it and its digits fit; for
-      // float-float vectors where one or four warps run a site group (8^4 x 2:
-      // 25.0 -> 23.5 us an iteration; at eight, 8^4 x 1, the float-float
-      // stencil is the faster one, 22.5 against 23.6, and needs no digits)
-      fix_ = lat->fix_ok && (kSeed64 || fix_split(g.V, L) <= 4) && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
+      // the integer stencil, when the links allow it and its digits fit
+      // (float-float loops: 8^4 x 1 22.1 -> 20.9 us an iteration, 8^4 x 2 25.0 ->
+      // 23.5; a launch on 16^3 x 32 90 -> 62 us)
+      fix_ = lat->fix_ok && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
              pex_.alloc(fix_exp_bytes(g.V) * L) == SSQCD_OK;
       fix_w_ = fix_split(g.V, L);
       if constexpr (kSeedDF) {
@@ -2910,11 +2913,10 @@ class CgRun final : public CgRunBase {
   }
 
   void launch_fix(dim3 grid, int par) {
-    switch (fix_w_) {
-      case 1: launch_fix<1>(grid, par); break;
-      case 4: launch_fix<4>(grid, par); break;
-      default: launch_fix<8>(grid, par); break;
-    }
+    if (fix_w_ == 1)
+      launch_fix<1>(grid, par);
+    else
+      launch_fix<4>(grid, par);
   }
 
   void iteration(int it) {

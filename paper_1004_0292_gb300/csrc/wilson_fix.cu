@@ -125,12 +125,13 @@ __device__ __noinline__ double2 hop_sum_fp64(const Geometry& g, const double2* _
 // fetched from L2 once for them.  Consecutive blocks take the further
 // right-hand sides of the same sites (nrb of them).
 template <int W, typename V2, bool USER>
-__global__ void __launch_bounds__(fix_threads(W), fix_min_blocks(W))
+__global__ void __launch_bounds__(kFixThreads, fix_min_blocks(W))
 wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const V2* __restrict__ in,
                   V2* __restrict__ out, int nrhs, int RB, int nrb) {
   constexpr bool kFF = std::is_same<V2, float4>::value;  // float-float fields
   static_assert(!(kFF && USER), "the caller's fields are FP64");
-  constexpr int kWarps = fix_threads(W) / 32;
+  static_assert(W == 1 || W == 4, "one or four warps a site group");
+  constexpr int kWarps = kFixThreads / 32;
   constexpr int kUnits = kWarps / W;  // (site group, rhs) units a block
   // W > 1: the warps' hop sums; W = 1: two operand stages a warp
   __shared__ longlong2 part[W > 1 ? kWarps * 6 * 32 : kWarps * kWarpStages];
@@ -173,7 +174,7 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
     });
     copy_wait<0>();
   } else {
-    hop_sums<W>(v, s, r, sub, h, up, lo);
+    hop_sums(v, s, r, sub, h, up, lo);
   }
   const double hf = hop_factor(h.E, -g.kappa);
   if (W > 1) {
@@ -254,7 +255,7 @@ void launch_apply(const Geometry& g, const FixView& v, const double2* u64, const
   while (2 * RB <= kUnits && 2 * RB <= nrhs) RB *= 2;
   const int nrb = (nrhs + RB - 1) / RB, gb = (groups + kUnits / RB - 1) / (kUnits / RB);
   const unsigned blocks = (unsigned)gb * nrb;
-  wilson_fix_kernel<W, V2, USER><<<blocks, fix_threads(W), 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
+  wilson_fix_kernel<W, V2, USER><<<blocks, kFixThreads, 0, s>>>(g, v, u64, in, out, nrhs, RB, nrb);
 }
 
 template <typename V2, bool USER>
@@ -272,11 +273,10 @@ int apply_block(ssqcd_lattice lat, const V2* in, V2* out, int nrhs, int4* dig, i
   const double2* u64 = lat->u64.as<double2>();
   SS_TRY((pack_fields<V2, USER>(in, nrhs, g.V, dig, ex, s)));
   const FixView v{lat->ufix.as<int4>(), lat->fnbr, dig, ex, fix_tiles(g.V)};
-  switch (fix_split(g.V, nrhs)) {
-    case 1: launch_apply<1, V2, USER>(g, v, u64, in, out, nrhs, s); break;
-    case 4: launch_apply<4, V2, USER>(g, v, u64, in, out, nrhs, s); break;
-    default: launch_apply<8, V2, USER>(g, v, u64, in, out, nrhs, s); break;
-  }
+  if (fix_split(g.V, nrhs) == 1)
+    launch_apply<1, V2, USER>(g, v, u64, in, out, nrhs, s);
+  else
+    launch_apply<4, V2, USER>(g, v, u64, in, out, nrhs, s);
   count_launches(1);
   SS_CHECK_LAUNCH();
   return SSQCD_OK;
@@ -322,13 +322,11 @@ int pack_fix(const float4* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t
 }
 
 // Warps that share the eight hops of 16 sites: 1 once the groups fill the
-// GPU's schedulers (8^4 x 4: 7.5 us against 9.4 with 4 and 11 with 8; 16^3 x 32:
-// 48 us against 57 and 70), 4 at half that, 8 below (8^4 x 1: 4.8 us against
-// 5.0 with 4 and 7.4 with 1).
-int fix_split(int V, int nrhs) {
-  const long long groups = (long long)fix_tiles(V) * nrhs;
-  return groups >= 608 ? 1 : groups >= 304 ? 4 : 8;
-}
+// GPU's schedulers (8^4 x 4, 1024 groups: 27.9 us an iteration against 29.6 with
+// 4; 16^3 x 32: 48 us an application against 57), 4 below (8^4 x 1, 256 groups:
+// 20.0 us an iteration; with eight warps, one hop each, it was 21.4, and 20.9
+// against 19.8 for the 64 groups of 4^4 x 4).
+int fix_split(int V, int nrhs) { return (long long)fix_tiles(V) * nrhs >= 608 ? 1 : 4; }
 
 int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s, void* work) {
   const Geometry& g = lat->g;

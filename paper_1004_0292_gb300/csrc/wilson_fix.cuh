@@ -411,50 +411,38 @@ __device__ __forceinline__ void hop_sums_piped(const FixView& v, int s, int i, i
   pipe_hops<0>(v, s, i, r, h, buf, up, lo, last);
 }
 
-// Hop sums of one warp's share (sub of W) of the eight hops for spin row r of
-// site s: up = upper output spin r, lo = lower output spin r, both in units
-// 2^(E - 57).  W = 8: hop sub; W = 4: direction sub; the direction is a
-// run-time value, since warps that each run their own copy of the code stall
-// on instruction fetches.  (W = 1: hop_sums_piped.)  All lanes of the warp
-// take part.
-template <int W>
+// Hop sums of one of four warps (sub: its direction, both hops) for spin row r
+// of site s: up = upper output spin r, lo = lower output spin r, both in units
+// 2^(E - 57).  The direction is a run-time value, since warps that each run
+// their own copy of the code stall on instruction fetches.  All lanes of the
+// warp take part.
 __device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub, Hops& h, Acc3& up, Acc3& lo) {
-  static_assert(W == 4 || W == 8, "W = 1: hop_sums_piped");
   clear(up);
   clear(lo);
-  const int mu = W == 4 ? sub : sub >> 1;
-  const bool back = W == 8 && (sub & 1) != 0;
+  const int mu = sub;
   const int nf = mu == 0 ? h.nb[0] : mu == 1 ? h.nb[2] : mu == 2 ? h.nb[4] : h.nb[6];
   const int nb = mu == 0 ? h.nb[1] : mu == 1 ? h.nb[3] : mu == 2 ? h.nb[5] : h.nb[7];
   HopData d;
-  if (back)
-    hop_fetch_at<true>(v, s, nb, mu, r, d);
-  else
-    hop_fetch_at<false>(v, s, nf, mu, r, d);
+  hop_fetch_at<false>(v, s, nf, mu, r, d);
   load_exponents(v, s, h);
   const unsigned s2 = (mu < 2 ? h.sh[0] : h.sh[1]) >> (16 * (mu & 1));
   const int sf = s2 & 0xff, sb = (s2 >> 8) & 0xff;
   Acc3 w;
-  if (!back) {
-    hop_math<-1, false>(d, mu, r, (nf & kNegBit) != 0, sf, w);
-    add_hop<false>(w, mu, r, up, lo);
-  }
-  if (W == 4) hop_fetch_at<true>(v, s, nb, mu, r, d);
-  if (W == 4 || back) {
-    hop_math<-1, true>(d, mu, r, (nb & kNegBit) != 0, sb, w);
-    add_hop<true>(w, mu, r, up, lo);
-  }
+  hop_math<-1, false>(d, mu, r, (nf & kNegBit) != 0, sf, w);
+  add_hop<false>(w, mu, r, up, lo);
+  hop_fetch_at<true>(v, s, nb, mu, r, d);
+  hop_math<-1, true>(d, mu, r, (nb & kNegBit) != 0, sb, w);
+  add_hop<true>(w, mu, r, up, lo);
   if (mu < 2) cross_over(lo);
 }
 
-// Launch shapes: warps a block, (site group, rhs) units a block, and the
-// blocks an SM that the registers are capped for (the fastest of those tried:
-// W = 1 at 3, 4, 5 blocks 368, 326, 386 us for 16^3 x 32 x 8; W = 4 at 7, 6, 5
-// 24.9, 24.1, 23.7 us an iteration of 8^4 x 2; W = 8 at 3, 4 the same for the
-// small lattices it serves).
-__host__ __device__ constexpr int fix_threads(int W) { return W == 8 ? 256 : 128; }
-__host__ __device__ constexpr int fix_units(int W) { return fix_threads(W) / 32 / W; }
-__host__ __device__ constexpr int fix_min_blocks(int W) { return W == 1 ? 4 : W == 4 ? 5 : 3; }
+// Launch shapes for W = 1 or 4 warps a site group: threads a block, (site group,
+// rhs) units a block, and the blocks an SM that the registers are capped for
+// (the fastest of those tried: W = 1 at 3, 4, 5 blocks 368, 326, 386 us for 16^3 x
+// 32 x 8; W = 4 at 7, 6, 5 24.9, 24.1, 23.7 us an iteration of 8^4 x 2).
+constexpr int kFixThreads = 128;
+__host__ __device__ constexpr int fix_units(int W) { return kFixThreads / 32 / W; }
+__host__ __device__ constexpr int fix_min_blocks(int W) { return W == 1 ? 4 : 5; }
 
 // psi - kappa D psi from a hop sum T in units 2^(E - 57): the sum is made a
 // double times 2^-200 (exact up to its rounding: |T| < 2^63) and the factor
