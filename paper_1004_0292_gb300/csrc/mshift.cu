@@ -91,8 +91,15 @@ struct Control {
   double* alpha;       // [L]     alpha_k
   double* inv_rr;      // [L]     1 / (r_k, r_k), kernel A
   double* vnorm2;      // [L]
-  int* live;           // [L]     shifts still iterating
-  int* live_total;     // [1]
+  // Shifts still iterating, [L] and their total, in kLiveEntries entries.  The
+  // Krylov-basis loop's kernel S of iteration k, on the side stream beside A and
+  // B of k + 1, goes from entry k - 1 to entry k; A, B and P of iteration k read entry
+  // k - 2, which A(k) has waited for: no kernel in flight writes it, so that
+  // all threads of an iteration see the same counts (A and B branch on them
+  // around block barriers).  The update form keeps to the last entry.
+  int* live;           // the entry that A, B and P read (in the update form B writes it)
+  int* live_prev;      // the entry that S reads
+  int* live_next;      // the entry that S writes
   int* ran;            // [1]     kernel A of this iteration did its work (read by B and P)
   int* rec_ran;        // [2]     the same per iteration parity (read by C, which may run
                        //         while the next iteration's A rewrites ran)
@@ -134,6 +141,11 @@ struct Control {
 
 constexpr int kUpdBlock = 256;
 constexpr int kSeedBlock = 256;
+constexpr int kLiveEntries = 4;  // a power of two, so that a chunk of iterations begins where the last one did
+// the entry of iteration k (k >= -kLiveEntries) in the counts that begin at live0
+__host__ __device__ __forceinline__ int* live_entry(int* live0, int k, int L) {
+  return live0 + (size_t)((k + kLiveEntries) & (kLiveEntries - 1)) * (L + 1);
+}
 
 // ---- Krylov-basis form ------------------------------------------------------------------
 // Instead of updating y_j and p-hat_j for every live shift in every iteration
@@ -234,13 +246,13 @@ __global__ void init_vectors_kernel(const double2* __restrict__ v, VR* __restric
 }
 
 // A source with ||v|| = 0 has the exact solution y = 0 and starts frozen.
-__global__ void init_control_kernel(Control c, const double* __restrict__ vn2, int L, int N) {
+__global__ void init_control_kernel(Control c, int* __restrict__ live0, const double* __restrict__ vn2, int L, int N) {
   for (int t = threadIdx.x; t < L; t += blockDim.x) {
     // rr_0, alpha_{-1} = 1, beta_{-1} = 0, scale 1, S = 1
     c.seed[t] = SeedState{vn2[t], 1.0, 0.0, 0.0, 1.0, {0.0, 1.0, 0.0}};
     c.alpha[t] = 0.0;
     c.vnorm2[t] = vn2[t];
-    c.live[t] = vn2[t] > 0.0 ? N : 0;
+    for (int e = 0; e < kLiveEntries; ++e) live_entry(live0, e, L)[t] = vn2[t] > 0.0 ? N : 0;
     c.list_n[t] = c.list_n[L + t] = 0;
     if (c.sprev != nullptr) {
       c.sprev[2 * t] = 1.0;  // alpha_{-1}
@@ -256,7 +268,7 @@ __global__ void init_control_kernel(Control c, const double* __restrict__ vn2, i
   if (threadIdx.x == 0) {
     int live = 0;
     for (int l = 0; l < L; ++l) live += vn2[l] > 0.0 ? N : 0;
-    *c.live_total = live;
+    for (int e = 0; e < kLiveEntries; ++e) live_entry(live0, e, L)[L] = live;
     *c.ran = 0;
     c.rec_ran[0] = c.rec_ran[1] = 0;
     *c.err = 0;
@@ -596,7 +608,7 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   typename Op::Pre ahead;
   op.pre(g, ahead);  // what no kernel of the loop writes
   pdl_wait();
-  const int err = *c.err, live_total = *c.live_total, live_l = c.live[blockIdx.y];
+  const int err = *c.err, live_total = c.live[L], live_l = c.live[blockIdx.y];
   if (err != 0 || live_total == 0) {
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *c.ran = c.rec_ran[par] = 0;
     return;
@@ -623,6 +635,7 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   // what the last block's tail needs of a source, loaded ahead of it
   const int lt = min((int)threadIdx.x, L - 1);
   const double rr_t = c.seed[lt].rr;
+  const int live_t = c.live[lt];
   d_pq = warp_sum(d_pq);
   if (lane == 0) sred[w] = d_pq;
   __syncthreads();
@@ -638,10 +651,6 @@ cg_stencil_kernel(Control c, int L, int par, Geometry g, Op op, double sigma, co
   }
   __syncthreads();
   if (!s_last) return;
-  // Kernel S of the iteration before may clear a count meanwhile: a block that
-  // reads zero adds nothing to its source's sum, so that the count read after
-  // every block's has to say whether the sum is used.
-  const int live_t = __ldcg(c.live + lt);
   tail_sums<kWarps>(c.partial, nbw, L, sums, spart);
   static_assert(kMaxSources <= Op::kThreads, "a thread a source");
   if ((int)threadIdx.x < L && live_t != 0) {
@@ -812,6 +821,7 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
   // what the last block's tail needs of a source, loaded ahead of it
   const int lt = min((int)threadIdx.x, L - 1);
   const double vn2_t = c.vnorm2[lt], irr_t = c.inv_rr[lt], alpha_t = c.alpha[lt], S_t = c.seed[lt].pad[1];
+  const int live_t = c.live[lt];
   char *slot1 = nullptr, *slot2 = nullptr;  // slots of the next iteration
   if (c.tab != nullptr) {
     slot1 = reinterpret_cast<char*>(basis_slot<V2>(c, kb + 1, (long long)L * n));
@@ -829,7 +839,6 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
   }
   __syncthreads();
   if (!s_last) return;
-  const int live_t = __ldcg(c.live + lt);  // after every block's, as in A
   tail_sums<kSeedBlock / 32>(c.partial_rr, nb, L, sums, sred);
   if ((int)threadIdx.x < L) {  // kMaxSources <= kSeedBlock
     const double a = sums[lt];
@@ -927,7 +936,7 @@ cg_seed_kernel(Control c, int L, int N, int par, double tol2, const V2* __restri
   if (threadIdx.x == 0) {
     int tot = 0;
     for (int ls = 0; ls < L; ++ls) tot += c.live[ls];
-    *c.live_total = tot;
+    c.live[L] = tot;
     c.done[1] = 0u;
     c.task_ctr[par] = 0u;
   }
@@ -1037,12 +1046,16 @@ cg_seed_p_fix_kernel(Control c, const V2* __restrict__ r, V2* __restrict__ p, in
 // b_j = s beta_k xi_{k+1} / xi_k into the coefficient records, the freeze
 // test |xi_{k+1}|^2 rr_{k+1} <= tol^2 ||v||^2, and the live counts.  It runs
 // beside P(k), A(k+1), B(k+1) of the main stream: they read the live counts
-// only to skip finished work, and a count one iteration old only makes them
-// do some of it once more (counts only fall).  A(k+2) waits for S(k), whose
-// records (alpha_rec, srec of this parity) it and B(k+2) rewrite.  One block.
+// of S(k-2) and S(k-1) (Control::live) only to skip finished work, and a count
+// one iteration old makes them do one iteration of it once more (counts only
+// fall).  A(k+2) waits for S(k), whose records (alpha_rec, srec of this parity)
+// it and B(k+2) rewrite.  One block.
 __global__ void __launch_bounds__(kSeedBlock)
 cg_shift_kernel(Control c, int L, int N, int par, double tol2, double rescale_by) {
-  if (c.rec_ran[par] == 0) return;
+  if (c.rec_ran[par] == 0) {  // the counts stay as they are
+    for (int t = threadIdx.x; t <= L; t += blockDim.x) c.live_next[t] = c.live_prev[t];
+    return;
+  }
   __shared__ int s_live[kMaxSources];
   const int NL = N * L;
   const int kb = c.srec_k[par];
@@ -1050,7 +1063,7 @@ cg_shift_kernel(Control c, int L, int N, int par, double tol2, double rescale_by
   __syncthreads();
   for (int qi = threadIdx.x; qi < NL; qi += blockDim.x) {
     const int ls = qi / N;
-    const int lv = c.live[ls], ac = c.act[qi];
+    const int lv = c.live_prev[ls], ac = c.act[qi];
     const double* rec = c.srec + ((size_t)par * L + ls) * 4;
     const double rr1 = rec[0], beta = rec[1], sc = rec[2], spad1 = rec[3];
     const double alpha = c.alpha_rec[par * L + ls], ap = c.sprev[2 * ls], bp = c.sprev[2 * ls + 1];
@@ -1090,17 +1103,17 @@ cg_shift_kernel(Control c, int L, int N, int par, double tol2, double rescale_by
   for (int ls = threadIdx.x; ls < L; ls += blockDim.x) {
     const double* rec = c.srec + ((size_t)par * L + ls) * 4;
     basis_scale(c, kb, NL, L)[ls] = rec[2];
-    if (c.live[ls] != 0) {
+    if (c.live_prev[ls] != 0) {
       c.sprev[2 * ls] = c.alpha_rec[par * L + ls];
       c.sprev[2 * ls + 1] = rec[1];
     }
-    c.live[ls] = s_live[ls];
+    c.live_next[ls] = s_live[ls];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     int tot = 0;
     for (int ls = 0; ls < L; ++ls) tot += s_live[ls];
-    *c.live_total = tot;
+    c.live_next[L] = tot;
   }
 }
 
@@ -2254,7 +2267,8 @@ class CgRun final : public CgRunBase {
   static constexpr bool kShiftDF = std::is_same<V2, float4>::value;  // shift vectors in float-float
   static constexpr bool kSeedDF = std::is_same<VR, float4>::value;   // seed vectors and stencil in float-float
   static constexpr bool kSeed64 = std::is_same<VR, double2>::value;  // seed vectors and stencil in FP64
-  static constexpr int kChunk = 16;  // even: every chunk starts at parity 0
+  static constexpr int kChunk = 16;  // every chunk starts at parity 0 and at the same entry of the live counts
+  static_assert(kChunk % 2 == 0 && kChunk % kLiveEntries == 0, "per-iteration records of a chunk");
   static constexpr int kSlots = 8;   // timing events per iteration: A, B, C, P start/stop
   static constexpr int kTimedEvery = 4;
   static constexpr int kInFlight = 2;  // chunks enqueued ahead of the poll
@@ -2367,7 +2381,7 @@ class CgRun final : public CgRunBase {
       return o;
     };
     const size_t o_seed = take(sizeof(SeedState) * L), o_alpha = take(sizeof(double) * L), o_irr = take(sizeof(double) * L),
-                 o_vn = take(sizeof(double) * L), o_live = take(sizeof(int) * L), o_tot = take(sizeof(int)),
+                 o_vn = take(sizeof(double) * L), o_live = take(sizeof(int) * kLiveEntries * (L + 1)),
                  o_ran = take(sizeof(int)), o_rran = take(sizeof(int) * 2), o_err = take(sizeof(int)),
                  o_si = take(sizeof(int) * 2), o_done = take(sizeof(unsigned) * 4),
                  o_s = take(sizeof(double2) * NL), o_xc = take(sizeof(double2) * NL),
@@ -2387,8 +2401,8 @@ class CgRun final : public CgRunBase {
     c.alpha = reinterpret_cast<double*>(base + o_alpha);
     c.inv_rr = reinterpret_cast<double*>(base + o_irr);
     c.vnorm2 = reinterpret_cast<double*>(base + o_vn);
-    c.live = reinterpret_cast<int*>(base + o_live);
-    c.live_total = reinterpret_cast<int*>(base + o_tot);
+    live0_ = reinterpret_cast<int*>(base + o_live);
+    c.live = c.live_prev = c.live_next = live_entry(live0_, -1, L);
     c.ran = reinterpret_cast<int*>(base + o_ran);
     c.rec_ran = reinterpret_cast<int*>(base + o_rran);
     c.err = reinterpret_cast<int*>(base + o_err);
@@ -2439,7 +2453,7 @@ class CgRun final : public CgRunBase {
     else
       init_vectors_kernel<<<dim3(nbu_, L), kUpdBlock, 0, st_>>>(v, r_.as<VR>(), p_.as<VR>(), yv_, ph_.as<V2>(), N, n);
     SS_CHECK_LAUNCH();
-    init_control_kernel<<<1, 256, 0, st_>>>(c, vn2, L, N);
+    init_control_kernel<<<1, 256, 0, st_>>>(c, live0_, vn2, L, N);
     SS_CHECK_LAUNCH();
     count_launches(2);
     if constexpr (kSeed64 || kSeedDF) {
@@ -2525,7 +2539,8 @@ class CgRun final : public CgRunBase {
       count_launches(1);
     }
     // live-shift count after the last iteration and the error flag
-    SS_CUDA(cudaMemcpyAsync(h_poll_ + 2 * slot, c_.live_total, sizeof(int), cudaMemcpyDeviceToHost, st_));
+    const int* live = basis_ ? live_entry(live0_, chunk - 1, L_) : c_.live;
+    SS_CUDA(cudaMemcpyAsync(h_poll_ + 2 * slot, live + L_, sizeof(int), cudaMemcpyDeviceToHost, st_));
     SS_CUDA(cudaMemcpyAsync(h_poll_ + 2 * slot + 1, c_.err, sizeof(int), cudaMemcpyDeviceToHost, st_));
     if (timing_)
       SS_CUDA(cudaMemcpyAsync(h_iters_ + (size_t)slot * N_ * L_, c_.iters, sizeof(int) * N_ * L_,
@@ -2578,7 +2593,7 @@ class CgRun final : public CgRunBase {
     const int live = h_poll_[2 * slot], err = h_poll_[2 * slot + 1];
     if (err == 2) return fail(SSQCD_ERR_NOCONV, "shift update: a device-side wait hit its limit");
     // every shift frozen: done, even if an iteration that ran after the last
-    // freeze (the Krylov-basis loop reads the live count one iteration late)
+    // freeze (the Krylov-basis loop reads the live counts one iteration late)
     // met a breakdown of the then useless seed recurrence
     if (live == 0) {
       *state = kPollDone;
@@ -2834,7 +2849,8 @@ class CgRun final : public CgRunBase {
     SS_CUDA(cudaStreamSynchronize(st_));
     int k = 0, live = 0, err = 0;
     SS_CUDA(cudaMemcpy(&k, c_.seed_iters, sizeof(int), cudaMemcpyDeviceToHost));
-    SS_CUDA(cudaMemcpy(&live, c_.live_total, sizeof(int), cudaMemcpyDeviceToHost));
+    // after whole chunks the newest counts are the last entry's
+    SS_CUDA(cudaMemcpy(&live, c_.live + L_, sizeof(int), cudaMemcpyDeviceToHost));
     SS_CUDA(cudaMemcpy(&err, c_.err, sizeof(int), cudaMemcpyDeviceToHost));
     *over = live == 0 || err != 0;  // what is launched now does nothing
     if (*over) return SSQCD_OK;
@@ -2901,10 +2917,10 @@ class CgRun final : public CgRunBase {
   }
 
   template <int W>
-  void launch_fix(dim3 grid, int par) {
+  void launch_fix(const Control& c, dim3 grid, int par) {
     if constexpr (kSeed64 || kSeedDF) {
       using Op = StencilFix<W, VR>;
-      launch_chain(cg_stencil_kernel<Op, VR>, grid, Op::kThreads, st_, prio_a_, basis_ && use_pdl(), c_, L_, par,
+      launch_chain(cg_stencil_kernel<Op, VR>, grid, Op::kThreads, st_, prio_a_, basis_ && use_pdl(), c, L_, par,
                    lat_->g,
                    Op{wfix::FixView{lat_->ufix.as<int4>(), lat_->fnbr, pdig_.as<int4>(), pex_.as<int>(),
                                     wfix::fix_tiles(lat_->g.V)}},
@@ -2912,18 +2928,23 @@ class CgRun final : public CgRunBase {
     }
   }
 
-  void launch_fix(dim3 grid, int par) {
+  void launch_fix(const Control& c, dim3 grid, int par) {
     if (fix_w_ == 1)
-      launch_fix<1>(grid, par);
+      launch_fix<1>(c, grid, par);
     else
-      launch_fix<4>(grid, par);
+      launch_fix<4>(c, grid, par);
   }
 
   void iteration(int it) {
     const Geometry& g = lat_->g;
     const long long n = n_;
     const int L = L_, N = N_;
-    Control& c = c_;
+    Control c = c_;
+    if (basis_) {
+      c.live = live_entry(live0_, it - 2, L);
+      c.live_prev = live_entry(live0_, it - 1, L);
+      c.live_next = live_entry(live0_, it, L);
+    }
     const dim3 grid_a(nbw_, L), grid_b(nbs_, L), grid_c(nbu_, L);
     const dim3 grid_p(p_blocks(n, L), L);
     VR* const r0 = r_.as<VR>();  // null in the Krylov-basis form (kernels B, P address the slots)
@@ -2944,7 +2965,7 @@ class CgRun final : public CgRunBase {
                     Stencil32<LinksF32>{LinksF32{lat_->u32.as<float4>(), g.V}}, sigma_, p_.as<VR>(), q_.as<VR>());
     } else if constexpr (kSeedDF) {
       if (fix_)
-        launch_fix(grid_a, par);
+        launch_fix(c, grid_a, par);
       else if (stencil_minb() == 3)
         launch_chain(cg_stencil_kernel<StencilDF<3>, VR>, grid_a, kStencilThreadsDF, st, prio_a_,
                      basis_ && use_pdl(), c, L, par, g, StencilDF<3>{lat_->udf.as<float4>()}, sigma_, p_.as<VR>(),
@@ -2954,7 +2975,7 @@ class CgRun final : public CgRunBase {
                      basis_ && use_pdl(), c, L, par, g, StencilDF<4>{lat_->udf.as<float4>()}, sigma_, p_.as<VR>(),
                      q_.as<VR>());
     } else if (fix_) {
-      launch_fix(grid_a, par);
+      launch_fix(c, grid_a, par);
     } else if (balanced_stencil()) {
       if (stencil_minb() == 8)
         launch_chain(cg_stencil_kernel<Stencil64h<8>, VR>, grid_a, kStencilThreads, st, prio_a_,
@@ -3057,6 +3078,7 @@ class CgRun final : public CgRunBase {
   DevBuf pdig_, pex_;  // p's digits and exponents
   DevBuf r_, p_, q_, ph_, y32_, x_, kx_, y_out_, ctl_;
   V2* yv_ = nullptr;
+  int* live0_ = nullptr;  // the live counts' entries
   Control c_{};
   std::vector<double2> shift_host_;
   std::vector<cudaEvent_t> ev_, tev_, ev_poll_;
