@@ -1451,6 +1451,16 @@ namespace {
 
 constexpr int kServerChunksAhead = 2;
 
+// Chunks of iterations up to kServerChunksAhead in flight, or as many as there
+// are before max_iter (launch then adds none: poll ends the run).
+int launch_ahead(CgRunBase& run) {
+  for (int before = -1; run.in_flight() < kServerChunksAhead && run.in_flight() > before;) {
+    before = run.in_flight();
+    SS_TRY(run.launch());
+  }
+  return SSQCD_OK;
+}
+
 // Device memory of one request at its peak: shift vectors (or the stored
 // residuals up to their cap), seed vectors and sources during the CG;
 // moments and the Rayleigh-Ritz basis afterwards.
@@ -1774,10 +1784,7 @@ extern "C" int ssqcd_server_progress(ssqcd_server srv, int wait, int* completed)
         ++done;
         break;
       }
-      while (r.run->in_flight() < kServerChunksAhead) {
-        s1 = r.run->launch();
-        if (s1 != SSQCD_OK) break;
-      }
+      s1 = launch_ahead(*r.run);
       if (s1 != SSQCD_OK) {
         request_fail(srv, r, s1);
         ++done;
@@ -1802,12 +1809,10 @@ extern "C" int ssqcd_server_progress(ssqcd_server srv, int wait, int* completed)
         ++done;
       }
     } else {
-      while (r.run->in_flight() < kServerChunksAhead)
-        if ((s1 = r.run->launch()) != SSQCD_OK) {
-          request_fail(srv, r, s1);
-          ++done;
-          break;
-        }
+      if ((s1 = launch_ahead(*r.run)) != SSQCD_OK) {
+        request_fail(srv, r, s1);
+        ++done;
+      }
     }
   }
   if (completed) *completed = done;
