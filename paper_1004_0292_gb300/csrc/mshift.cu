@@ -2334,6 +2334,9 @@ class CgRun final : public CgRunBase {
       fix_ = lat->fix_ok && pdig_.alloc(fix_field_bytes(g.V) * L) == SSQCD_OK &&
              pex_.alloc(fix_exp_bytes(g.V) * L) == SSQCD_OK;
       fix_w_ = fix_split(g.V, L);
+      if (fix_)
+        fix_view_ = wfix::FixView{lat->ufix.as<int4>(), lat->fnbr, pdig_.as<int4>(), pex_.as<int>(),
+                                  wfix::fix_tiles(g.V)};
       if constexpr (kSeedDF) {
         AllocStream plain(st_, false);  // lattice-owned
         if (!fix_) SS_TRY(ensure_df_links(lat));
@@ -2921,10 +2924,7 @@ class CgRun final : public CgRunBase {
     if constexpr (kSeed64 || kSeedDF) {
       using Op = StencilFix<W, VR>;
       launch_chain(cg_stencil_kernel<Op, VR>, grid, Op::kThreads, st_, prio_a_, basis_ && use_pdl(), c, L_, par,
-                   lat_->g,
-                   Op{wfix::FixView{lat_->ufix.as<int4>(), lat_->fnbr, pdig_.as<int4>(), pex_.as<int>(),
-                                    wfix::fix_tiles(lat_->g.V)}},
-                   sigma_, p_.as<VR>(), q_.as<VR>());
+                   lat_->g, Op{fix_view_}, sigma_, p_.as<VR>(), q_.as<VR>());
     }
   }
 
@@ -3076,6 +3076,7 @@ class CgRun final : public CgRunBase {
   bool fix_ = false;  // the integer stencil
   int fix_w_ = 0;
   DevBuf pdig_, pex_;  // p's digits and exponents
+  wfix::FixView fix_view_{};  // links and p as init found them: an upload meanwhile may leave the lattice without
   DevBuf r_, p_, q_, ph_, y32_, x_, kx_, y_out_, ctl_;
   V2* yv_ = nullptr;
   int* live0_ = nullptr;  // the live counts' entries

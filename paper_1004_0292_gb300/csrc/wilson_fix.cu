@@ -405,7 +405,6 @@ void give_workspace(ssqcd_lattice lat, std::unique_ptr<DevBuf> ws) {
 int build_fix_links(ssqcd_lattice lat) {
   const int V = lat->g.V;
   lat->fix_ok = false;
-  lat->fnbr = nullptr;
   // links, neighbour table and the check's flag in one allocation
   const size_t lb = 3 * fix_field_bytes(V), nb = 8 * fix_exp_bytes(V);
   if (lat->ufix.alloc(lb + nb + sizeof(int)) != SSQCD_OK) return SSQCD_OK;  // no room: the FP64 kernel serves
@@ -421,9 +420,11 @@ int build_fix_links(ssqcd_lattice lat) {
   SS_CUDA(cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, lat->stream));
   SS_CUDA(cudaStreamSynchronize(lat->stream));
   lat->fix_ok = h == 0;
+  // Once links have suited, the memory stays the lattice's: a run in flight
+  // (ssqcd_server) may hold it, whatever is uploaded meanwhile.
   if (lat->fix_ok)
     lat->fnbr = nbr;
-  else
+  else if (lat->fnbr == nullptr)
     lat->ufix.release();
   return SSQCD_OK;
 }
