@@ -240,7 +240,13 @@ int ssqcd_upload_gauge(ssqcd_lattice lat, const double* links, int on_device);
 
 /* out = A in for nrhs spinor fields ([nrhs][V][4][3] complex128; in and out
  * both host, or both device, per on_device; they must not overlap).  A is
- * the Hermitian fermion matrix of Section 4, applied in FP64. */
+ * the Hermitian fermion matrix of Section 4.  Links whose rows and columns
+ * have unit length to 2^-10 (SU(3) fields) are applied in 60-bit fixed point
+ * relative to a site's largest component, and in FP64 to a component whose
+ * hop terms are all far below that: every component lies within 2^-46 of the
+ * sum of its terms' sizes (typically 2^-52 and less; FP64's own bound is
+ * ~2^-48), the field within 2^-52 of its norm.  Other links are applied in
+ * FP64. */
 int ssqcd_apply_H(ssqcd_lattice lat, const double* in, double* out, int nrhs, int on_device);
 
 /* Same as ssqcd_apply_H with the mixed path's operator: links stored FP16

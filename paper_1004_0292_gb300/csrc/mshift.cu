@@ -407,8 +407,9 @@ struct StencilFix {
         if (k < 6) own[j] = p[(size_t)((k < 3 ? 0 : 6) + r * 3 + k % 3) * V + s];
     }
     wfix::Acc3 up, lo;
+    wfix::Witness<false> none;
     if constexpr (W == 1) {
-      wfix::hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * wfix::kWarpStages), up, lo,
+      wfix::hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * wfix::kWarpStages), up, lo, none,
                            [&](int4* to) {  // the diagonal term's p, a row of lanes a component
 #pragma unroll
                              for (int k = 0; k < 6; ++k)
@@ -418,7 +419,7 @@ struct StencilFix {
                            });
       wfix::copy_wait<0>();  // each lane reads back its own copies
     } else {
-      wfix::hop_sums(v, s, r, sub, h, up, lo);
+      wfix::hop_sums(v, s, r, sub, h, up, lo, none);
     }
     const bool special = h.E > wfix::kMaxExp;
     const double hf = special ? __longlong_as_double(0x7ff8000000000000ll) : wfix::hop_factor(h.E, -g.kappa);
@@ -1028,11 +1029,11 @@ cg_seed_p_fix_kernel(Control c, const V2* __restrict__ r, V2* __restrict__ p, in
 #pragma unroll
     for (int a = 0; a < 3; ++a) p[o + (size_t)a * V] = v[a];
   }
-  const int e = wfix::quad_site_exp(v);
+  const int word = wfix::quad_site_word(v, q), e = wfix::word_exp(word);
   if (s < V) {
     const bool none = e == wfix::kZeroExp || e == wfix::kSpecialExp;
     const int tiles = wfix::fix_tiles(V);
-    if (q == 0) ex[(size_t)l * tiles * wfix::kTile + s] = e;
+    if (q == 0) ex[(size_t)l * tiles * wfix::kTile + s] = word;
     int4* d = dig + wfix::field_at(tiles, l, s) + 3 * q * wfix::kTile;
 #pragma unroll
     for (int a = 0; a < 3; ++a) d[a * wfix::kTile] = none ? make_int4(0, 0, 0, 0) : wfix::to_site_digits(v[a], e);

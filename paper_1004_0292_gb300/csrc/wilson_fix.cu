@@ -62,19 +62,24 @@ pack_fix_kernel(const V2* __restrict__ in, int4* __restrict__ dig, int* __restri
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     v[a] = s >= V ? V2{} : USER ? __ldg(in + (f * V + s) * 12 + 3 * q + a) : __ldg(in + (f * 12 + 3 * q + a) * V + s);
-  const int e = quad_site_exp(v);
+  const int word = quad_site_word(v, q), e = word_exp(word);
   if (s >= V) return;
   const int tiles = fix_tiles(V);
-  if (q == 0) ex[f * tiles * kTile + s] = e;
+  if (q == 0) ex[f * tiles * kTile + s] = word;
   const bool none = e == kZeroExp || e == kSpecialExp;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     dig[field_at(tiles, f, s) + (3 * q + a) * kTile] = none ? make_int4(0, 0, 0, 0) : to_site_digits(v[a], e);
 }
 
+__device__ __forceinline__ bool is_zero(double2 v) {  // by integers
+  return ((unsigned)(__double2hiint(v.x) | __double2hiint(v.y)) << 1 | (unsigned)(__double2loint(v.x) | __double2loint(v.y))) == 0;
+}
+
 // (D psi)(s), component comp, in FP64 from the links and the field as they
-// are: the sites next to a value the digits cannot hold (above 2^800, not
-// finite).  The sums are those of the FP64 kernel up to their order.
+// are: next to a value the digits cannot hold (above 2^800, not finite), and
+// where the digits' roundings may not be small (Witness).  The sums are those of the
+// FP64 kernel up to their order.
 template <bool USER>
 __device__ __noinline__ double2 hop_sum_fp64(const Geometry& g, const double2* __restrict__ u,
                                              const double2* __restrict__ in, size_t f, int s, int comp) {
@@ -94,12 +99,19 @@ __device__ __noinline__ double2 hop_sum_fp64(const Geometry& g, const double2* _
     const bool swap = (mu & 1) == 0;
     const int sb = (mu == 1 && r == 0) || (mu == 2 && r == 1) ? -1 : 1;
     const int sp = back ? sb : -sb;
-    double2 t = make_double2(0.0, 0.0);
+    double2 x[3], l[3];
+#pragma unroll
     for (int b = 0; b < 3; ++b) {
       const int cu = r * 3 + b, cl = 6 + lr * 3 + b;
-      const double2 x = USER ? in[(f * V + nb) * 12 + cu] : in[(f * 12 + cu) * V + nb];
-      const double2 l = USER ? in[(f * V + nb) * 12 + cl] : in[(f * 12 + cl) * V + nb];
-      double2 h = swap ? make_double2(x.x - sp * l.y, x.y + sp * l.x) : make_double2(x.x + sp * l.x, x.y + sp * l.y);
+      x[b] = USER ? in[(f * V + nb) * 12 + cu] : in[(f * 12 + cu) * V + nb];
+      l[b] = USER ? in[(f * V + nb) * 12 + cl] : in[(f * 12 + cl) * V + nb];
+    }
+    double2 t = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      if (is_zero(x[b]) && is_zero(l[b])) continue;
+      double2 h = swap ? make_double2(x[b].x - sp * l[b].y, x[b].y + sp * l[b].x)
+                       : make_double2(x[b].x + sp * l[b].x, x[b].y + sp * l[b].y);
       if (neg) h = make_double2(-h.x, -h.y);
       const double2 w = u[(size_t)(mu * 9 + (back ? 3 * b + a : 3 * a + b)) * V + (back ? nb : s)];
       if (back)
@@ -136,6 +148,7 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
   // W > 1: the warps' hop sums; W = 1: two operand stages a warp
   __shared__ longlong2 part[W > 1 ? kWarps * 6 * 32 : kWarps * kWarpStages];
   __shared__ V2 stage[USER && W > 1 ? kUnits * kFixSites * 13 : 1];
+  __shared__ unsigned evidence[W > 1 && !kFF ? kWarps * 6 * 32 : 1];  // the warps' Witness
   const int V = g.V;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int unit = w / W, sub = w % W;
@@ -164,8 +177,9 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
   Hops h;
   load_neighbours(v, s, h);
   Acc3 up, lo;
+  Witness<!kFF> wit;
   if constexpr (W == 1) {
-    hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * kWarpStages), up, lo, [&](int4* to) {
+    hop_sums_piped(v, s, i, r, h, reinterpret_cast<int4*>(part + w * kWarpStages), up, lo, wit, [&](int4* to) {
       if (USER) {
         const int4* src = reinterpret_cast<const int4*>(inf + (size_t)s0 * 12);
         for (int t = lane; t < own; t += 32) copy16(to + stage_at(t), src + t);
@@ -174,7 +188,7 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
     });
     copy_wait<0>();
   } else {
-    hop_sums(v, s, r, sub, h, up, lo);
+    hop_sums(v, s, r, sub, h, up, lo, wit);
   }
   const double hf = hop_factor(h.E, -g.kappa);
   if (W > 1) {
@@ -182,10 +196,32 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
     for (int a = 0; a < 3; ++a) {
       part[(w * 6 + a) * 32 + lane] = make_longlong2(up.re[a], up.im[a]);
       part[(w * 6 + 3 + a) * 32 + lane] = make_longlong2(lo.re[a], lo.im[a]);
+      if constexpr (!kFF) {
+        evidence[(w * 6 + a) * 32 + lane] = wit.up[a];
+        evidence[(w * 6 + 3 + a) * 32 + lane] = wit.lo[a];
+      }
     }
     __syncthreads();
   } else {
     __syncwarp();
+  }
+  unsigned again = 0;  // components whose hops are taken in FP64
+  if constexpr (!kFF) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      if (W > 1 && k % W != sub) continue;
+      unsigned x = k < 3 ? wit.up[k % 3] : wit.lo[k % 3];
+      if constexpr (W > 1) {
+        x = 0;
+#pragma unroll
+        for (int q = 0; q < W; ++q) x |= evidence[((unit * W + q) * 6 + k) * 32 + lane];
+      }
+      if ((x & kWitnessBits) == 0) again |= 1u << k;
+    }
+    // zero hops, as of a diluted source, are exact
+    if (!any_hop(h.spins, r, false)) again &= 56u;
+    if (!any_hop(h.spins, r, true)) again &= 7u;
+    if (h.E > kMaxExp) again = 63u;
   }
   // component k of this lane: 0..2 spin r, 3..5 spin 2 + r
 #pragma unroll
@@ -221,19 +257,25 @@ wilson_fix_kernel(Geometry g, FixView v, const double2* __restrict__ u64, const 
         outf[(size_t)comp * V + s] = o;
     }
   }
-  if constexpr (!kFF) if (work && s0 + i < V && h.E > kMaxExp) {  // next to a value the digits do not hold: FP64
-    for (int k = sub; k < 6; k += W) {
-      const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
-      const double2 p = USER ? in[((size_t)fc * V + s) * 12 + comp] : inf[(size_t)comp * V + s];
-      const double2 d = hop_sum_fp64<USER>(g, u64, in, fc, s, comp);
-      const double sg = k < 3 ? 1.0 : -1.0;
-      double2 o;
-      o.x = fma(sg, fma(-g.kappa, d.x, p.x), 0.0 * p.x);
-      o.y = fma(sg, fma(-g.kappa, d.y, p.y), 0.0 * p.y);
-      if (USER)
-        st[i * 13 + comp] = o;
-      else
-        outf[(size_t)comp * V + s] = o;
+  if constexpr (!kFF) {
+    if (work && s0 + i < V && again != 0) {
+      const double small = fabs(hf) * 0x1p-148;  // kappa 2^(E - 5)
+      for (int k = sub; k < 6; k += W) {
+        if ((again >> k & 1) == 0) continue;
+        const int comp = (k < 3 ? 0 : 6) + r * 3 + k % 3;
+        const double2 p = USER ? in[((size_t)fc * V + s) * 12 + comp] : inf[(size_t)comp * V + s];
+        // beside diagonal terms of that size the hops' roundings are as small
+        if (h.E <= kMaxExp && fmin(fabs(p.x), fabs(p.y)) >= small) continue;
+        const double2 d = hop_sum_fp64<USER>(g, u64, in, fc, s, comp);
+        const double sg = k < 3 ? 1.0 : -1.0;
+        double2 o;
+        o.x = fma(sg, fma(-g.kappa, d.x, p.x), 0.0 * p.x);
+        o.y = fma(sg, fma(-g.kappa, d.y, p.y), 0.0 * p.y);
+        if (USER)
+          st[i * 13 + comp] = o;
+        else
+          outf[(size_t)comp * V + s] = o;
+      }
     }
   }
   if (USER) {

@@ -5,10 +5,13 @@
 // multiply-adds (32 x 32 + 64 -> 64 bits; both measured), so a hop's link
 // product -- a sum of six real products an output, three multiply-adds a
 // product -- costs a fifth as much in 60-bit fixed point as in FP64, and the
-// additions almost nothing.  It is more accurate as well: every
-// product and sum is exact but for the low-by-low digit product and two
-// roundings at 2^-58 of the site's largest component (FP64 rounds each
-// operation at 2^-53 of its own result).
+// additions almost nothing.  Every product and sum is exact but for the
+// low-by-low digit product and two roundings at 2^-58 of the site's largest
+// component.  In the norm of a site that is less than FP64's roundings; a
+// component far below its site's or its neighbours' largest has fewer bits here
+// than FP64 gives it, so that the stand-alone operator looks for such
+// components (Witness) and takes their hops in FP64.  The CG loop, whose
+// stopping test and solutions are bounded in the norm, does not.
 //
 // Format.  The 24 reals of a site share one exponent e with every |v| < 2^e;
 // a real is the integer X = round(v 2^(59 - e)), |X| <= 2^59, kept as two
@@ -96,7 +99,10 @@ __device__ __forceinline__ int4 to_site_digits(float4 v, int e) {
 }
 
 // Four lanes a site (lane = 8 q + j: spin q of site j of eight), three
-// components each: the site's exponent, the same in its four lanes.
+// components each: the site's word, 16 e + one bit a spin that is not zero
+// throughout, the same in its four lanes.
+constexpr int kSpinBits = 4;
+__device__ __forceinline__ int word_exp(int word) { return word >> kSpinBits; }
 __device__ __forceinline__ void site_key(const double2& v, int& key, int& low) {
   key = max(key, max(abs_key(v.x), abs_key(v.y)));
   low |= __double2loint(v.x) | __double2loint(v.y);
@@ -110,24 +116,24 @@ __device__ __forceinline__ int key_exp(float4, int key, int) {
   return key == 0 ? kZeroExp : ex == 255 ? kSpecialExp : max(ex, 1) - 126;
 }
 template <typename V2>
-__device__ __forceinline__ int quad_site_exp(const V2 (&v)[3]) {
+__device__ __forceinline__ int quad_site_word(const V2 (&v)[3], int q) {
   int key = 0, low = 0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) site_key(v[a], key, low);
-  int nz = (key | low) != 0;
+  int nz = (key | low) != 0 ? 1 << q : 0;
 #pragma unroll
   for (int o = 8; o <= 16; o <<= 1) {
     key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
     nz |= __shfl_xor_sync(0xffffffffu, nz, o);
   }
-  return key_exp(v[0], key, nz);
+  return key_exp(v[0], key, nz) << kSpinBits | nz;
 }
 
 // ---- layout -----------------------------------------------------------------------------
 // Tiles of 16 consecutive sites, so that every component of a site lies at a
 // constant distance from its first one (one address a hop, the loads take
 // their offsets as immediates): fields [f][tile][12][16] int4, links
-// [mu][tile][9][16] int4, exponents [f][tile 16].
+// [mu][tile][9][16] int4, site words (exponents) [f][tile 16].
 constexpr int kTile = kFixSites;
 __host__ __device__ __forceinline__ int fix_tiles(int V) { return (V + kTile - 1) / kTile; }
 __device__ __forceinline__ size_t field_at(int tiles, size_t f, int s) {
@@ -235,6 +241,46 @@ __device__ __forceinline__ void hop_math(const HopData& d, int mu_rt, int r, boo
   }
 }
 
+// Evidence that the terms of a component's hop sum are not all far below 2^E,
+// the scale of the sum's roundings: the largest (as an OR) of its shares from the
+// hops, for the three colours of upper spin r and of lower spin 2 + r.  The roundings stay
+// below 48 units of 2^(E - 57) (six a hop), ~2 in the root mean square; a share of 2^52
+// units and more bounds them by 2^-46, ~2^-51, of the sum of the terms' sizes, where FP64's
+// own bound is ~2^-49.  Dense fields always have it: the sixteen reals of a
+// component would all have to be below a fourteenth of their spread.
+template <bool ON>
+struct Witness {
+  unsigned up[ON ? 3 : 1] = {}, lo[ON ? 3 : 1] = {};
+  // a hop of direction 0 or 1 (both for spin row r: crossed later) or 2 or 3
+  template <bool LOWER>
+  __device__ __forceinline__ void add(const Acc3& w) {
+    if constexpr (ON) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int re = (int)(w.re[a] >> 32), im = (int)(w.im[a] >> 32);
+        const unsigned x = (unsigned)(re ^ (re >> 31)) | (unsigned)(im ^ (im >> 31));
+        up[a] |= x;
+        if constexpr (LOWER) lo[a] |= x;
+      }
+    }
+  }
+  // after directions 0 and 1, which feed lower spin 3 - r: hand over what they gave
+  __device__ __forceinline__ void cross() {
+    if constexpr (ON) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) lo[a] = __shfl_xor_sync(0xffffffffu, up[a], 16);
+    }
+  }
+};
+constexpr unsigned kWitnessBits = ~((1u << 20) - 1);  // of the words above: 2^52 and more
+// Whether the upper spin r (lower: 2 + r) gets a hop from a spin that is not zero:
+// spin row r takes spins r and 2 + r (directions 2 and 3) or 3 - r (0 and 1) and
+// feeds spins r and 2 + r, or 3 - r.
+__device__ __forceinline__ bool any_hop(const int (&spins)[2], int r, bool lower) {
+  const int a = lower ? 1 << (1 - r) | 4 << r : 1 << r | 8 >> r;
+  return ((spins[0] & a) | (spins[1] & (5 << r))) != 0;
+}
+
 // neighbour of s in direction mu, forward or backward
 template <bool BACK>
 __device__ __forceinline__ int neighbour_rt(int s, const wcore::Coords& c, const Geometry& g, int mu, bool& twrap) {
@@ -260,7 +306,7 @@ struct FixView {
   const int4* __restrict__ u;    // links
   const int* __restrict__ nbr;   // neighbour table
   const int4* __restrict__ dig;  // the field's digits
-  const int* __restrict__ ex;    // its site exponents
+  const int* __restrict__ ex;    // its site words
   int tiles;
 };
 
@@ -270,6 +316,7 @@ struct Hops {
   int nb[8];
   unsigned sh[2];  // eight shifts of a byte
   int E;
+  int spins[2];    // bits of the spins that are not zero in the hops of directions 0 and 1, 2 and 3
 };
 // In two parts: the copies or loads of the hops' operands need the neighbours
 // alone, so that they are under way while the exponents come.
@@ -280,9 +327,13 @@ __device__ __forceinline__ void load_neighbours(const FixView& v, int s, Hops& h
 }
 __device__ __forceinline__ void load_exponents(const FixView& v, int s, Hops& h) {
   int e[8];
-  const int own = __ldg(v.ex + s);
+  const int own = word_exp(__ldg(v.ex + s));
 #pragma unroll
   for (int k = 0; k < 8; ++k) e[k] = __ldg(v.ex + (h.nb[k] & (kNegBit - 1)));
+  h.spins[0] = e[0] | e[1] | e[2] | e[3];
+  h.spins[1] = e[4] | e[5] | e[6] | e[7];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) e[k] = word_exp(e[k]);
   h.E = kZeroExp;
 #pragma unroll
   for (int k = 0; k < 8; ++k) h.E = max(h.E, e[k]);
@@ -366,8 +417,9 @@ __device__ __forceinline__ void stage_hop(const FixView& v, int s, int nbe, int 
 }
 
 // the arithmetic of hop K from its stage
-template <int K>
-__device__ __forceinline__ void staged_hop(const int4* buf, int nbe, int sh, int i, int r, Acc3& up, Acc3& d) {
+template <int K, bool WIT>
+__device__ __forceinline__ void staged_hop(const int4* buf, int nbe, int sh, int i, int r, Acc3& up, Acc3& d,
+                                           Witness<WIT>& wit) {
   constexpr int MU = K >> 1;
   constexpr bool BACK = (K & 1) != 0;
   const int lr = MU < 2 ? 1 - r : r;
@@ -375,16 +427,18 @@ __device__ __forceinline__ void staged_hop(const int4* buf, int nbe, int sh, int
   Acc3 w;
   hop_fetch<true>(buf + 12 * kTile + i, buf + r * 3 * kTile + i, buf + (6 + lr * 3) * kTile + i, o);
   hop_math<MU, BACK>(o, MU, r, (nbe & kNegBit) != 0, sh, w);
+  wit.template add<(MU >= 2)>(w);
   add_hop<BACK>(w, MU, r, up, d);
 }
 
-template <int K, typename Last>
+template <int K, bool WIT, typename Last>
 __device__ __forceinline__ void pipe_hops(const FixView& v, int s, int i, int r, const Hops& h, int4* buf, Acc3& up,
-                                          Acc3& lo, Last last) {
+                                          Acc3& lo, Witness<WIT>& wit, Last last) {
   if constexpr (K < 8) {
     copy_wait<1>();
     __syncwarp();
-    staged_hop<K>(buf + (K & 1) * kStageElems, h.nb[K], (int)(h.sh[K >> 2] >> (8 * (K & 3))) & 0xff, i, r, up, lo);
+    staged_hop<K>(buf + (K & 1) * kStageElems, h.nb[K], (int)(h.sh[K >> 2] >> (8 * (K & 3))) & 0xff, i, r, up, lo,
+                  wit);
     __syncwarp();
     if constexpr (K + 2 < 8)
       stage_hop<K + 2>(v, s, h.nb[K + 2], i, r, buf + (K & 1) * kStageElems);
@@ -392,23 +446,26 @@ __device__ __forceinline__ void pipe_hops(const FixView& v, int s, int i, int r,
       last(buf + (K & 1) * kStageElems);  // commits a group of its own
     else
       copy_commit();
-    if constexpr (K == 3) cross_over(lo);
-    pipe_hops<K + 1>(v, s, i, r, h, buf, up, lo, last);
+    if constexpr (K == 3) {
+      cross_over(lo);
+      wit.cross();
+    }
+    pipe_hops<K + 1>(v, s, i, r, h, buf, up, lo, wit, last);
   }
 }
 
 // The eight hops of the warp's 16 sites, whose neighbours are loaded (the
 // exponents are loaded here); last(stage) starts the copy of what
 // the caller needs after them (committed, complete after copy_wait<1>).
-template <typename Last>
+template <bool WIT, typename Last>
 __device__ __forceinline__ void hop_sums_piped(const FixView& v, int s, int i, int r, Hops& h, int4* buf,
-                                               Acc3& up, Acc3& lo, Last last) {
+                                               Acc3& up, Acc3& lo, Witness<WIT>& wit, Last last) {
   clear(up);
   clear(lo);
   stage_hop<0>(v, s, h.nb[0], i, r, buf);
   stage_hop<1>(v, s, h.nb[1], i, r, buf + kStageElems);
   load_exponents(v, s, h);
-  pipe_hops<0>(v, s, i, r, h, buf, up, lo, last);
+  pipe_hops<0>(v, s, i, r, h, buf, up, lo, wit, last);
 }
 
 // Hop sums of one of four warps (sub: its direction, both hops) for spin row r
@@ -416,7 +473,9 @@ __device__ __forceinline__ void hop_sums_piped(const FixView& v, int s, int i, i
 // 2^(E - 57).  The direction is a run-time value, since warps that each run
 // their own copy of the code stall on instruction fetches.  All lanes of the
 // warp take part.
-__device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub, Hops& h, Acc3& up, Acc3& lo) {
+template <bool WIT>
+__device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub, Hops& h, Acc3& up, Acc3& lo,
+                                         Witness<WIT>& wit) {
   clear(up);
   clear(lo);
   const int mu = sub;
@@ -429,11 +488,16 @@ __device__ __forceinline__ void hop_sums(const FixView& v, int s, int r, int sub
   const int sf = s2 & 0xff, sb = (s2 >> 8) & 0xff;
   Acc3 w;
   hop_math<-1, false>(d, mu, r, (nf & kNegBit) != 0, sf, w);
+  wit.template add<true>(w);
   add_hop<false>(w, mu, r, up, lo);
   hop_fetch_at<true>(v, s, nb, mu, r, d);
   hop_math<-1, true>(d, mu, r, (nb & kNegBit) != 0, sb, w);
+  wit.template add<true>(w);
   add_hop<true>(w, mu, r, up, lo);
-  if (mu < 2) cross_over(lo);
+  if (mu < 2) {
+    cross_over(lo);
+    wit.cross();
+  }
 }
 
 // Launch shapes for W = 1 or 4 warps a site group: threads a block, (site group,
