@@ -296,9 +296,16 @@ int ssqcd_shifted_cg(ssqcd_lattice lat, int N, const double* z, int L, const dou
 
 /* ---- moments (Eq. 2) ------------------------------------------------------------ */
 
-/* s_hat[l][k] = sum_j w_j zeta_j^k y[l][j] for k < M (Eq. 2), on the device,
- * FP64.  y: [L][N][V][4][3] complex128 and s_hat: [L][M][V][4][3] complex128,
- * both host or both device per on_device; w, zeta: [N] complex128 host. */
+/* s_hat[l][k] = sum_j w_j zeta_j^k y[l][j] for k < M (Eq. 2), on the device.
+ * y: [L][N][V][4][3] complex128 and s_hat: [L][M][V][4][3] complex128,
+ * both host or both device per on_device; w, zeta: [N] complex128 host.
+ * In FP64, or for larger sums of dense vectors (on average within five
+ * binades of their largest component) in 56-bit fixed point relative to each
+ * vector's largest component and each output's largest coefficient, within
+ * 2^-52 of FP64's result in the norm.  A real or imaginary part none of
+ * whose terms comes within 2^-11 of that scale is summed in FP64 all the same, so
+ * that every part lies within N 2^-42 of the sum of its terms' sizes
+ * (typically sqrt(N) 2^-48). */
 int ssqcd_moments(ssqcd_lattice lat, int N, int M, int L, const double* w, const double* zeta,
                   const double* y, double* s_hat, int on_device);
 

@@ -654,7 +654,7 @@ int combine(const double2* S, int ms, long long n, const double2* C, int mc, dou
   if (ms <= 0 || mc <= 0 || n <= 0 || nl <= 0) return SSQCD_OK;
   if (combine_tc_enabled() && combine_tc_applicable(n, 1, ms) && (double)nl * ms * mc * (double)n >= kTcCombineTerms) {
     DevBuf work;
-    if (work.alloc(combine_tc_work_bytes(nl, ms)) == SSQCD_OK) {
+    if (work.alloc(combine_tc_vectors_work_bytes(n, nl, ms)) == SSQCD_OK) {
       bool suits = false;
       SS_TRY(combine_tc_vectors(S, ms, n, C, mc, Q, nl, work.p, s, &suits));
       if (suits) return SSQCD_OK;

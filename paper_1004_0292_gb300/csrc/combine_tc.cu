@@ -440,7 +440,8 @@ __global__ void tc_scales_kernel(const unsigned* __restrict__ mx, CoefView C, in
   for (int s = threadIdx.x; s < cnt; s += blockDim.x) {
     const unsigned key = mx[(size_t)lz * S + s];
     const bool fin = key < kBadKey;
-    const int e = fin && key != 0 ? max((int)(key >> 20) - 1022, -950) : 0;  // 2^(e - 1) <= max < 2^e
+    // 2^(e - 1) <= max < 2^e; a vector of zeros has no share in its outputs' scales
+    const int e = !fin ? 0 : key != 0 ? max((int)(key >> 20) - 1022, -950) : -950;
     bad |= !fin;
     if (ex != nullptr && o == 0 && key != 0 &&
         (unsigned long long)(key >> 20) * (unsigned long long)(2 * n) >
@@ -452,7 +453,7 @@ __global__ void tc_scales_kernel(const unsigned* __restrict__ mx, CoefView C, in
       for (int k = 0; k < (C.cplx ? 2 : 1); ++k) {
         const double c = C.get(l, o ^ k, s);
         bad |= !isfinite(c);
-        if (isfinite(c)) m = fmax(m, fabs(ldexp(c, e)));
+        if (isfinite(c) && key != 0) m = fmax(m, fabs(ldexp(c, e)));
       }
     }
   }
@@ -514,6 +515,122 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
   }
   unsigned char* dst = bimg + ((size_t)lz * ksteps_cap + kk) * (kSlices * OUT * kKStep * 2) + core_off(row, 8 * h);
   *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(f);
+}
+
+// ---- components far below their vectors' largest ---------------------------------------------
+// The roundings of an output are relative to its scale, sig: at most S 2^-53 sig,
+// ~sqrt(S) 2^-57 in the root mean square.  A part (real or imaginary) of an output element
+// one of whose terms is at least 2^-(kCoefBits + kVecBits + 1) sig is served by
+// that: such a term is a coefficient within kCoefBits binades of its output's scale times a component
+// within kVecBits of its vector's.  The elements with a part that has terms, but none such, go
+// on a list (tc_witness_kernel) and take the FP64 sum behind the pass
+// (tc_rest_kernel); more of them than the list holds, and the vectors do not suit.
+// Dense vectors have next to none, and their elements show it by the one to
+// six slots where an output's coefficient is largest: 45 us more for the 16^3 x 32 moments' 1.16 ms.
+constexpr int kCoefBits = 3, kVecBits = 7;
+constexpr int kMaxPass = kWideOut / 2;  // complex outputs a pass
+struct Components {
+  uint4* mask;                  // [l][slot] bits of the pass's outputs: re and im of the coefficient large, not zero
+  unsigned long long* largest;  // [l][kMaxPass] coefficient (as float bits) and slot of the largest, per output
+  long long* list;              // l' n + element
+  unsigned* count;
+  unsigned cap;
+};
+__global__ void tc_masks_kernel(CoefView C, int O, int S, int stride, const unsigned* __restrict__ mx,
+                                const int* __restrict__ eslot, const double* __restrict__ sig, Components k) {
+  const int lz = blockIdx.y;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < S * O; t += gridDim.x * blockDim.x) {
+    const int s = t / O, o = t % O;
+    if (mx[(size_t)lz * S + s] == 0) continue;
+    const double2 c = C.c[lz * C.sl + o * C.so + s * C.ss];
+    const int d = eslot[(size_t)lz * padded(S) + s] - (exp_above(sig[(size_t)lz * stride + 2 * o]) - 1);
+    const double re = fabs(ldexp(c.x, d)), im = fabs(ldexp(c.y, d));
+    uint4* m = k.mask + (size_t)lz * S + s;
+    const unsigned bit = 1u << o;
+    if (re >= ldexp(1.0, -kCoefBits)) atomicOr(&m->x, bit);
+    if (im >= ldexp(1.0, -kCoefBits)) atomicOr(&m->y, bit);
+    if (c.x != 0.0) atomicOr(&m->z, bit);
+    if (c.y != 0.0) atomicOr(&m->w, bit);
+    atomicMax(k.largest + lz * kMaxPass + o,
+              (unsigned long long)__float_as_uint((float)fmax(re, im)) << 32 | (unsigned)s);
+  }
+}
+__global__ void __launch_bounds__(256)
+tc_witness_kernel(SlotMap map, long long n, int l0, int O, int S, const int* __restrict__ eslot, Components k,
+                  int* __restrict__ err) {
+  const int lz = blockIdx.y;
+  const unsigned all = (1u << O) - 1;
+  // the slots of the outputs' largest coefficients, each once, four to a turn
+  // (their loads together: a turn is a pass over four vectors)
+  __shared__ int s_slot[kMaxPass];
+  __shared__ int s_slots;
+  if (threadIdx.x < 32) {
+    const int o = threadIdx.x;
+    const int s = o < O ? (int)(unsigned)k.largest[lz * kMaxPass + o] : -1 - o;
+    const bool first = (int)__ffs(__match_any_sync(0xffffffffu, s)) - 1 == o && o < O;
+    const unsigned f = __ballot_sync(0xffffffffu, first);
+    if (first) s_slot[__popc(f & ((1u << o) - 1))] = s;
+    if (o == 0) s_slots = __popc(f);
+  }
+  __syncthreads();
+  const int slots = s_slots;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    unsigned fr = 0, fi = 0, nr = 0, ni = 0;  // outputs whose real, imaginary part has a large term, a term
+    auto at = [&](int s) { return __ldg(reinterpret_cast<const uint4*>(slot_ptr(map, n, l0 + lz, s)) + e); };
+    auto visit = [&](uint4 x, int s) {
+      const uint4 m = __ldg(k.mask + (size_t)lz * S + s);
+      const int low = __ldg(eslot + (size_t)lz * padded(S) + s) + 1023 - kVecBits;
+      const bool br = (int)(x.y >> 20 & 0x7FF) >= low, bi = (int)(x.w >> 20 & 0x7FF) >= low;
+      const bool zr = (x.y << 1 | x.x) != 0, zi = (x.w << 1 | x.z) != 0;
+      fr |= (br ? m.x : 0) | (bi ? m.y : 0);
+      fi |= (bi ? m.x : 0) | (br ? m.y : 0);
+      nr |= (zr ? m.z : 0) | (zi ? m.w : 0);
+      ni |= (zi ? m.z : 0) | (zr ? m.w : 0);
+      return (fr & fi) == all;
+    };
+    bool ok = false;
+    for (int o = 0; o < slots && !ok; o += 4) {
+      uint4 x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = at(s_slot[min(o + i, slots - 1)]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) ok = visit(x[i], s_slot[min(o + i, slots - 1)]);
+    }
+    for (int s = 0; s < S && !ok; ++s) ok = visit(at(s), s);
+    if (!ok && ((nr & ~fr) | (ni & ~fi)) != 0) {
+      const unsigned place = atomicAdd(k.count, 1u);
+      if (place < k.cap)
+        k.list[place] = (long long)lz * n + e;
+      else
+        atomicOr(err, kErrSpread);
+    }
+  }
+}
+// the listed elements' outputs in FP64: a warp an element, its lanes the slots
+__global__ void __launch_bounds__(256)
+tc_rest_kernel(SlotMap map, long long n, int l0, CoefView C, int O, int S, Components k, long long out_l,
+               double2* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const unsigned cnt = min(*k.count, k.cap);
+  for (unsigned i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < cnt; i += gridDim.x * (blockDim.x >> 5)) {
+    const int lz = (int)(k.list[i] / n), l = l0 + lz;
+    const long long e = k.list[i] % n;
+    for (int o = 0; o < O; ++o) {
+      double re = 0.0, im = 0.0;
+      for (int s = lane; s < S; s += 32) {
+        const double2 x = reinterpret_cast<const double2*>(slot_ptr(map, n, l, s))[e];
+        const double2 c = C.c[lz * C.sl + o * C.so + s * C.ss];
+        re = fma(c.x, x.x, fma(-c.y, x.y, re));
+        im = fma(c.x, x.y, fma(c.y, x.x, im));
+      }
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, d);
+        im += __shfl_xor_sync(0xffffffffu, im, d);
+      }
+      if (lane == 0) out[l * out_l + (long long)o * n + e] = make_double2(re, im);
+    }
+  }
 }
 
 // A sum xh 2^32 + xl (|xh| < 2^50) times 2^e as a double, rounded to nearest
@@ -947,6 +1064,18 @@ bool combine_tc_applicable(long long n, int O, int S) {
   return O >= 1 && O <= kOut && n > 0 && S >= 1 && S <= kMaxCount;
 }
 
+namespace {
+// elements that the list of tc_witness_kernel holds: a 64th of all, whose FP64
+// sums take a few percent of all elements'
+unsigned rest_cap(long long n, int nl) { return (unsigned)std::min(n * nl / 64 + 64, 1LL << 28); }
+}  // namespace
+
+size_t combine_tc_vectors_work_bytes(long long n, int nl, int S) {
+  return combine_tc_work_bytes(nl, S) + align256(sizeof(uint4) * (size_t)nl * S) +
+         align256(sizeof(unsigned long long) * (size_t)nl * kMaxPass) + 256 +
+         sizeof(long long) * (size_t)rest_cap(n, nl);
+}
+
 size_t combine_tc_work_bytes(int nl, int S) {
   const int ks = (S + kKStep - 1) / kKStep;
   return align256(sizeof(unsigned long long) * (size_t)nl * S) + align256(sizeof(unsigned) * (size_t)nl * S) +
@@ -960,10 +1089,11 @@ namespace {
 // suits (may be null): set to false, the outputs then not to be used, when a
 // vector has too wide a spread (kMaxSpread), an infinity or a NaN; with add
 // (complex coefficients: the sums are added to out) that is found out before
-// out is touched.
+// out is touched.  comps (may be null; complex coefficients, not with add):
+// elements with small components take the FP64 sum.
 int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const int* count, double2* out,
                 long long out_l, int l0, int nl, void* work, cudaStream_t st, bool* suits, bool add = false,
-                bool ff = false) {
+                bool ff = false, const Components* comps = nullptr) {
   const int ks = (S + kKStep - 1) / kKStep;
   TcWork w = carve(work, nl, S, ks);
   unsigned long long* ex = suits != nullptr ? w.ex : nullptr;
@@ -1026,6 +1156,16 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     }
     scales(o0);
     SS_CHECK_LAUNCH();
+    if (comps != nullptr) {
+      SS_CUDA(cudaMemsetAsync(comps->mask, 0, (char*)(comps->count + 1) - (char*)comps->mask, st));
+      tc_masks_kernel<<<dim3(std::min((S * (Op / 2) + 255) / 256, 64), nl), 256, 0, st>>>(
+          Cp, Op / 2, S, wide ? kWideOut : kOut, w.mx, w.eslot, w.sig, *comps);
+      SS_CHECK_LAUNCH();
+      tc_witness_kernel<<<dim3((unsigned)std::min((n + 255) / 256, 16LL * sms), nl), 256, 0, st>>>(
+          map, n, l0, Op / 2, S, w.eslot, *comps, w.err);
+      SS_CHECK_LAUNCH();
+      count_launches(2);
+    }
     if (wide)
       tc_bslices_kernel<kWideOut><<<dim3(ks, nl), 2 * Form<true>::kBRows, 0, st>>>(Cp, Op, S, l0, count, w.eslot, w.sig,
                                                                                    ks, w.bimg);
@@ -1037,6 +1177,11 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
         map, n, l0, nl, count, S, w.eslot, w.bimg, ks, w.sig, Op, out_l, out + (long long)o0 * n, w.err);
     SS_CHECK_LAUNCH();
     count_launches(3);
+    if (comps != nullptr) {
+      tc_rest_kernel<<<4 * sms, 256, 0, st>>>(map, n, l0, Cp, Op / 2, S, *comps, out_l, out + (long long)o0 * n);
+      SS_CHECK_LAUNCH();
+      count_launches(1);
+    }
   }
   count_launches(1);
   SS_CUDA(cudaMemcpyAsync(&h_err, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1066,8 +1211,17 @@ int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, cons
 int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,
                        cudaStream_t st, bool* suits) {
   if (O < 1 || nl < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
+  Components k;
+  char* p = static_cast<char*>(work) + combine_tc_work_bytes(nl, S);
+  k.mask = reinterpret_cast<uint4*>(p);
+  p += align256(sizeof(uint4) * (size_t)nl * S);
+  k.largest = reinterpret_cast<unsigned long long*>(p);
+  p += align256(sizeof(unsigned long long) * (size_t)nl * kMaxPass);
+  k.count = reinterpret_cast<unsigned*>(p);  // cleared with the two before it
+  k.list = reinterpret_cast<long long*>(p + 256);
+  k.cap = rest_cap(n, nl);
   return combine_all(SlotMap{nullptr, 0, 1, x, S}, n, CoefView{C, 0, 1, O, true, true}, O, S, nullptr, out, (long long)O * n,
-                     0, nl, work, st, suits);
+                     0, nl, work, st, suits, false, false, &k);
 }
 
 }  // namespace ssqcd

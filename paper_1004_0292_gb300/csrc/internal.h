@@ -290,7 +290,10 @@ int combine_tc(char* const* tab, int basis_log, long long n, int L, const double
 int combine_tc_complex(char* const* tab, int basis_log, long long n, int L, const double2* C, int O, int S,
                        const int* count, double2* out, int l0, int nl, void* work, cudaStream_t st, bool* suits,
                        bool add = false);
-// out[l][o] = sum_s C[s][o] x[l][s] for l < nl, vectors of n complex elements
+// out[l][o] = sum_s C[s][o] x[l][s] for l < nl, vectors of n complex elements;
+// work: combine_tc_vectors_work_bytes.  Elements whose terms are all far below
+// the vectors' largest take the FP64 sum.
+size_t combine_tc_vectors_work_bytes(long long n, int nl, int S);
 int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, int O, double2* out, int nl, void* work,
                        cudaStream_t st, bool* suits);
 
