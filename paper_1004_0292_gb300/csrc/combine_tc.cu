@@ -564,15 +564,20 @@ tc_witness_kernel(SlotMap map, long long n, int l0, int O, int S, const int* __r
   // (their loads together: a turn is a pass over four vectors)
   __shared__ int s_slot[kMaxPass];
   __shared__ int s_slots;
+  __shared__ bool s_done;  // the whole sum in FP64 already (other blocks of this launch may say so: read once)
   if (threadIdx.x < 32) {
     const int o = threadIdx.x;
     const int s = o < O ? (int)(unsigned)k.largest[lz * kMaxPass + o] : -1 - o;
     const bool first = (int)__ffs(__match_any_sync(0xffffffffu, s)) - 1 == o && o < O;
     const unsigned f = __ballot_sync(0xffffffffu, first);
     if (first) s_slot[__popc(f & ((1u << o) - 1))] = s;
-    if (o == 0) s_slots = __popc(f);
+    if (o == 0) {
+      s_slots = __popc(f);
+      s_done = (*reinterpret_cast<volatile int*>(err) & kErrSpread) != 0;
+    }
   }
   __syncthreads();
+  if (s_done) return;
   const int slots = s_slots;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     unsigned fr = 0, fi = 0, nr = 0, ni = 0;  // outputs whose real, imaginary part has a large term, a term
@@ -609,7 +614,8 @@ tc_witness_kernel(SlotMap map, long long n, int l0, int O, int S, const int* __r
 // the listed elements' outputs in FP64: a warp an element, its lanes the slots
 __global__ void __launch_bounds__(256)
 tc_rest_kernel(SlotMap map, long long n, int l0, CoefView C, int O, int S, Components k, long long out_l,
-               double2* __restrict__ out) {
+               double2* __restrict__ out, const int* __restrict__ err) {
+  if ((*err & kErrSpread) != 0) return;
   const int lane = threadIdx.x & 31;
   const unsigned cnt = min(*k.count, k.cap);
   for (unsigned i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < cnt; i += gridDim.x * (blockDim.x >> 5)) {
@@ -669,6 +675,8 @@ combine_tc_kernel(SlotMap map, long long n, int l0, int nl, const int* __restric
                   const double* __restrict__ sig, int O, long long out_l, double2* __restrict__ out,
                   int* __restrict__ err) {
   extern __shared__ unsigned char tc_smem_raw[];
+  // vectors that do not suit, known before this launch: the FP64 sum follows
+  if ((*err & kErrSpread) != 0) return;
   using F = Form<WIDE>;
   static_assert(CPLX || !WIDE, "the wide form's bound is that of signed digits");
   constexpr int kSliceStages = F::kSliceStages, kChunkSteps = F::kChunkSteps, kBBytes = F::kBBytes;
@@ -1178,7 +1186,8 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     SS_CHECK_LAUNCH();
     count_launches(3);
     if (comps != nullptr) {
-      tc_rest_kernel<<<4 * sms, 256, 0, st>>>(map, n, l0, Cp, Op / 2, S, *comps, out_l, out + (long long)o0 * n);
+      tc_rest_kernel<<<4 * sms, 256, 0, st>>>(map, n, l0, Cp, Op / 2, S, *comps, out_l, out + (long long)o0 * n,
+                                             w.err);
       SS_CHECK_LAUNCH();
       count_launches(1);
     }
