@@ -298,7 +298,8 @@ int ssqcd_shifted_cg(ssqcd_lattice lat, int N, const double* z, int L, const dou
 
 /* s_hat[l][k] = sum_j w_j zeta_j^k y[l][j] for k < M (Eq. 2), on the device.
  * y: [L][N][V][4][3] complex128 and s_hat: [L][M][V][4][3] complex128,
- * both host or both device per on_device; w, zeta: [N] complex128 host.
+ * both host or both device per on_device, s_hat possibly over y (by way of a
+ * copy); w, zeta: [N] complex128 host.
  * In FP64, or for larger sums of dense vectors (on average within five
  * binades of their largest component) in 56-bit fixed point relative to each
  * vector's largest component and each output's largest coefficient, within

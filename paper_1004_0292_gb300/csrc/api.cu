@@ -284,16 +284,23 @@ extern "C" int ssqcd_moments(ssqcd_lattice lat, int N, int M, int L, const doubl
   const long long n = 12LL * lat->g.V;
   const double2* src = reinterpret_cast<const double2*>(y);
   double2* dst = reinterpret_cast<double2*>(s_hat);
+  const size_t y_bytes = sizeof(double2) * n * N * L, s_bytes = sizeof(double2) * n * M * L;
+  // moments over the solutions themselves (a buffer used again) by way of a copy
+  const uintptr_t y0 = reinterpret_cast<uintptr_t>(y), s0 = reinterpret_cast<uintptr_t>(s_hat);
+  const bool copy_out = !on_device || (y0 < s0 + s_bytes && s0 < y0 + y_bytes);
   if (!on_device) {
-    SS_TRY(yd.alloc(sizeof(double2) * n * N * L));
-    SS_TRY(sd.alloc(sizeof(double2) * n * M * L));
-    SS_CUDA(cudaMemcpyAsync(yd.p, y, sizeof(double2) * n * N * L, cudaMemcpyHostToDevice, lat->stream));
+    SS_TRY(yd.alloc(y_bytes));
+    SS_CUDA(cudaMemcpyAsync(yd.p, y, y_bytes, cudaMemcpyHostToDevice, lat->stream));
     src = yd.as<double2>();
+  }
+  if (copy_out) {
+    SS_TRY(sd.alloc(s_bytes));
     dst = sd.as<double2>();
   }
   SS_TRY(moments_device(src, N, M, L, n, coef.data(), dst, scratch, lat->stream));
-  if (!on_device)
-    SS_CUDA(cudaMemcpyAsync(s_hat, dst, sizeof(double2) * n * M * L, cudaMemcpyDeviceToHost, lat->stream));
+  if (copy_out)
+    SS_CUDA(cudaMemcpyAsync(s_hat, dst, s_bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                            lat->stream));
   SS_CUDA(cudaStreamSynchronize(lat->stream));
   return SSQCD_OK;
 }
