@@ -652,6 +652,12 @@ int combine_fp64(const double2* S, int ms, long long n, const double2* C, int mc
 
 int combine(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s, int nl) {
   if (ms <= 0 || mc <= 0 || n <= 0 || nl <= 0) return SSQCD_OK;
+  constexpr int kBlocks = 32768;  // blocks of vectors at a time: a dimension of the kernels' grids
+  if (nl > kBlocks) {
+    for (int l = 0; l < nl; l += kBlocks)
+      SS_TRY(combine(S + (long long)l * ms * n, ms, n, C, mc, Q + (long long)l * mc * n, s, std::min(kBlocks, nl - l)));
+    return SSQCD_OK;
+  }
   if (combine_tc_enabled() && combine_tc_applicable(n, 1, ms) && (double)nl * ms * mc * (double)n >= kTcCombineTerms) {
     DevBuf work;
     if (work.alloc(combine_tc_vectors_work_bytes(n, nl, ms)) == SSQCD_OK) {
