@@ -1119,7 +1119,14 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
   const long long tiles = ((2 * n + kRows - 1) / kRows) * nl;
   const int grid = (int)(tiles < sms ? tiles : sms);
   // a pass: its first output, its outputs, and whether it is a wide one
-  auto wide_at = [&](int o0) { return C.cplx && O - o0 > kOut / 2; };
+  auto* wide_kern = add ? combine_tc_kernel<true, false, true, true, false> : combine_tc_kernel<true, false, false, true, false>;
+  bool wide_ok = C.cplx && O > kOut / 2;
+  if (wide_ok) {  // its warps share out the registers of the launch: as many as the shares add up to, or the narrow form
+    cudaFuncAttributes at;
+    SS_CUDA(cudaFuncGetAttributes(&at, wide_kern));
+    wide_ok = at.numRegs >= Form<true>::kRegs;
+  }
+  auto wide_at = [&](int o0) { return wide_ok && O - o0 > kOut / 2; };
   auto outs_at = [&](int o0) { return std::min(O - o0, !C.cplx ? kOut : wide_at(o0) ? kWideOut / 2 : kOut / 2); };
   auto scales = [&](int o0) {
     CoefView Cp = C;
@@ -1147,8 +1154,7 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     CoefView Cp = C;
     Cp.c += o0 * C.so;
     const int Op = (C.cplx ? 2 : 1) * outs_at(o0);
-    auto* kern = wide    ? (add ? combine_tc_kernel<true, false, true, true, false>
-                               : combine_tc_kernel<true, false, false, true, false>)
+    auto* kern = wide    ? wide_kern
                  : add    ? combine_tc_kernel<true, false, true, false, false>
                  : C.cplx ? (S <= 64 ? combine_tc_kernel<true, true, false, false, false>
                                      : combine_tc_kernel<true, false, false, false, false>)
@@ -1157,11 +1163,6 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
                            : combine_tc_kernel<false, false, false, false, false>;
     const size_t smem = (wide ? sizeof(TcShared<true>) : sizeof(TcShared<false>)) + 1024;
     SS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));  // the same every time
-    if (wide) {  // its warps share out the registers of the launch
-      cudaFuncAttributes at;
-      SS_CUDA(cudaFuncGetAttributes(&at, kern));
-      if (at.numRegs < Form<true>::kRegs) return fail(SSQCD_ERR_CUDA, "combination (tensor cores): too few registers");
-    }
     scales(o0);
     SS_CHECK_LAUNCH();
     if (comps != nullptr) {
