@@ -288,11 +288,25 @@ int ssqcd_contour(int path, double gamma, double rho, double beta, int N, double
  * mixed ones need a lattice created with that code, the others run on any
  * lattice (reliable_every as in ssqcd_opts).
  * Returns SSQCD_ERR_BREAKDOWN or SSQCD_ERR_NOCONV when the loop cannot finish
- * (outputs then hold the last iterate). */
+ * (outputs then hold the last iterate).
+ * With SSQCD_FP64 and SSQCD_FP64_DFSHIFT larger systems (N >= 4, N L n >= 4e5)
+ * keep the seed residuals in device memory and form the solutions out of
+ * them, at the end and whenever that memory is full, in FP64 throughout
+ * (rounded at 2^-56 of the largest term of a solution, in its norm as an FP64
+ * sum is): up to 512 N L n bytes, at least 4 GiB, and at most half of the memory left
+ * once the solutions have theirs (ssqcd_set_residual_bytes).  Where that is below
+ * 3072 L n bytes the solutions are updated in every iteration, in the
+ * precision asked for.  Of the memory it took from the device's pool of
+ * stream-ordered allocations a call leaves at most 4 GiB there. */
 int ssqcd_shifted_cg(ssqcd_lattice lat, int N, const double* z, int L, const double* v,
                      int on_device, double sigma, double tol, int max_iter, int precision,
                      int reliable_every,
                      double* y, int* iters, double* xi, int* seed_iters);
+
+/* Device memory that the stored seed residuals of ssqcd_shifted_cg on this
+ * lattice may take: 0 (default) by the rule above, > 0 at most so many bytes
+ * (below 3072 L n none), < 0 none. */
+int ssqcd_set_residual_bytes(ssqcd_lattice lat, double bytes);
 
 /* ---- moments (Eq. 2) ------------------------------------------------------------ */
 

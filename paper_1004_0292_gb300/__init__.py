@@ -24,7 +24,7 @@ __all__ = [
     "OK", "ERR_ARG", "ERR_OOM", "ERR_BREAKDOWN", "ERR_NOCONV", "ERR_CUDA",
     "FP64", "MIXED", "MIXED_F32LINKS", "FP64_SHIFT32", "FP64_DFSHIFT", "DF", "EXTRACT_RR", "EXTRACT_HANKEL", "PATH_LINES", "PATH_CIRCLE", "SsqcdError",
     "library_path", "lib", "Server", "time_stencil", "create_lattice", "upload_gauge", "apply_H", "apply_H_mixed",
-    "contour", "shifted_cg", "moments", "moments_noalloc", "ss_solve", "ss_solve_windows", "ss_eigpairs", "small_eigh",
+    "contour", "shifted_cg", "set_residual_bytes", "moments", "moments_noalloc", "ss_solve", "ss_solve_windows", "ss_eigpairs", "small_eigh",
     "kernel_launches", "set_kernel_timing", "set_stencil_variant", "stencil_tuning", "Lattice", "Result", "Opts", "Stats",
 ]
 
@@ -105,6 +105,7 @@ def lib():
         "ssqcd_lattice_destroy": (None, [vp]),
         "ssqcd_contour": (i, [i, d, d, d, i, vp, vp]),
         "ssqcd_shifted_cg": (i, [vp, i, vp, i, vp, i, d, d, i, i, i, vp, vp, vp, vp]),
+        "ssqcd_set_residual_bytes": (i, [vp, d]),
         "ssqcd_moments": (i, [vp, i, i, i, vp, vp, vp, vp, i]),
         "ssqcd_default_opts": (None, [vp]),
         "ssqcd_ss_solve": (i, [vp, vp, i, i, i, vp, vp]),
@@ -260,6 +261,11 @@ def shifted_cg(lat: Lattice, z, v, sigma=0.0, tol=1e-12, max_iter=100000, precis
     if code not in (OK, ERR_BREAKDOWN, ERR_NOCONV):
         _check(code)
     return code, y, iters, xi, si.value
+
+
+def set_residual_bytes(lat: Lattice, nbytes):
+    """Device memory that shifted_cg's stored residuals may take: 0 by its own rule, < 0 none."""
+    _check(lib().ssqcd_set_residual_bytes(lat.handle, float(nbytes)))
 
 
 def moments(lat: Lattice, w, zeta, y, M):

@@ -114,6 +114,13 @@ extern "C" void ssqcd_lattice_destroy(ssqcd_lattice lat) {
   delete lat;
 }
 
+extern "C" int ssqcd_set_residual_bytes(ssqcd_lattice lat, double bytes) {
+  SS_TRY(check_lattice(lat, false));
+  if (std::isnan(bytes)) return fail(SSQCD_ERR_ARG, "ssqcd_set_residual_bytes: not a number");
+  lat->residual_bytes = bytes;
+  return SSQCD_OK;
+}
+
 extern "C" int ssqcd_upload_gauge(ssqcd_lattice lat, const double* links, int on_device) {
   SS_TRY(check_lattice(lat, false));
   if (links == nullptr) return fail(SSQCD_ERR_ARG, "NULL links");
@@ -240,6 +247,14 @@ extern "C" int ssqcd_shifted_cg(ssqcd_lattice lat, int N, const double* z, int L
     return fail(SSQCD_ERR_ARG, "bad shifted_cg arguments");
   if (is_mixed(precision) && precision != lat->precision)
     return fail(SSQCD_ERR_ARG, "a mixed-precision solve needs a lattice created with that precision");
+  // what the run leaves in the pool of stream-ordered memory is given back above
+  // what it found there, or kPoolIdle
+  struct Pool {
+    size_t before = pool_bytes();
+    ~Pool() {
+      if (pool_bytes() > before) trim_pool(before);
+    }
+  } pool;
   DevBuf vd, yd;
   SS_TRY(to_device_layout(lat, v, L, on_device, vd));
   std::vector<int> it(iters ? (size_t)L * N : 0);
@@ -259,6 +274,7 @@ extern "C" int ssqcd_shifted_cg(ssqcd_lattice lat, int N, const double* z, int L
     else std::memcpy(xi, xx.data(), sizeof(double2) * xx.size());
   }
   if (seed_iters) *seed_iters = o.seed_iters;
+  yd.release();  // (on the stream, before its last wait)
   SS_CUDA(cudaStreamSynchronize(lat->stream));
   return st;
 }

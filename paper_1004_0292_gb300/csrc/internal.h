@@ -90,6 +90,15 @@ struct AllocStream {
   bool prev_on_;
 };
 
+// Device memory that allocations can still have: free, or idle in the pool of
+// the stream-ordered ones (which keeps what they give back).
+size_t available_device_memory();
+// What the pool holds, and its idle memory given back down to `keep` bytes held
+// (and at least kPoolIdle of it idle).
+size_t pool_bytes();
+void trim_pool(size_t keep);
+constexpr size_t kPoolIdle = (size_t)4 << 30;
+
 // ---- lattice -------------------------------------------------------------------
 struct Geometry {
   int X, Y, Z, T;
@@ -118,6 +127,7 @@ struct ssqcd_lattice_s {
   // work spaces of finished apply calls, kept for the next ones (take_workspace)
   std::mutex ws_mutex;
   std::vector<std::unique_ptr<ssqcd::DevBuf>> ws;
+  double residual_bytes = 0.0;  // ssqcd_set_residual_bytes
 };
 
 namespace ssqcd {
@@ -314,13 +324,16 @@ class CgRunBase {
 };
 // basis_cap: bytes the stored residuals may take (Krylov-basis form, FP64 and
 // DF precisions); 0 selects the per-iteration shift-vector updates.  want_y:
-// the solutions are wanted, not the stored residuals; their memory and that of
-// p-hat is taken at once, so that the residuals only use what is left
+// the solutions are wanted, not the stored residuals; their memory, that of
+// p-hat and of the segments' coefficients is taken at once, and a negative
+// basis_cap stands for at most half of what is left (SSQCD_ERR_OOM below kSolutionBlocks blocks)
+constexpr int kSolutionBlocks = 12;
 int make_cg_run(ssqcd_lattice lat, int N, const double2* z_host, int L, const double2* v, double sigma, double tol,
                 int max_iter, int precision, int reliable_every, double basis_cap, cudaStream_t st,
                 std::unique_ptr<CgRunBase>* out, bool want_y = false);
 // the basis_cap of a solve from its options and size (n, N points, L
 // sources): 0 when the form does not apply
+double solve_residual_bytes(double n, int N, int L);  // where nothing is set and the device has it
 double basis_cap_for(int precision, int basis, double basis_max_bytes, long long n, int N, int L);
 int shifted_cg_device(ssqcd_lattice lat, int N, const double2* z_host, int L, const double2* v,
                       double sigma, double tol, int max_iter, int precision, int reliable_every,

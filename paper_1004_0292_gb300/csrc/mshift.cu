@@ -1795,12 +1795,6 @@ segment_state_kernel(const double2* __restrict__ gp, const double2* __restrict__
     if (pp != nullptr) ph[q * n + e] = make_double2(b.x * x.x - b.y * x.y, b.x * x.y + b.y * x.x);
   }
 }
-__global__ void __launch_bounds__(kUpdBlock)
-add_vectors_kernel(double2* __restrict__ y, const double2* __restrict__ x, long long count) {
-  for (long long e = blockIdx.x * (long long)kUpdBlock + threadIdx.x; e < count; e += (long long)gridDim.x * kUpdBlock)
-    y[e] = make_double2(y[e].x + x[e].x, y[e].y + x[e].y);
-}
-
 // Moment coefficients of one window: G[l][m][s] = sum_j W[j][m] gam[l][j][s]
 // (j ascending: a fixed order).
 __global__ void basis_window_kernel(const double2* __restrict__ gam, const double2* __restrict__ W, int N, int M,
@@ -1857,7 +1851,7 @@ constexpr int kCombThreads = 64;
 template <typename VR, typename VO, int OUT, bool RC>
 __global__ void __launch_bounds__(kCombThreads, 2)
 basis_combine_kernel(char* const* __restrict__ tab, long long n, int L, const double2* __restrict__ C, int O, int S,
-                     const int* __restrict__ count, VO* __restrict__ out, int l0) {
+                     const int* __restrict__ count, VO* __restrict__ out, int l0, bool add) {
   __shared__ double s_w[RC ? 1 : 3][kCombTile][OUT];
   __shared__ const VR* s_p[kCombTile];
   const int l = blockIdx.y + l0, o0 = blockIdx.z * OUT;
@@ -1914,9 +1908,13 @@ basis_combine_kernel(char* const* __restrict__ tab, long long n, int L, const do
   if (e < n) {
 #pragma unroll
     for (int o = 0; o < OUT; ++o)
-      if (o < no)
-        put_out(out[((size_t)l * O + o0 + o) * n + e],
-                RC ? make_double2(a1[o], a2[o]) : make_double2(a1[o] - a2[o], (a3[RC ? 0 : o] - a1[o]) - a2[o]));
+      if (o < no) {
+        VO& at = out[((size_t)l * O + o0 + o) * n + e];
+        const double2 sum =
+            RC ? make_double2(a1[o], a2[o]) : make_double2(a1[o] - a2[o], (a3[RC ? 0 : o] - a1[o]) - a2[o]);
+        const double2 old = add ? to_d2(at) : make_double2(0.0, 0.0);
+        put_out(at, add ? make_double2(old.x + sum.x, old.y + sum.y) : sum);
+      }
   }
 }
 
@@ -2009,10 +2007,10 @@ basis_combine_df_kernel(char* const* __restrict__ tab, long long n, int L, const
     for (int o = 0; o < no; ++o) out[((size_t)l * O + o0 + o) * n + e] = accd[o];
 }
 
-// sources [l0, l0 + nl) of L (all by default); rc: real coefficients
+// sources [l0, l0 + nl) of L (all by default); rc: real coefficients; add: onto out
 template <typename VR, typename VO>
 int launch_combine(char* const* tab, long long n, int L, const double2* C, int O, int S, const int* count, VO* out,
-                   cudaStream_t st, int l0 = 0, int nl = -1, bool rc = false) {
+                   cudaStream_t st, int l0 = 0, int nl = -1, bool rc = false, bool add = false) {
   if (nl < 0) nl = L - l0;
   // outputs a thread accumulates: 16 when there are at least 16 (a
   // 16-moment window reads the residuals once instead of twice, 48
@@ -2025,13 +2023,13 @@ int launch_combine(char* const* tab, long long n, int L, const double2* C, int O
   const int per = (out_per_thread == 16 && O >= 16) ? 16 : kCombOut;
   const dim3 grid((unsigned)((n + kCombThreads - 1) / kCombThreads), nl, (O + per - 1) / per);
   if (per == 16 && rc)
-    basis_combine_kernel<VR, VO, 16, true><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0);
+    basis_combine_kernel<VR, VO, 16, true><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0, add);
   else if (per == 16)
-    basis_combine_kernel<VR, VO, 16, false><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0);
+    basis_combine_kernel<VR, VO, 16, false><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0, add);
   else if (rc)
-    basis_combine_kernel<VR, VO, kCombOut, true><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0);
+    basis_combine_kernel<VR, VO, kCombOut, true><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0, add);
   else
-    basis_combine_kernel<VR, VO, kCombOut, false><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0);
+    basis_combine_kernel<VR, VO, kCombOut, false><<<grid, kCombThreads, 0, st>>>(tab, n, L, C, O, S, count, out, l0, add);
   SS_CHECK_LAUNCH();
   count_launches(1);
   return SSQCD_OK;
@@ -2296,7 +2294,7 @@ class CgRun final : public CgRunBase {
     want_y_ = want_y;
     // the Krylov-basis form: 16-byte seed vectors (FP64 or float-float) and
     // shift vectors of the same type, no reliable updates
-    basis_ = basis_cap > 0.0 && kBasisCapable && reliable_every <= 0;
+    basis_ = basis_cap != 0.0 && kBasisCapable && reliable_every <= 0;
     basis_cap_ = basis_cap;
     basis_state_ = basis_ ? 1 : 0;
     N_ = N;
@@ -2359,7 +2357,7 @@ class CgRun final : public CgRunBase {
 
     SS_TRY(p_.alloc(sizeof(VR) * n * L));
     SS_TRY(q_.alloc(sizeof(VR) * n * L));
-    if (basis_ && want_y_) SS_TRY(alloc_update_vectors());
+    if (basis_ && want_y_) SS_TRY(reserve_solutions());
     if (basis_) {
       // block table (pinned host mirror, written once per entry) and the
       // first two blocks: slot 0 and the first chunk's residuals
@@ -2718,6 +2716,30 @@ class CgRun final : public CgRunBase {
     return SSQCD_OK;
   }
 
+  // Where the solutions are wanted: y and p-hat, and what a segment's end
+  // needs (the coefficients of its slots; the combination on the tensor cores, whose
+  // work space may fail, has the FP64 one behind it), so that a run under way
+  // has no more than blocks to ask for.  A cap that is not the caller's
+  // (basis_cap < 0) then takes half of what is left at most.
+  int reserve_solutions() {
+    SS_TRY(alloc_update_vectors());
+    const bool ours = basis_cap_ < 0.0;
+    basis_cap_ = std::abs(basis_cap_);
+    const int NL = N_ * L_;
+    const double slot = (double)sizeof(VR) * L_ * n_;
+    const double left = ours ? std::min(basis_cap_, 0.5 * (double)available_device_memory()) : basis_cap_;
+    if (left < kSolutionBlocks * kBasisBlock * slot) return fail(SSQCD_ERR_OOM, "stored residuals: no room for them");
+    // slots between two formings of the solutions: what the cap holds, and a block of leeway
+    seg_slots_ = (int)std::min((double)max_iter_ + 1.0, left / slot + kBasisBlock);
+    const size_t coef = sizeof(double2) * (size_t)NL * seg_slots_;
+    SS_TRY(gam_.alloc(coef));
+    SS_TRY(seg_gp_.alloc(coef));
+    SS_TRY(seg_go_.alloc(2 * sizeof(double2) * NL));
+    SS_TRY(count_.alloc(sizeof(int) * L_));
+    basis_cap_ = left;
+    return SSQCD_OK;
+  }
+
   // Blocks for every slot up to kend (and the coefficient records of the
   // iterations before it); at the memory cap, the next segment.
   int ensure_blocks(int kend) {
@@ -2732,7 +2754,7 @@ class CgRun final : public CgRunBase {
         const int st = b->alloc(blk_bytes_);
         if (st != SSQCD_OK) {
           // where the solutions' memory is at hand, no more room is the cap
-          if (!want_y_ || blocks_.size() < 3) return st;
+          if (!want_y_ || blocks_.size() < 2) return st;
           b.reset();
           basis_cap_ = (double)basis_bytes_;
         } else {
@@ -2789,15 +2811,14 @@ class CgRun final : public CgRunBase {
     const int NL = N_ * L_;
     SS_TRY(gam_.alloc(sizeof(double2) * (size_t)NL * basis_S_));
     const bool old = k0_ > 0;
-    DevBuf gp;
-    if (old) SS_TRY(gp.alloc(sizeof(double2) * NL));
+    if (old) SS_TRY(seg_go_.alloc(2 * sizeof(double2) * NL));
     basis_gamma_kernel<<<(NL + kGammaQ - 1) / kGammaQ, kGammaBlock, 0, st_>>>(c_, L_, N_, basis_S_, gam_.as<double2>(), k0_,
-                                                          gp.as<double2>());
+                                                          old ? seg_go_.as<double2>() : nullptr);
     SS_CHECK_LAUNCH();
     count_launches(1);
     if (!old && !want_y_) return SSQCD_OK;
     if constexpr (kBasisCapable) {
-      if (old) SS_TRY(add_old_state(gp.as<double2>(), nullptr));
+      if (old) SS_TRY(add_old_state(seg_go_.as<double2>(), nullptr));
       SS_TRY(combine_solutions(gam_, basis_S_, yv_, old));
     }
     blocks_.clear();
@@ -2831,18 +2852,8 @@ class CgRun final : public CgRunBase {
                                   st_, &suits, add));
         if (suits) return SSQCD_OK;
       }
-      if (add) {
-        DevBuf t;
-        const long long cnt = n_ * N_ * L_;
-        SS_TRY(t.alloc(sizeof(double2) * cnt));
-        SS_TRY((launch_combine<VR, V2>(tab, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), t.as<double2>(), st_)));
-        add_vectors_kernel<<<1216, kUpdBlock, 0, st_>>>(out, t.as<double2>(), cnt);
-        SS_CHECK_LAUNCH();
-        count_launches(1);
-        return SSQCD_OK;
-      }
     }
-    return launch_combine<VR, V2>(tab, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), out, st_);
+    return launch_combine<VR, V2>(tab, n_, L_, g.as<double2>(), N_, S, count_.as<int>(), out, st_, 0, -1, false, add);
   }
 
   // At the memory cap: form y_j and p-hat_j from the segment's residuals.  FP64
@@ -2864,11 +2875,13 @@ class CgRun final : public CgRunBase {
     const bool old = k0_ > 0;
     if (!old && !want_y_) SS_TRY(alloc_update_vectors());
     const int NL = N_ * L_;
-    DevBuf gy, gp, go;
+    // (reserved where the solutions are wanted)
+    DevBuf &gy = gam_, &gp = seg_gp_, &go = seg_go_;
     SS_TRY(gy.alloc(sizeof(double2) * (size_t)NL * S));
     SS_TRY(gp.alloc(sizeof(double2) * (size_t)NL * S));
     if (old) SS_TRY(go.alloc(2 * sizeof(double2) * NL));
-    basis_gamma_kernel<<<(NL + kGammaQ - 1) / kGammaQ, kGammaBlock, 0, st_>>>(c_, L_, N_, S, gy.as<double2>(), k0_, go.as<double2>());
+    basis_gamma_kernel<<<(NL + kGammaQ - 1) / kGammaQ, kGammaBlock, 0, st_>>>(c_, L_, N_, S, gy.as<double2>(), k0_,
+                                                                             old ? go.as<double2>() : nullptr);
     SS_CHECK_LAUNCH();
     basis_phat_kernel<<<(NL + 127) / 128, 128, 0, st_>>>(c_, L_, N_, k, S, gp.as<double2>(), k0_,
                                                          old ? go.as<double2>() + NL : nullptr);
@@ -2898,6 +2911,7 @@ class CgRun final : public CgRunBase {
     SS_CUDA(cudaStreamSynchronize(st_));
     gy.release();
     gp.release();
+    go.release();
     blocks_.clear();
     spare_.clear();
     basis_bytes_ = 0;
@@ -3073,6 +3087,8 @@ class CgRun final : public CgRunBase {
   int k0_ = 0;           // its first iteration
   bool want_y_ = false;  // the solutions, not the stored residuals, are wanted
   DevBuf tab_, gam_, count_;
+  DevBuf seg_gp_, seg_go_;  // a segment's coefficients beside gam_: of p-hat; of the old y and p-hat
+  int seg_slots_ = 0;       // slots that the reserved ones have room for (where the solutions are wanted)
   char** h_tab_ = nullptr;
   bool fix_ = false;  // the integer stencil
   int fix_w_ = 0;
@@ -3142,15 +3158,20 @@ int drive(CgRunBase* run) {
 
 namespace {
 
-// Memory for the stored residuals of a run that wants the solutions, 0 for the
+// Memory for the stored residuals of a run that wants the solutions (negative:
+// by this rule, the run takes half of what is left at most; positive: as the caller
+// set it), 0 for the
 // update form: a twentieth of the time an iteration's update takes goes into
 // the combination per iteration (8^4 x 4, 32 shifts: 102 us against 5), but it
 // has launches and coefficients of its own, ~200 us, that a run of few or short
 // vectors does not earn back.
-double solutions_cap(long long n, int N, int L, int precision) {
-  if (!(precision == SSQCD_FP64 || precision == SSQCD_FP64_DFSHIFT) || !combine_tc_enabled() || N < 4 || (double)n * N * L < 4e5) return 0.0;
-  const double cap = basis_cap_for(SSQCD_FP64, 1, 0.0, n, N, L);
-  return cap >= 12.0 * 16.0 * 16.0 * (double)n * L ? cap : 0.0;  // at least twelve blocks
+double solutions_cap(ssqcd_lattice lat, int N, int L, int precision) {
+  const double n = 12.0 * lat->g.V;
+  if (!(precision == SSQCD_FP64 || precision == SSQCD_FP64_DFSHIFT) || !combine_tc_enabled() || N < 4 ||
+      n * N * L < 4e5 || lat->residual_bytes < 0.0)
+    return 0.0;
+  const double cap = lat->residual_bytes > 0.0 ? lat->residual_bytes : -solve_residual_bytes(n, N, L);
+  return std::abs(cap) >= kSolutionBlocks * 16.0 * 16.0 * n * L ? cap : 0.0;
 }
 
 }  // namespace
@@ -3163,10 +3184,11 @@ int shifted_cg_device(ssqcd_lattice lat, int N, const double2* z_host, int L, co
   // every cap) instead of an update of y and p-hat in every iteration.  The
   // seed is FP64 with float-float shift vectors as well, and the solutions then
   // FP64 throughout.
-  const double cap = solutions_cap(12LL * lat->g.V, N, L, precision);
-  int made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, cap > 0.0 ? SSQCD_FP64 : precision, reliable_every,
-                         cap, lat->stream, &run, cap > 0.0);
-  if (made == SSQCD_ERR_OOM && cap > 0.0)  // the update form needs less
+  const double cap = solutions_cap(lat, N, L, precision);
+  const bool stored = cap != 0.0;
+  int made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, stored ? SSQCD_FP64 : precision, reliable_every,
+                         cap, lat->stream, &run, stored);
+  if (made == SSQCD_ERR_OOM && stored)  // the update form needs less
     made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, precision, reliable_every, 0.0, lat->stream, &run);
   SS_TRY(made);
   const int status = drive(run.get());
@@ -3189,18 +3211,19 @@ int shifted_cg_solve(ssqcd_lattice lat, int N, const double2* z_host, int L, con
   return status;
 }
 
-double basis_cap_for(int precision, int basis, double basis_max_bytes, long long n, int N, int L) {
-  if (basis == 0 || !(precision == SSQCD_FP64 || precision == SSQCD_DF)) return 0.0;
-  if (basis_max_bytes > 0.0) return basis_max_bytes;
+double solve_residual_bytes(double n, int N, int L) {
   // sixteen times the memory of the shift vectors the update form would
   // hold (y and p-hat, 16 B a complex element: 32 N L n bytes), i.e. up to
   // 32 N iterations, and at least 4 GiB; a function of the problem only, so
   // that a solve makes the same choice (and the same arithmetic) wherever it
-  // runs, unless the device has less than twice that free
-  const double cap = std::max(16.0 * 32.0 * (double)n * N * L, 4.0 * (1ull << 30));
-  size_t free_b = 0, total_b = 0;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0.0;
-  return std::min(cap, 0.5 * (double)free_b);
+  // runs, unless the device has less than twice that to give
+  return std::max(16.0 * 32.0 * n * N * L, 4.0 * (1ull << 30));
+}
+
+double basis_cap_for(int precision, int basis, double basis_max_bytes, long long n, int N, int L) {
+  if (basis == 0 || !(precision == SSQCD_FP64 || precision == SSQCD_DF)) return 0.0;
+  if (basis_max_bytes > 0.0) return basis_max_bytes;
+  return std::min(solve_residual_bytes((double)n, N, L), 0.5 * (double)available_device_memory());
 }
 
 void KrylovBasis::release() {

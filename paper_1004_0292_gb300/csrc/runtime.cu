@@ -1,4 +1,5 @@
 // Error reporting, device buffers and launch accounting shared by the library.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstring>
@@ -66,6 +67,44 @@ void keep_pool_memory() {
   (void)cudaGetLastError();
 }
 }  // namespace
+
+namespace {
+bool default_pool(cudaMemPool_t* pool) {
+  int dev = 0;
+  const bool ok = cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(pool, dev) == cudaSuccess;
+  if (!ok) (void)cudaGetLastError();
+  return ok;
+}
+size_t pool_attribute(cudaMemPoolAttr what) {
+  cudaMemPool_t pool;
+  unsigned long long v = 0;
+  if (!default_pool(&pool)) return 0;
+  if (cudaMemPoolGetAttribute(pool, what, &v) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return (size_t)v;
+}
+}  // namespace
+
+size_t pool_bytes() { return pool_attribute(cudaMemPoolAttrReservedMemCurrent); }
+
+size_t available_device_memory() {
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  const size_t held = pool_bytes(), used = pool_attribute(cudaMemPoolAttrUsedMemCurrent);
+  return free_b + (held > used ? held - used : 0);
+}
+
+void trim_pool(size_t keep) {
+  cudaMemPool_t pool;
+  if (!default_pool(&pool)) return;
+  keep = std::max(keep, pool_attribute(cudaMemPoolAttrUsedMemCurrent) + kPoolIdle);
+  if (cudaMemPoolTrimTo(pool, keep) != cudaSuccess) (void)cudaGetLastError();
+}
 
 int DevBuf::alloc(size_t nbytes) {
   if (p && bytes >= nbytes) return SSQCD_OK;
