@@ -3186,7 +3186,8 @@ int shifted_cg_device(ssqcd_lattice lat, int N, const double2* z_host, int L, co
   // FP64 throughout.
   const double cap = solutions_cap(lat, N, L, precision);
   const bool stored = cap != 0.0;
-  int made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, stored ? SSQCD_FP64 : precision, reliable_every,
+  int made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, stored ? SSQCD_FP64 : precision,
+                         stored ? 0 : reliable_every,  // of the mixed precisions only
                          cap, lat->stream, &run, stored);
   if (made == SSQCD_ERR_OOM && stored)  // the update form needs less
     made = make_cg_run(lat, N, z_host, L, v, sigma, tol, max_iter, precision, reliable_every, 0.0, lat->stream, &run);
