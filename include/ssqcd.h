@@ -59,11 +59,15 @@ extern "C" {
 #define SSQCD_FP64_DFSHIFT 4    /* as SSQCD_FP64_SHIFT32 with y and p-hat in
                                    float-float (hi + lo FP32 pair, 48-bit
                                    significand) updated on the FP32 pipes      */
-#define SSQCD_DF           5    /* links, stencil, seed and shift vectors all in
-                                   float-float on the FP32 pipes, and so are
-                                   the Rayleigh-Ritz basis (CGS2), A T and the
-                                   projected matrix; recurrence scalars, moment
-                                   sums, eigenvectors and residuals in FP64    */
+#define SSQCD_DF           5    /* seed and shift vectors in float-float on the
+                                   FP32 pipes, and so are the Rayleigh-Ritz
+                                   basis (CGS2) and the projected matrix; links
+                                   and hops in 60-bit fixed point as in
+                                   ssqcd_apply_H, in float-float for links that
+                                   it does not take; recurrence scalars, moment
+                                   sums (more than eight moments: as FP64 ones,
+                                   see ssqcd_stats.real_moments), eigenvectors
+                                   and residuals in FP64                       */
 
 /* ---- eigenvalue extraction from the moments ---------------------------------- */
 #define SSQCD_EXTRACT_RR     0  /* Rayleigh-Ritz on span(S_hat) (Section 2.1): eigenpairs
@@ -211,7 +215,8 @@ typedef struct {
                              are conjugate and sum to a real number; 0: complex
                              coefficients (circle points, shift-vector updates,
                              or SSQCD_REAL_MOMENTS=0 in the environment).
-                             With real coefficients and FP64 residuals the
+                             With real coefficients and FP64 residuals, or
+                             float-float ones and more than eight moments, the
                              combination runs on the tensor cores: residuals
                              and coefficients are split exactly into seven
                              8-bit fp16 slices on power-of-two grids and the
@@ -253,8 +258,9 @@ int ssqcd_apply_H(ssqcd_lattice lat, const double* in, double* out, int nrhs, in
  * (SSQCD_MIXED) or FP32 (SSQCD_MIXED_F32LINKS) as their first two rows, the
  * third rebuilt as conj(row0 x row1) (exact for SU(3)); spinors and
  * arithmetic in FP32.  Input and output stay complex128 at the boundary.
- * On a SSQCD_DF lattice: links, spinors and arithmetic in float-float
- * (relative error ~1e-14).  Requires a lattice created with one of the two
+ * On a SSQCD_DF lattice: as ssqcd_apply_H where that works in fixed point
+ * (nothing is rounded to float-float), else links, spinors and arithmetic in
+ * float-float (relative error ~1e-14).  Requires a lattice created with one of the two
  * mixed precisions or with SSQCD_DF. */
 int ssqcd_apply_H_mixed(ssqcd_lattice lat, const double* in, double* out, int nrhs, int on_device);
 
@@ -494,8 +500,8 @@ const char* ssqcd_last_error(void);
 
 /* Device time of the stencil alone: `reps` applications of A (after two
  * warm-up applications) to nrhs device-resident fields, in the lattice's
- * precision (SSQCD_FP64 / _FP64_SHIFT32 / _FP64_DFSHIFT: FP64; SSQCD_DF:
- * float-float; the mixed ones: FP32 spinors with their 12-parameter links),
+ * precision (SSQCD_FP64 / _FP64_SHIFT32 / _FP64_DFSHIFT: FP64 fields; SSQCD_DF:
+ * float-float ones; the mixed ones: FP32 spinors with their 12-parameter links),
  * CUDA events on the lattice stream.  *ms_per_call receives the mean time of
  * one application (all nrhs fields). */
 int ssqcd_time_stencil(ssqcd_lattice lat, int nrhs, int reps, double* ms_per_call);
