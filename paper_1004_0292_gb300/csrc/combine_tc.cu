@@ -498,7 +498,9 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
     int d = 0;
     if (o < O && s < cnt) {
       const int g = exp_above(sig[(size_t)lz * OUT + o]) - 1;  // sig = 2^g
-      const double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * padded(S) + s] - g);
+      double b = ldexp(C.get(l, o, s), eslot[(size_t)lz * padded(S) + s] - g);
+      // no share of a vector of zeros, whatever its coefficient (of one that is no number sig tells)
+      if (!(fabs(b) <= 1.0)) b = 0.0;
       if (C.sgn) {
         long long X = llrint(ldexp(b, 56));
         for (int k = 6; k >= q; --k) {

@@ -2867,7 +2867,9 @@ class CgRun final : public CgRunBase {
     // after whole chunks the newest counts are the last entry's
     SS_CUDA(cudaMemcpy(&live, c_.live + L_, sizeof(int), cudaMemcpyDeviceToHost));
     SS_CUDA(cudaMemcpy(&err, c_.err, sizeof(int), cudaMemcpyDeviceToHost));
-    *over = live == 0 || err != 0;  // what is launched now does nothing
+    // what is launched now does nothing, or (the counts being read one iteration
+    // late) one iteration more, whose slot and record are in the last block
+    *over = live == 0 || err != 0;
     if (*over) return SSQCD_OK;
     std::vector<int> it_all, act_all;
     int S = 0;
