@@ -185,6 +185,8 @@ __device__ __forceinline__ double* basis_scale(const Control& c, int k, int NL, 
 size_t basis_block_bytes(size_t vec_bytes, int NL, int L) {
   return vec_bytes + (size_t)2 * kBasisBlock * NL * sizeof(double2) + (size_t)kBasisBlock * L * sizeof(double);
 }
+// blocks the table holds at most: a million iterations, whatever max_iter is
+constexpr size_t kTableBlocks = 1 << 16;
 constexpr int kMaxShifts = 512;   // quadrature points per source
 constexpr int kMaxTotal = 1024;   // (source, point) pairs in one solve
 constexpr int kMaxSources = 64;
@@ -2363,7 +2365,7 @@ class CgRun final : public CgRunBase {
       // first two blocks: slot 0 and the first chunk's residuals
       blk_vec_ = (sizeof(VR) * kBasisBlock * (size_t)L * n + 255) / 256 * 256;
       blk_bytes_ = basis_block_bytes(blk_vec_, NL, L);
-      tab_cap_ = (max_iter + kChunk) / kBasisBlock + 2;
+      tab_cap_ = std::min((size_t)(((long long)max_iter + kChunk) / kBasisBlock + 2), kTableBlocks);
       SS_TRY(tab_.alloc(sizeof(char*) * tab_cap_));
       SS_CUDA(cudaMallocHost(&h_tab_, sizeof(char*) * (tab_cap_ + 2)));  // + the first two slot pointers
       SS_TRY(ensure_blocks(kChunk + 1));
@@ -2716,11 +2718,11 @@ class CgRun final : public CgRunBase {
     return SSQCD_OK;
   }
 
-  // Where the solutions are wanted: y and p-hat, and what a segment's end
-  // needs (the coefficients of its slots; the combination on the tensor cores, whose
-  // work space may fail, has the FP64 one behind it), so that a run under way
-  // has no more than blocks to ask for.  A cap that is not the caller's
-  // (basis_cap < 0) then takes half of what is left at most.
+  // Where the solutions are wanted: y and p-hat at once; what a segment's end
+  // needs, the coefficients of its slots, ahead of the slots (reserve_slots; the
+  // combination on the tensor cores, whose work space may fail, has the FP64 one
+  // behind it), so that a run under way can always form its solutions.  A
+  // cap that is not the caller's (basis_cap < 0) is half of what is left then at most.
   int reserve_solutions() {
     SS_TRY(alloc_update_vectors());
     const bool ours = basis_cap_ < 0.0;
@@ -2729,29 +2731,43 @@ class CgRun final : public CgRunBase {
     const double slot = (double)sizeof(VR) * L_ * n_;
     const double left = ours ? std::min(basis_cap_, 0.5 * (double)available_device_memory()) : basis_cap_;
     if (left < kSolutionBlocks * kBasisBlock * slot) return fail(SSQCD_ERR_OOM, "stored residuals: no room for them");
-    // slots between two formings of the solutions: what the cap holds, and a block of leeway
-    seg_slots_ = (int)std::min((double)max_iter_ + 1.0, left / slot + kBasisBlock);
-    const size_t coef = sizeof(double2) * (size_t)NL * seg_slots_;
-    SS_TRY(gam_.alloc(coef));
-    SS_TRY(seg_gp_.alloc(coef));
     SS_TRY(seg_go_.alloc(2 * sizeof(double2) * NL));
     SS_TRY(count_.alloc(sizeof(int) * L_));
     basis_cap_ = left;
+    return reserve_slots(2 * kBasisBlock);
+  }
+
+  // Room for the coefficients of a segment of so many slots; what is there
+  // stays where there is none.
+  int reserve_slots(int slots) {
+    if (slots <= seg_slots_) return SSQCD_OK;
+    DevBuf g, p;
+    const size_t bytes = sizeof(double2) * (size_t)N_ * L_ * slots;
+    SS_TRY(g.alloc(bytes));
+    SS_TRY(p.alloc(bytes));
+    gam_.swap(g);
+    seg_gp_.swap(p);
+    seg_slots_ = slots;
     return SSQCD_OK;
   }
+  size_t coef_bytes(int slots) const { return want_y_ ? 2 * sizeof(double2) * (size_t)N_ * L_ * slots : 0; }
 
   // Blocks for every slot up to kend (and the coefficient records of the
   // iterations before it); at the memory cap, the next segment.
   int ensure_blocks(int kend) {
     while (basis_ && blocks_.size() < (size_t)(kend >> kBasisLog) + 1 - blk0_) {
-      if (blk0_ + blocks_.size() >= tab_cap_) return fail(SSQCD_ERR_ARG, "stored residuals: block table full");
       std::unique_ptr<DevBuf> b;
-      if (!spare_.empty()) {
+      const bool full = blk0_ + blocks_.size() >= tab_cap_;
+      // the slots with this block, and room for their coefficients twice as fast
+      const int slots = (int)(blocks_.size() + 1) * kBasisBlock, room = slots <= seg_slots_ ? seg_slots_ : 2 * slots;
+      if (full) {
+      } else if (!spare_.empty()) {
         b = std::move(spare_.back());
         spare_.pop_back();
-      } else if ((double)(basis_bytes_ + blk_bytes_) <= basis_cap_ || blocks_.size() < 2) {
+      } else if ((double)(basis_bytes_ + blk_bytes_ + coef_bytes(room)) <= basis_cap_ || blocks_.size() < 2) {
         b = std::make_unique<DevBuf>();
-        const int st = b->alloc(blk_bytes_);
+        int st = want_y_ ? reserve_slots(room) : SSQCD_OK;
+        if (st == SSQCD_OK) st = b->alloc(blk_bytes_);
         if (st != SSQCD_OK) {
           // where the solutions' memory is at hand, no more room is the cap
           if (!want_y_ || blocks_.size() < 2) return st;
@@ -2764,7 +2780,7 @@ class CgRun final : public CgRunBase {
       }
       if (b == nullptr) {
         bool over = false;
-        SS_TRY(next_segment(&over));
+        SS_TRY(next_segment(&over, full));
         if (over) return SSQCD_OK;
         continue;
       }
@@ -2859,8 +2875,9 @@ class CgRun final : public CgRunBase {
   // At the memory cap: form y_j and p-hat_j from the segment's residuals.  FP64
   // runs then begin the next segment with the blocks they have, r_k where it
   // is; float-float ones free the blocks and continue with the per-iteration
-  // updates (new chunk graphs).  *over: no shift is live any more.
-  int next_segment(bool* over) {
+  // updates (new chunk graphs), and so do those that fill the block table
+  // (updates).  *over: no shift is live any more.
+  int next_segment(bool* over, bool updates = false) {
     SS_CUDA(cudaStreamSynchronize(st_));
     int k = 0, live = 0, err = 0;
     SS_CUDA(cudaMemcpy(&k, c_.seed_iters, sizeof(int), cudaMemcpyDeviceToHost));
@@ -2899,7 +2916,7 @@ class CgRun final : public CgRunBase {
     // end and r_k the first slot of its block.  Segments of 128 iterations and
     // more: a segment's combinations read its residuals 4 N L / 16 times.
     const size_t keep = (size_t)(k >> kBasisLog) - blk0_;
-    if (std::is_same<V2, double2>::value && k % kBasisBlock == 0 && keep >= 8) {
+    if (std::is_same<V2, double2>::value && k % kBasisBlock == 0 && keep >= 8 && !updates) {
       std::vector<std::unique_ptr<DevBuf>> rest;
       for (size_t i = 0; i < blocks_.size(); ++i) (i < keep ? spare_ : rest).push_back(std::move(blocks_[i]));
       blocks_.swap(rest);
@@ -3090,7 +3107,7 @@ class CgRun final : public CgRunBase {
   bool want_y_ = false;  // the solutions, not the stored residuals, are wanted
   DevBuf tab_, gam_, count_;
   DevBuf seg_gp_, seg_go_;  // a segment's coefficients beside gam_: of p-hat; of the old y and p-hat
-  int seg_slots_ = 0;       // slots that the reserved ones have room for (where the solutions are wanted)
+  int seg_slots_ = 0;       // slots that they have room for (where the solutions are wanted)
   char** h_tab_ = nullptr;
   bool fix_ = false;  // the integer stencil
   int fix_w_ = 0;
