@@ -27,7 +27,7 @@ solves an independent replica (its own sources): the path has no data
 exchange, so scaling is weak and there is no collective on the data path.
 
 ``mixed`` reports the same metric on the same workload for the solve
-precision SSQCD_DF (float-float links, stencil, seed vectors, stored
+precision SSQCD_DF (float-float seed vectors, stored
 residuals and the Rayleigh-Ritz basis on the FP32 pipes; FP64 recurrence
 scalars, eigenvectors and residuals), with
 its ratio to the plain FP64 value.  ``mixed_fp32_fp16`` records the FP32
@@ -98,9 +98,10 @@ STENCIL_FLOP_PER_SITE = 1368
 # link-times-spin-row products; the wide multiply-add runs at 32 lanes a clock and SM.
 STENCIL_MADS_PER_SITE = 8 * 2 * 9 * 4 * 3
 WIDE_MAD_PEAK = 152 * 32 * 2.07e9 / 1e12
-# DRAM traffic of one launch of that kernel (1 rhs, 16^3 x 32) from an ncu capture;
-# None until captured for the current kernel.
-STENCIL_FP64_TRAFFIC = None
+# DRAM traffic of one launch of that kernel (1 rhs, 16^3 x 32) from an ncu capture
+# (dram__bytes_read.sum + dram__bytes_write.sum,
+# profiles/stencil_integer_fp64_16x16x16x32.md); None once the kernel changes.
+STENCIL_FP64_TRAFFIC = 132803584.0 + 12933120.0
 # DRAM traffic of one launch of each update kernel with all 128 (source,
 # shift) pairs live on this workload (ncu dram__bytes_read.sum +
 # dram__bytes_write.sum, one capture per kernel; the algorithmic bytes of such
@@ -355,7 +356,7 @@ def run_ours(args):
         e2e = {"value": float(sum(e2e_pairs) / sum(e2e_times)), "unit": UNIT,
                "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h)}
 
-    # ---- mixed arm: float-float links, stencil, seed vectors and stored residuals (SSQCD_DF) ----
+    # ---- mixed arm: float-float seed vectors and stored residuals (SSQCD_DF) ----
     mixed = None
     if not args.no_mixed:
         lat_m = ss.create_lattice(w["dims"], w["kappa"], w["bc_t"], precision=ss.DF, stream=stream)
@@ -379,9 +380,9 @@ def run_ours(args):
         value_m = pairs_m / (ms_m / 1e3)
         it_m = max(1, sum(x["launches_update"] for x in s_m))
         mixed = {
-            "precision": "SSQCD_DF: float-float (FP32 pair, 48-bit significand) links, stencil, seed vectors and "
-                         "stored residuals, and the Rayleigh-Ritz basis and products, on the FP32 pipes; FP64 "
-                         "recurrence scalars, eigenvectors and residuals",
+            "precision": "SSQCD_DF: float-float (FP32 pair, 48-bit significand) seed vectors and stored residuals, and "
+                         "the Rayleigh-Ritz basis and products, on the FP32 pipes; links and hops in 60-bit fixed point; "
+                         "FP64 recurrence scalars, eigenvectors and residuals",
             "value": value_m, "unit": UNIT, "ms_per_step": ms_m / args.steps,
             "vs_plain_fp64": value_m / value, "eigenpairs_per_step": c_m[-1],
             "max_accepted_residual": r_m[-1], "iterations_per_step": p_m[-1]["iterations"],
@@ -453,8 +454,8 @@ def run_ours(args):
                 "bound": "alu", "achieved": sten_mads, "peak": WIDE_MAD_PEAK,
                 "unit": "T 32 x 32 + 64-bit integer multiply-adds/s",
                 "frac": sten_mads / WIDE_MAD_PEAK if sten_mads else None, "traffic": STENCIL_FP64_TRAFFIC,
-                "traffic_note": "no capture of this kernel on this workload; algorithmic 192 + 192 B of digits and p in, "
-                                "192 out, 576 of links a site = 151 MB",
+                "traffic_note": "one launch; algorithmic 192 + 192 B of digits and p in, 192 out, 576 of links a site = "
+                                "151 MB",
                 "peak_source": "derived: 152 SMs x 32 lanes/clk (measured by a probe) x 2.07 GHz (no integer entry in "
                                "MEASURED_PEAKS.json)",
                 "op_count": "1728 a site and rhs: 8 hops x 18 complex products x 4 real ones x 3 digit products",

@@ -44,7 +44,7 @@
 // behind a dependent load of the block table (3200 cycles a K-step), the epilogue
 // converted to 64-bit integers on the FP64 pipe, and a digit took twice the
 // integer operations.  Those of the slicing warps (~20 an element, the integer
-// pipe 69% busy) and the scale pass bound it now.
+// pipe 58% busy) and the scale pass bound it now.
 //
 // One persistent CTA per SM (26 warps; wide form 28):
 // * warp 25: bulk copies (cp.async.bulk, a lane a slot) of a tile's 16 slots x
@@ -528,7 +528,7 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
 // on a list (tc_witness_kernel) and take the FP64 sum behind the pass
 // (tc_rest_kernel); more of them than the list holds, and the vectors do not suit.
 // Dense vectors have next to none, and their elements show it by the one to
-// six slots where an output's coefficient is largest: 45 us more for the 16^3 x 32 moments' 1.16 ms.
+// six slots where an output's coefficient is largest: 40 us of the 16^3 x 32 moments' 1.07 ms.
 constexpr int kCoefBits = 3, kVecBits = 7;
 constexpr int kMaxPass = kWideOut / 2;  // complex outputs a pass
 struct Components {

@@ -156,13 +156,13 @@ int wilson64(const Geometry& g, const double2* u, const double2* in, double2* ou
 int wilson64_lat(ssqcd_lattice lat, const double2* in, bool user, double2* out, int nrhs, cudaStream_t s,
                  void* work = nullptr);
 int wilson_df_lat(ssqcd_lattice lat, const float4* in, float4* out, int nrhs, cudaStream_t s);  // float-float fields
-// Integer stencil (wilson_fix.cu): fields as digits with one exponent a site,
-// bytes of each for one field; the links take three fields' bytes
+// Integer stencil (wilson_fix.cu): fields as digits with one word (exponent, spins
+// that are not zero) a site, bytes of each for one field; the links take three fields' bytes
 size_t fix_field_bytes(int V);
 size_t fix_exp_bytes(int V);
 int pack_fix(const double2* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
 int pack_fix(const float4* in, int nrhs, int V, int4* dig, int* ex, cudaStream_t s);
-int fix_split(int V, int nrhs);  // warps that share the hops of 16 sites: 1, 4 or 8
+int fix_split(int V, int nrhs);  // warps that share the hops of 16 sites: 1 or 4
 int fix_block(int V, int nrhs);  // right-hand sides converted at a time
 // A work space of the lattice with at least `bytes`: one that an earlier call
 // gave back, or a new one.  give_workspace takes it back once its stream has
