@@ -522,17 +522,21 @@ __global__ void tc_bslices_kernel(CoefView C, int O, int S, int l0, const int* _
 // ---- components far below their vectors' largest ---------------------------------------------
 // The roundings of an output are relative to its scale, sig: at most S 2^-53 sig,
 // ~sqrt(S) 2^-57 in the root mean square.  A part (real or imaginary) of an output element
-// one of whose terms is at least 2^-(kCoefBits + kVecBits + 1) sig is served by
-// that: such a term is a coefficient within kCoefBits binades of its output's scale times a component
-// within kVecBits of its vector's.  The elements with a part that has terms, but none such, go
-// on a list (tc_witness_kernel) and take the FP64 sum behind the pass
-// (tc_rest_kernel); more of them than the list holds, and the vectors do not suit.
-// Dense vectors have next to none, and their elements show it by the one to
-// six slots where an output's coefficient is largest: 40 us of the 16^3 x 32 moments' 1.07 ms.
-constexpr int kCoefBits = 3, kVecBits = 7;
+// one of whose terms is at least 2^-kTermBits sig is served by that.  The elements with a
+// part that has terms, but none such, go on a list (tc_witness_kernel) and take the FP64
+// sum behind the pass (tc_rest_kernel); more of them than the list holds, and the
+// vectors do not suit.  Dense vectors have next to none, and their elements show it
+// by the one to six slots where an output's coefficient is largest: 35 us of the 16^3 x 32
+// moments' 1.07 ms.
+constexpr int kTermBits = 11;
 constexpr int kMaxPass = kWideOut / 2;  // complex outputs a pass
+// Words a slot: word d - 1 for components within d binades of the vector's scale,
+// the outputs (bits, the real parts of coefficients below, the imaginary ones above)
+// whose coefficients make a large term with them; the last but one the coefficients
+// that are not zero.
+constexpr int kLevels = kTermBits - 1, kMaskWords = kLevels + 2;
 struct Components {
-  uint4* mask;                  // [l][slot] bits of the pass's outputs: re and im of the coefficient large, not zero
+  unsigned* mask;               // [l][slot][kMaskWords]
   unsigned long long* largest;  // [l][kMaxPass] coefficient (as float bits) and slot of the largest, per output
   long long* list;              // l' n + element
   unsigned* count;
@@ -547,12 +551,14 @@ __global__ void tc_masks_kernel(CoefView C, int O, int S, int stride, const unsi
     const double2 c = C.c[lz * C.sl + o * C.so + s * C.ss];
     const int d = eslot[(size_t)lz * padded(S) + s] - (exp_above(sig[(size_t)lz * stride + 2 * o]) - 1);
     const double re = fabs(ldexp(c.x, d)), im = fabs(ldexp(c.y, d));
-    uint4* m = k.mask + (size_t)lz * S + s;
-    const unsigned bit = 1u << o;
-    if (re >= ldexp(1.0, -kCoefBits)) atomicOr(&m->x, bit);
-    if (im >= ldexp(1.0, -kCoefBits)) atomicOr(&m->y, bit);
-    if (c.x != 0.0) atomicOr(&m->z, bit);
-    if (c.y != 0.0) atomicOr(&m->w, bit);
+    unsigned* m = k.mask + ((size_t)lz * S + s) * kMaskWords;
+    const unsigned br = 1u << o, bi = 0x10000u << o;
+    for (int v = 1; v <= kLevels; ++v) {
+      const double least = ldexp(1.0, v - kTermBits);
+      const unsigned bits = (re >= least ? br : 0) | (im >= least ? bi : 0);
+      if (bits != 0) atomicOr(m + v - 1, bits);
+    }
+    atomicOr(m + kLevels, (c.x != 0.0 ? br : 0) | (c.y != 0.0 ? bi : 0));
     atomicMax(k.largest + lz * kMaxPass + o,
               (unsigned long long)__float_as_uint((float)fmax(re, im)) << 32 | (unsigned)s);
   }
@@ -585,15 +591,17 @@ tc_witness_kernel(SlotMap map, long long n, int l0, int O, int S, const int* __r
     unsigned fr = 0, fi = 0, nr = 0, ni = 0;  // outputs whose real, imaginary part has a large term, a term
     auto at = [&](int s) { return __ldg(reinterpret_cast<const uint4*>(slot_ptr(map, n, l0 + lz, s)) + e); };
     auto visit = [&](uint4 x, int s) {
-      const uint4 m = __ldg(k.mask + (size_t)lz * S + s);
-      const int low = __ldg(eslot + (size_t)lz * padded(S) + s) + 1023 - kVecBits;
-      const bool br = (int)(x.y >> 20 & 0x7FF) >= low, bi = (int)(x.w >> 20 & 0x7FF) >= low;
-      const bool zr = (x.y << 1 | x.x) != 0, zi = (x.w << 1 | x.z) != 0;
-      fr |= (br ? m.x : 0) | (bi ? m.y : 0);
-      fi |= (bi ? m.x : 0) | (br ? m.y : 0);
-      nr |= (zr ? m.z : 0) | (zi ? m.w : 0);
-      ni |= (zi ? m.z : 0) | (zr ? m.w : 0);
-      return (fr & fi) == all;
+      const unsigned* m = k.mask + ((size_t)lz * S + s) * kMaskWords;
+      const int top = __ldg(eslot + (size_t)lz * padded(S) + s) + 1023;
+      // binades below the scale, at least one; past the levels: none
+      const unsigned dr = (unsigned)(top - (int)(x.y >> 20 & 0x7FF)) - 1, di = (unsigned)(top - (int)(x.w >> 20 & 0x7FF)) - 1;
+      const unsigned mr = dr < kLevels ? __ldg(m + dr) : 0, mi = di < kLevels ? __ldg(m + di) : 0, nz = __ldg(m + kLevels);
+      const unsigned zr = (x.y << 1 | x.x) != 0 ? nz : 0, zi = (x.w << 1 | x.z) != 0 ? nz : 0;
+      fr |= mr | mi >> 16;
+      fi |= mi | mr >> 16;
+      nr |= zr | zi >> 16;
+      ni |= zi | zr >> 16;
+      return (fr & fi & all) == all;
     };
     bool ok = false;
     for (int o = 0; o < slots && !ok; o += 4) {
@@ -604,7 +612,7 @@ tc_witness_kernel(SlotMap map, long long n, int l0, int O, int S, const int* __r
       for (int i = 0; i < 4; ++i) ok = visit(x[i], s_slot[min(o + i, slots - 1)]);
     }
     for (int s = 0; s < S && !ok; ++s) ok = visit(at(s), s);
-    if (!ok && ((nr & ~fr) | (ni & ~fi)) != 0) {
+    if (!ok && (((nr & ~fr) | (ni & ~fi)) & all) != 0) {
       const unsigned place = atomicAdd(k.count, 1u);
       if (place < k.cap)
         k.list[place] = (long long)lz * n + e;
@@ -613,31 +621,25 @@ tc_witness_kernel(SlotMap map, long long n, int l0, int O, int S, const int* __r
     }
   }
 }
-// the listed elements' outputs in FP64: a warp an element, its lanes the slots
+// The listed elements' outputs in FP64, a thread each: the outputs of an element
+// side by side read its components together.
 __global__ void __launch_bounds__(256)
 tc_rest_kernel(SlotMap map, long long n, int l0, CoefView C, int O, int S, Components k, long long out_l,
                double2* __restrict__ out, const int* __restrict__ err) {
   if ((*err & kErrSpread) != 0) return;
-  const int lane = threadIdx.x & 31;
-  const unsigned cnt = min(*k.count, k.cap);
-  for (unsigned i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < cnt; i += gridDim.x * (blockDim.x >> 5)) {
-    const int lz = (int)(k.list[i] / n), l = l0 + lz;
-    const long long e = k.list[i] % n;
-    for (int o = 0; o < O; ++o) {
-      double re = 0.0, im = 0.0;
-      for (int s = lane; s < S; s += 32) {
-        const double2 x = reinterpret_cast<const double2*>(slot_ptr(map, n, l, s))[e];
-        const double2 c = C.c[lz * C.sl + o * C.so + s * C.ss];
-        re = fma(c.x, x.x, fma(-c.y, x.y, re));
-        im = fma(c.x, x.y, fma(c.y, x.x, im));
-      }
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, d);
-        im += __shfl_xor_sync(0xffffffffu, im, d);
-      }
-      if (lane == 0) out[l * out_l + (long long)o * n + e] = make_double2(re, im);
+  const long long work = (long long)min(*k.count, k.cap) * O;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < work; t += (long long)gridDim.x * blockDim.x) {
+    const long long at = k.list[t / O], e = at % n;
+    const int o = (int)(t % O), lz = (int)(at / n), l = l0 + lz;
+    const double2* c = C.c + lz * C.sl + o * C.so;
+    double re = 0.0, im = 0.0;
+#pragma unroll 4
+    for (int s = 0; s < S; ++s) {
+      const double2 x = __ldg(reinterpret_cast<const double2*>(slot_ptr(map, n, l, s)) + e), w = c[s * C.ss];
+      re = fma(w.x, x.x, fma(-w.y, x.y, re));
+      im = fma(w.x, x.y, fma(w.y, x.x, im));
     }
+    out[l * out_l + (long long)o * n + e] = make_double2(re, im);
   }
 }
 
@@ -1075,13 +1077,14 @@ bool combine_tc_applicable(long long n, int O, int S) {
 }
 
 namespace {
-// elements that the list of tc_witness_kernel holds: a 64th of all, whose FP64
-// sums take a few percent of all elements'
+// Elements that the list of tc_witness_kernel holds: a 64th of all, whose FP64
+// sums cost a few percent of everyone's.  (Where one slot has an output's only
+// large coefficient, 1.3% of a Gaussian vector's elements are on it.)
 unsigned rest_cap(long long n, int nl) { return (unsigned)std::min(n * nl / 64 + 64, 1LL << 28); }
 }  // namespace
 
 size_t combine_tc_vectors_work_bytes(long long n, int nl, int S) {
-  return combine_tc_work_bytes(nl, S) + align256(sizeof(uint4) * (size_t)nl * S) +
+  return combine_tc_work_bytes(nl, S) + align256(sizeof(unsigned) * kMaskWords * (size_t)nl * S) +
          align256(sizeof(unsigned long long) * (size_t)nl * kMaxPass) + 256 +
          sizeof(long long) * (size_t)rest_cap(n, nl);
 }
@@ -1189,7 +1192,7 @@ int combine_all(const SlotMap& map, long long n, CoefView C, int O, int S, const
     SS_CHECK_LAUNCH();
     count_launches(3);
     if (comps != nullptr) {
-      tc_rest_kernel<<<4 * sms, 256, 0, st>>>(map, n, l0, Cp, Op / 2, S, *comps, out_l, out + (long long)o0 * n,
+      tc_rest_kernel<<<8 * sms, 256, 0, st>>>(map, n, l0, Cp, Op / 2, S, *comps, out_l, out + (long long)o0 * n,
                                              w.err);
       SS_CHECK_LAUNCH();
       count_launches(1);
@@ -1225,8 +1228,8 @@ int combine_tc_vectors(const double2* x, int S, long long n, const double2* C, i
   if (O < 1 || nl < 1 || !combine_tc_applicable(n, 1, S)) return fail(SSQCD_ERR_ARG, "combine_tc: shape not supported");
   Components k;
   char* p = static_cast<char*>(work) + combine_tc_work_bytes(nl, S);
-  k.mask = reinterpret_cast<uint4*>(p);
-  p += align256(sizeof(uint4) * (size_t)nl * S);
+  k.mask = reinterpret_cast<unsigned*>(p);
+  p += align256(sizeof(unsigned) * kMaskWords * (size_t)nl * S);
   k.largest = reinterpret_cast<unsigned long long*>(p);
   p += align256(sizeof(unsigned long long) * (size_t)nl * kMaxPass);
   k.count = reinterpret_cast<unsigned*>(p);  // cleared with the two before it
