@@ -626,6 +626,11 @@ namespace {
 // four launches and the read of its error word take ~40 us, what the FP64 pipe
 // (four operations a term, 152 x 2 a clock) does for six million terms.
 constexpr double kTcCombineTerms = 8e6;
+// And vectors times outputs of a pass (8 to 16 of them: fewer cost the FP64 kernel as
+// much) that a pass needs to pay, as it costs what sixteen vectors do however few there
+// are.  16^3 x 32, tensor cores against FP64 pipe: 1 vector x 64 outputs 3.2 ms, 0.89; 4
+// x 16 1.00, 0.87; 5 x 16 1.08, 1.03; 6 x 16 1.00, 1.20; 8 x 8 0.84, 0.87; 12 x 8 0.80, 1.20.
+constexpr int kTcCombinePass = 96;
 
 int combine_fp64(const double2* S, int ms, long long n, const double2* C, int mc, double2* Q, cudaStream_t s) {
   const int cy = (mc + kCC - 1) / kCC;
@@ -658,7 +663,8 @@ int combine(const double2* S, int ms, long long n, const double2* C, int mc, dou
       SS_TRY(combine(S + (long long)l * ms * n, ms, n, C, mc, Q + (long long)l * mc * n, s, std::min(kBlocks, nl - l)));
     return SSQCD_OK;
   }
-  if (combine_tc_enabled() && combine_tc_applicable(n, 1, ms) && (double)nl * ms * mc * (double)n >= kTcCombineTerms) {
+  if (combine_tc_enabled() && combine_tc_applicable(n, 1, ms) && (double)nl * ms * mc * (double)n >= kTcCombineTerms &&
+      ms * std::clamp(mc, 8, 16) >= kTcCombinePass) {
     DevBuf work;
     if (work.alloc(combine_tc_vectors_work_bytes(n, nl, ms)) == SSQCD_OK) {
       bool suits = false;
