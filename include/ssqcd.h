@@ -49,7 +49,10 @@ extern "C" {
 #define SSQCD_ERR_CUDA      5  /* a CUDA runtime call failed                     */
 
 /* ---- precision of the solve loop ------------------------------------------ */
-#define SSQCD_FP64  0  /* everything in FP64 ("plain")                          */
+#define SSQCD_FP64  0  /* FP64 ("plain"); the hops of the loop in 60-bit fixed
+                          point relative to the largest component of a site and its
+                          neighbours where the links suit it (ssqcd_apply_H),
+                          which in a vector's norm is no coarser              */
 #define SSQCD_MIXED 1  /* FP32 stencil + shift updates with FP16 12-parameter
                           links, FP64 reliable updates of the seed residual,
                           FP64 moments and Rayleigh-Ritz                       */
