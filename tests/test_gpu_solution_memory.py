@@ -110,3 +110,28 @@ def test_memory_given_back(ss):
     torch.cuda.synchronize()
     left = free - torch.cuda.mem_get_info()[0]
     assert left <= y.nbytes + (4 << 30) + (600 << 20)  # the links' digits and work spaces among them
+
+
+def test_segments_of_residuals_that_keep_the_fp64_sum(ss):
+    # diagonal links keep the colours apart: a source of one colour leaves zeros
+    # in every residual, so that each segment's FP64 sum is added to the last one's
+    import torch
+    L, N = 2, 8
+    lat = ss.create_lattice(DIMS, 0.15, -1)
+    phases = synthetic.rng(8).uniform(-1.0, 1.0, (4, synthetic.volume(DIMS), 3))
+    ss.upload_gauge(lat, np.exp(1j * phases)[..., None] * np.eye(3))
+    v = synthetic.gaussian_sources(DIMS, L, seed=6)
+    v[:, :, :, 1:] = 0.0
+    v = torch.from_numpy(v).cuda()
+    z = 0.01 + 0.002 * np.arange(N) + 0.002j * (-1.0) ** np.arange(N)
+    ss.set_residual_bytes(lat, -1)
+    code, ref, iters, _, it = ss.shifted_cg(lat, z, v, tol=TOL)
+    assert code == ss.OK and it > 300  # two segments
+    block = 16 * 16 * 12 * synthetic.volume(DIMS) * L
+    for nbytes in (13 * block, 200 * block):
+        ss.set_residual_bytes(lat, nbytes)
+        code, y, iters2, _, _ = ss.shifted_cg(lat, z, v, tol=TOL)
+        assert code == ss.OK
+        assert bool((y[..., 1:] == 0).all())
+        assert int((iters2 - iters).abs().max()) <= 0.02 * it + 2
+        assert _close(y, ref, v, z)
